@@ -20,13 +20,13 @@ constexpr size_t kCacheCap = 1024;
 int plan_free(b200sp_plan* p, bool stream_ordered = false, cudaStream_t stream = nullptr) {
   if (!p) return B200SP_OK;
   int rc = B200SP_OK;
-  if (p->block || p->cuts_block || p->compact_block || p->flat_tile_row || p->quad_block) {
+  if (p->block || p->cuts_block || p->compact_block || p->spmm_split || p->quad_block) {
     cudaError_t e = cudaSuccess;
     if (stream_ordered) {
       if (p->block) e = cudaFreeAsync(p->block, stream);
       if (p->cuts_block && e == cudaSuccess) e = cudaFreeAsync(p->cuts_block, stream);
       if (p->compact_block && e == cudaSuccess) e = cudaFreeAsync(p->compact_block, stream);
-      if (p->flat_tile_row && e == cudaSuccess) e = cudaFreeAsync(p->flat_tile_row, stream);
+      if (p->spmm_split && e == cudaSuccess) e = cudaFreeAsync(p->spmm_split, stream);
       if (p->quad_block && e == cudaSuccess) e = cudaFreeAsync(p->quad_block, stream);
     } else {
       int cur = 0;
@@ -36,7 +36,7 @@ int plan_free(b200sp_plan* p, bool stream_ordered = false, cudaStream_t stream =
       if (e == cudaSuccess && p->block) e = cudaFree(p->block);
       if (e == cudaSuccess && p->cuts_block) e = cudaFree(p->cuts_block);
       if (e == cudaSuccess && p->compact_block) e = cudaFree(p->compact_block);
-      if (e == cudaSuccess && p->flat_tile_row) e = cudaFree(p->flat_tile_row);
+      if (e == cudaSuccess && p->spmm_split) e = cudaFree(p->spmm_split);
       if (e == cudaSuccess && p->quad_block) e = cudaFree(p->quad_block);
       if (cur != p->device) cudaSetDevice(cur);
     }
@@ -47,7 +47,7 @@ int plan_free(b200sp_plan* p, bool stream_ordered = false, cudaStream_t stream =
 }
 
 // The list of the rows that have nonzeros (their numbers and their offsets), built on the device in stream order and kept with
-// the plan: used by the merge-tile SpMV kernel under the switch "merge_empty" and by the nnz-balanced SpMM kernel.  Needs
+// the plan: used by the merge-tile SpMV kernel under the switch "merge_empty".  Needs
 // info.bin_rows[0] (the number of empty rows).  No synchronisation.
 int plan_compact_rows(b200sp_plan* p, cudaStream_t stream, DeviceInfo* dev) {
   if (p->compact_block) return B200SP_OK;

@@ -248,7 +248,8 @@ struct b200sp_plan {
   unsigned long long* probe_out = nullptr;  // two counters for the column-locality probe
   int num_medium = 0, num_long = 0;
   const void* probed_col_idx = nullptr;   // col_idx the column-locality probe last ran on
-  int32_t* flat_tile_row = nullptr;       // tile starts of the nnz-balanced SpMM kernel (a pool block of its own, built on first use)
+  int32_t* spmm_split = nullptr;          // warp shares of the nnz-balanced SpMM kernel (a pool block of its own, built on first use)
+  int spmm_witems = 0, spmm_shares = 0;   // merge items per share, consecutive shares per warp
   // merge list over the rows that have nonzeros (matrices with many empty rows)
   void* compact_block = nullptr;          // one pool block: row ids, their offsets, block counts
   int compact_rows = 0;                   // number of rows that have nonzeros (0 = the list has not been built)

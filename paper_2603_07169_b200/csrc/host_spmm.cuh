@@ -4,6 +4,7 @@
 #include "host_spmv.cuh"
 #include "spmm_kernels.cuh"
 #include "spmm_bstage_kernels.cuh"
+#include "spmm_merge_kernels.cuh"
 #include "format_kernels.cuh"
 
 namespace {
@@ -297,10 +298,6 @@ int spmm_column_ranges(b200sp_plan* p, const int32_t* col_idx, int slice_bytes, 
   return B200SP_OK;
 }
 
-// nnz-balanced SpMM (spmm_flat_kernel) for matrices whose rows are too uneven for one lane group per row.
-constexpr int kFlatChunk = 32;                          // nonzeros per lane group
-constexpr int kFlatTile = (kSpmmThreads / 8) * kFlatChunk;   // nonzeros per CTA
-
 bool spmm_rows_are_uneven(const b200sp_plan_info_t& I) {
   if (I.nnz <= 0 || I.m <= 0) return false;
   const int64_t nonempty = I.m - I.bin_rows[0];
@@ -310,55 +307,69 @@ bool spmm_rows_are_uneven(const b200sp_plan_info_t& I) {
          || (double)I.max_row_len > 4.0 * mean + 8.0;       // or the longest row is far above the mean
 }
 
-template <typename T, int VEC>
-int run_spmm_flat(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
-                  cudaStream_t stream, DeviceInfo* dev) {
+template <typename T, int V, int J>
+int launch_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
+                      cudaStream_t stream, DeviceInfo* dev) {
   const b200sp_plan_info_t& I = p->info;
-  constexpr int KS = 8 * VEC;
-  const int tiles = (int)((I.nnz + kFlatTile - 1) / kFlatTile);
+  constexpr int KS = 32 * V * J;
+  const int witems = p->spmm_witems, shares = p->spmm_shares;
+  const long long per_tile = (long long)witems * shares * kMergeWarps;
+  const int tiles = (int)((I.m + I.nnz + per_tile - 1) / per_tile);
   const int slices = (k + KS - 1) / KS;
   if ((long long)slices * tiles >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
-  int rc;
-  if (I.bin_rows[0] > 0) {   // the rows that have nonzeros, listed once per plan (stream order, no synchronisation)
-    rc = plan_compact_rows(p, stream, dev);
-    if (rc != B200SP_OK) return rc;
-  }
-  const int rows = I.bin_rows[0] > 0 ? p->compact_rows : (int)I.m;
-  const int* rp = I.bin_rows[0] > 0 ? p->compact_row_ptr : p->row_ptr;
-  const int* rid = I.bin_rows[0] > 0 ? p->compact_row_id : nullptr;
-  if (!p->flat_tile_row) {   // tile starts: once per plan, a small kernel in stream order
-    rc = pool_alloc(dev, (void**)&p->flat_tile_row, (size_t)(tiles + 1) * sizeof(int32_t), stream);
-    if (rc != B200SP_OK) return rc;
-    rc = launch(plan_nnz_tile_rows_kernel, dim3((unsigned)((tiles + 1 + 255) / 256)), dim3(256), stream, nullptr, 0, dev, rp, rows,
-                (int)I.nnz, kFlatTile, tiles, (int*)p->flat_tile_row);
-    if (rc != B200SP_OK) return rc;
-  }
   // per-call scratch: what each tile leaves unfinished and what it finishes for an earlier tile, KS floats per (slice, tile)
   float* scratch = nullptr;
   const size_t per = (size_t)slices * tiles * KS;
-  rc = pool_alloc(dev, (void**)&scratch, 2 * per * sizeof(float), stream);
+  int rc = pool_alloc(dev, (void**)&scratch, 2 * per * sizeof(float), stream);
   if (rc != B200SP_OK) return rc;
-  if (I.bin_rows[0] > 0) {
-    long long blocks = ((long long)I.m * (k / VEC) + 255) / 256;
-    if (blocks > (long long)dev->sms * 16) blocks = (long long)dev->sms * 16;
-    rc = launch(spmm_empty_rows_kernel<T, VEC>, dim3((unsigned)blocks), dim3(256), stream, nullptr, 0, dev, (int)I.m, k, p->row_ptr, Y, beta);
-  }
-  if (rc == B200SP_OK) {
-    tl_pdl_kernel = true;
-    rc = launch(spmm_flat_kernel<T, VEC, kSpmmThreads, kFlatChunk>, dim3((unsigned)(slices * tiles)), dim3(kSpmmThreads), stream, B,
-                (size_t)I.n * k * sizeof(T), dev, rows, (int)I.nnz, k, tiles, rp, rid, (const int*)p->flat_tile_row, col_idx, vals, B, Y,
-                scratch, scratch + per, alpha, beta);
-  }
+  tl_pdl_kernel = true;
+  rc = launch(spmm_merge_kernel<T, V, J>, dim3((unsigned)(slices * tiles)), dim3(kMergeWarps * 32), stream, B, (size_t)I.n * k * sizeof(T), dev,
+              (int)I.m, (int)I.nnz, k, tiles, witems, shares, (const int*)p->spmm_split, p->row_ptr, col_idx, vals, B, Y, scratch, scratch + per, alpha, beta);
   if (rc == B200SP_OK && tiles > 1) {
-    const long long groups = (long long)slices * tiles;
     tl_pdl_kernel = true;
-    rc = launch(spmm_flat_fixup_kernel<T, VEC, kSpmmThreads, kFlatTile>, dim3((unsigned)((groups * 8 + kSpmmThreads - 1) / kSpmmThreads)),
-                dim3(kSpmmThreads), stream, nullptr, 0, dev, rows, (int)I.nnz, k, tiles, slices, rp, rid, (const int*)p->flat_tile_row,
-                (const float*)scratch, (const float*)(scratch + per), Y, alpha, beta);
+    rc = launch(spmm_merge_fixup_kernel<T>, dim3((unsigned)(((long long)slices * tiles + 7) / 8)), dim3(256), stream, nullptr, 0, dev, (int)I.m,
+                (int)I.nnz, k, tiles, slices, KS, witems, shares, (const int*)p->spmm_split, p->row_ptr, (const float*)scratch, (const float*)(scratch + per), Y,
+                alpha, beta);
   }
   const cudaError_t e = cudaFreeAsync(scratch, stream);
   if (e != cudaSuccess && rc == B200SP_OK) rc = cuda_fail(e, "cudaFreeAsync");
   return rc;
+}
+
+// nnz-balanced SpMM (spmm_merge_kernel), any k.  The widest pieces (16 bytes per lane at most) that k allows, narrowed while half as
+// wide a piece still covers all of k with one load; then as many loads per nonzero as it takes (at most 4) before k is cut into slices.
+template <typename T, int VMAX>
+int run_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
+                   cudaStream_t stream, DeviceInfo* dev) {
+  const b200sp_plan_info_t& I = p->info;
+  int v = 1;
+  while (v < VMAX && k % (2 * v) == 0 && 32 * v < k) v *= 2;
+  if (!p->spmm_split) {   // shares: once per plan, a small kernel in stream order
+    int w = kMergeWarpItems, per_warp = kMergeShares;
+    while (per_warp > 1 && I.m + I.nnz < (int64_t)dev->sms * 128 * w * per_warp) per_warp /= 2;   // fewer and shorter shares for small problems,
+    while (w > 32 && I.m + I.nnz < (int64_t)dev->sms * 48 * w) w /= 2;                            // so that every SM has enough warps
+    const long long shares = (I.m + I.nnz + w - 1) / w;
+    int rc = pool_alloc(dev, (void**)&p->spmm_split, (size_t)(shares + 1) * sizeof(int32_t), stream);
+    if (rc != B200SP_OK) return rc;
+    rc = launch(plan_merge_split_kernel, dim3((unsigned)((shares + 1 + 255) / 256)), dim3(256), stream, nullptr, 0, dev, p->row_ptr, (int)I.m,
+                (int)I.nnz, w, (int)shares, (int*)p->spmm_split);
+    if (rc != B200SP_OK) return rc;
+    p->spmm_witems = w;
+    p->spmm_shares = per_warp;
+  }
+  const int loads = (k + 32 * v - 1) / (32 * v);
+#define B200SP_MERGE_J(V)                                                                                                   \
+  do {                                                                                                                      \
+    if (loads == 1) return launch_spmm_merge<T, V, 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);                 \
+    if (loads == 2) return launch_spmm_merge<T, V, 2>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);                 \
+    return launch_spmm_merge<T, V, (V * sizeof(T) >= 16 ? 2 : 4)>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);     \
+  } while (0)
+  if (v == 1) B200SP_MERGE_J(1);
+  if (v == 2) B200SP_MERGE_J(2);
+  if (v == 4) B200SP_MERGE_J(4);
+  if constexpr (VMAX == 8) { if (v == 8) B200SP_MERGE_J(8); }
+  return B200SP_ERR_UNSUPPORTED;
+#undef B200SP_MERGE_J
 }
 
 template <typename T, int VEC>
@@ -397,6 +408,10 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
       if (rc != B200SP_ERR_UNSUPPORTED) return rc;   // unsupported shape for the tensor map: fall through to the sliced kernel
     }
   }
+  if (g_opt.spmm_sliced && (g_opt.spmm_flat == 1 || (g_opt.spmm_flat == 2 && (spmm_rows_are_uneven(I) || k % VEC != 0)))) {
+    const int rc = run_spmm_merge<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
+    if (rc != B200SP_ERR_UNSUPPORTED) return rc;
+  }
   if (k % VEC == 0 && g_opt.spmm_sliced) {
     // lanes per row: eight (a 128-byte slice) unless k is narrower than that
     const int vecs_k = k / VEC;
@@ -405,8 +420,6 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     const int slices = (k + KS - 1) / KS;
     const int row_blocks = (int)((I.m + GROUPS - 1) / GROUPS);
     if ((long long)slices * row_blocks >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
-    if (lanes == 8 && (g_opt.spmm_flat == 1 || (g_opt.spmm_flat == 2 && spmm_rows_are_uneven(I))))
-      return run_spmm_flat<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
     int rc;
     const int mid_blocks = (p->num_medium + GROUPS - 1) / GROUPS;
     int ranges = 1;

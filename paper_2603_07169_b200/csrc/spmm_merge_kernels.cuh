@@ -1,0 +1,374 @@
+// nnz-balanced CSR SpMM: Y = alpha * A * B + beta * Y, B (n x k) and Y (m x k) row-major
+// (paper, Appendix C, Table 6, task 13, with alpha/beta).
+//
+// The work list is the merge of the m row-end markers with the nnz nonzeros, cut into equal shares of `witems` items per WARP,
+// whatever rows they belong to: neither long rows nor empty ones unbalance it, and Y of the empty rows is written by the same
+// pass.  A warp walks its nonzeros one after another with all 32 lanes along k, so the end of a row is one warp-uniform branch
+// and no sum is ever combined across lanes.
+#pragma once
+#include "common.cuh"
+
+namespace b200sp {
+
+__device__ __forceinline__ float bf16_lo(unsigned w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(unsigned w) { return __uint_as_float(w & 0xFFFF0000u); }
+__device__ __forceinline__ unsigned bf16_pair(float a, float b) {
+  return (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(a)) | ((unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
+}
+
+// V consecutive stored values as one load / store, converted to FP32 only when consumed.
+template <typename T, int V> struct Piece;
+template <> struct Piece<float, 1> {
+  typedef float raw;
+  static __device__ __forceinline__ void widen(raw b, float (&o)[1]) { o[0] = b; }
+  static __device__ __forceinline__ raw pack(const float (&o)[1]) { return o[0]; }
+};
+template <> struct Piece<float, 2> {
+  typedef float2 raw;
+  static __device__ __forceinline__ void widen(raw b, float (&o)[2]) { o[0] = b.x; o[1] = b.y; }
+  static __device__ __forceinline__ raw pack(const float (&o)[2]) { return make_float2(o[0], o[1]); }
+};
+template <> struct Piece<float, 4> {
+  typedef float4 raw;
+  static __device__ __forceinline__ void widen(raw b, float (&o)[4]) { o[0] = b.x; o[1] = b.y; o[2] = b.z; o[3] = b.w; }
+  static __device__ __forceinline__ raw pack(const float (&o)[4]) { return make_float4(o[0], o[1], o[2], o[3]); }
+};
+template <> struct Piece<bf16_t, 1> {
+  typedef bf16_t raw;
+  static __device__ __forceinline__ void widen(raw b, float (&o)[1]) { o[0] = to_f32(b); }
+  static __device__ __forceinline__ raw pack(const float (&o)[1]) { return __bfloat16_as_ushort(__float2bfloat16_rn(o[0])); }
+};
+template <> struct Piece<bf16_t, 2> {
+  typedef unsigned raw;
+  static __device__ __forceinline__ void widen(raw b, float (&o)[2]) { o[0] = bf16_lo(b); o[1] = bf16_hi(b); }
+  static __device__ __forceinline__ raw pack(const float (&o)[2]) { return bf16_pair(o[0], o[1]); }
+};
+template <> struct Piece<bf16_t, 4> {
+  typedef uint2 raw;
+  static __device__ __forceinline__ void widen(raw b, float (&o)[4]) { o[0] = bf16_lo(b.x); o[1] = bf16_hi(b.x); o[2] = bf16_lo(b.y); o[3] = bf16_hi(b.y); }
+  static __device__ __forceinline__ raw pack(const float (&o)[4]) { return make_uint2(bf16_pair(o[0], o[1]), bf16_pair(o[2], o[3])); }
+};
+template <> struct Piece<bf16_t, 8> {
+  typedef uint4 raw;
+  static __device__ __forceinline__ void widen(raw b, float (&o)[8]) {
+    o[0] = bf16_lo(b.x); o[1] = bf16_hi(b.x); o[2] = bf16_lo(b.y); o[3] = bf16_hi(b.y);
+    o[4] = bf16_lo(b.z); o[5] = bf16_hi(b.z); o[6] = bf16_lo(b.w); o[7] = bf16_hi(b.w);
+  }
+  static __device__ __forceinline__ raw pack(const float (&o)[8]) {
+    return make_uint4(bf16_pair(o[0], o[1]), bf16_pair(o[2], o[3]), bf16_pair(o[4], o[5]), bf16_pair(o[6], o[7]));
+  }
+};
+
+template <typename T, int V>
+__device__ __forceinline__ void piece_fma(const typename Piece<T, V>::raw& b, float v, float (&acc)[V]) {
+  float w[V];
+  Piece<T, V>::widen(b, w);
+#pragma unroll
+  for (int i = 0; i < V; ++i) acc[i] = fmaf(v, w[i], acc[i]);
+}
+
+template <typename T, int V>
+__device__ __forceinline__ void piece_store(T* yp, const float (&acc)[V], float alpha, float beta) {
+  typedef typename Piece<T, V>::raw raw;
+  float out[V];
+#pragma unroll
+  for (int j = 0; j < V; ++j) out[j] = alpha * acc[j];
+  if (beta != 0.0f) {
+    float old[V];
+    Piece<T, V>::widen(*(const raw*)yp, old);
+#pragma unroll
+    for (int j = 0; j < V; ++j) out[j] += beta * old[j];
+  }
+  *(raw*)yp = Piece<T, V>::pack(out);
+}
+
+// N consecutive words of shared memory (N 2, 4 or 8; aligned to 4 N or 16 bytes) with vector loads
+template <int N, typename W>
+__device__ __forceinline__ void lds_group(const W* p, W (&o)[N]) {
+  if constexpr (N >= 4) {
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+      const int4 t = *(const int4*)(p + i);
+      o[i] = *(const W*)&t.x; o[i + 1] = *(const W*)&t.y; o[i + 2] = *(const W*)&t.z; o[i + 3] = *(const W*)&t.w;
+    }
+  } else {
+    const int2 t = *(const int2*)p;
+    o[0] = *(const W*)&t.x; o[1] = *(const W*)&t.y;
+  }
+}
+
+// A value that is the same in all lanes, made known as such: branches on it need no reconvergence code.
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xFFFFFFFFu, v, 0); }
+
+// 4-byte asynchronous copy global -> shared of which the first `bytes` (2 or 4) are read and the rest is zero
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, int bytes = 4) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+constexpr int kMergeWarps = 8;       // warps per CTA of spmm_merge_kernel
+constexpr int kMergeWarpItems = 128; // most merge items per share
+constexpr int kMergeShares = 4;      // most consecutive shares per warp
+
+// Resident CTAs per SM that the registers are capped for, by the registers the loads in flight and the sums take.
+template <typename T, int V, int J>
+constexpr int merge_ctas() {
+  constexpr int need = (8 * V * (int)sizeof(T) + 3) / 4 + 2 * V * J;
+  return need <= 20 ? 5 : need <= 40 ? 4 : 3;
+}
+
+// What a warp keeps in shared memory of one share: its columns, its values and the ends of its rows, and room to read a group ahead.
+template <typename T> struct MergeStage;
+template <> struct MergeStage<float> {
+  int col[kMergeWarpItems + 8];
+  float val[kMergeWarpItems + 8];
+  int end[kMergeWarpItems + 4];
+};
+template <> struct MergeStage<bf16_t> {
+  int col[kMergeWarpItems + 8];
+  unsigned raw[kMergeWarpItems / 2 + 4];      // the 4-byte words that hold the values, as stored
+  int end[kMergeWarpItems + 4];
+};
+
+// A warp takes `shares` consecutive shares; the (col, val) pairs and row ends of the next one arrive in shared memory (cp.async)
+// while it walks the current one.  Lane l holds columns slice * 32 * V * J + 32 * V * j + l * V + (0 .. V-1), j < J, of the current
+// row in FP32 registers (acc: products of the current share; tot: of the row's earlier shares); U = 8 / J nonzeros, 8 loads of B, are
+// in flight.  A warp leaves two partial sums in shared memory: `head` for a first row that began before its shares, `carry` for
+// the row it leaves unfinished; after one barrier the warp that holds a row's end adds the carries of the warps before it in
+// order, and what crosses the CTA's own ends goes to tile_tail / tile_carry and is finished by spmm_merge_fixup_kernel.  No
+// chain is longer than kMergeWarpItems products + kMergeShares + kMergeWarps partial sums + the tiles' terms.
+// split[i]: row ends before item i * witems.
+template <typename T, int V, int J>
+__global__ void __launch_bounds__(kMergeWarps * 32, (merge_ctas<T, V, J>()))
+spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, const int* __restrict__ split, const int* __restrict__ row_ptr,
+                  const int* __restrict__ col_idx, const T* __restrict__ vals, const T* __restrict__ B, T* __restrict__ Y,
+                  float* __restrict__ tile_carry, float* __restrict__ tile_tail, float alpha, float beta) {
+  constexpr int U = 8 / J, KS = 32 * V * J;
+  typedef typename Piece<T, V>::raw raw;
+  __shared__ __align__(16) MergeStage<T> stage_s[kMergeWarps][2];
+  __shared__ __align__(16) float wide_s[sizeof(T) == 2 ? kMergeWarps : 1][sizeof(T) == 2 ? kMergeWarpItems + 8 : 4];   // BF16: the current share's values widened
+  __shared__ float head_s[kMergeWarps][KS];
+  static_assert(sizeof(stage_s[0]) >= KS * sizeof(float), "a warp's carry takes the place of its stages");
+  auto carry_s = [&](int w) { return reinterpret_cast<float*>(&stage_s[w][0]); };
+  grid_dependency_wait();
+  const int slice = blockIdx.x / tiles, t = blockIdx.x - slice * tiles;
+  const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const long long total = (long long)m + nnz;
+  const int last = (int)((total + witems - 1) / witems);
+  const int s0 = (int)min(((long long)t * kMergeWarps + warp) * shares, (long long)last), s1 = min(s0 + shares, last);
+  const int r_first = uniform(__ldg(split + s0));
+  int r_lo = r_first, r_hi = uniform(__ldg(split + min(s0 + 1, last)));
+  const int start0 = uniform(__ldg(row_ptr + r_first));      // start of the first row (nnz when there is none)
+  const int p_first = (int)(min((long long)s0 * witems, total) - r_first);
+  bool head = start0 < p_first;                              // the current row began before this warp's shares
+
+  // copies of share s (rows r0 .. r1 end in it) into stage st
+  auto fetch = [&](int s, int r0, int r1, MergeStage<T>& st) {
+    const int p0 = (int)((long long)s * witems - r0), cnt = (int)(min((long long)(s + 1) * witems, total) - r1) - p0, rows = r1 - r0;
+#pragma unroll
+    for (int i = 0; i < kMergeWarpItems; i += 32) {
+      if (i + lane < cnt) {
+        cp_async4(&st.col[i + lane], col_idx + p0 + i + lane);
+        if constexpr (sizeof(T) == 4) cp_async4(&st.val[i + lane], vals + p0 + i + lane);
+      }
+      if (i + lane < rows) cp_async4(&st.end[i + lane], row_ptr + r0 + 1 + i + lane);
+    }
+    if constexpr (sizeof(T) == 2) {
+      const int w0 = p0 & ~1, words = (p0 + cnt - w0 + 1) >> 1;
+#pragma unroll
+      for (int i = 0; i < kMergeWarpItems / 2 + 32; i += 32)
+        if (i + lane < words) cp_async4(&st.raw[i + lane], vals + w0 + 2 * (i + lane), min(4, 2 * (nnz - w0 - 2 * (i + lane))));
+    }
+    if (lane < U) st.col[cnt + lane] = 0;                    // read ahead of the end, never multiplied
+    if (lane == 0) st.end[rows] = 0x7FFFFFFF;
+  };
+
+  const int col0 = slice * KS + lane * V;
+  bool on[J];
+  float acc[J][V], tot[J][V];
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    on[j] = col0 + 32 * V * j < k;
+#pragma unroll
+    for (int i = 0; i < V; ++i) { acc[j][i] = 0.0f; tot[j][i] = 0.0f; }
+  }
+  const char* const Bc = (const char*)(B + col0);
+  const int row_bytes = k * (int)sizeof(T);
+  T* yp = Y + (long long)r_first * k + col0;
+
+  if (s0 < s1) fetch(s0, r_lo, r_hi, stage_s[warp][0]);
+  cp_async_commit();
+  int r_next = uniform(__ldg(split + min(s0 + 2, last)));
+  for (int s = s0; s < s1; ++s) {
+    const int cur = (s - s0) & 1;
+    if (s + 1 < s1) fetch(s + 1, r_hi, r_next, stage_s[warp][cur ^ 1]);
+    cp_async_commit();
+    const int r_after = __ldg(split + min(s + 3, last));
+    cp_async_wait<1>();
+    __syncwarp();
+    MergeStage<T>& st = stage_s[warp][cur];
+    const int p0 = (int)((long long)s * witems - r_lo), cnt = (int)(min((long long)(s + 1) * witems, total) - r_hi) - p0, rows = r_hi - r_lo;
+    const float* vls;
+    if constexpr (sizeof(T) == 2) {
+      const bf16_t* const raw_v = (const bf16_t*)st.raw + (p0 & 1);
+#pragma unroll
+      for (int i = 0; i < kMergeWarpItems; i += 32) if (i + lane < cnt) wide_s[warp][i + lane] = to_f32(raw_v[i + lane]);
+      __syncwarp();
+      vls = wide_s[warp];
+    } else {
+      vls = st.val;
+    }
+    const int* const ends = st.end;
+    int j_row = 0, end = uniform(ends[0]) - p0;              // the current row ends before nonzero `end` of the share
+    // the current row has been added up to its end: stored, or left as the warp's head when it began earlier
+    auto finish_row = [&]() {
+#pragma unroll
+      for (int j = 0; j < J; ++j)
+#pragma unroll
+        for (int i = 0; i < V; ++i) { acc[j][i] += tot[j][i]; tot[j][i] = 0.0f; }
+      if (head) {
+        head = false;
+#pragma unroll
+        for (int j = 0; j < J; ++j)
+#pragma unroll
+          for (int i = 0; i < V; ++i) head_s[warp][32 * V * j + lane * V + i] = acc[j][i];
+      } else {
+#pragma unroll
+        for (int j = 0; j < J; ++j) if (on[j]) piece_store<T, V>(yp + 32 * V * j, acc[j], alpha, beta);
+      }
+#pragma unroll
+      for (int j = 0; j < J; ++j)
+#pragma unroll
+        for (int i = 0; i < V; ++i) acc[j][i] = 0.0f;
+      yp += k;
+      end = uniform(ends[++j_row]) - p0;
+    };
+    for (int q = 0; q < cnt; q += U) {
+      int c[U];
+      float v[U];
+      raw b[U][J];
+      lds_group<U>(st.col + q, c);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int j = 0; j < J; ++j) if (on[j]) b[u][j] = __ldg((const raw*)(Bc + (long long)c[u] * row_bytes) + 32 * j);
+      lds_group<U>(vls + q, v);
+      if (q + U > cnt) {                                     // the last, partly filled group: (0, 0) instead of what was read ahead
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (q + u >= cnt) {
+            v[u] = 0.0f;
+#pragma unroll
+            for (int j = 0; j < J; ++j) b[u][j] = raw();
+          }
+      }
+      if (end >= q + U) {                                    // no row ends inside this group
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int j = 0; j < J; ++j) piece_fma<T, V>(b[u][j], v[u], acc[j]);
+      } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          while (end == q + u) finish_row();
+#pragma unroll
+          for (int j = 0; j < J; ++j) piece_fma<T, V>(b[u][j], v[u], acc[j]);
+        }
+      }
+    }
+    while (j_row < rows) finish_row();
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+#pragma unroll
+      for (int i = 0; i < V; ++i) { tot[j][i] += acc[j][i]; acc[j][i] = 0.0f; }
+    __syncwarp();                                            // every lane is done with the stage: the next copies may land in it
+    r_lo = r_hi; r_hi = r_next; r_next = uniform(r_after);
+  }
+#pragma unroll
+  for (int j = 0; j < J; ++j)
+#pragma unroll
+    for (int i = 0; i < V; ++i) carry_s(warp)[32 * V * j + lane * V + i] = tot[j][i];   // zero when the shares end with a row
+  __syncthreads();
+
+  // (r_lo is now the number of row ends before this warp's end)
+  const int region = witems * shares;
+  const long long slot = ((long long)slice * tiles + t) * KS;
+  if (start0 < p_first && r_lo > r_first) {                  // complete the row that ends here: the carries before it, in order, then the head
+    const long long ws = ((long long)start0 + r_first) / region - (long long)t * kMergeWarps;   // the warp that holds the row's start
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      float s[V];
+#pragma unroll
+      for (int i = 0; i < V; ++i) s[i] = 0.0f;
+      for (int w = ws > 0 ? (int)ws : 0; w < warp; ++w)
+#pragma unroll
+        for (int i = 0; i < V; ++i) s[i] += carry_s(w)[32 * V * j + lane * V + i];
+#pragma unroll
+      for (int i = 0; i < V; ++i) s[i] += head_s[warp][32 * V * j + lane * V + i];
+      if (ws >= 0) { if (on[j]) piece_store<T, V>(Y + (long long)r_first * k + col0 + 32 * V * j, s, alpha, beta); }
+      else {
+#pragma unroll
+        for (int i = 0; i < V; ++i) tile_tail[slot + 32 * V * j + lane * V + i] = s[i];
+      }
+    }
+  }
+  if (warp == kMergeWarps - 1) {                             // what the tile leaves unfinished
+    long long ws = kMergeWarps;
+    if (r_lo < m) ws = ((long long)__ldg(row_ptr + r_lo) + r_lo) / region - (long long)t * kMergeWarps;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      float s[V];
+#pragma unroll
+      for (int i = 0; i < V; ++i) s[i] = 0.0f;
+      for (int w = ws > 0 ? (int)ws : 0; w < kMergeWarps; ++w)
+#pragma unroll
+        for (int i = 0; i < V; ++i) s[i] += carry_s(w)[32 * V * j + lane * V + i];
+#pragma unroll
+      for (int i = 0; i < V; ++i) tile_carry[slot + 32 * V * j + lane * V + i] = s[i];
+    }
+  }
+}
+
+// Finishes the rows that a tile boundary of spmm_merge_kernel cut: tile t completes such a row when its first row began in an
+// earlier tile and ends in this one.  The row's value is tile_carry[first .. t-1] + tile_tail[t], the carries added in trees of
+// 16 whose sums form a chain; one warp per (slice, tile), fixed order.
+template <typename T>
+__global__ void __launch_bounds__(256)
+spmm_merge_fixup_kernel(int m, int nnz, int k, int tiles, int slices, int ks, int witems, int shares, const int* __restrict__ split,
+                        const int* __restrict__ row_ptr, const float* __restrict__ tile_carry, const float* __restrict__ tile_tail,
+                        T* __restrict__ Y, float alpha, float beta) {
+  grid_dependency_wait();
+  const long long id = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (id >= (long long)slices * tiles) return;
+  const int slice = (int)(id / tiles), t = (int)(id - (long long)slice * tiles);
+  if (t < 1) return;
+  const long long total = (long long)m + nnz;
+  const int items = witems * shares * kMergeWarps, per = shares * kMergeWarps;
+  const int last = (int)((total + witems - 1) / witems);
+  const int r0 = __ldg(split + (long long)t * per), r1 = __ldg(split + min((long long)(t + 1) * per, (long long)last));
+  if (r0 >= r1) return;                                      // no row ends in the tile
+  const long long p0 = (long long)t * items - r0;
+  const int rs = __ldg(row_ptr + r0);
+  if (rs >= p0) return;                                      // its first row starts inside it
+  const int tf = (int)(((long long)rs + r0) / items);
+  for (int c = lane; c < ks && slice * ks + c < k; c += 32) {
+    const float* const cp = tile_carry + (long long)slice * tiles * ks + c;
+    float acc = 0.0f;
+    for (int u = tf; u < t; u += 16) {
+      float part[16];
+#pragma unroll
+      for (int v = 0; v < 16; ++v) part[v] = u + v < t ? cp[(long long)(u + v) * ks] : 0.0f;
+#pragma unroll
+      for (int w = 8; w > 0; w >>= 1)
+#pragma unroll
+        for (int v = 0; v < w; ++v) part[v] += part[v + w];
+      acc += part[0];
+    }
+    acc += tile_tail[((long long)slice * tiles + t) * ks + c];
+    epilogue_store(Y, (long long)r0 * k + slice * ks + c, acc, alpha, beta);
+  }
+}
+
+}  // namespace b200sp

@@ -1,0 +1,64 @@
+"""nnz-balanced SpMM (spmm_merge_kernel): every piece width, odd k, and matrices whose items end at the edges of shares, warps and tiles."""
+import numpy as np
+import pytest
+
+import gen
+import paper_2603_07169_b200 as b200sp
+from gpu_util import assert_within, run_spmm
+
+pytestmark = pytest.mark.gpu
+
+
+def matrices():
+    rng = np.random.default_rng(3)
+    skew = (rng.pareto(1.3, 3000) * 3).astype(np.int64).clip(0, 900)
+    skew[5] = 6000                                                            # a row over several CTAs
+    return {
+        "skewed": skew,
+        "one_share": np.array([32 - 4, 0, 0]),                                 # rows + nonzeros = 31, then exactly 32
+        "share_edge": np.array([28, 0, 0, 0]),
+        "cta_edge": np.concatenate([np.full(7, 31), [32]]),                    # 8 warps x 32 items, all rows ending at share ends
+        "cta_edge_plus_one": np.concatenate([np.full(8, 31), [1]]),
+        "one_row": np.array([5000]),
+        "all_empty_but_last": np.concatenate([np.zeros(5000, np.int64), [3]]),
+        "large": rng.integers(0, 60, 120_000),                                 # shares of 128 items, several to a warp
+    }
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("case", sorted(matrices()))
+def test_merge_spmm_against_oracle(case, dtype):
+    lens = matrices()[case]
+    rng = np.random.default_rng(len(case))
+    n = 40_000                                                                 # too many columns for the shared-memory-B kernel
+    A = gen.random_csr(len(lens), n, lens, seed=5, sort_cols=False)
+    b200sp.b200sp_set_option("spmm_flat", 1)
+    try:
+        for k in ((50,) if case == "large" else (2, 3, 16, 33, 50, 64, 65, 100, 127, 130, 256, 300)):
+            B = rng.standard_normal(n * k).astype(np.float32)
+            Y0 = rng.standard_normal(A.m * k).astype(np.float32)
+            Y, Y_ref, S = run_spmm(A, B, k, None, 1.0, 0.0, dtype)
+            assert_within(Y, Y_ref, S, dtype, what="%s k=%d" % (case, k))
+            Y, Y_ref, S = run_spmm(A, B, k, Y0, -0.5, 1.25, dtype)
+            y0f = Y0 if dtype == "f32" else gen.bf16_to_f32(gen.to_bf16(Y0))
+            assert_within(Y, Y_ref, S, dtype, 1.0, np.abs(1.25 * y0f.astype(np.float64)).reshape(A.m, k), what="%s k=%d ab" % (case, k))
+    finally:
+        b200sp.b200sp_set_option("spmm_flat", 2)
+
+
+def test_non_finite_rows_of_b_touch_only_the_rows_that_use_them():
+    """What a warp reads ahead of its last nonzero (row 0 of B) is never multiplied."""
+    n, k = 9000, 64
+    lens = np.full(77, 5)
+    lens[::4] = 0
+    A = gen.random_csr(len(lens), n, lens, seed=1)
+    A.col_idx[:] = np.maximum(A.col_idx, 1)
+    B = np.ones(n * k, np.float32)
+    B[:k] = np.inf
+    b200sp.b200sp_set_option("spmm_flat", 1)
+    try:
+        Y, Y_ref, S = run_spmm(A, B, k, None, 1.0, 0.0, "f32")
+        assert np.isfinite(Y).all()
+        assert_within(Y, Y_ref, S, "f32")
+    finally:
+        b200sp.b200sp_set_option("spmm_flat", 2)
