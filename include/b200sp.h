@@ -25,7 +25,7 @@
  *    col_idx, vals, x / B and y / Y must be 16-byte aligned, row_ptr 4-byte aligned.
  *  - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  Calls enqueue
  *    work and return without synchronising, except where stated (plan creation reads back a few
- *    hundred bytes and synchronises the stream once).
+ *    hundred bytes, through pinned host memory that the library keeps, and synchronises the stream once).
  *  - beta == 0: y / Y is write-only (its old contents, NaN included, are ignored).  alpha == 0 or
  *    nnz == 0: y = beta * y without reading A.  m == 0: nothing is done.  x / B must not alias y / Y.
  *  - The compute kernels are launched with programmatic stream serialisation (option "pdl"): a kernel waits for the
@@ -111,12 +111,12 @@ int spmm_csr(int64_t m, int64_t n, int64_t nnz, int64_t k, const int32_t* row_pt
 /* ---- plan API --------------------------------------------------------------------------------
  * The plan pass depends on the sparsity pattern's row structure only (row_ptr): it computes the
  * row-length statistics and bins, chooses the kernels, and computes the nnz-balanced split points
- * (a merge-path search over rows + nonzeros) and the lists of rows of 129-1024 and of more than 1024 nonzeros that
- * SpMM treats separately, all on the device.  From the same statistics it decides whether SpMM gives every row to a
- * group of eight lanes (even rows) or cuts the nonzeros into equal chunks whatever rows they belong to (uneven rows:
- * many empty rows, or a share of the nonzeros in rows of more than 128); the list of non-empty rows that the second
- * form needs is built on the first SpMM call, in stream order, and so is the order of the rows by length that SpMM
- * uses when A has so few columns that a slice of B is kept in shared memory.
+ * (a merge-path search over rows + nonzeros), all on the device and in one launch.  From the same statistics it decides
+ * whether SpMM gives every row to a group of eight lanes (even rows) or cuts rows + nonzeros into equal shares per warp
+ * (uneven rows: many empty rows, or a share of the nonzeros in rows of more than 128).  What only some SpMM kernels need is
+ * built on the first SpMM call that uses them, in stream order: the lists of rows of 129-1024 and of more than 1024 nonzeros,
+ * the shares of large matrices, and the order of the rows by length that SpMM uses when A has so few columns that a slice
+ * of B is kept in shared memory.
  * When the row statistics select the row-direct SpMV kernel, the first b200sp_spmv / spmv_csr call with a given
  * col_idx additionally samples how local the columns are (one small kernel and one synchronisation of the stream)
  * and falls back to the merge-tile kernel for matrices with scattered columns.

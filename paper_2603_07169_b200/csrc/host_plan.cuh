@@ -3,6 +3,7 @@
 #pragma once
 #include "host_runtime.cuh"
 #include "plan_kernels.cuh"
+#include "spmm_merge_kernels.cuh"
 
 namespace {
 
@@ -20,26 +21,20 @@ constexpr size_t kCacheCap = 1024;
 int plan_free(b200sp_plan* p, bool stream_ordered = false, cudaStream_t stream = nullptr) {
   if (!p) return B200SP_OK;
   int rc = B200SP_OK;
-  if (p->block || p->cuts_block || p->compact_block || p->spmm_split || p->quad_block) {
+  void* const blocks[] = {p->block, p->cuts_block, p->compact_block, p->split_block, p->quad_block, p->lists_block};
+  bool any = false;
+  for (void* b : blocks) any |= b != nullptr;
+  if (any) {
     cudaError_t e = cudaSuccess;
-    if (stream_ordered) {
-      if (p->block) e = cudaFreeAsync(p->block, stream);
-      if (p->cuts_block && e == cudaSuccess) e = cudaFreeAsync(p->cuts_block, stream);
-      if (p->compact_block && e == cudaSuccess) e = cudaFreeAsync(p->compact_block, stream);
-      if (p->spmm_split && e == cudaSuccess) e = cudaFreeAsync(p->spmm_split, stream);
-      if (p->quad_block && e == cudaSuccess) e = cudaFreeAsync(p->quad_block, stream);
-    } else {
-      int cur = 0;
+    int cur = p->device;
+    if (!stream_ordered) {
       e = cudaGetDevice(&cur);
       if (e == cudaSuccess && cur != p->device) e = cudaSetDevice(p->device);
       if (e == cudaSuccess) e = cudaDeviceSynchronize();
-      if (e == cudaSuccess && p->block) e = cudaFree(p->block);
-      if (e == cudaSuccess && p->cuts_block) e = cudaFree(p->cuts_block);
-      if (e == cudaSuccess && p->compact_block) e = cudaFree(p->compact_block);
-      if (e == cudaSuccess && p->spmm_split) e = cudaFree(p->spmm_split);
-      if (e == cudaSuccess && p->quad_block) e = cudaFree(p->quad_block);
-      if (cur != p->device) cudaSetDevice(cur);
     }
+    for (void* b : blocks)
+      if (b && e == cudaSuccess) e = stream_ordered ? cudaFreeAsync(b, stream) : cudaFree(b);
+    if (cur != p->device) cudaSetDevice(cur);
     if (e != cudaSuccess) rc = cuda_fail(e, "freeing a plan");
   }
   delete p;
@@ -77,6 +72,66 @@ int plan_compact_rows(b200sp_plan* p, cudaStream_t stream, DeviceInfo* dev) {
   return B200SP_OK;
 }
 
+// Pinned host memory for the results of plan passes, one slot per pass in flight; a pass holds its slot (and the accumulators of
+// the same index in g_plan_slots) from before its launch until its results have been read.
+struct PlanSlots {
+  std::mutex mutex;
+  std::condition_variable freed;
+  PlanStats* host = nullptr;
+  std::vector<int> idle;
+} g_slots;
+
+int plan_slot_take(int* slot) {
+  std::unique_lock<std::mutex> lock(g_slots.mutex);
+  if (!g_slots.host) {
+    CU(cudaHostAlloc((void**)&g_slots.host, kPlanSlots * sizeof(PlanStats), cudaHostAllocPortable | cudaHostAllocMapped));
+    for (int i = kPlanSlots - 1; i >= 0; --i) g_slots.idle.push_back(i);
+  }
+  g_slots.freed.wait(lock, [] { return !g_slots.idle.empty(); });
+  *slot = g_slots.idle.back();
+  g_slots.idle.pop_back();
+  return B200SP_OK;
+}
+
+void plan_slot_give(int slot) {
+  { std::lock_guard<std::mutex> lock(g_slots.mutex); g_slots.idle.push_back(slot); }
+  g_slots.freed.notify_one();
+}
+
+// Warp shares of the nnz-balanced SpMM kernel: items per share and shares per warp, fewer and shorter for small problems so that
+// every SM has enough warps.  Returns the number of shares.
+long long spmm_shares(const b200sp_plan_info_t& I, const DeviceInfo* dev, int* witems, int* per_warp) {
+  int w = kMergeWarpItems, s = kMergeShares;
+  while (s > 1 && I.m + I.nnz < (int64_t)dev->sms * 128 * w * s) s /= 2;
+  while (w > 32 && I.m + I.nnz < (int64_t)dev->sms * 48 * w) w /= 2;
+  *witems = w;
+  *per_warp = s;
+  return (I.m + I.nnz + w - 1) / w;
+}
+
+// The lists of rows of kMediumRow + 1 .. kLongRow and of more than kLongRow nonzeros, built on the device in stream order on the
+// first SpMM call that needs them; their lengths are known from the plan pass.
+int plan_row_lists(b200sp_plan* p, cudaStream_t stream, DeviceInfo* dev) {
+  if (p->lists_block || p->num_medium + p->num_long == 0) return B200SP_OK;
+  const size_t n_mid = (size_t)p->num_medium, n_long = (size_t)p->num_long;
+  int* blk = nullptr;
+  int rc = pool_alloc(dev, (void**)&blk, (4 + n_mid + n_long) * sizeof(int32_t), stream);
+  if (rc != B200SP_OK) return rc;
+  cudaError_t e = cudaMemsetAsync(blk, 0, 2 * sizeof(int), stream);
+  if (e == cudaSuccess) {
+    const int blocks = (int)((p->info.m + 255) / 256);
+    plan_row_lists_kernel<<<blocks < dev->sms * 8 ? blocks : dev->sms * 8, 256, 0, stream>>>(
+        p->row_ptr, (int)p->info.m, kMediumRow, kLongRow, (int)n_mid, (int)n_long, blk + 4, blk + 4 + n_mid, blk);
+    g_launches++;
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) { cudaFreeAsync(blk, stream); return cuda_fail(e, "lists of medium and long rows"); }
+  p->lists_block = blk;
+  p->medium_rows = blk + 4;
+  p->long_rows = blk + 4 + n_mid;
+  return B200SP_OK;
+}
+
 int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32_t* row_ptr, cudaStream_t stream) {
   DeviceInfo* dev = nullptr;
   int rc = device_info(&dev);
@@ -92,63 +147,43 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
   I.spmv_kernel = g_opt.spmv_kernel >= 0 ? g_opt.spmv_kernel : 0;
   if (m == 0) { *out = p; return B200SP_OK; }
 
-  // one block from the pool: statistics, counters, split points, carries, tails, medium- and long-row lists
+  // one block from the pool: the probe's counters, split points, carries, tails; for small matrices also the shares of the
+  // nnz-balanced SpMM kernel, which then cost no launch of their own (large ones search them on first use)
   const size_t nt = (size_t)I.spmv_tiles;
-  const size_t long_cap = (size_t)(nnz / (kLongRow + 1)) + 1;     // rows longer than kLongRow: at most this many
-  const size_t mid_cap = (size_t)(nnz / (kMediumRow + 1)) + 1;    // rows longer than kMediumRow
+  int witems = 0, per_warp = 0;
+  const long long shares = spmm_shares(I, dev, &witems, &per_warp);
+  const bool with_shares = shares <= 65536;
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-  const size_t o_stats = 0, o_count = o_stats + up(sizeof(PlanStats)), o_split = o_count + 256, o_carry = o_split + up((nt + 1) * 4),
-               o_tail = o_carry + up((nt + 1) * 4), o_mid = o_tail + up((nt + 1) * 4), o_long = o_mid + up(mid_cap * 4),
-               total = o_long + up(long_cap * 4);
-  PlanStats h = {};
-  h.min_len = 0x7FFFFFFF;
+  const size_t o_split = 256, o_carry = o_split + up((nt + 1) * 4), o_tail = o_carry + up((nt + 1) * 4), o_share = o_tail + up((nt + 1) * 4),
+               total = o_share + (with_shares ? up((size_t)(shares + 1) * 4) : 0);
   auto fail = [&](int code) { plan_free(p, true, stream); cudaStreamSynchronize(stream); return code; };
 #define CUP(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) return fail(cuda_fail(e_, #call)); } while (0)
   rc = pool_alloc(dev, &p->block, total, stream);
   if (rc != B200SP_OK) { delete p; return rc; }
   char* base = (char*)p->block;
-  PlanStats* d_stats = (PlanStats*)(base + o_stats);
-  int* d_count = (int*)(base + o_count);                       // two list counters
-  p->probe_out = (unsigned long long*)(base + o_count + 16);   // two probe counters
+  p->probe_out = (unsigned long long*)base;   // two probe counters
   p->split_row = (int32_t*)(base + o_split);
   p->carry = (float*)(base + o_carry);
   p->tail = (float*)(base + o_tail);
-  p->medium_rows = (int32_t*)(base + o_mid);
-  p->long_rows = (int32_t*)(base + o_long);
+  if (with_shares) { p->spmm_split = (int32_t*)(base + o_share); p->spmm_witems = witems; p->spmm_shares = per_warp; }
   I.scratch_bytes = (int64_t)total;
-  CUP(cudaMemcpyAsync(d_stats, &h, sizeof h, cudaMemcpyHostToDevice, stream));
+  int slot = 0;
+  rc = plan_slot_take(&slot);
+  if (rc != B200SP_OK) return fail(rc);
+  PlanStats h;
   {
-    const int blocks = (int)((m + 256 * 8 - 1) / (256 * 8));
-    const int grid = blocks < dev->sms * 8 ? (blocks > 0 ? blocks : 1) : dev->sms * 8;
-    plan_stats_kernel<<<grid, 256, 0, stream>>>(row_ptr, (int)m, d_stats);
+    const long long blocks = (m + 256 * 4 - 1) / (256 * 4);
+    const int grid = (int)(blocks < dev->sms * 8 ? blocks : dev->sms * 8);
+    plan_pass_kernel<<<grid, 256, 0, stream>>>(row_ptr, (int)m, (int)nnz, slot, g_slots.host + slot, items, (int)nt, p->split_row,
+                                               with_shares ? witems : 0, (int)shares, p->spmm_split);
     g_launches++;
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    h = g_slots.host[slot];
+    plan_slot_give(slot);
+    if (e != cudaSuccess) return fail(cuda_fail(e, "plan pass"));
   }
-  plan_merge_split_kernel<<<(unsigned)((nt + 1 + 255) / 256), 256, 0, stream>>>(row_ptr, (int)m, (int)nnz, items, (int)nt, p->split_row);
-  g_launches++;
-  CUP(cudaGetLastError());
-  CUP(cudaMemcpyAsync(&h, d_stats, sizeof h, cudaMemcpyDeviceToHost, stream));
-  CUP(cudaStreamSynchronize(stream));
-  if (!h.bad && h.bin_rows[4] + h.bin_rows[5] > 0) {   // lists of the rows in the last two length bins, sorted on the host
-    const size_t n_mid = (size_t)h.bin_rows[4], n_long = (size_t)h.bin_rows[5];
-    if (n_mid > mid_cap || n_long > long_cap) return fail(B200SP_ERR_BAD_CSR);   // cannot happen for a monotone row_ptr
-    CUP(cudaMemsetAsync(d_count, 0, 2 * sizeof(int), stream));
-    const int blocks = (int)((m + 255) / 256);
-    plan_row_lists_kernel<<<blocks < dev->sms * 8 ? blocks : dev->sms * 8, 256, 0, stream>>>(
-        row_ptr, (int)m, kMediumRow, kLongRow, (int)n_mid, (int)n_long, p->medium_rows, p->long_rows, d_count);
-    g_launches++;
-    CUP(cudaGetLastError());
-    std::vector<int32_t> tmp(n_mid + n_long);
-    if (n_mid) CUP(cudaMemcpyAsync(tmp.data(), p->medium_rows, n_mid * sizeof(int32_t), cudaMemcpyDeviceToHost, stream));
-    if (n_long) CUP(cudaMemcpyAsync(tmp.data() + n_mid, p->long_rows, n_long * sizeof(int32_t), cudaMemcpyDeviceToHost, stream));
-    CUP(cudaStreamSynchronize(stream));
-    std::sort(tmp.begin(), tmp.begin() + n_mid);
-    std::sort(tmp.begin() + n_mid, tmp.end());
-    if (n_mid) CUP(cudaMemcpyAsync(p->medium_rows, tmp.data(), n_mid * sizeof(int32_t), cudaMemcpyHostToDevice, stream));
-    if (n_long) CUP(cudaMemcpyAsync(p->long_rows, tmp.data() + n_mid, n_long * sizeof(int32_t), cudaMemcpyHostToDevice, stream));
-    CUP(cudaStreamSynchronize(stream));
-    p->num_medium = (int)n_mid;
-    p->num_long = (int)n_long;
-  }
+  if (!h.bad) { p->num_medium = (int)h.bin_rows[4]; p->num_long = (int)h.bin_rows[5]; }
   // Many rows without nonzeros (a quarter or more): the merge list is built over the rows that have nonzeros only, and the
   // split points are searched again over that list.
   if (!h.bad && g_opt.merge_empty && nnz > 0 && (int64_t)h.bin_rows[0] * 4 >= m) {

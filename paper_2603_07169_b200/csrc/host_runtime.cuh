@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <condition_variable>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -243,12 +244,14 @@ struct b200sp_plan {
   int32_t* split_row = nullptr;       // spmv tiles + 1
   float* carry = nullptr;             // spmv tiles
   float* tail = nullptr;              // spmv tiles
-  int32_t* medium_rows = nullptr;     // rows of kMediumRow + 1 .. kLongRow nonzeros, ascending
-  int32_t* long_rows = nullptr;       // rows longer than kLongRow, ascending
+  void* lists_block = nullptr;        // one pool block for the two lists below, built on the first SpMM call that needs them
+  int32_t* medium_rows = nullptr;     // rows of kMediumRow + 1 .. kLongRow nonzeros, in any order
+  int32_t* long_rows = nullptr;       // rows longer than kLongRow, in any order
   unsigned long long* probe_out = nullptr;  // two counters for the column-locality probe
   int num_medium = 0, num_long = 0;
   const void* probed_col_idx = nullptr;   // col_idx the column-locality probe last ran on
-  int32_t* spmm_split = nullptr;          // warp shares of the nnz-balanced SpMM kernel (a pool block of its own, built on first use)
+  int32_t* spmm_split = nullptr;          // warp shares of the nnz-balanced SpMM kernel (part of `block` for small matrices, else a pool block of its own, built on first use)
+  void* split_block = nullptr;            // that block
   int spmm_witems = 0, spmm_shares = 0;   // merge items per share, consecutive shares per warp
   // merge list over the rows that have nonzeros (matrices with many empty rows)
   void* compact_block = nullptr;          // one pool block: row ids, their offsets, block counts

@@ -16,8 +16,10 @@ int launch_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, co
   const b200sp_plan_info_t& I = p->info;
   constexpr int GROUPS = kSpmmThreads / LANES;
   const unsigned grid = (unsigned)((I.m + GROUPS - 1) / GROUPS);
+  int rc = plan_row_lists(p, stream, dev);
+  if (rc != B200SP_OK) return rc;
   tl_pdl_kernel = true;
-  int rc = launch(spmm_row_group_kernel<T, VEC, LANES, NCH, kSpmmThreads>, dim3(grid), dim3(kSpmmThreads), stream, B,
+  rc = launch(spmm_row_group_kernel<T, VEC, LANES, NCH, kSpmmThreads>, dim3(grid), dim3(kSpmmThreads), stream, B,
                   (size_t)I.n * k * sizeof(T), dev, (int)I.m, k, p->row_ptr, col_idx, vals, B, Y, alpha, beta, kLongRow);
   if (rc != B200SP_OK || p->num_long == 0) return rc;
   const long long ctas = (long long)((k + 8 * VEC - 1) / (8 * VEC)) * p->num_long;
@@ -196,6 +198,7 @@ int launch_spmm_bstage_quads(b200sp_plan* p, int k, const int32_t* col_idx, cons
                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS) return B200SP_ERR_UNSUPPORTED;
   int rc = plan_quad_order(p, GPW, stream, dev);
+  if (rc == B200SP_OK) rc = plan_row_lists(p, stream, dev);
   if (rc != B200SP_OK) return rc;
   auto kernel = spmm_bstage_quads_kernel<T, VEC, LANES, THREADS>;
   static bool configured[64] = {};
@@ -345,15 +348,14 @@ int run_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals,
   int v = 1;
   while (v < VMAX && k % (2 * v) == 0 && 32 * v < k) v *= 2;
   if (!p->spmm_split) {   // shares: once per plan, a small kernel in stream order
-    int w = kMergeWarpItems, per_warp = kMergeShares;
-    while (per_warp > 1 && I.m + I.nnz < (int64_t)dev->sms * 128 * w * per_warp) per_warp /= 2;   // fewer and shorter shares for small problems,
-    while (w > 32 && I.m + I.nnz < (int64_t)dev->sms * 48 * w) w /= 2;                            // so that every SM has enough warps
-    const long long shares = (I.m + I.nnz + w - 1) / w;
-    int rc = pool_alloc(dev, (void**)&p->spmm_split, (size_t)(shares + 1) * sizeof(int32_t), stream);
+    int w = 0, per_warp = 0;
+    const long long shares = spmm_shares(I, dev, &w, &per_warp);
+    int rc = pool_alloc(dev, &p->split_block, (size_t)(shares + 1) * sizeof(int32_t), stream);
     if (rc != B200SP_OK) return rc;
     rc = launch(plan_merge_split_kernel, dim3((unsigned)((shares + 1 + 255) / 256)), dim3(256), stream, nullptr, 0, dev, p->row_ptr, (int)I.m,
-                (int)I.nnz, w, (int)shares, (int*)p->spmm_split);
+                (int)I.nnz, w, (int)shares, (int*)p->split_block);
     if (rc != B200SP_OK) return rc;
+    p->spmm_split = (int32_t*)p->split_block;
     p->spmm_witems = w;
     p->spmm_shares = per_warp;
   }
@@ -420,7 +422,8 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     const int slices = (k + KS - 1) / KS;
     const int row_blocks = (int)((I.m + GROUPS - 1) / GROUPS);
     if ((long long)slices * row_blocks >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
-    int rc;
+    int rc = plan_row_lists(p, stream, dev);
+    if (rc != B200SP_OK) return rc;
     const int mid_blocks = (p->num_medium + GROUPS - 1) / GROUPS;
     int ranges = 1;
     if (lanes == 8) {

@@ -1,0 +1,58 @@
+"""The plan pass (statistics written to pinned memory by its last block): sizes around its block and grid edges, passes one after
+another (the accumulators must come back clean) and from several threads at once."""
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2603_07169_b200 as b200sp
+
+pytestmark = pytest.mark.gpu
+EDGES = [(0, 0), (1, 4), (5, 32), (33, 128), (129, 1024), (1025, 1 << 30)]
+
+
+def expect(lens):
+    rows = [int(((lens >= a) & (lens <= b)).sum()) for a, b in EDGES]
+    nnz = [int(lens[(lens >= a) & (lens <= b)].sum()) for a, b in EDGES]
+    return int(lens.min()), int(lens.max()), rows, nnz
+
+
+def check(lens, stream=None):
+    row_ptr = torch.from_numpy(np.concatenate([[0], lens.cumsum()]).astype(np.int32)).to("cuda:0")
+    torch.cuda.synchronize()
+    plan = b200sp.b200sp_plan_create(len(lens), 1 << 20, int(lens.sum()), row_ptr, stream)
+    info = b200sp.b200sp_plan_info(plan)
+    b200sp.b200sp_plan_destroy(plan)
+    assert (info["min_row_len"], info["max_row_len"], info["bin_rows"], info["bin_nnz"]) == expect(lens)
+
+
+def lengths(m, seed):
+    rng = np.random.default_rng(seed)
+    return rng.choice([0, 1, 4, 5, 32, 33, 128, 129, 700, 1024, 1025, 3000], m, p=[.2, .2, .1, .1, .1, .1, .05, .05, .04, .03, .02, .01]).astype(np.int64)
+
+
+@pytest.mark.parametrize("m", [1, 31, 255, 256, 257, 1023, 1024, 1025, 4097, 1_300_000])
+def test_statistics_match_numpy(m):
+    for seed in range(3):
+        check(lengths(m, seed))
+    check(np.full(m, 7, np.int64))       # nothing left over from the passes before
+
+
+def test_passes_from_several_threads():
+    failures = []
+
+    def work(i):
+        try:
+            s = torch.cuda.Stream()
+            for j in range(20):
+                check(lengths(1000 * i + 17 * j + 1, j), s)
+        except BaseException as e:      # noqa: BLE001 - reported below
+            failures.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(6)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failures, failures[0]
