@@ -491,19 +491,25 @@ int b200sp_cache_drop(const void* key_ptr) {
   std::vector<void*> blocks;
   {
     std::lock_guard<std::mutex> lock(g_mutex);
-    for (auto it = g_cache.begin(); it != g_cache.end();) {
-      if (std::get<0>(it->first) == dev && std::get<1>(it->first) == key_ptr) { plans.push_back(it->second.plan); it = g_cache.erase(it); }
-      else ++it;
-    }
+    std::vector<const void*> row_ptrs{key_ptr};   // plans are cached under the row offsets that a dropped COO or CSC entry owned as well
     for (auto it = g_coo_cache.begin(); it != g_coo_cache.end();) {
-      if (std::get<0>(it->first) == dev && std::get<1>(it->first) == key_ptr) { blocks.push_back(it->second.row_ptr); it = g_coo_cache.erase(it); }
+      if (std::get<0>(it->first) == dev && std::get<1>(it->first) == key_ptr) {
+        blocks.push_back(it->second.row_ptr);
+        row_ptrs.push_back(it->second.row_ptr);
+        it = g_coo_cache.erase(it);
+      }
       else ++it;
     }
     for (auto it = g_csc_cache.begin(); it != g_csc_cache.end();) {
       if (std::get<0>(it->first) == dev && std::get<1>(it->first) == key_ptr) {
-        blocks.push_back(it->second.block);
+        for (void* q : {it->second.block, it->second.csr_block, it->second.prod_block}) blocks.push_back(q);
+        row_ptrs.push_back(it->second.row_ptr);
         it = g_csc_cache.erase(it);
       } else ++it;
+    }
+    for (auto it = g_cache.begin(); it != g_cache.end();) {
+      if (std::get<0>(it->first) == dev && std::find(row_ptrs.begin(), row_ptrs.end(), std::get<1>(it->first)) != row_ptrs.end()) { plans.push_back(it->second.plan); it = g_cache.erase(it); }
+      else ++it;
     }
   }
   int rc = B200SP_OK;

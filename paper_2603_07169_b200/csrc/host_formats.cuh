@@ -3,6 +3,7 @@
 #pragma once
 #include "host_spmm.cuh"
 #include "format_kernels.cuh"
+#include "csc_kernels.cuh"
 
 // ---- COO front end: row offsets from sorted row indices, then the CSR path ----
 struct CooEntry { int32_t* row_ptr = nullptr; };
@@ -46,17 +47,32 @@ static int coo_row_ptr(const int32_t** out, int64_t m, int64_t n, int64_t nnz, c
   return B200SP_OK;
 }
 
-// ---- CSC front end: a transpose plan built on the device (see format_kernels.cuh), then the CSR path ----
-// One pool block per pattern: row offsets, columns and CSC positions in row-major order, and room for the permuted values.
-struct CscEntry { void* block = nullptr; int32_t* row_ptr = nullptr; int32_t* col = nullptr; int32_t* perm = nullptr; void* vals_t = nullptr; };
+// ---- CSC front end: a transpose plan built on the device (see format_kernels.cuh and csc_kernels.cuh) ----
+// Per pattern: row offsets and CSC positions in row-major order; for SpMV the places of the products (csc_kernels.cuh); for SpMM, and
+// for SpMV where those do not apply, the columns in row-major order and room for the permuted values.  The last two are built on first use.
+struct CscEntry {
+  void* block = nullptr;
+  int32_t* row_ptr = nullptr;
+  int32_t* perm = nullptr;
+  void* csr_block = nullptr;
+  int32_t* col = nullptr;
+  void* vals_t = nullptr;
+  void* prod_block = nullptr;
+  bool prod_tried = false;
+  int tile = 0, tiles = 0, buckets = 0, cap = 0;
+  int *bucket_row = nullptr, *bucket_start = nullptr, *tile_col = nullptr, *run_shift = nullptr;
+  unsigned short *src = nullptr, *dst = nullptr, *dcol = nullptr, *run_before = nullptr;
+  float* prod = nullptr;
+};
 static std::map<std::tuple<int, const void*, const void*, int64_t, int64_t, int64_t>, CscEntry> g_csc_cache;
+static std::mutex g_csc_build;      // one thread at a time adds parts to an entry
 
 static void csc_free(CscEntry& e) {
-  if (e.block) cudaFree(e.block);
+  for (void* b : {e.block, e.csr_block, e.prod_block}) if (b) cudaFree(b);
   e = CscEntry();
 }
 
-static int csc_plan(CscEntry* out, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr, const int32_t* row_idx, cudaStream_t stream) {
+static int csc_plan(CscEntry** out, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr, const int32_t* row_idx, cudaStream_t stream) {
   DeviceInfo* dev = nullptr;
   int rc = device_info(&dev);
   if (rc != B200SP_OK) return rc;
@@ -66,21 +82,18 @@ static int csc_plan(CscEntry* out, int64_t m, int64_t n, int64_t nnz, const int3
   {
     std::lock_guard<std::mutex> lock(g_mutex);
     auto it = g_csc_cache.find(key);
-    if (it != g_csc_cache.end()) { *out = it->second; return B200SP_OK; }
+    if (it != g_csc_cache.end()) { *out = &it->second; return B200SP_OK; }
   }
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
   const size_t nz = nnz > 0 ? (size_t)nnz : 1;
   const size_t blocks = (size_t)((m + 1 + kScanBlock - 1) / kScanBlock);
-  const size_t o_rp = 0, o_col = o_rp + up(((size_t)m + 2) * 4), o_perm = o_col + up(nz * 4), o_vals = o_perm + up(nz * 4),
-               o_fill = o_vals + up(nz * 4), o_bs = o_fill + up(((size_t)m + 2) * 4), o_bad = o_bs + up((blocks + 1) * 4), total = o_bad + 256;
+  const size_t o_rp = 0, o_perm = o_rp + up(((size_t)m + 2) * 4), o_fill = o_perm + up(nz * 4), o_bs = o_fill + up(((size_t)m + 2) * 4), o_bad = o_bs + up((blocks + 1) * 4), total = o_bad + 256;
   CscEntry e;
   rc = pool_alloc(dev, &e.block, total, stream);
   if (rc != B200SP_OK) return rc;
   char* base = (char*)e.block;
   e.row_ptr = (int32_t*)(base + o_rp);
-  e.col = (int32_t*)(base + o_col);
   e.perm = (int32_t*)(base + o_perm);
-  e.vals_t = base + o_vals;
   int* fill = (int*)(base + o_fill);
   int* bsum = (int*)(base + o_bs);
   int* d_bad = (int*)(base + o_bad);
@@ -108,17 +121,138 @@ static int csc_plan(CscEntry* out, int64_t m, int64_t n, int64_t nnz, const int3
   if (nnz > 0) {
     csc_place_kernel<<<grid_for(nnz), 256, 0, stream>>>(row_idx, (long long)nnz, e.row_ptr, fill, e.perm);
     csc_sort_rows_kernel<<<(unsigned)((m + 255) / 256), 256, 0, stream>>>((int)m, e.row_ptr, e.perm);
-    csc_cols_kernel<<<grid_for(nnz), 256, 0, stream>>>((long long)nnz, (int)n, col_ptr, e.perm, e.col);
-    g_launches += 3;
+    g_launches += 2;
     CUF(cudaGetLastError());
   }
   CUF(cudaStreamSynchronize(stream));
 #undef CUF
   std::lock_guard<std::mutex> lock(g_mutex);
   auto ins = g_csc_cache.emplace(key, e);
-  if (!ins.second) { cudaFreeAsync(e.block, stream); e = ins.first->second; }
-  *out = e;
+  if (!ins.second) cudaFreeAsync(e.block, stream);
+  *out = &ins.first->second;
   return B200SP_OK;
+}
+
+// Columns in row-major order and room for the permuted values: what the CSR kernels need.
+static int csc_csr_part(CscEntry* e, int64_t n, int64_t nnz, const int32_t* col_ptr, cudaStream_t stream, DeviceInfo* dev) {
+  std::lock_guard<std::mutex> lock(g_csc_build);
+  if (e->csr_block) return B200SP_OK;
+  const size_t bytes = ((size_t)(nnz > 0 ? nnz : 1) * 4 + 255) & ~(size_t)255;
+  void* blk = nullptr;
+  const int rc = pool_alloc(dev, &blk, 2 * bytes, stream);
+  if (rc != B200SP_OK) return rc;
+  if (nnz > 0) {
+    long long blocks = (nnz + 255) / 256;
+    if (blocks > (long long)dev->sms * 16) blocks = (long long)dev->sms * 16;
+    csc_cols_kernel<<<(unsigned)blocks, 256, 0, stream>>>((long long)nnz, (int)n, col_ptr, e->perm, (int*)blk);
+    g_launches++;
+    const cudaError_t err = cudaGetLastError();
+    if (err != cudaSuccess) { cudaFreeAsync(blk, stream); return cuda_fail(err, "CSC columns"); }
+  }
+  e->col = (int32_t*)blk;
+  e->vals_t = (char*)blk + bytes;
+  e->csr_block = blk;
+  return B200SP_OK;
+}
+
+// The places of the products of csc_kernels.cuh; leaves e->prod_block null where they do not apply.  Synchronises the stream once.
+// Sizes: below 4.8 M nonzeros tiles and buckets of 2048 or 4096, so that every SM gets several; else one tile of 24576 .. 32768 entries
+// per SM and round (96 .. 128 KB of products), the size that leaves the least of the last round idle, and buckets of 8192 nonzeros,
+// 16384 above 2^25.  A run (a tile's products for one bucket) then averages tile * C / nnz = 3.5 .. 55 words: 2^24 nonzeros take 78 us,
+// 81 us with tiles of 32768, 84 us with two tiles of 16384 per SM.  Above 2^26
+// nonzeros, with a row of more than kCscSlack nonzeros or a tile over more than 65536 columns, SpMV takes the CSR kernels.
+static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr, const int32_t* row_idx, cudaStream_t stream,
+                            DeviceInfo* dev) {
+  std::lock_guard<std::mutex> lock(g_csc_build);
+  if (e->prod_tried) return B200SP_OK;
+  if (nnz <= 0 || nnz > ((int64_t)1 << 26)) { e->prod_tried = true; return B200SP_OK; }
+  const int64_t sms = dev->sms;
+  int tile = nnz < sms * 4 * 2048 ? 2048 : 4096;
+  if (nnz >= sms * 8 * 4096) {
+    int64_t best = INT64_MAX;
+    for (int t : {32768, 28672, 24576}) {
+      const int64_t time = (((nnz + t - 1) / t + sms - 1) / sms) * t;     // rounds of one tile per SM
+      if (time < best) { best = time; tile = t; }
+    }
+  }
+  const int shift = nnz < sms * 4 * 2048 ? 11 : nnz < sms * 8 * 4096 ? 12 : nnz <= ((int64_t)1 << 25) ? 13 : 14;
+  const int tiles = (int)((nnz + tile - 1) / tile), buckets = (int)(((nnz - 1) >> shift) + 1), cap = (1 << shift) + kCscSlack;
+  if (buckets > kCscMaxBuckets) { e->prod_tried = true; return B200SP_OK; }
+  auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  const size_t nz = (size_t)tiles * tile;
+  const size_t o_src = 0, o_dst = o_src + up(nz * 2), o_dcol = o_dst + up(nz * 2), o_before = o_dcol + up(nz * 2), o_shift = o_before + up(nz / 32 * 2),
+               o_brow = o_shift + up((size_t)tiles * buckets * 4), o_bstart = o_brow + up((size_t)(buckets + 1) * 4), o_tcol = o_bstart + up((size_t)(buckets + 1) * 4), o_prod = o_tcol + up((size_t)tiles * 4),
+               total = o_prod + up(nz * 4);
+  char* blk = nullptr;
+  int rc = pool_alloc(dev, (void**)&blk, total, stream);
+  if (rc != B200SP_OK) return rc;
+  auto fail = [&](int code) { cudaFreeAsync(blk, stream); cudaStreamSynchronize(stream); return code; };
+#define CUP(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) return fail(cuda_fail(e_, #call)); } while (0)
+  int* stat = (int*)(blk + o_before);            // not needed yet
+  int* count = (int*)(blk + o_shift);            // counts, then starts, then shifts of the runs
+  int* place = (int*)(blk + o_prod);             // the products come later
+  int* brow = (int*)(blk + o_brow);
+  int* tcol = (int*)(blk + o_tcol);
+  int h[2] = {0, 0};
+  CUP(cudaMemsetAsync(stat, 0, 2 * sizeof(int), stream));
+  csc_bucket_rows_plan<<<(buckets + 1 + 255) / 256, 256, 0, stream>>>(e->row_ptr, (int)m, buckets, shift, brow, (int*)(blk + o_bstart));
+  const int wider = buckets > tiles ? buckets : tiles;
+  csc_extents_plan<<<(wider + 255) / 256, 256, 0, stream>>>(e->row_ptr, brow, buckets, col_ptr, (int)n, (int)nnz, tile, tiles, tcol, stat);
+  g_launches += 2;
+  CUP(cudaGetLastError());
+  CUP(cudaMemcpyAsync(h, stat, sizeof h, cudaMemcpyDeviceToHost, stream));
+  CUP(cudaStreamSynchronize(stream));
+  if (h[0] > cap || h[1] > 65535) { e->prod_tried = true; return fail(B200SP_OK); }
+  const size_t slots_smem = (size_t)buckets * 12 + (size_t)tile * 2;
+  CUP(cudaFuncSetAttribute(csc_tile_slots_plan, cudaFuncAttributeMaxDynamicSharedMemorySize, kCscMaxBuckets * 12 + kCscMaxTile * 2));
+  csc_tile_counts_plan<<<tiles, 512, (size_t)buckets * 4, stream>>>(row_idx, e->row_ptr, (int)nnz, tile, shift, buckets, count);
+  csc_run_starts_plan<<<(buckets + 31) / 32, 1024, 0, stream>>>(e->row_ptr, brow, buckets, tiles, count);
+  csc_tile_slots_plan<<<tiles, 1024, slots_smem, stream>>>(row_idx, e->row_ptr, col_ptr, tcol, (int)n, (int)nnz, tile, shift, buckets,
+                                                          (unsigned short*)(blk + o_src), (unsigned short*)(blk + o_before), count,
+                                                          (unsigned short*)(blk + o_dcol), place);
+  csc_bucket_places_plan<<<buckets, 512, 0, stream>>>(brow, e->row_ptr, e->perm, place, (unsigned short*)(blk + o_dst));
+  g_launches += 4;
+  CUP(cudaGetLastError());
+#undef CUP
+  e->tile = tile; e->tiles = tiles; e->buckets = buckets; e->cap = cap;
+  e->bucket_row = brow; e->bucket_start = (int*)(blk + o_bstart); e->tile_col = tcol; e->run_shift = (int*)(blk + o_shift);
+  e->src = (unsigned short*)(blk + o_src); e->dst = (unsigned short*)(blk + o_dst); e->dcol = (unsigned short*)(blk + o_dcol);
+  e->run_before = (unsigned short*)(blk + o_before);
+  e->prod = (float*)(blk + o_prod);
+  e->prod_block = blk;
+  e->prod_tried = true;
+  return B200SP_OK;
+}
+
+template <typename T, int TILE, int THREADS>
+static int launch_csc_products(const CscEntry* e, int64_t nnz, const T* vals, const T* x, cudaStream_t stream, DeviceInfo* dev) {
+  auto kernel = csc_products_kernel<T, TILE, THREADS>;
+  const size_t smem = (size_t)e->tile * 4 + (size_t)e->buckets * 4;
+  CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCscMaxTile * 4 + kCscMaxBuckets * 4));
+  tl_pdl_kernel = true;
+  return launch_smem(kernel, dim3((unsigned)e->tiles), dim3(THREADS), smem, stream, nullptr, 0, dev, (int)nnz, e->buckets, vals, x,
+                     (const unsigned short*)e->dcol, (const int*)e->tile_col, (const unsigned short*)e->src, (const unsigned short*)e->run_before,
+                     (const int*)e->run_shift, e->prod);
+}
+
+// SpMV by products: two launches.
+template <typename T>
+static int run_csc_products(const CscEntry* e, int64_t nnz, const T* vals, const T* x, T* y, float alpha, float beta, cudaStream_t stream, DeviceInfo* dev) {
+  int rc;
+  switch (e->tile) {
+    case 2048: rc = launch_csc_products<T, 2048, 512>(e, nnz, vals, x, stream, dev); break;
+    case 4096: rc = launch_csc_products<T, 4096, 512>(e, nnz, vals, x, stream, dev); break;
+    case 24576: rc = launch_csc_products<T, 24576, 1024>(e, nnz, vals, x, stream, dev); break;
+    case 28672: rc = launch_csc_products<T, 28672, 1024>(e, nnz, vals, x, stream, dev); break;
+    default: rc = launch_csc_products<T, 32768, 1024>(e, nnz, vals, x, stream, dev); break;
+  }
+  if (rc != B200SP_OK) return rc;
+  auto kernel = csc_bucket_sums_kernel<T>;
+  const size_t smem = (size_t)(e->cap + e->cap / 32 + 2) * 4 + (size_t)(e->cap / (kCscShortRow + 1) + 1) * 4;
+  CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+  tl_pdl_kernel = true;
+  return launch_smem(kernel, dim3((unsigned)e->buckets), dim3(kCscThreads), smem, stream, nullptr, 0, dev, e->cap, (const int*)e->bucket_row,
+                     (const int*)e->bucket_start, (const int*)e->row_ptr, (const float*)e->prod, (const unsigned short*)e->dst, y, alpha, beta);
 }
 
 static int csc_call(bool is_mm, int64_t m, int64_t n, int64_t nnz, int64_t k, const int32_t* col_ptr, const int32_t* row_idx, const void* vals,
@@ -133,9 +267,19 @@ static int csc_call(bool is_mm, int64_t m, int64_t n, int64_t nnz, int64_t k, co
   rc = device_info(&dev);
   if (rc != B200SP_OK) return rc;
   cudaStream_t stream = (cudaStream_t)stream_v;
-  CscEntry e;
-  rc = csc_plan(&e, m, n, nnz, col_ptr, row_idx, stream);
+  CscEntry* entry = nullptr;
+  rc = csc_plan(&entry, m, n, nnz, col_ptr, row_idx, stream);
   if (rc != B200SP_OK) return rc;
+  if (!is_mm && nnz > 0 && alpha != 0.0f && in && out && aligned16(vals) && aligned16(in) && aligned16(out)) {
+    rc = csc_product_part(entry, m, n, nnz, col_ptr, row_idx, stream, dev);
+    if (rc != B200SP_OK) return rc;
+    if (entry->prod_block)
+      return dtype == B200SP_F32 ? run_csc_products<float>(entry, nnz, (const float*)vals, (const float*)in, (float*)out, alpha, beta, stream, dev)
+                                 : run_csc_products<bf16_t>(entry, nnz, (const bf16_t*)vals, (const bf16_t*)in, (bf16_t*)out, alpha, beta, stream, dev);
+  }
+  rc = csc_csr_part(entry, n, nnz, col_ptr, stream, dev);
+  if (rc != B200SP_OK) return rc;
+  const CscEntry& e = *entry;
   if (nnz > 0) {
     long long blocks = (nnz + 255) / 256;
     if (blocks > (long long)dev->sms * 16) blocks = (long long)dev->sms * 16;

@@ -111,11 +111,18 @@ constexpr int kMergeWarps = 8;       // warps per CTA of spmm_merge_kernel
 constexpr int kMergeWarpItems = 128; // most merge items per share
 constexpr int kMergeShares = 4;      // most consecutive shares per warp
 
-// Resident CTAs per SM that the registers are capped for, by the registers the loads in flight and the sums take.
+// Nonzeros whose loads of B (J each) are in flight per warp: 8 loads, 16 where a nonzero takes four of them (100,000 uneven rows, k = 127
+// FP32: 84 us against 89 us with 8; with one or two loads per nonzero 16 in flight are slower).
+template <int V, int J>
+constexpr int kMergeUnroll = J >= 4 ? (V >= 4 ? 2 : 4) : 8 / J;
+
+// Resident CTAs per SM that the registers are capped for, by the registers the loads in flight and the sums take: warps resident, not
+// loads per warp, hide the latency (R-MAT 2^22, k = 64 FP32: 828 us with 6 CTAs, 854 us with 5), as long as little spills.  (Two or four
+// nonzeros per step on half or quarter warps, 16 bytes per lane, measured 905 us: the sums of the halves at every row end cost more.)
 template <typename T, int V, int J>
 constexpr int merge_ctas() {
-  constexpr int need = (8 * V * (int)sizeof(T) + 3) / 4 + 2 * V * J;
-  return need <= 20 ? 5 : need <= 40 ? 4 : 3;
+  constexpr int need = kMergeUnroll<V, J> * J * ((V * (int)sizeof(T) + 3) / 4) + 2 * V * J;
+  return need <= 20 ? 6 : need <= 24 ? 5 : need <= 40 ? 4 : 3;
 }
 
 // What a warp keeps in shared memory of one share: its columns, its values and the ends of its rows, and room to read a group ahead.
@@ -133,7 +140,7 @@ template <> struct MergeStage<bf16_t> {
 
 // A warp takes `shares` consecutive shares; the (col, val) pairs and row ends of the next one arrive in shared memory (cp.async)
 // while it walks the current one.  Lane l holds columns slice * 32 * V * J + 32 * V * j + l * V + (0 .. V-1), j < J, of the current
-// row in FP32 registers (acc: products of the current share; tot: of the row's earlier shares); U = 8 / J nonzeros, 8 loads of B, are
+// row in FP32 registers (acc: products of the current share; tot: of the row's earlier shares); U nonzeros, U J loads of B, are
 // in flight.  A warp leaves two partial sums in shared memory: `head` for a first row that began before its shares, `carry` for
 // the row it leaves unfinished; after one barrier the warp that holds a row's end adds the carries of the warps before it in
 // order, and what crosses the CTA's own ends goes to tile_tail / tile_carry and is finished by spmm_merge_fixup_kernel.  No
@@ -144,7 +151,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32, (merge_ctas<T, V, J>()))
 spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, const int* __restrict__ split, const int* __restrict__ row_ptr,
                   const int* __restrict__ col_idx, const T* __restrict__ vals, const T* __restrict__ B, T* __restrict__ Y,
                   float* __restrict__ tile_carry, float* __restrict__ tile_tail, float alpha, float beta) {
-  constexpr int U = 8 / J, KS = 32 * V * J;
+  constexpr int U = kMergeUnroll<V, J>, KS = 32 * V * J;
   typedef typename Piece<T, V>::raw raw;
   __shared__ __align__(16) MergeStage<T> stage_s[kMergeWarps][2];
   __shared__ __align__(16) float wide_s[sizeof(T) == 2 ? kMergeWarps : 1][sizeof(T) == 2 ? kMergeWarpItems + 8 : 4];   // BF16: the current share's values widened
@@ -181,7 +188,7 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
         if (i + lane < words) cp_async4(&st.raw[i + lane], vals + w0 + 2 * (i + lane), min(4, 2 * (nnz - w0 - 2 * (i + lane))));
     }
     if (lane < U) st.col[cnt + lane] = 0;                    // read ahead of the end, never multiplied
-    if (lane == 0) st.end[rows] = 0x7FFFFFFF;
+    if (lane == 0) st.end[rows] = (int)((unsigned)p0 + 0x100000u);   // no end inside this share
   };
 
   const int col0 = slice * KS + lane * V;
@@ -219,8 +226,8 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
     } else {
       vls = st.val;
     }
-    const int* const ends = st.end;
-    int j_row = 0, end = uniform(ends[0]) - p0;              // the current row ends before nonzero `end` of the share
+    auto share_end = [&](int j) { return (int)((unsigned)uniform(st.end[j]) - (unsigned)p0); };
+    int j_row = 0, end = share_end(0);             // the current row ends before nonzero `end` of the share
     // the current row has been added up to its end: stored, or left as the warp's head when it began earlier
     auto finish_row = [&]() {
 #pragma unroll
@@ -242,7 +249,7 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
 #pragma unroll
         for (int i = 0; i < V; ++i) acc[j][i] = 0.0f;
       yp += k;
-      end = uniform(ends[++j_row]) - p0;
+      end = share_end(++j_row);
     };
     for (int q = 0; q < cnt; q += U) {
       int c[U];

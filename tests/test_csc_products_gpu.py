@@ -1,0 +1,105 @@
+"""SpMV of CSC matrices by products written in runs (csc_kernels.cuh): every tile and bucket size, ragged ends, rows and columns at the
+limits of the path and beyond them (where the CSR kernels take over), and reproducible sums."""
+import numpy as np
+import pytest
+import torch
+
+import gen
+import oracle
+import paper_2603_07169_b200 as b200sp
+from gpu_util import assert_within, empty_out, store, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+def matrices():
+    rng = np.random.default_rng(12)
+    tail = np.zeros(4000, np.int64)
+    tail[:50] = 30
+    return {
+        "one_entry": (np.array([0, 1, 0]), 5),
+        "tile_less_one": (np.full(23, 89), 300),                  # 2047 nonzeros
+        "tile_exact": (np.full(32, 64), 300),                     # 2048 nonzeros: one tile, one bucket
+        "tile_plus_one": (np.full(3, 683), 900),                  # 2049 nonzeros
+        "rows_at_the_limit": (np.array([1024] * 5 + [0, 1, 1024, 33, 32]), 2000),
+        "row_over_the_limit": (np.array([1025] + [3] * 500), 2000),   # a bucket may still hold it
+        "row_far_over": (np.array([5000] + [3] * 2000), 6000),    # CSR kernels
+        "wide_tile": (np.full(3000, 2), 900_000),                 # a tile spans more than 65536 columns: CSR kernels
+        "trailing_empty_rows": (tail, 100),
+        "power_law": ((rng.pareto(1.5, 30_000) * 2).astype(np.int64).clip(0, 900), 20_000),
+        "tile_4096": (rng.integers(0, 30, 100_000), 50_000),
+        "tile_24576": (16, 328_000),                              # 5.2 M nonzeros (equal rows: drawn by the fast generator)
+        "tile_28672": (16, 500_000),
+        "tile_32768": (16, 560_000),
+    }
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("case", sorted(matrices()))
+def test_csc_products_against_oracle(case, dtype):
+    lens, n = matrices()[case]
+    A = gen.uniform_rows(n, n, lens, 3) if isinstance(lens, int) else gen.random_csr(len(lens), n, lens, seed=3, sort_cols=True)
+    rng = np.random.default_rng(1)
+    cp, ri, va = gen.csr_to_csc(A)
+    v_s, x_s, y0_s = store(va, dtype), store(rng.standard_normal(n).astype(np.float32), dtype), store(rng.standard_normal(A.m).astype(np.float32), dtype)
+    d = [to_dev(a) for a in (cp, ri, v_s, x_s)]
+    y_ref, S = oracle.spmm_csc(A.m, n, 1, cp, ri, v_s, x_s, None, 1.0, 0.0, dtype)
+    outs = []
+    for _ in range(2):
+        y = empty_out(A.m, dtype)
+        b200sp.spmv_csc(A.m, n, A.nnz, d[0], d[1], d[2], d[3], y, 1.0, 0.0, dtype)
+        outs.append(to_host(y, dtype))
+        b200sp.b200sp_cache_drop(d[0])                            # the second pass plans again: the same sums in the same order
+    assert_within(outs[0], y_ref[:, 0], S[:, 0], dtype, what=case)
+    assert np.array_equal(outs[0], outs[1])
+    y = to_dev(y0_s).clone()
+    b200sp.spmv_csc(A.m, n, A.nnz, d[0], d[1], d[2], d[3], y, -0.5, 1.25, dtype)
+    y_ref, S = oracle.spmm_csc(A.m, n, 1, cp, ri, v_s, x_s, y0_s, -0.5, 1.25, dtype)
+    y0f = y0_s if dtype == "f32" else gen.bf16_to_f32(y0_s)
+    assert_within(to_host(y, dtype), y_ref[:, 0], S[:, 0], dtype, 1.0, np.abs(1.25 * y0f.astype(np.float64)), what=case + " ab")
+    b200sp.b200sp_cache_clear()
+
+
+@pytest.mark.parametrize("per_row", [31, 33])
+def test_csc_products_around_the_largest_bucket_size(per_row):
+    """2^20 rows: nonzeros on both sides of 2^25, where buckets double; against 64-bit sums on the GPU."""
+    m = 1 << 20
+    g = torch.Generator("cuda").manual_seed(per_row)
+    row = torch.arange(m, device="cuda").repeat_interleave(per_row)
+    col = torch.randint(0, m, (m * per_row,), generator=g, device="cuda")
+    key = (col * m + row).sort().values
+    col, row = key // m, (key % m).int()
+    cp = torch.searchsorted(col, torch.arange(m + 1, device="cuda")).int()
+    vals = torch.randn(m * per_row, generator=g, device="cuda")
+    x = torch.randn(m, generator=g, device="cuda")
+    y = torch.full((m,), float("nan"), device="cuda")
+    b200sp.spmv_csc(m, m, m * per_row, cp, row, vals, x, y, 1.0, 0.0, "f32")
+    p = vals.double() * x.double()[col]
+    ref = torch.zeros(m, dtype=torch.float64, device="cuda").index_add_(0, row.long(), p)
+    S = torch.zeros(m, dtype=torch.float64, device="cuda").index_add_(0, row.long(), p.abs())
+    assert float(((y.double() - ref).abs() / (1e-5 * S + 1e-30)).max()) <= 1.0
+    b200sp.b200sp_cache_clear()
+
+
+def test_dropping_a_csc_pattern_drops_the_plans_of_its_row_offsets():
+    """Two patterns of the same sizes one after another under one address: the second must not meet anything of the first."""
+    rng = np.random.default_rng(4)
+    m, n = 4000, 3000
+    lens1 = np.full(m, 8)
+    lens2 = rng.integers(0, 17, m)
+    lens2[:8] += 1500                                             # too long for the products: the CSR kernels and their plan
+    lens1[0] += lens2.sum() - lens1.sum()
+    ptr = None
+    for lens in (lens1, lens2, lens1):
+        A = gen.random_csr(m, n, lens, seed=2, sort_cols=True)
+        cp, ri, va = gen.csr_to_csc(A)
+        x = rng.standard_normal(n).astype(np.float32)
+        if ptr is None:
+            ptr, idx = to_dev(cp), to_dev(ri)
+        ptr.copy_(torch.from_numpy(cp)), idx.copy_(torch.from_numpy(ri))
+        y = empty_out(m, "f32")
+        b200sp.spmv_csc(m, n, A.nnz, ptr, idx, to_dev(va), to_dev(x), y, 1.0, 0.0, "f32")
+        y_ref, S = oracle.spmm_csc(m, n, 1, cp, ri, va, x, None, 1.0, 0.0, "f32")
+        assert_within(to_host(y, "f32"), y_ref[:, 0], S[:, 0], "f32")
+        b200sp.b200sp_cache_drop(ptr)
+    b200sp.b200sp_cache_clear()
