@@ -242,14 +242,14 @@ __device__ __forceinline__ int block_exclusive_sum(int v, int* s, int* total) {
   return (warp ? s[warp - 1] : 0) + incl - v;
 }
 
-// The slots of a tile: src, run_before, run_shift (see pass 1), the columns, and place_of[p]: where in the product buffer entry p goes.  One
-// CTA of 1024 threads per tile.  The order inside a run is arbitrary: place_of records it, and pass 2 undoes it.
+// The slots of a tile: src, run_before, run_shift (see pass 1), the columns, and position[i]: the CSC position of product i of the buffer.  One
+// CTA of 1024 threads per tile.  The order inside a run is arbitrary: pass 2 undoes it.
 // start: where the tile's run in each bucket begins; on return the shifts of its runs, one after another.
 // Dynamic shared memory: 3 * buckets ints, then tile 16-bit words.
 __global__ void __launch_bounds__(1024) csc_tile_slots_plan(const int* __restrict__ row_idx, const int* __restrict__ row_ptr, const int* __restrict__ col_ptr,
                                                             const int* __restrict__ tile_col, int n, int nnz, int tile, int shift, int buckets,
                                                             int unsigned short* __restrict__ src, unsigned short* __restrict__ run_before, int* start,
-                                                            unsigned short* __restrict__ dcol, int* __restrict__ place_of) {
+                                                            unsigned short* __restrict__ dcol, int* __restrict__ position) {
   extern __shared__ int csc_slots_smem[];
   __shared__ int s_scan[33];
   int* const cursor = csc_slots_smem;            // counts, then the next free slot of each run
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(1024) csc_tile_slots_plan(const int* __restric
     const int p = p0 + i, b = __ldg(row_ptr + row_idx[p]) >> shift;
     const int j = atomicAdd(&cursor[b], 1);
     src_s[j] = (unsigned short)(i | (j == first[b] ? 0x8000 : 0));
-    place_of[p] = p0 + j + shift_s[b];
+    position[p0 + j + shift_s[b]] = p;
     int lo = c0, hi = c1;                        // the last column with col_ptr <= p
     while (lo < hi) { const int mid = (lo + hi) >> 1; if (__ldg(col_ptr + mid + 1) <= p) lo = mid + 1; else hi = mid; }
     dcol[p] = (unsigned short)(lo - c0);
@@ -305,12 +305,37 @@ __global__ void __launch_bounds__(1024) csc_tile_slots_plan(const int* __restric
   }
 }
 
-// dst of the entry at row-major place q, whose CSC position is perm[q].  One CTA per bucket.
-__global__ void __launch_bounds__(512) csc_bucket_places_plan(const int* __restrict__ bucket_row, const int* __restrict__ row_ptr, const int* __restrict__ perm,
-                                                              const int* __restrict__ place_of, unsigned short* __restrict__ dst) {
-  const int s0 = row_ptr[bucket_row[blockIdx.x]], s1 = row_ptr[bucket_row[blockIdx.x + 1]];
+// dst: the place of the bucket's product i in row order, the entries of a row in the order of their CSC positions.  One CTA per bucket.
+// The positions go to their rows' ranges in shared memory in any order (slots claimed with atomics, on counters in shared memory
+// where the bucket has at most cap rows); an entry's place in its row is the number of smaller ones there.  Dynamic shared memory:
+// cap ints, cap pairs of 16 bits, cap ints.
+__global__ void __launch_bounds__(1024) csc_bucket_places_plan(int cap, const int* __restrict__ bucket_row, const int* __restrict__ bucket_start,
+                                                               const int* __restrict__ row_ptr, const int* __restrict__ row_idx,
+                                                               const int* __restrict__ position, int* __restrict__ fill, unsigned short* __restrict__ dst) {
+  extern __shared__ int csc_places_smem[];
+  int* const key_s = csc_places_smem;
+  ushort2* const row_s = (ushort2*)(key_s + cap);            // of product i: its row's range among the bucket's nonzeros
+  int* const claimed_s = (int*)(row_s + cap);
+  const int r0 = bucket_row[blockIdx.x], rows = bucket_row[blockIdx.x + 1] - r0;
+  const int s0 = bucket_start[blockIdx.x], cnt = bucket_start[blockIdx.x + 1] - s0;
+  const bool few = rows <= cap;
+  if (few) for (int i = threadIdx.x; i < rows; i += 1024) claimed_s[i] = 0;
+  __syncthreads();
 #pragma unroll 4
-  for (int q = s0 + threadIdx.x; q < s1; q += 512) dst[place_of[perm[q]]] = (unsigned short)(q - s0);
+  for (int i = threadIdx.x; i < cnt; i += 1024) {
+    const int p = position[s0 + i], r = row_idx[p];
+    const int rs = __ldg(row_ptr + r) - s0, re = __ldg(row_ptr + r + 1) - s0;
+    key_s[rs + (few ? atomicAdd(claimed_s + (r - r0), 1) : atomicAdd(fill + r, 1))] = p;
+    row_s[i] = make_ushort2((unsigned short)rs, (unsigned short)re);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < cnt; i += 1024) {
+    const int p = position[s0 + i], rs = row_s[i].x, re = row_s[i].y;
+    int place = rs;
+#pragma unroll 4
+    for (int q = rs; q < re; ++q) place += key_s[q] < p;
+    dst[s0 + i] = (unsigned short)place;
+  }
 }
 
 }  // namespace b200sp

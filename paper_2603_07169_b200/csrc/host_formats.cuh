@@ -48,13 +48,14 @@ static int coo_row_ptr(const int32_t** out, int64_t m, int64_t n, int64_t nnz, c
 }
 
 // ---- CSC front end: a transpose plan built on the device (see format_kernels.cuh and csc_kernels.cuh) ----
-// Per pattern: row offsets and CSC positions in row-major order; for SpMV the places of the products (csc_kernels.cuh); for SpMM, and
-// for SpMV where those do not apply, the columns in row-major order and room for the permuted values.  The last two are built on first use.
+// Per pattern: row offsets; for SpMV the places of the products (csc_kernels.cuh); for SpMM, and for SpMV where those do not apply, the
+// CSC positions and columns in row-major order and room for the permuted values.  The last two are built on first use.
 struct CscEntry {
   void* block = nullptr;
   int32_t* row_ptr = nullptr;
-  int32_t* perm = nullptr;
+  int32_t* fill = nullptr;            // m + 2 counters, for building the parts below
   void* csr_block = nullptr;
+  int32_t* perm = nullptr;
   int32_t* col = nullptr;
   void* vals_t = nullptr;
   void* prod_block = nullptr;
@@ -85,16 +86,15 @@ static int csc_plan(CscEntry** out, int64_t m, int64_t n, int64_t nnz, const int
     if (it != g_csc_cache.end()) { *out = &it->second; return B200SP_OK; }
   }
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-  const size_t nz = nnz > 0 ? (size_t)nnz : 1;
   const size_t blocks = (size_t)((m + 1 + kScanBlock - 1) / kScanBlock);
-  const size_t o_rp = 0, o_perm = o_rp + up(((size_t)m + 2) * 4), o_fill = o_perm + up(nz * 4), o_bs = o_fill + up(((size_t)m + 2) * 4), o_bad = o_bs + up((blocks + 1) * 4), total = o_bad + 256;
+  const size_t o_rp = 0, o_fill = o_rp + up(((size_t)m + 2) * 4), o_bs = o_fill + up(((size_t)m + 2) * 4), o_bad = o_bs + up((blocks + 1) * 4), total = o_bad + 256;
   CscEntry e;
   rc = pool_alloc(dev, &e.block, total, stream);
   if (rc != B200SP_OK) return rc;
   char* base = (char*)e.block;
   e.row_ptr = (int32_t*)(base + o_rp);
-  e.perm = (int32_t*)(base + o_perm);
-  int* fill = (int*)(base + o_fill);
+  e.fill = (int32_t*)(base + o_fill);
+  int* fill = e.fill;
   int* bsum = (int*)(base + o_bs);
   int* d_bad = (int*)(base + o_bad);
   int h_bad = 0;
@@ -117,13 +117,6 @@ static int csc_plan(CscEntry** out, int64_t m, int64_t n, int64_t nnz, const int
   scan_apply_kernel<<<(unsigned)blocks, 256, 0, stream>>>(fill, (long long)m + 1, bsum, e.row_ptr);
   g_launches += 4;
   CUF(cudaGetLastError());
-  CUF(cudaMemsetAsync(fill, 0, ((size_t)m + 2) * 4, stream));
-  if (nnz > 0) {
-    csc_place_kernel<<<grid_for(nnz), 256, 0, stream>>>(row_idx, (long long)nnz, e.row_ptr, fill, e.perm);
-    csc_sort_rows_kernel<<<(unsigned)((m + 255) / 256), 256, 0, stream>>>((int)m, e.row_ptr, e.perm);
-    g_launches += 2;
-    CUF(cudaGetLastError());
-  }
   CUF(cudaStreamSynchronize(stream));
 #undef CUF
   std::lock_guard<std::mutex> lock(g_mutex);
@@ -133,24 +126,33 @@ static int csc_plan(CscEntry** out, int64_t m, int64_t n, int64_t nnz, const int
   return B200SP_OK;
 }
 
-// Columns in row-major order and room for the permuted values: what the CSR kernels need.
-static int csc_csr_part(CscEntry* e, int64_t n, int64_t nnz, const int32_t* col_ptr, cudaStream_t stream, DeviceInfo* dev) {
+// CSC positions and columns in row-major order and room for the permuted values: what the CSR kernels need.
+static int csc_csr_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr, const int32_t* row_idx, cudaStream_t stream,
+                        DeviceInfo* dev) {
   std::lock_guard<std::mutex> lock(g_csc_build);
   if (e->csr_block) return B200SP_OK;
   const size_t bytes = ((size_t)(nnz > 0 ? nnz : 1) * 4 + 255) & ~(size_t)255;
-  void* blk = nullptr;
-  const int rc = pool_alloc(dev, &blk, 2 * bytes, stream);
+  char* blk = nullptr;
+  const int rc = pool_alloc(dev, (void**)&blk, 3 * bytes, stream);
   if (rc != B200SP_OK) return rc;
+  int* perm = (int*)blk;
+  int* col = (int*)(blk + bytes);
   if (nnz > 0) {
     long long blocks = (nnz + 255) / 256;
     if (blocks > (long long)dev->sms * 16) blocks = (long long)dev->sms * 16;
-    csc_cols_kernel<<<(unsigned)blocks, 256, 0, stream>>>((long long)nnz, (int)n, col_ptr, e->perm, (int*)blk);
-    g_launches++;
-    const cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) { cudaFreeAsync(blk, stream); return cuda_fail(err, "CSC columns"); }
+    cudaError_t err = cudaMemsetAsync(e->fill, 0, ((size_t)m + 2) * 4, stream);
+    if (err == cudaSuccess) {
+      csc_place_kernel<<<(unsigned)blocks, 256, 0, stream>>>(row_idx, (long long)nnz, e->row_ptr, e->fill, perm);
+      csc_sort_rows_kernel<<<(unsigned)((m + 255) / 256), 256, 0, stream>>>((int)m, e->row_ptr, perm);
+      csc_cols_kernel<<<(unsigned)blocks, 256, 0, stream>>>((long long)nnz, (int)n, col_ptr, perm, col);
+      g_launches += 3;
+      err = cudaGetLastError();
+    }
+    if (err != cudaSuccess) { cudaFreeAsync(blk, stream); return cuda_fail(err, "CSC row-major order"); }
   }
-  e->col = (int32_t*)blk;
-  e->vals_t = (char*)blk + bytes;
+  e->perm = perm;
+  e->col = col;
+  e->vals_t = blk + 2 * bytes;
   e->csr_block = blk;
   return B200SP_OK;
 }
@@ -190,7 +192,7 @@ static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, cons
 #define CUP(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) return fail(cuda_fail(e_, #call)); } while (0)
   int* stat = (int*)(blk + o_before);            // not needed yet
   int* count = (int*)(blk + o_shift);            // counts, then starts, then shifts of the runs
-  int* place = (int*)(blk + o_prod);             // the products come later
+  int* place = (int*)(blk + o_prod);             // the products' CSC positions; the products come later
   int* brow = (int*)(blk + o_brow);
   int* tcol = (int*)(blk + o_tcol);
   int h[2] = {0, 0};
@@ -210,7 +212,10 @@ static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, cons
   csc_tile_slots_plan<<<tiles, 1024, slots_smem, stream>>>(row_idx, e->row_ptr, col_ptr, tcol, (int)n, (int)nnz, tile, shift, buckets,
                                                           (unsigned short*)(blk + o_src), (unsigned short*)(blk + o_before), count,
                                                           (unsigned short*)(blk + o_dcol), place);
-  csc_bucket_places_plan<<<buckets, 512, 0, stream>>>(brow, e->row_ptr, e->perm, place, (unsigned short*)(blk + o_dst));
+  CUP(cudaMemsetAsync(e->fill, 0, ((size_t)m + 2) * 4, stream));
+  CUP(cudaFuncSetAttribute(csc_bucket_places_plan, cudaFuncAttributeMaxDynamicSharedMemorySize, ((1 << 14) + kCscSlack) * 12));
+  csc_bucket_places_plan<<<buckets, 1024, (size_t)cap * 12, stream>>>(cap, brow, (const int*)(blk + o_bstart), e->row_ptr, row_idx, place, e->fill,
+                                                                    (unsigned short*)(blk + o_dst));
   g_launches += 4;
   CUP(cudaGetLastError());
 #undef CUP
@@ -277,7 +282,7 @@ static int csc_call(bool is_mm, int64_t m, int64_t n, int64_t nnz, int64_t k, co
       return dtype == B200SP_F32 ? run_csc_products<float>(entry, nnz, (const float*)vals, (const float*)in, (float*)out, alpha, beta, stream, dev)
                                  : run_csc_products<bf16_t>(entry, nnz, (const bf16_t*)vals, (const bf16_t*)in, (bf16_t*)out, alpha, beta, stream, dev);
   }
-  rc = csc_csr_part(entry, n, nnz, col_ptr, stream, dev);
+  rc = csc_csr_part(entry, m, n, nnz, col_ptr, row_idx, stream, dev);
   if (rc != B200SP_OK) return rc;
   const CscEntry& e = *entry;
   if (nnz > 0) {

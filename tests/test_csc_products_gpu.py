@@ -26,6 +26,7 @@ def matrices():
         "row_far_over": (np.array([5000] + [3] * 2000), 6000),    # CSR kernels
         "wide_tile": (np.full(3000, 2), 900_000),                 # a tile spans more than 65536 columns: CSR kernels
         "trailing_empty_rows": (tail, 100),
+        "more_rows_than_a_bucket": (np.concatenate([tail, np.zeros(4000, np.int64), tail]), 100),
         "power_law": ((rng.pareto(1.5, 30_000) * 2).astype(np.int64).clip(0, 900), 20_000),
         "tile_4096": (rng.integers(0, 30, 100_000), 50_000),
         "tile_24576": (16, 328_000),                              # 5.2 M nonzeros (equal rows: drawn by the fast generator)
