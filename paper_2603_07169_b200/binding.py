@@ -128,6 +128,31 @@ def _ptr(t) -> Optional[int]:
     return t.ctypes.data
 
 
+_product = _ell_product = _plan_product = None      # csrc/marshal.cpp, and the library's entry points as addresses
+_address = {}
+
+
+def _load_native():
+    """Loads the native marshalling (built with the library): the checks below and the call in one step.  Its functions return the
+    library's status, or -1 for arguments they do not take as they stand; the Python code that follows each call then handles
+    them or raises the precise error."""
+    global _product, _ell_product, _plan_product
+    import importlib.util
+    import torch  # noqa: F401 - the extension resolves its symbols against the libraries that this loads
+    path = os.path.join(_HERE, "_marshal.so")
+    if not os.path.exists(path):
+        raise ImportError("_marshal.so is not built (%s); run `python -c 'import __graft_entry__ as g; g.build()'` "
+                          "or `python -m paper_2603_07169_b200.build`" % path)
+    spec = importlib.util.spec_from_file_location("_marshal", path)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    L = lib()
+    for name in ("spmv_csr", "spmm_csr", "spmv_csr_noalloc", "spmv_coo", "spmm_coo", "spmv_csc", "spmm_csc", "spmv_ell", "spmm_ell",
+                 "b200sp_spmv", "b200sp_spmm", "b200sp_plan_info", "b200sp_spmv_naive", "b200sp_spmm_naive"):
+        _address[name] = ctypes.cast(getattr(L, name), ctypes.c_void_p).value
+    _ell_product, _plan_product, _product = mod.ell_product, mod.plan_product, mod.product
+
+
 def _esize(dtype) -> int:
     return 4 if _dt(dtype) == F32 else 2
 
@@ -221,11 +246,25 @@ def _csr_args(m, n, nnz, k, row_ptr, col_idx, vals, dense_in, dense_out, dtype, 
 
 
 def spmv_csr(m, n, nnz, row_ptr, col_idx, vals, x, y, alpha, beta, dtype, stream=None):
+    if _product is None:
+        _load_native()
+    rc = _product(_address["spmv_csr"], 0, m, n, nnz, 0, row_ptr, col_idx, vals, x, y, alpha, beta, dtype, stream)
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "spmv_csr")
     a = _csr_args(m, n, nnz, 0, row_ptr, col_idx, vals, x, y, dtype, "spmv_csr")
     _ck(lib().spmv_csr(m, n, nnz, a[0], a[1], a[2], a[3], a[4], alpha, beta, _dt(dtype), _stream(stream)), "spmv_csr")
 
 
 def spmm_csr(m, n, nnz, k, row_ptr, col_idx, vals, B, Y, alpha, beta, dtype, stream=None):
+    if _product is None:
+        _load_native()
+    rc = _product(_address["spmm_csr"], 0, m, n, nnz, k, row_ptr, col_idx, vals, B, Y, alpha, beta, dtype, stream) if k > 0 else -1
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "spmm_csr")
     a = _csr_args(m, n, nnz, k, row_ptr, col_idx, vals, B, Y, dtype, "spmm_csr")
     _ck(lib().spmm_csr(m, n, nnz, k, a[0], a[1], a[2], a[3], a[4], alpha, beta, _dt(dtype), _stream(stream)), "spmm_csr")
 
@@ -233,6 +272,13 @@ def spmm_csr(m, n, nnz, k, row_ptr, col_idx, vals, B, Y, alpha, beta, dtype, str
 def spmv_csr_noalloc(m, n, nnz, row_ptr, col_idx, vals, x, y, alpha, beta, dtype, stream=None):
     """SpMV for callers that may not allocate device memory: scratch comes from a fixed array inside the
     library (m + nnz <= b200sp_noalloc_max_items()); overlapping calls race on that array."""
+    if _product is None:
+        _load_native()
+    rc = _product(_address["spmv_csr_noalloc"], 0, m, n, nnz, 0, row_ptr, col_idx, vals, x, y, alpha, beta, dtype, stream)
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "spmv_csr_noalloc")
     if 0 <= m + nnz <= b200sp_noalloc_max_items():
         a = _csr_args(m, n, nnz, 0, row_ptr, col_idx, vals, x, y, dtype, "spmv_csr_noalloc")
     else:   # refused by the library on the sizes alone: nothing is dereferenced
@@ -241,6 +287,13 @@ def spmv_csr_noalloc(m, n, nnz, row_ptr, col_idx, vals, x, y, alpha, beta, dtype
 
 
 def spmv_coo(m, n, nnz, row_idx, col_idx, vals, x, y, alpha, beta, dtype, stream=None):
+    if _product is None:
+        _load_native()
+    rc = _product(_address["spmv_coo"], 1, m, n, nnz, 0, row_idx, col_idx, vals, x, y, alpha, beta, dtype, stream)
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "spmv_coo")
     e = _esize(dtype)
     _ck(lib().spmv_coo(m, n, nnz, _dev(row_idx, nnz, 4, "spmv_coo row_idx"), _dev(col_idx, nnz, 4, "spmv_coo col_idx"),
                        _dev(vals, nnz, e, "spmv_coo vals"), _dev(x, n if nnz > 0 else 0, e, "spmv_coo x"), _dev(y, m, e, "spmv_coo y"),
@@ -248,6 +301,13 @@ def spmv_coo(m, n, nnz, row_idx, col_idx, vals, x, y, alpha, beta, dtype, stream
 
 
 def spmm_coo(m, n, nnz, k, row_idx, col_idx, vals, B, Y, alpha, beta, dtype, stream=None):
+    if _product is None:
+        _load_native()
+    rc = _product(_address["spmm_coo"], 1, m, n, nnz, k, row_idx, col_idx, vals, B, Y, alpha, beta, dtype, stream) if k > 0 else -1
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "spmm_coo")
     e = _esize(dtype)
     _ck(lib().spmm_coo(m, n, nnz, k, _dev(row_idx, nnz, 4, "spmm_coo row_idx"), _dev(col_idx, nnz, 4, "spmm_coo col_idx"),
                        _dev(vals, nnz, e, "spmm_coo vals"), _dev(B, n * k if nnz > 0 else 0, e, "spmm_coo B"), _dev(Y, m * k, e, "spmm_coo Y"),
@@ -255,6 +315,13 @@ def spmm_coo(m, n, nnz, k, row_idx, col_idx, vals, B, Y, alpha, beta, dtype, str
 
 
 def spmv_csc(m, n, nnz, col_ptr, row_idx, vals, x, y, alpha, beta, dtype, stream=None):
+    if _product is None:
+        _load_native()
+    rc = _product(_address["spmv_csc"], 2, m, n, nnz, 0, col_ptr, row_idx, vals, x, y, alpha, beta, dtype, stream)
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "spmv_csc")
     e = _esize(dtype)
     _ck(lib().spmv_csc(m, n, nnz, _dev(col_ptr, n + 1, 4, "spmv_csc col_ptr"), _dev(row_idx, nnz, 4, "spmv_csc row_idx"),
                        _dev(vals, nnz, e, "spmv_csc vals"), _dev(x, n if nnz > 0 else 0, e, "spmv_csc x"), _dev(y, m, e, "spmv_csc y"),
@@ -262,6 +329,13 @@ def spmv_csc(m, n, nnz, col_ptr, row_idx, vals, x, y, alpha, beta, dtype, stream
 
 
 def spmm_csc(m, n, nnz, k, col_ptr, row_idx, vals, B, Y, alpha, beta, dtype, stream=None):
+    if _product is None:
+        _load_native()
+    rc = _product(_address["spmm_csc"], 2, m, n, nnz, k, col_ptr, row_idx, vals, B, Y, alpha, beta, dtype, stream) if k > 0 else -1
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "spmm_csc")
     e = _esize(dtype)
     _ck(lib().spmm_csc(m, n, nnz, k, _dev(col_ptr, n + 1, 4, "spmm_csc col_ptr"), _dev(row_idx, nnz, 4, "spmm_csc row_idx"),
                        _dev(vals, nnz, e, "spmm_csc vals"), _dev(B, n * k if nnz > 0 else 0, e, "spmm_csc B"), _dev(Y, m * k, e, "spmm_csc Y"),
@@ -269,12 +343,26 @@ def spmm_csc(m, n, nnz, k, col_ptr, row_idx, vals, B, Y, alpha, beta, dtype, str
 
 
 def spmv_ell(m, n, width, col_ids, vals, x, y, alpha, beta, dtype, stream=None):
+    if _product is None:
+        _load_native()
+    rc = _ell_product(_address["spmv_ell"], m, n, width, 0, col_ids, vals, x, y, alpha, beta, dtype, stream)
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "spmv_ell")
     e = _esize(dtype)
     _ck(lib().spmv_ell(m, n, width, _dev(col_ids, m * width, 4, "spmv_ell col_ids"), _dev(vals, m * width, e, "spmv_ell vals"),
                        _dev(x, n if m * width > 0 else 0, e, "spmv_ell x"), _dev(y, m, e, "spmv_ell y"), alpha, beta, _dt(dtype), _stream(stream)), "spmv_ell")
 
 
 def spmm_ell(m, n, width, k, col_ids, vals, B, Y, alpha, beta, dtype, stream=None):
+    if _product is None:
+        _load_native()
+    rc = _ell_product(_address["spmm_ell"], m, n, width, k, col_ids, vals, B, Y, alpha, beta, dtype, stream) if k > 0 else -1
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "spmm_ell")
     e = _esize(dtype)
     _ck(lib().spmm_ell(m, n, width, k, _dev(col_ids, m * width, 4, "spmm_ell col_ids"), _dev(vals, m * width, e, "spmm_ell vals"),
                        _dev(B, n * k if m * width > 0 else 0, e, "spmm_ell B"), _dev(Y, m * k, e, "spmm_ell Y"), alpha, beta, _dt(dtype),
@@ -282,11 +370,25 @@ def spmm_ell(m, n, width, k, col_ids, vals, B, Y, alpha, beta, dtype, stream=Non
 
 
 def b200sp_spmv_naive(m, n, nnz, row_ptr, col_idx, vals, x, y, alpha, beta, dtype, stream=None):
+    if _product is None:
+        _load_native()
+    rc = _product(_address["b200sp_spmv_naive"], 0, m, n, nnz, 0, row_ptr, col_idx, vals, x, y, alpha, beta, dtype, stream)
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "b200sp_spmv_naive")
     a = _csr_args(m, n, nnz, 0, row_ptr, col_idx, vals, x, y, dtype, "b200sp_spmv_naive")
     _ck(lib().b200sp_spmv_naive(m, n, nnz, a[0], a[1], a[2], a[3], a[4], alpha, beta, _dt(dtype), _stream(stream)), "b200sp_spmv_naive")
 
 
 def b200sp_spmm_naive(m, n, nnz, k, row_ptr, col_idx, vals, B, Y, alpha, beta, dtype, stream=None):
+    if _product is None:
+        _load_native()
+    rc = _product(_address["b200sp_spmm_naive"], 0, m, n, nnz, k, row_ptr, col_idx, vals, B, Y, alpha, beta, dtype, stream) if k > 0 else -1
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "b200sp_spmm_naive")
     a = _csr_args(m, n, nnz, k, row_ptr, col_idx, vals, B, Y, dtype, "b200sp_spmm_naive")
     _ck(lib().b200sp_spmm_naive(m, n, nnz, k, a[0], a[1], a[2], a[3], a[4], alpha, beta, _dt(dtype), _stream(stream)), "b200sp_spmm_naive")
 
@@ -360,12 +462,26 @@ def b200sp_plan_info(plan) -> dict:
 
 
 def b200sp_spmv(plan, col_idx, vals, x, y, alpha, beta, dtype, stream=None):
+    if _product is None:
+        _load_native()
+    rc = _plan_product(_address["b200sp_plan_info"], _address["b200sp_spmv"], plan, 0, col_idx, vals, x, y, alpha, beta, dtype, stream)
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "b200sp_spmv")
     I = b200sp_plan_info(plan)      # the plan knows m, n, nnz
     a = _csr_args(I["m"], I["n"], I["nnz"], 0, None, col_idx, vals, x, y, dtype, "b200sp_spmv")
     _ck(lib().b200sp_spmv(plan, a[1], a[2], a[3], a[4], alpha, beta, _dt(dtype), _stream(stream)), "b200sp_spmv")
 
 
 def b200sp_spmm(plan, k, col_idx, vals, B, Y, alpha, beta, dtype, stream=None):
+    if _product is None:
+        _load_native()
+    rc = _plan_product(_address["b200sp_plan_info"], _address["b200sp_spmm"], plan, k, col_idx, vals, B, Y, alpha, beta, dtype, stream) if k > 0 else -1
+    if rc == 0:
+        return
+    if rc > 0:
+        raise B200spError(rc, "b200sp_spmm")
     I = b200sp_plan_info(plan)
     a = _csr_args(I["m"], I["n"], I["nnz"], k, None, col_idx, vals, B, Y, dtype, "b200sp_spmm")
     _ck(lib().b200sp_spmm(plan, k, a[1], a[2], a[3], a[4], alpha, beta, _dt(dtype), _stream(stream)), "b200sp_spmm")

@@ -1,4 +1,5 @@
-"""Builds libb200sp.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libb200sp.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _marshal.so (the binding's native argument
+marshalling, a CPython extension on torch's C++ headers) with g++."""
 from __future__ import annotations
 
 import glob
@@ -8,6 +9,7 @@ import subprocess
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libb200sp.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
 LIB_CHECKED = os.path.join(HERE, "libb200sp_check.so")     # the same sources with -DB200SP_BOUNDS_CHECK
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared"]
@@ -38,6 +40,24 @@ def build(force: bool = False, verbose: bool = False, checked: bool = False) -> 
     return lib
 
 
+def build_marshal(force: bool = False) -> str:
+    """Compile csrc/marshal.cpp into _marshal.so if it is missing or older than its source."""
+    src = os.path.join(CSRC, "marshal.cpp")
+    if force or not os.path.exists(MARSHAL) or os.path.getmtime(MARSHAL) < os.path.getmtime(src):
+        import sysconfig
+        import torch
+        from torch.utils.cpp_extension import include_paths, library_paths
+        tmp = MARSHAL + ".tmp.%d" % os.getpid()
+        cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+        incs = ["-I" + d for d in include_paths() + [sysconfig.get_paths()["include"], os.path.join(cuda, "include")]]
+        libs = ["-L" + d for d in library_paths()] + ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+        subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-w",
+                               "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI)] + incs + ["-o", tmp, src] + libs)
+        os.replace(tmp, MARSHAL)
+    return MARSHAL
+
+
 if __name__ == "__main__":
     import sys
+    print(build_marshal())
     print(build(force=True, verbose=True, checked="--bounds-check" in sys.argv))
