@@ -128,7 +128,7 @@ def _ptr(t) -> Optional[int]:
     return t.ctypes.data
 
 
-_product = _ell_product = _plan_product = None      # csrc/marshal.cpp, and the library's entry points as addresses
+_product = _ell_product = _plan_product = _plan_create = None      # csrc/marshal.cpp, and the library's entry points as addresses
 _address = {}
 
 
@@ -136,7 +136,7 @@ def _load_native():
     """Loads the native marshalling (built with the library): the checks below and the call in one step.  Its functions return the
     library's status, or -1 for arguments they do not take as they stand; the Python code that follows each call then handles
     them or raises the precise error."""
-    global _product, _ell_product, _plan_product
+    global _product, _ell_product, _plan_product, _plan_create
     import importlib.util
     import torch  # noqa: F401 - the extension resolves its symbols against the libraries that this loads
     path = os.path.join(_HERE, "_marshal.so")
@@ -148,9 +148,9 @@ def _load_native():
     spec.loader.exec_module(mod)
     L = lib()
     for name in ("spmv_csr", "spmm_csr", "spmv_csr_noalloc", "spmv_coo", "spmm_coo", "spmv_csc", "spmm_csc", "spmv_ell", "spmm_ell",
-                 "b200sp_spmv", "b200sp_spmm", "b200sp_plan_info", "b200sp_spmv_naive", "b200sp_spmm_naive"):
+                 "b200sp_spmv", "b200sp_spmm", "b200sp_plan_info", "b200sp_plan_create", "b200sp_spmv_naive", "b200sp_spmm_naive"):
         _address[name] = ctypes.cast(getattr(L, name), ctypes.c_void_p).value
-    _ell_product, _plan_product, _product = mod.ell_product, mod.plan_product, mod.product
+    _ell_product, _plan_product, _plan_create, _product = mod.ell_product, mod.plan_product, mod.plan_create, mod.product
 
 
 def _esize(dtype) -> int:
@@ -445,6 +445,13 @@ def spmm_csr_host(m, n, nnz, k, row_ptr, col_idx, vals, B, Y, alpha, beta, dtype
 
 
 def b200sp_plan_create(m, n, nnz, row_ptr, stream=None) -> int:
+    if _product is None:
+        _load_native()
+    plan = _plan_create(_address["b200sp_plan_create"], m, n, nnz, row_ptr, stream)
+    if plan >= 0:
+        return plan
+    if plan < -1:
+        raise B200spError(-2 - plan, "b200sp_plan_create")
     out = ctypes.c_void_p()
     _ck(lib().b200sp_plan_create(ctypes.byref(out), m, n, nnz, _dev(row_ptr, m + 1 if m > 0 else 0, 4, "b200sp_plan_create row_ptr"),
                                  _stream(stream)), "b200sp_plan_create")

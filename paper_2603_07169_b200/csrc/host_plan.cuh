@@ -98,15 +98,11 @@ void plan_slot_give(int slot) {
   g_slots.freed.notify_one();
 }
 
-// Warp shares of the nnz-balanced SpMM kernel: items per share and shares per warp, fewer and shorter for small problems so that
-// every SM has enough warps.  Returns the number of shares.
-long long spmm_shares(const b200sp_plan_info_t& I, const DeviceInfo* dev, int* witems, int* per_warp) {
-  int w = kMergeWarpItems, s = kMergeShares;
-  while (s > 1 && I.m + I.nnz < (int64_t)dev->sms * 128 * w * s) s /= 2;
-  while (w > 32 && I.m + I.nnz < (int64_t)dev->sms * 48 * w) w /= 2;
-  *witems = w;
-  *per_warp = s;
-  return (I.m + I.nnz + w - 1) / w;
+// Merge items per share of the nnz-balanced SpMM kernel: 128, fewer for small problems (20,011 rows, 220,121 items, k = 128 with a fresh
+// plan: 64 us with shares of 56 and 64, 71 us with 32, 70 us with 128).
+int spmm_share_items(const b200sp_plan_info_t& I, const DeviceInfo* dev) {
+  const int64_t w = (I.m + I.nnz + (int64_t)dev->sms * 24 - 1) / ((int64_t)dev->sms * 24);
+  return w >= kMergeWarpItems ? kMergeWarpItems : w <= 32 ? 32 : (int)((w + 7) / 8 * 8);
 }
 
 // The lists of rows of kMediumRow + 1 .. kLongRow and of more than kLongRow nonzeros, built on the device in stream order on the
@@ -150,8 +146,8 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
   // one block from the pool: the probe's counters, split points, carries, tails; for small matrices also the shares of the
   // nnz-balanced SpMM kernel, which then cost no launch of their own (large ones search them on first use)
   const size_t nt = (size_t)I.spmv_tiles;
-  int witems = 0, per_warp = 0;
-  const long long shares = spmm_shares(I, dev, &witems, &per_warp);
+  const int witems = spmm_share_items(I, dev);
+  const long long shares = (m + nnz + witems - 1) / witems;
   const bool with_shares = shares <= 65536;
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
   const size_t o_split = 256, o_carry = o_split + up((nt + 1) * 4), o_tail = o_carry + up((nt + 1) * 4), o_share = o_tail + up((nt + 1) * 4),
@@ -165,14 +161,15 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
   p->split_row = (int32_t*)(base + o_split);
   p->carry = (float*)(base + o_carry);
   p->tail = (float*)(base + o_tail);
-  if (with_shares) { p->spmm_split = (int32_t*)(base + o_share); p->spmm_witems = witems; p->spmm_shares = per_warp; }
+  if (with_shares) { p->spmm_split = (int32_t*)(base + o_share); p->spmm_witems = witems; }
   I.scratch_bytes = (int64_t)total;
   int slot = 0;
   rc = plan_slot_take(&slot);
   if (rc != B200SP_OK) return fail(rc);
   PlanStats h;
   {
-    const long long blocks = (m + 256 * 4 - 1) / (256 * 4);
+    const long long searches = (long long)nt + 1 + (with_shares ? shares + 1 : 0), work = m > searches * 4 ? m : searches * 4;
+    const long long blocks = (work + 256 * 4 - 1) / (256 * 4);   // four rows and at most one search per thread
     const int grid = (int)(blocks < dev->sms * 8 ? blocks : dev->sms * 8);
     plan_pass_kernel<<<grid, 256, 0, stream>>>(row_ptr, (int)m, (int)nnz, slot, g_slots.host + slot, items, (int)nt, p->split_row,
                                                with_shares ? witems : 0, (int)shares, p->spmm_split);

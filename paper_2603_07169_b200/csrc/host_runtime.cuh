@@ -252,7 +252,7 @@ struct b200sp_plan {
   const void* probed_col_idx = nullptr;   // col_idx the column-locality probe last ran on
   int32_t* spmm_split = nullptr;          // warp shares of the nnz-balanced SpMM kernel (part of `block` for small matrices, else a pool block of its own, built on first use)
   void* split_block = nullptr;            // that block
-  int spmm_witems = 0, spmm_shares = 0;   // merge items per share, consecutive shares per warp
+  int spmm_witems = 0;                    // merge items per share
   // merge list over the rows that have nonzeros (matrices with many empty rows)
   void* compact_block = nullptr;          // one pool block: row ids, their offsets, block counts
   int compact_rows = 0;                   // number of rows that have nonzeros (0 = the list has not been built)

@@ -315,7 +315,27 @@ int launch_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* va
                       cudaStream_t stream, DeviceInfo* dev) {
   const b200sp_plan_info_t& I = p->info;
   constexpr int KS = 32 * V * J;
-  const int witems = p->spmm_witems, shares = p->spmm_shares;
+  const int witems = p->spmm_witems;
+  auto kernel = spmm_merge_kernel<T, V, J>;
+  static int per_sm[64] = {};   // per instantiation and device: resident CTAs
+  if (!per_sm[p->device]) {
+    int nb = 0;
+    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kMergeWarps * 32, 0));
+    per_sm[p->device] = nb > 0 ? nb : 1;
+  }
+  // Shares per warp, by a model of the time: a wave of resident warps costs their items and about 40 more (what a warp does before its first
+  // and after its last nonzero); the last of several waves is, on average, a third full, and a single wave has nothing to fill in behind
+  // its slower warps.  40,000 rows of 20, k = 256 FP32 with a fresh plan: 131 us with two shares (one wave), 149 us with one (1.8 waves);
+  // 100,000 rows of 12, k = 127: 84 us with one (1.7 waves), 94 us with two; 155,787 rows of 12, k = 96: 80 us with two, 84 us with one.
+  int shares = 1;
+  {
+    const double resident = (double)per_sm[p->device] * dev->sms * kMergeWarps, total = (double)(I.m + I.nnz) / witems;
+    double best = 0.0;
+    for (int s = 1; s <= kMergeShares; ++s) {
+      const double waves = total / (s * resident), cost = (s * witems + 40.0) * (waves > 0.95 ? waves + 0.35 : 1.15);
+      if (s == 1 || cost < best) { best = cost; shares = s; }
+    }
+  }
   const long long per_tile = (long long)witems * shares * kMergeWarps;
   const int tiles = (int)((I.m + I.nnz + per_tile - 1) / per_tile);
   const int slices = (k + KS - 1) / KS;
@@ -326,7 +346,7 @@ int launch_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* va
   int rc = pool_alloc(dev, (void**)&scratch, 2 * per * sizeof(float), stream);
   if (rc != B200SP_OK) return rc;
   tl_pdl_kernel = true;
-  rc = launch(spmm_merge_kernel<T, V, J>, dim3((unsigned)(slices * tiles)), dim3(kMergeWarps * 32), stream, B, (size_t)I.n * k * sizeof(T), dev,
+  rc = launch(kernel, dim3((unsigned)(slices * tiles)), dim3(kMergeWarps * 32), stream, B, (size_t)I.n * k * sizeof(T), dev,
               (int)I.m, (int)I.nnz, k, tiles, witems, shares, (const int*)p->spmm_split, p->row_ptr, col_idx, vals, B, Y, scratch, scratch + per, alpha, beta);
   if (rc == B200SP_OK && tiles > 1) {
     tl_pdl_kernel = true;
@@ -348,8 +368,8 @@ int run_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals,
   int v = 1;
   while (v < VMAX && k % (2 * v) == 0 && 32 * v < k) v *= 2;
   if (!p->spmm_split) {   // shares: once per plan, a small kernel in stream order
-    int w = 0, per_warp = 0;
-    const long long shares = spmm_shares(I, dev, &w, &per_warp);
+    const int w = spmm_share_items(I, dev);
+    const long long shares = (I.m + I.nnz + w - 1) / w;
     int rc = pool_alloc(dev, &p->split_block, (size_t)(shares + 1) * sizeof(int32_t), stream);
     if (rc != B200SP_OK) return rc;
     rc = launch(plan_merge_split_kernel, dim3((unsigned)((shares + 1 + 255) / 256)), dim3(256), stream, nullptr, 0, dev, p->row_ptr, (int)I.m,
@@ -357,7 +377,6 @@ int run_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals,
     if (rc != B200SP_OK) return rc;
     p->spmm_split = (int32_t*)p->split_block;
     p->spmm_witems = w;
-    p->spmm_shares = per_warp;
   }
   const int loads = (k + 32 * v - 1) / (32 * v);
 #define B200SP_MERGE_J(V)                                                                                                   \

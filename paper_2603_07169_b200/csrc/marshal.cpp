@@ -177,7 +177,33 @@ PyObject* plan_product(PyObject*, PyObject* const* v, Py_ssize_t argc) {
   });
 }
 
+// (fn, m, n, nnz, row_ptr, stream): the new plan's address, or -1 / -2 - status (a plan's address is never negative as a signed number).
+PyObject* plan_create(PyObject*, PyObject* const* v, Py_ssize_t argc) {
+  long long result = -1;
+  try {
+    if (argc == 6) {
+      Reader r;
+      void* const fn = r.address(v[0]);
+      const int64_t m = r.size(v[1]), n = r.size(v[2]), nnz = r.size(v[3]);
+      const int32_t* row_ptr = (const int32_t*)r.operand(v[4], m > 0 ? m + 1 : 0, 4);
+      void* const stream = r.stream(v[5]);
+      if (r.ok) {
+        b200sp_plan* plan = nullptr;
+        int status;
+        Py_BEGIN_ALLOW_THREADS
+        status = ((decltype(&b200sp_plan_create))fn)(&plan, m, n, nnz, row_ptr, stream);
+        Py_END_ALLOW_THREADS
+        result = status == B200SP_OK ? (long long)(intptr_t)plan : -2 - status;
+      }
+    }
+  } catch (...) {
+    result = -1;
+  }
+  return PyLong_FromLongLong(result);
+}
+
 PyMethodDef methods[] = {
+    {"plan_create", (PyCFunction)(void (*)(void))plan_create, METH_FASTCALL, nullptr},
     {"product", (PyCFunction)(void (*)(void))product, METH_FASTCALL, nullptr},
     {"ell_product", (PyCFunction)(void (*)(void))ell_product, METH_FASTCALL, nullptr},
     {"plan_product", (PyCFunction)(void (*)(void))plan_product, METH_FASTCALL, nullptr},

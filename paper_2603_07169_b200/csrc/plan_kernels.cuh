@@ -57,9 +57,11 @@ __global__ void __launch_bounds__(256) plan_pass_kernel(const int* __restrict__ 
   if (threadIdx.x == 0) { s_short = 0; s_max = 0; s_bad = 0; }
   __syncthreads();
   const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
-  for (long long t = i0; t <= tiles; t += stride) split_row[t] = merge_split(row_ptr, m, nnz, items, (int)t);
-  if (share_items > 0)
-    for (long long t = i0; t <= shares; t += stride) share_split[t] = merge_split(row_ptr, m, nnz, share_items, (int)t);
+  const long long first_tile = share_items > 0 ? (long long)shares + 1 : 0;      // one search per thread, whichever set it belongs to
+  for (long long t = i0; t <= first_tile + tiles; t += stride) {
+    if (t < first_tile) share_split[t] = merge_split(row_ptr, m, nnz, share_items, (int)t);
+    else split_row[t - first_tile] = merge_split(row_ptr, m, nnz, items, (int)(t - first_tile));
+  }
   int lshort = 0, lmax = 0, bad = 0;
   unsigned rows[6] = {0, 0, 0, 0, 0, 0}, nz[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll 4
