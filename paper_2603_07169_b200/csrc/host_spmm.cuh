@@ -343,16 +343,17 @@ int launch_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* va
   // per-call scratch: what each tile leaves unfinished and what it finishes for an earlier tile, KS floats per (slice, tile)
   float* scratch = nullptr;
   const size_t per = (size_t)slices * tiles * KS;
-  int rc = pool_alloc(dev, (void**)&scratch, 2 * per * sizeof(float), stream);
+  int rc = pool_alloc(dev, (void**)&scratch, 2 * per * sizeof(float) + (size_t)tiles * sizeof(int2), stream);
+  int2* const tile_row = (int2*)(scratch + 2 * per);
   if (rc != B200SP_OK) return rc;
   tl_pdl_kernel = true;
   rc = launch(kernel, dim3((unsigned)(slices * tiles)), dim3(kMergeWarps * 32), stream, B, (size_t)I.n * k * sizeof(T), dev,
-              (int)I.m, (int)I.nnz, k, tiles, witems, shares, (const int*)p->spmm_split, p->row_ptr, col_idx, vals, B, Y, scratch, scratch + per, alpha, beta);
+              (int)I.m, (int)I.nnz, k, tiles, witems, shares, (const int*)p->spmm_split, p->row_ptr, col_idx, vals, B, Y, scratch, scratch + per, tile_row, alpha, beta);
   if (rc == B200SP_OK && tiles > 1) {
     tl_pdl_kernel = true;
-    rc = launch(spmm_merge_fixup_kernel<T>, dim3((unsigned)(((long long)slices * tiles + 7) / 8)), dim3(256), stream, nullptr, 0, dev, (int)I.m,
-                (int)I.nnz, k, tiles, slices, KS, witems, shares, (const int*)p->spmm_split, p->row_ptr, (const float*)scratch, (const float*)(scratch + per), Y,
-                alpha, beta);
+    const int lanes = KS >= 128 ? 128 : KS;      // a power of two
+    rc = launch(spmm_merge_fixup_kernel<T>, dim3((unsigned)(((long long)slices * tiles * lanes + 255) / 256)), dim3(256), stream, nullptr, 0, dev, k,
+                tiles, slices, KS, lanes, (const int2*)tile_row, (const float*)scratch, (const float*)(scratch + per), Y, alpha, beta);
   }
   const cudaError_t e = cudaFreeAsync(scratch, stream);
   if (e != cudaSuccess && rc == B200SP_OK) rc = cuda_fail(e, "cudaFreeAsync");
@@ -429,7 +430,9 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
       if (rc != B200SP_ERR_UNSUPPORTED) return rc;   // unsupported shape for the tensor map: fall through to the sliced kernel
     }
   }
-  if (g_opt.spmm_sliced && (g_opt.spmm_flat == 1 || (g_opt.spmm_flat == 2 && (spmm_rows_are_uneven(I) || k % VEC != 0)))) {
+  // Uneven rows, and k that is no multiple of 16 bytes unless it is so narrow that a lane per column and a group of lanes per row lose
+  // little (100,000 rows of 13: k = 13 18 us by rows, 27 us by shares; k = 23 35 / 27 us; k = 50 47 / 35 us FP32, 42 / 34 us BF16)
+  if (g_opt.spmm_sliced && (g_opt.spmm_flat == 1 || (g_opt.spmm_flat == 2 && (spmm_rows_are_uneven(I) || (k % VEC != 0 && k > 16))))) {
     const int rc = run_spmm_merge<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
     if (rc != B200SP_ERR_UNSUPPORTED) return rc;
   }
@@ -501,6 +504,7 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     if (k <= 2) return launch_spmm<T, 1, 2, 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
     if (k <= 4) return launch_spmm<T, 1, 4, 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
     if (k <= 8) return launch_spmm<T, 1, 8, 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
+    if (k <= 16) return launch_spmm<T, 1, 16, 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
     return launch_spmm<T, 1, 32, 2>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
   }
   const int vecs = k / VEC;  // vector columns per row

@@ -150,12 +150,13 @@ template <typename T, int V, int J>
 __global__ void __launch_bounds__(kMergeWarps * 32, (merge_ctas<T, V, J>()))
 spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, const int* __restrict__ split, const int* __restrict__ row_ptr,
                   const int* __restrict__ col_idx, const T* __restrict__ vals, const T* __restrict__ B, T* __restrict__ Y,
-                  float* __restrict__ tile_carry, float* __restrict__ tile_tail, float alpha, float beta) {
+                  float* __restrict__ tile_carry, float* __restrict__ tile_tail, int2* __restrict__ tile_row, float alpha, float beta) {
   constexpr int U = kMergeUnroll<V, J>, KS = 32 * V * J;
   typedef typename Piece<T, V>::raw raw;
   __shared__ __align__(16) MergeStage<T> stage_s[kMergeWarps][2];
   __shared__ __align__(16) float wide_s[sizeof(T) == 2 ? kMergeWarps : 1][sizeof(T) == 2 ? kMergeWarpItems + 8 : 4];   // BF16: the current share's values widened
   __shared__ float head_s[kMergeWarps][KS];
+  __shared__ int first_s[2];                                 // the tile's first row and where it starts, -1 when inside the tile
   static_assert(sizeof(stage_s[0]) >= KS * sizeof(float), "a warp's carry takes the place of its stages");
   auto carry_s = [&](int w) { return reinterpret_cast<float*>(&stage_s[w][0]); };
   grid_dependency_wait();
@@ -296,19 +297,21 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
   for (int j = 0; j < J; ++j)
 #pragma unroll
     for (int i = 0; i < V; ++i) carry_s(warp)[32 * V * j + lane * V + i] = tot[j][i];   // zero when the shares end with a row
+  if (warp == 0 && lane == 0) { first_s[0] = r_first; first_s[1] = start0 < p_first ? start0 : -1; }
   __syncthreads();
 
   // (r_lo is now the number of row ends before this warp's end)
-  const int region = witems * shares;
+  // Merge items are counted in 32 bits (m + nnz < 2^32): three divisions in 64 bits would be calls, and spills in the loop above.
+  const unsigned region = (unsigned)(witems * shares);
   const long long slot = ((long long)slice * tiles + t) * KS;
   if (start0 < p_first && r_lo > r_first) {                  // complete the row that ends here: the carries before it, in order, then the head
-    const long long ws = ((long long)start0 + r_first) / region - (long long)t * kMergeWarps;   // the warp that holds the row's start
+    const int ws = (int)(((unsigned)start0 + (unsigned)r_first) / region) - t * kMergeWarps;   // the warp that holds the row's start
 #pragma unroll
     for (int j = 0; j < J; ++j) {
       float s[V];
 #pragma unroll
       for (int i = 0; i < V; ++i) s[i] = 0.0f;
-      for (int w = ws > 0 ? (int)ws : 0; w < warp; ++w)
+      for (int w = ws > 0 ? ws : 0; w < warp; ++w)
 #pragma unroll
         for (int i = 0; i < V; ++i) s[i] += carry_s(w)[32 * V * j + lane * V + i];
 #pragma unroll
@@ -321,14 +324,18 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
     }
   }
   if (warp == kMergeWarps - 1) {                             // what the tile leaves unfinished
-    long long ws = kMergeWarps;
-    if (r_lo < m) ws = ((long long)__ldg(row_ptr + r_lo) + r_lo) / region - (long long)t * kMergeWarps;
+    if (slice == 0 && lane == 0) {                           // and for the fix-up: the row that it completes for earlier tiles, and the first of them
+      const int r = first_s[0], rs = first_s[1];
+      tile_row[t] = rs >= 0 && r_lo > r ? make_int2(r, (int)(((unsigned)rs + (unsigned)r) / (region * kMergeWarps))) : make_int2(-1, 0);
+    }
+    int ws = kMergeWarps;
+    if (r_lo < m) ws = (int)(((unsigned)__ldg(row_ptr + r_lo) + (unsigned)r_lo) / region) - t * kMergeWarps;
 #pragma unroll
     for (int j = 0; j < J; ++j) {
       float s[V];
 #pragma unroll
       for (int i = 0; i < V; ++i) s[i] = 0.0f;
-      for (int w = ws > 0 ? (int)ws : 0; w < kMergeWarps; ++w)
+      for (int w = ws > 0 ? ws : 0; w < kMergeWarps; ++w)
 #pragma unroll
         for (int i = 0; i < V; ++i) s[i] += carry_s(w)[32 * V * j + lane * V + i];
 #pragma unroll
@@ -337,33 +344,25 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
   }
 }
 
-// Finishes the rows that a tile boundary of spmm_merge_kernel cut: tile t completes such a row when its first row began in an
-// earlier tile and ends in this one.  The row's value is tile_carry[first .. t-1] + tile_tail[t], the carries added in trees of
-// 16 whose sums form a chain; one warp per (slice, tile), fixed order.
+// Finishes the rows that a tile boundary of spmm_merge_kernel cut: the row's value is tile_carry[first .. t-1] + tile_tail[t], the carries
+// added in trees of 16 whose sums form a chain; `lanes` threads per (slice, tile), fixed order.  Latency-bound: which row and from which
+// tile on comes from the tile itself (tile_row), so that only one load stands before those of the partial sums.
 template <typename T>
 __global__ void __launch_bounds__(256)
-spmm_merge_fixup_kernel(int m, int nnz, int k, int tiles, int slices, int ks, int witems, int shares, const int* __restrict__ split,
-                        const int* __restrict__ row_ptr, const float* __restrict__ tile_carry, const float* __restrict__ tile_tail,
-                        T* __restrict__ Y, float alpha, float beta) {
+spmm_merge_fixup_kernel(int k, int tiles, int slices, int ks, int lanes, const int2* __restrict__ tile_row, const float* __restrict__ tile_carry,
+                        const float* __restrict__ tile_tail, T* __restrict__ Y, float alpha, float beta) {
   grid_dependency_wait();
-  const long long id = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
+  const long long id = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / lanes;
+  const int lane = threadIdx.x & (lanes - 1);
   if (id >= (long long)slices * tiles) return;
   const int slice = (int)(id / tiles), t = (int)(id - (long long)slice * tiles);
-  if (t < 1) return;
-  const long long total = (long long)m + nnz;
-  const int items = witems * shares * kMergeWarps, per = shares * kMergeWarps;
-  const int last = (int)((total + witems - 1) / witems);
-  const int r0 = __ldg(split + (long long)t * per), r1 = __ldg(split + min((long long)(t + 1) * per, (long long)last));
-  if (r0 >= r1) return;                                      // no row ends in the tile
-  const long long p0 = (long long)t * items - r0;
-  const int rs = __ldg(row_ptr + r0);
-  if (rs >= p0) return;                                      // its first row starts inside it
-  const int tf = (int)(((long long)rs + r0) / items);
-  for (int c = lane; c < ks && slice * ks + c < k; c += 32) {
+  const int2 row = __ldg(tile_row + t);
+  if (row.x < 0) return;                                     // no row that began in an earlier tile ends in this one
+  for (int c = lane; c < ks && slice * ks + c < k; c += lanes) {
     const float* const cp = tile_carry + (long long)slice * tiles * ks + c;
+    const float tail = tile_tail[((long long)slice * tiles + t) * ks + c];
     float acc = 0.0f;
-    for (int u = tf; u < t; u += 16) {
+    for (int u = row.y; u < t; u += 16) {
       float part[16];
 #pragma unroll
       for (int v = 0; v < 16; ++v) part[v] = u + v < t ? cp[(long long)(u + v) * ks] : 0.0f;
@@ -373,8 +372,7 @@ spmm_merge_fixup_kernel(int m, int nnz, int k, int tiles, int slices, int ks, in
         for (int v = 0; v < w; ++v) part[v] += part[v + w];
       acc += part[0];
     }
-    acc += tile_tail[((long long)slice * tiles + t) * ks + c];
-    epilogue_store(Y, (long long)r0 * k + slice * ks + c, acc, alpha, beta);
+    epilogue_store(Y, (long long)row.x * k + slice * ks + c, acc + tail, alpha, beta);
   }
 }
 

@@ -46,6 +46,17 @@ def test_merge_spmm_against_oracle(case, dtype):
         b200sp.b200sp_set_option("spmm_flat", 2)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_even_rows_of_ragged_width_on_both_sides_of_the_rule(dtype):
+    """k that is no multiple of a vector: by rows up to 16 columns (a group of 2 to 16 lanes per row), by shares above."""
+    rng = np.random.default_rng(2)
+    A = gen.random_csr(3000, 20_000, rng.integers(10, 16, 3000), seed=8)
+    for k in (2, 3, 5, 7, 9, 13, 15, 17, 18, 31):
+        B = rng.standard_normal(A.n * k).astype(np.float32)
+        Y, Y_ref, S = run_spmm(A, B, k, None, 1.0, 0.0, dtype)
+        assert_within(Y, Y_ref, S, dtype, what="k=%d" % k)
+
+
 def test_non_finite_rows_of_b_touch_only_the_rows_that_use_them():
     """What a warp reads ahead of its last nonzero (row 0 of B) is never multiplied."""
     n, k = 9000, 64
