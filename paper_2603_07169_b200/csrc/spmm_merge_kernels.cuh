@@ -59,12 +59,33 @@ template <> struct Piece<bf16_t, 8> {
   }
 };
 
+// acc += v * b.  BF16 pairs by the mixed-precision FMA of sm_100 (BF16 factors, FP32 addend and result, one rounding; v is a widened BF16
+// value): the same value as fmaf on the widened factors without the widening (100 columns of 2^18 rows of 32: 198 -> 173 us).
+__device__ __forceinline__ void mixed_fma(unsigned w, float v, float& a0, float& a1) {
+  asm("{ .reg .b16 lo, hi;\n\t"
+      "mov.b32 {lo, hi}, %3;\n\t"
+      "fma.rn.f32.bf16 %0, %2, lo, %0;\n\t"
+      "fma.rn.f32.bf16 %1, %2, hi, %1; }"
+      : "+f"(a0), "+f"(a1) : "h"((unsigned short)(__float_as_uint(v) >> 16)), "r"(w));
+}
 template <typename T, int V>
 __device__ __forceinline__ void piece_fma(const typename Piece<T, V>::raw& b, float v, float (&acc)[V]) {
-  float w[V];
-  Piece<T, V>::widen(b, w);
+  if constexpr (sizeof(T) == 2 && V == 2) {
+    mixed_fma(b, v, acc[0], acc[1]);
+  } else if constexpr (sizeof(T) == 2 && V == 4) {
+    mixed_fma(b.x, v, acc[0], acc[1]);
+    mixed_fma(b.y, v, acc[2], acc[3]);
+  } else if constexpr (sizeof(T) == 2 && V == 8) {
+    mixed_fma(b.x, v, acc[0], acc[1]);
+    mixed_fma(b.y, v, acc[2], acc[3]);
+    mixed_fma(b.z, v, acc[4], acc[5]);
+    mixed_fma(b.w, v, acc[6], acc[7]);
+  } else {
+    float w[V];
+    Piece<T, V>::widen(b, w);
 #pragma unroll
-  for (int i = 0; i < V; ++i) acc[i] = fmaf(v, w[i], acc[i]);
+    for (int i = 0; i < V; ++i) acc[i] = fmaf(v, w[i], acc[i]);
+  }
 }
 
 template <typename T, int V>
@@ -146,7 +167,8 @@ template <> struct MergeStage<bf16_t> {
 // order, and what crosses the CTA's own ends goes to tile_tail / tile_carry and is finished by spmm_merge_fixup_kernel.  No
 // chain is longer than kMergeWarpItems products + kMergeShares + kMergeWarps partial sums + the tiles' terms.
 // split[i]: row ends before item i * witems.
-template <typename T, int V, int J>
+// LIST: for matrices with empty rows and beta != 0 (see below); the listing costs 2-5 % where there are none.
+template <typename T, int V, int J, bool LIST>
 __global__ void __launch_bounds__(kMergeWarps * 32, (merge_ctas<T, V, J>()))
 spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, const int* __restrict__ split, const int* __restrict__ row_ptr,
                   const int* __restrict__ col_idx, const T* __restrict__ vals, const T* __restrict__ B, T* __restrict__ Y,
@@ -155,6 +177,7 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
   typedef typename Piece<T, V>::raw raw;
   __shared__ __align__(16) MergeStage<T> stage_s[kMergeWarps][2];
   __shared__ __align__(16) float wide_s[sizeof(T) == 2 ? kMergeWarps : 1][sizeof(T) == 2 ? kMergeWarpItems + 8 : 4];   // BF16: the current share's values widened
+  __shared__ unsigned char empty_s[LIST ? kMergeWarps : 1][LIST ? kMergeWarpItems : 4];
   __shared__ float head_s[kMergeWarps][KS];
   __shared__ int first_s[2];                                 // the tile's first row and where it starts, -1 when inside the tile
   static_assert(sizeof(stage_s[0]) >= KS * sizeof(float), "a warp's carry takes the place of its stages");
@@ -189,7 +212,7 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
         if (i + lane < words) cp_async4(&st.raw[i + lane], vals + w0 + 2 * (i + lane), min(4, 2 * (nnz - w0 - 2 * (i + lane))));
     }
     if (lane < U) st.col[cnt + lane] = 0;                    // read ahead of the end, never multiplied
-    if (lane == 0) st.end[rows] = (int)((unsigned)p0 + 0x100000u);   // no end inside this share
+    if (!LIST && lane == 0) st.end[rows] = (int)((unsigned)p0 + 0x100000u);   // no end inside this share
   };
 
   const int col0 = slice * KS + lane * V;
@@ -203,7 +226,35 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
   }
   const char* const Bc = (const char*)(B + col0);
   const int row_bytes = k * (int)sizeof(T);
-  T* yp = Y + (long long)r_first * k + col0;
+  T* yrow = Y + (long long)r_first * k + col0;
+  int begin = start0;                                        // start of the current row
+  // rows empty_s[warp][0 .. count) of the share whose first row is at ys: y = beta * y over the slice's columns
+  auto scale_rows = [&](T* ys, int count) {
+    const int width = min(KS, k - slice * KS);
+    const bool wide = V * sizeof(T) < 16 && k * (int)sizeof(T) % 16 == 0;       // 16 bytes a lane where the rows allow it
+    const int per = wide ? 16 / (int)sizeof(T) : V;
+    int lanes = 32;                                          // lanes to a row: a power of two
+    while (lanes > 1 && (lanes / 2) * per >= width) lanes /= 2;
+    const int sub = lane / lanes, step = 32 / lanes;
+    for (int c = (lane & (lanes - 1)) * per; c < width; c += lanes * per) {
+      T* const yc = ys + slice * KS + c;
+#pragma unroll 4
+      for (int i = sub; i < count; i += step) {
+        T* const y = yc + (long long)empty_s[warp][i] * k;
+        if (wide) {
+          float zero[16 / sizeof(T)];
+#pragma unroll
+          for (int x = 0; x < 16 / (int)sizeof(T); ++x) zero[x] = 0.0f;
+          piece_store<T, 16 / (int)sizeof(T)>(y, zero, 0.0f, beta);
+        } else {
+          float zero[V];
+#pragma unroll
+          for (int x = 0; x < V; ++x) zero[x] = 0.0f;
+          piece_store<T, V>(y, zero, 0.0f, beta);
+        }
+      }
+    }
+  };
 
   if (s0 < s1) fetch(s0, r_lo, r_hi, stage_s[warp][0]);
   cp_async_commit();
@@ -227,8 +278,34 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
     } else {
       vls = st.val;
     }
-    auto share_end = [&](int j) { return (int)((unsigned)uniform(st.end[j]) - (unsigned)p0); };
-    int j_row = 0, end = share_end(0);             // the current row ends before nonzero `end` of the share
+    int listed = rows, empties = 0;
+    if constexpr (LIST) {
+      listed = 0;
+      // The rows of the share that have nonzeros, in order, written over the ends: (number among the share's rows) << 8 | (nonzero before
+      // which it ends).  The others are listed apart and scaled (set to zero) at once, as many lanes to a row as it has pieces and several
+      // rows in flight: one by one between the others, each would cost the walk a wait for its old values.
+      for (int i0 = 0; i0 < rows; i0 += 32) {
+        const int i = i0 + lane;
+        const int e = i < rows ? st.end[i] : 0;
+        int before = __shfl_up_sync(0xFFFFFFFFu, e, 1);
+        if (lane == 0) before = begin;
+        begin = __shfl_sync(0xFFFFFFFFu, e, min(31, rows - 1 - i0));
+        const bool full = i < rows && e != before, empty = i < rows && e == before;
+        const unsigned fulls = __ballot_sync(0xFFFFFFFFu, full), empty_rows = __ballot_sync(0xFFFFFFFFu, empty), below = (1u << lane) - 1u;
+        if (full) st.end[listed + __popc(fulls & below)] = (i << 8) | (e - p0);     // (behind what has been read: the list is never ahead of i)
+        if (empty) empty_s[warp][empties + __popc(empty_rows & below)] = (unsigned char)i;
+        listed += __popc(fulls);
+        empties += __popc(empty_rows);
+        __syncwarp();
+      }
+      if (lane == 0) st.end[listed] = 0xFF;                    // no end inside this share
+      __syncwarp();
+    }
+    T* const ys = LIST ? Y + (long long)r_lo * k : nullptr;
+    if constexpr (LIST) { if (empties > 0) scale_rows(ys, empties); }
+    // the current row ends before nonzero `end` of the share
+    auto share_end = [&](int j) { return LIST ? uniform(st.end[j]) : (int)((unsigned)uniform(st.end[j]) - (unsigned)p0); };
+    int j_row = 0, row = share_end(0), end = LIST ? row & 0xFF : row;
     // the current row has been added up to its end: stored, or left as the warp's head when it began earlier
     auto finish_row = [&]() {
 #pragma unroll
@@ -242,6 +319,7 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
 #pragma unroll
           for (int i = 0; i < V; ++i) head_s[warp][32 * V * j + lane * V + i] = acc[j][i];
       } else {
+        T* const yp = LIST ? ys + (long long)(row >> 8) * k + col0 : yrow;
 #pragma unroll
         for (int j = 0; j < J; ++j) if (on[j]) piece_store<T, V>(yp + 32 * V * j, acc[j], alpha, beta);
       }
@@ -249,8 +327,9 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
       for (int j = 0; j < J; ++j)
 #pragma unroll
         for (int i = 0; i < V; ++i) acc[j][i] = 0.0f;
-      yp += k;
-      end = share_end(++j_row);
+      row = share_end(++j_row);
+      end = LIST ? row & 0xFF : row;
+      if constexpr (!LIST) yrow += k;
     };
     for (int q = 0; q < cnt; q += U) {
       int c[U];
@@ -279,13 +358,14 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
       } else {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          while (end == q + u) finish_row();
+          if constexpr (LIST) { if (end == q + u) finish_row(); }
+          else while (end == q + u) finish_row();
 #pragma unroll
           for (int j = 0; j < J; ++j) piece_fma<T, V>(b[u][j], v[u], acc[j]);
         }
       }
     }
-    while (j_row < rows) finish_row();
+    while (j_row < listed) finish_row();                     // the row (rows) that end with the share
 #pragma unroll
     for (int j = 0; j < J; ++j)
 #pragma unroll
