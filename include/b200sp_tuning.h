@@ -32,7 +32,7 @@ extern "C" {
  *                    launch gathers from stay in L2: 1 = no ranges (default: measured slower, see the benchmarks' record),
  *                    0 = as many as make a range of B fit L2, 2, 3, 4 or 8 = that many
  *  merge-tile SpMV kernel
- *   "merge_items"    merge items per tile: 1024, 2048 (default) or 4096
+ *   "merge_items"    merge items per tile: 1024, 2048 (default; 1024 below 12 million rows + nonzeros) or 4096
  *   "merge_threads"  threads per CTA: 64, 128 (default) or 256
  *   "merge_carve"    shared-memory carveout in percent requested for it: 0, 25, 45 (default), 60, 75, 100 or -1 = leave to the driver
  *   "merge_short"    rows of up to this many products are added by one thread: 8, 16, 32 (default) or 64
@@ -41,7 +41,7 @@ extern "C" {
  *                    measured 3 % slower on the power-law workload with 61 % empty rows)
  *  row-direct SpMV kernel
  *   "row_stages"     shared-memory stages per CTA, 2 (default) .. 4
- *   "row_ctas"       CTAs per SM the tiles are sized for, 1..4, default 3
+ *   "row_ctas"       CTAs per SM the tiles are sized for, 1..4, default 3 (3 and 4 are raised to 5 at most where short rows leave room)
  *   "row_smem_kb"    shared memory per SM it may use for stages: 48, 96, 160, 220 (default) or 227 (what is left stays L1)
  *   "row_threads"    threads per CTA, 128 or 256 (default)
  *   "row_unroll"     gathers in flight per thread, 8 (default) or 16

@@ -128,6 +128,15 @@ int plan_row_lists(b200sp_plan* p, cudaStream_t stream, DeviceInfo* dev) {
   return B200SP_OK;
 }
 
+// Lanes per row of the sub-warp kernel: by the mean row length, raised so that no lane adds more than kSubwarpChain terms in sequence.
+int subwarp_lanes(int64_t m, int64_t nnz, int max_len) {
+  const double mean = m > 0 ? (double)nnz / (double)m : 0.0;
+  int lpr = g_opt.sub_lanes;
+  if (lpr <= 0) lpr = mean <= 3 ? 1 : mean <= 6 ? 2 : mean <= 12 ? 4 : mean <= 24 ? 8 : mean <= 64 ? 16 : 32;
+  while (lpr < 32 && ((long long)max_len + lpr - 1) / lpr > kSubwarpChain) lpr *= 2;
+  return lpr;
+}
+
 int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32_t* row_ptr, cudaStream_t stream) {
   DeviceInfo* dev = nullptr;
   int rc = device_info(&dev);
@@ -137,7 +146,9 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
   p->row_ptr = row_ptr;
   b200sp_plan_info_t& I = p->info;
   I.m = m; I.n = n; I.nnz = nnz;
-  const int items = g_opt.merge_items;
+  // SpMV tiles of 1024 items instead of 2048 below 12 M: more CTAs (R-MAT 2^17 10.4 / 11.5 us, 2^18 15.9 / 16.5 us, 2^19 23.7 / 25.4 us,
+  // 2^20 40.6 / 42.2 us; equal from 2^21 on)
+  const int items = g_opt.merge_items == 2048 && m + nnz < 12000000 ? 1024 : g_opt.merge_items;
   I.spmv_tile_items = items;
   I.spmv_tiles = (int32_t)((m + nnz + items - 1) / items);
   I.spmv_kernel = g_opt.spmv_kernel >= 0 ? g_opt.spmv_kernel : 0;
@@ -211,7 +222,10 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
   int choice = uniform_ok ? 2 : (row_direct_ok ? 1 : 0);
   // Small problems (launch-latency regime): one sub-warp per row, no scratch, maximum spread over the SMs -- unless the
   // rows are uniform (the uniform-row kernel is as flat) or the row-direct kernel would still get a tile for every SM.
-  if (nnz > 0 && nnz <= kSmallNnz && h.max_len <= 32 * kSubwarpChain && !uniform_ok && !(row_direct_ok && m >= (int64_t)kRowThreads * dev->sms)) choice = 3;
+  // A lane that adds more than some 40 products in sequence makes the launch wait for it (0.27 us for two): the merge-tile kernel with its
+  // second launch is then faster (R-MAT 2^14 / 2^15 / 2^16: 7.5 / 9.3 / 17.7 us by sub-warps, 6.5 / 7.3 / 7.8 us by tiles).
+  const int sub = subwarp_lanes(m, nnz, h.max_len);
+  if (nnz > 0 && nnz <= kSmallNnz && (h.max_len + sub - 1) / sub <= 40 && !uniform_ok && !(row_direct_ok && m >= (int64_t)kRowThreads * dev->sms)) choice = 3;
   if (g_opt.spmv_kernel == 3) choice = h.max_len <= 32 * kSubwarpChain ? 3 : 0;
   if (g_opt.spmv_kernel == 0) choice = 0;
   if (g_opt.spmv_kernel == 1) choice = row_direct_possible ? 1 : 0;

@@ -20,14 +20,25 @@ int run_scale(long long count, T* y, float beta, cudaStream_t stream, DeviceInfo
 
 int gcd_int(int a, int b) { while (b) { const int t = a % b; a = b; b = t; } return a; }
 
+// CTAs per SM that the row-direct kernel's tiles are sized for: the switch, raised to at most 5 (what the registers allow) where rows are so short
+// that tiles of a row per thread leave shared memory unused: 5-point Laplacian 1000^2 FP32 13.5 us with 5, 17.2 us with 3.
+template <typename T>
+int row_ctas_for(int threads, int max_len, int stages, int sm_budget) {
+  int ctas = g_opt.row_ctas;
+  const int full = stages * row_tile_stage_bytes<T>(threads, (threads * max_len + 16 + 7) & ~7) + 1024 + 256 + 128;
+  while (ctas >= 3 && ctas < 5 && (ctas + 1) * full <= sm_budget) ++ctas;
+  return ctas;
+}
+
 template <typename T, int THREADS, int UNROLL, bool ROT>
 int launch_row_direct(b200sp_plan* p, const int32_t* col_idx, const T* vals, const T* x, T* y, float alpha, float beta,
                       cudaStream_t stream, DeviceInfo* dev, int rot_lanes) {
   const b200sp_plan_info_t& I = p->info;
   const int max_len = I.max_row_len > 0 ? I.max_row_len : 1;
-  const int stages = g_opt.row_stages, ctas = g_opt.row_ctas;
+  const int stages = g_opt.row_stages;
   int sm_budget = g_opt.row_smem_kb * 1024;
   if (sm_budget > kSmemPerSm) sm_budget = kSmemPerSm;
+  const int ctas = row_ctas_for<T>(THREADS, max_len, stages, sm_budget);
   const int cta_budget = sm_budget / ctas - 1024 - 256;
   const int stage_budget = cta_budget / stages;
   const int cap_max = (stage_budget - (THREADS + 4) * 4 - 64) / (4 + (int)sizeof(T));
@@ -60,9 +71,10 @@ template <typename T>
 int launch_row_direct_ell(int64_t m, int width, const int32_t* col_ids, const T* vals, const T* x, T* y, float alpha, float beta,
                           cudaStream_t stream, DeviceInfo* dev) {
   constexpr int THREADS = kRowThreads, UNROLL = 8;
-  const int stages = g_opt.row_stages, ctas = g_opt.row_ctas;
+  const int stages = g_opt.row_stages;
   int sm_budget = g_opt.row_smem_kb * 1024;
   if (sm_budget > kSmemPerSm) sm_budget = kSmemPerSm;
+  const int ctas = row_ctas_for<T>(THREADS, width, stages, sm_budget);
   const int stage_budget = (sm_budget / ctas - 1024 - 256) / stages;
   const int cap_max = (stage_budget - (THREADS + 4) * 4 - 64) / (4 + (int)sizeof(T));
   int R = (cap_max - 16) / width;
@@ -219,12 +231,7 @@ template <typename T>
 int run_spmv_subwarp(b200sp_plan* p, const int32_t* col_idx, const T* vals, const T* x, T* y, float alpha, float beta,
                      cudaStream_t stream, DeviceInfo* dev) {
   const b200sp_plan_info_t& I = p->info;
-  const double mean = I.m > 0 ? (double)I.nnz / (double)I.m : 0.0;
-  int lpr = g_opt.sub_lanes;
-  if (lpr <= 0) lpr = mean <= 3 ? 1 : mean <= 6 ? 2 : mean <= 12 ? 4 : mean <= 24 ? 8 : mean <= 64 ? 16 : 32;
-  // no lane adds more than kSubwarpChain terms in sequence, whatever the mean says (the plan sends matrices with a row
-  // longer than 32 * kSubwarpChain to the merge-tile kernel)
-  while (lpr < 32 && ((long long)I.max_row_len + lpr - 1) / lpr > kSubwarpChain) lpr *= 2;
+  const int lpr = subwarp_lanes(I.m, I.nnz, I.max_row_len);
   switch (lpr) {
     case 1: return launch_subwarp<T, 1>(p, col_idx, vals, x, y, alpha, beta, stream, dev);
     case 2: return launch_subwarp<T, 2>(p, col_idx, vals, x, y, alpha, beta, stream, dev);
