@@ -170,6 +170,23 @@ int run_spmv_uniform(b200sp_plan* p, const int32_t* col_idx, const T* vals, cons
   return B200SP_ERR_UNSUPPORTED;
 }
 
+// Rows all of one length that the kernel above does not take (spmv_equal_rows_kernel).
+bool spmv_rows_are_equal(const b200sp_plan_info_t& I) { return I.nnz > 0 && I.min_row_len == I.max_row_len && I.max_row_len >= 3 && I.max_row_len <= 64; }
+
+template <typename T>
+int run_spmv_equal_rows(b200sp_plan* p, const int32_t* col_idx, const T* vals, const T* x, T* y, float alpha, float beta,
+                        cudaStream_t stream, DeviceInfo* dev) {
+  constexpr int THREADS = 128;
+  const b200sp_plan_info_t& I = p->info;
+  const int L = I.max_row_len, G = L <= 16 ? 1 : L <= 32 ? 2 : 4, stride = G * ((L + G - 1) / G | 1);
+  const long long rows = THREADS / G, blocks = (I.m + rows - 1) / rows;
+  const size_t smem = (size_t)rows * stride * sizeof(float);
+  auto kernel = G == 1 ? spmv_equal_rows_kernel<T, THREADS, 1> : G == 2 ? spmv_equal_rows_kernel<T, THREADS, 2> : spmv_equal_rows_kernel<T, THREADS, 4>;
+  tl_pdl_kernel = true;
+  return launch_smem(kernel, dim3((unsigned)blocks), dim3(THREADS), smem, stream, x, (size_t)I.n * sizeof(T), dev, (int)I.m, (int)I.nnz, L, stride,
+                     (unsigned)((65536 + L - 1) / L), col_idx, vals, x, y, alpha, beta);
+}
+
 // y of the rows that are not in a merge list of non-empty rows: y = beta * y (zero when beta == 0).
 template <typename T>
 int run_empty_rows(b200sp_plan* p, T* y, float beta, cudaStream_t stream, DeviceInfo* dev) {
@@ -292,6 +309,7 @@ int run_spmv(b200sp_plan* p, const int32_t* col_idx, const T* vals, const T* x, 
     const int rc = probe_col_locality(p, col_idx, stream);
     if (rc != B200SP_OK) return rc;
     if (!p->cols_local) {
+      if (spmv_rows_are_equal(I)) return run_spmv_equal_rows<T>(p, col_idx, vals, x, y, alpha, beta, stream, dev);
       return run_spmv_merge_any<T>(p, col_idx, vals, x, y, alpha, beta, stream, dev);
     }
   }

@@ -63,6 +63,59 @@ spmv_uniform_vec_kernel(long long quads, const int* __restrict__ col_idx, const 
   }
 }
 
+// The same for rows of any one length L of 3 .. 64: a warp takes 32 / G rows (G = 1, 2, 4 for L to 16, 32, 64), whose nonzeros are contiguous
+// and start on a multiple of four, so that they stream with the same 128-bit loads; the products go to the warp's own shared memory, and G
+// lanes per row add them up.  Bound like the kernel above by the gathers' L1 misses: no more than 512 products a warp, because with 1024
+// (32 rows of 24) shared memory left the gathers no L1 and the time doubled.  `stride` is an odd multiple of G: no bank conflicts in the sums.
+// Against the merge-tile kernel, which scattered columns took before, FP32: 4.2 M nonzeros in rows of 5 / 12 / 50 19.7 / 20.0 / 20.6 us (25.0 / 23.0 / 26.7 us),
+// 16.8 M in rows of 5 / 12 / 40 70 / 67 / 66 us (82 / 73 / 91 us).
+template <typename T, int THREADS, int G>
+__global__ void __launch_bounds__(THREADS, 2048 / THREADS)
+spmv_equal_rows_kernel(int m, int nnz, int L, int stride, unsigned inv, const int* __restrict__ col_idx, const T* __restrict__ vals, const T* __restrict__ x,
+                       T* __restrict__ y, float alpha, float beta) {
+  extern __shared__ float equal_rows_prod[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int rows = 32 / G;
+  float* const prod = equal_rows_prod + warp * rows * stride;
+  grid_dependency_wait();
+  const long long warps = (long long)gridDim.x * (THREADS / 32);
+  for (long long w = (long long)blockIdx.x * (THREADS / 32) + warp; w * rows < m; w += warps) {
+    const long long row = w * rows + lane / G;
+    const float yold = beta != 0.0f && row < m ? to_f32(y[row]) : 0.0f;   // asked for now: its latency overlaps the gathers
+    const int p0 = (int)(w * rows * L), cnt = min(rows * L, nnz - p0);
+    for (int e = lane * 4; e < cnt; e += 128) {
+      int c[4];
+      float v[4];
+      if (e + 4 <= cnt) {
+        const int4 cc = ld_stream_i4(col_idx + p0 + e);
+        c[0] = cc.x; c[1] = cc.y; c[2] = cc.z; c[3] = cc.w;
+        ld_stream_vals4(vals + p0 + e, v);
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { c[u] = e + u < cnt ? ld_stream_i1(col_idx + p0 + e + u) : -1; v[u] = e + u < cnt ? ld_stream_val1(vals + p0 + e + u) : 0.0f; }
+      }
+      float g[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) g[u] = c[u] >= 0 ? ld_gather(x + c[u]) : 0.0f;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)   // (e + u) / L: inv = ceil(2^16 / L) gives it exactly below 512
+        prod[e + u + (int)(((unsigned)(e + u) * inv) >> 16) * (stride - L)] = v[u] * g[u];
+    }
+    __syncwarp();
+    float acc = 0.0f;
+    if (row < m)
+      for (int j = lane & (G - 1); j < L; j += G) acc += prod[lane / G * stride + j];
+    #pragma unroll
+    for (int d = G >> 1; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+    if (row < m && (lane & (G - 1)) == 0) {
+      float r = alpha * acc;
+      if (beta != 0.0f) r += beta * yold;
+      store_elem(y + row, r);
+    }
+    __syncwarp();
+  }
+}
+
 }  // namespace b200sp
 
 namespace b200sp {
