@@ -265,11 +265,13 @@ struct b200sp_plan {
   int cuts_ranges = 0;                    // number of ranges they describe (0 = none computed)
   bool cols_sorted = false;               // every row's columns ascend
   // processing order of the SpMM kernel with B in shared memory: rows of at most kLongRow nonzeros sorted by length, in blocks of quad_gpw
-  void* quad_block = nullptr;             // one pool block: row numbers, row lengths, block offsets (built on first use)
-  int32_t* quad_row = nullptr;            // quad_blocks * quad_gpw row numbers (-1 = unused slot)
-  int32_t* quad_len = nullptr;            // their lengths
-  int32_t* quad_pos = nullptr;            // quad_blocks + 1: where each block's quads start in the per-call copy of A
-  int quad_gpw = 0, quad_blocks = 0;
+  struct QuadOrder {
+    void* block = nullptr;                // one pool block: row numbers, row lengths, block offsets (built on first use)
+    int32_t* row = nullptr;               // blocks * gpw row numbers (-1 = unused slot)
+    int32_t* len = nullptr;               // their lengths
+    int32_t* pos = nullptr;               // blocks + 1: where each block's quads start in the per-call copy of A
+    int blocks = 0;
+  } quad[4];                              // for 4, 8, 16 and 32 rows per warp
   const void* probed_key = nullptr;       // host entry points: the HOST col_idx that verdict belongs to
   bool cols_local = true;                 // its verdict: adjacent rows share most of their lines of x
 };

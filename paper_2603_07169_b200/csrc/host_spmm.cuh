@@ -113,14 +113,15 @@ int device_scan_in_place(int* data, long long count, int* bsum, cudaStream_t str
 
 // The processing order of spmm_bstage_quads_kernel (see plan_kernels.cuh), built once per plan and lane-group width, on the
 // device and in stream order: no synchronisation.  B200SP_ERR_UNSUPPORTED when the positions would not fit 32 bits.
-int plan_quad_order(b200sp_plan* p, int gpw, cudaStream_t stream, DeviceInfo* dev) {
+int plan_quad_order(b200sp_plan* p, int gpw, b200sp_plan::QuadOrder** out, cudaStream_t stream, DeviceInfo* dev) {
   static_assert(kLongRow == 1024, "quad_key() assumes rows of at most 1024 nonzeros");
-  if (p->quad_block && p->quad_gpw == gpw) return B200SP_OK;
+  b200sp_plan::QuadOrder& Q = p->quad[gpw == 4 ? 0 : gpw == 8 ? 1 : gpw == 16 ? 2 : 3];
+  *out = &Q;
+  if (Q.block) return B200SP_OK;
   const b200sp_plan_info_t& I = p->info;
   const long long listed = I.m - p->num_long;
   const long long blocks = (listed + gpw - 1) / gpw;
   if ((I.nnz + 3 * I.m) / 4 + (long long)(kLongRow / 4 + 2) * gpw >= (1LL << 31) - 64 || blocks < 1) return B200SP_ERR_UNSUPPORTED;
-  if (p->quad_block) { CU(cudaFreeAsync(p->quad_block, stream)); p->quad_block = nullptr; p->quad_gpw = 0; }
   long long rows_per_blk = (I.m + 65535) / 65536;
   if (rows_per_blk < 256) rows_per_blk = 256;
   rows_per_blk = (rows_per_blk + 31) / 32 * 32;
@@ -158,22 +159,22 @@ int plan_quad_order(b200sp_plan* p, int gpw, cudaStream_t stream, DeviceInfo* de
   if (rc != B200SP_OK) return fail(rc);
   CUQ(cudaFreeAsync(tmp, stream));
 #undef CUQ
-  p->quad_block = blk;
-  p->quad_row = row_of;
-  p->quad_len = len_of;
-  p->quad_pos = pos;
-  p->quad_gpw = gpw;
-  p->quad_blocks = (int)blocks;
+  Q.block = blk;
+  Q.row = row_of;
+  Q.len = len_of;
+  Q.pos = pos;
+  Q.blocks = (int)blocks;
   return B200SP_OK;
 }
 
 // The same with the rows in the plan's sorted order and A re-laid once per call into padded quads (spmm_bstage_prep_kernel),
 // which the main kernel's warps fetch with bulk copies; rows longer than kLongRow by spmm_long_row_kernel.
-template <typename T, int VEC, int LANES, int THREADS = 1024>
-int launch_spmm_bstage_quads(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
+template <typename T, int VEC, int SLICE_LANES, int PIECES, int THREADS>
+int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
                              cudaStream_t stream, DeviceInfo* dev, EncodeTiledFn encode) {
   const b200sp_plan_info_t& I = p->info;
-  constexpr int KS = LANES * VEC, ROW_BYTES = LANES * 16, GPW = 32 / LANES, WARPS = THREADS / 32;
+  constexpr int LANES = SLICE_LANES / PIECES;
+  constexpr int KS = SLICE_LANES * VEC, ROW_BYTES = SLICE_LANES * 16, GPW = 32 / LANES, WARPS = THREADS / 32;
   const int box_rows = I.n < 256 ? (int)I.n : 256;
   const int boxes = (int)((I.n + box_rows - 1) / box_rows);
   const size_t bslice = (((size_t)boxes * box_rows * ROW_BYTES) + 127) & ~(size_t)127;
@@ -197,17 +198,18 @@ int launch_spmm_bstage_quads(b200sp_plan* p, int k, const int32_t* col_idx, cons
                              gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS) return B200SP_ERR_UNSUPPORTED;
-  int rc = plan_quad_order(p, GPW, stream, dev);
+  b200sp_plan::QuadOrder* Q = nullptr;
+  int rc = plan_quad_order(p, GPW, &Q, stream, dev);
   if (rc == B200SP_OK) rc = plan_row_lists(p, stream, dev);
   if (rc != B200SP_OK) return rc;
-  auto kernel = spmm_bstage_quads_kernel<T, VEC, LANES, THREADS>;
+  auto kernel = spmm_bstage_quads_kernel<T, VEC, LANES, PIECES, THREADS>;
   static bool configured[64] = {};
   if (!configured[p->device]) {
     CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerSm - 2048));
     configured[p->device] = true;
   }
   const int slices = (k + KS - 1) / KS;
-  const int blocks = p->quad_blocks;
+  const int blocks = Q->blocks;
   const long long most = (blocks + WARPS - 1) / WARPS;   // a block per warp at least
   long long chunks;
   if (g_opt.bstage_nnz > 0) {
@@ -235,18 +237,23 @@ int launch_spmm_bstage_quads(b200sp_plan* p, int k, const int32_t* col_idx, cons
   // the per-call copy of A: at most the rows' quads plus (kLongRow / 4 + 2) * GPW of padding where the length changes along the list
   const size_t entries = (((size_t)((I.nnz + 3 * I.m) / 4) + (size_t)(kLongRow / 4 + 2) * GPW) * 4 + 15) & ~(size_t)7;
   void* scratch = nullptr;
-  rc = pool_alloc(dev, &scratch, entries * (2 + sizeof(T)), stream);
+  const long long slots = (long long)blocks * GPW;
+  // 64-byte rows of the slice: the copy of A changes the order of a block's rows to have fewer bank conflicts, if there are slices enough to pay
+  // for it (2^14 rows of 20: 8 slices 18.5 us without, 19.5 us with; 16 slices 27.5 / 27.7; 32 slices, 2^15 rows 85.1 / 83.0; 256 slices 276 / 258)
+  const bool reorder = ROW_BYTES == 64 && slices >= 24;
+  rc = pool_alloc(dev, &scratch, entries * (2 + sizeof(T)) + (reorder ? (size_t)slots * 8 : 0), stream);
   if (rc != B200SP_OK) return rc;
   unsigned short* qoff = (unsigned short*)scratch;       // entries 16-bit offsets, then entries values (16-byte aligned: entries is a multiple of 8)
   T* qval = (T*)((char*)scratch + entries * 2);
-  const long long slots = (long long)blocks * GPW;
+  int* slot_row = reorder ? (int*)((char*)scratch + entries * (2 + sizeof(T))) : Q->row;
+  int* slot_len = reorder ? slot_row + slots : Q->len;
   tl_pdl_kernel = true;
   rc = launch(spmm_bstage_prep_kernel<T, ROW_BYTES>, dim3((unsigned)((slots * 8 + 255) / 256)), dim3(256), stream, nullptr, 0, dev, (int)slots, GPW,
-              (const int*)p->quad_row, (const int*)p->quad_pos, p->row_ptr, col_idx, vals, qoff, qval);
+              (const int*)Q->row, (const int*)Q->pos, p->row_ptr, col_idx, vals, qoff, qval, (int)reorder, slot_row, slot_len);
   if (rc == B200SP_OK) {
     tl_pdl_kernel = true;
     rc = launch_smem(kernel, dim3((unsigned)(slices * row_chunks)), dim3(THREADS), smem, stream, nullptr, 0, dev, map, (int)I.n, k, row_chunks,
-                     blocks, box_rows, (int)bslice, capq, (const int*)p->quad_row, (const int*)p->quad_len, (const int*)p->quad_pos,
+                     blocks, box_rows, (int)bslice, capq, (const int*)slot_row, (const int*)slot_len, (const int*)Q->pos,
                      (const unsigned short*)qoff, (const T*)qval, Y, alpha, beta, dev->err_flag, g_opt.spin_limit, g_opt.debug_no_copies);
   }
   const cudaError_t e = cudaFreeAsync(scratch, stream);
@@ -259,6 +266,21 @@ int launch_spmm_bstage_quads(b200sp_plan* p, int k, const int32_t* col_idx, cons
                 (const int*)p->long_rows, p->row_ptr, col_idx, vals, B, Y, alpha, beta);
   }
   return rc;
+}
+
+// Pieces of 16 bytes per lane and row: two where the slice has at least 64 bytes a row and the warps of all SMs get a step at least (half as
+// many reads of A and half as many address instructions per product).  2^16 rows of 20 x 4096 FP32 1017 us with two, 1092 us with one; 2^14 rows
+// of 10 (128-byte slices) 156 / 203 us; but 2^10 rows x 256 columns, 1024 steps, 12.1 / 10.8 us.  BF16 with 16 columns a lane wants
+// 80 registers: 768 threads (512 threads 285 us, 768 threads 270 us on 2^16 rows x 2048 columns, one piece 308 us).
+template <typename T, int VEC, int SLICE_LANES, int THREADS>
+int launch_spmm_bstage_quads(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
+                             cudaStream_t stream, DeviceInfo* dev, EncodeTiledFn encode) {
+  if constexpr (SLICE_LANES >= 4 && THREADS == 1024) {
+    const long long slices = (k + SLICE_LANES * VEC - 1) / (SLICE_LANES * VEC), steps = (p->info.m * SLICE_LANES / 64 + 1) * slices;
+    if (steps >= 32LL * dev->sms)
+      return launch_spmm_bstage_quads_as<T, VEC, SLICE_LANES, 2, sizeof(T) == 2 ? 768 : 1024>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev, encode);
+  }
+  return launch_spmm_bstage_quads_as<T, VEC, SLICE_LANES, 1, THREADS>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev, encode);
 }
 
 // Column ranges for the k-sliced kernel: how many, and the per-row cut positions (computed once per col_idx; one small

@@ -203,29 +203,52 @@ spmm_bstage_kernel(const __grid_constant__ CUtensorMap tmapB, int m, int n, int 
 //   their rows are equally long they read different parts of the bank line.  (The order of a row's products
 //   changes; each lane still adds them in one fixed order.)
 //
+// With two rows to a bank line (64-byte rows, n = 2048) the rows of a block are also re-ordered by how many of their columns are even.
+//
 // spmm_bstage_quads_kernel then needs no alignment steps and gets a block's quads with ONE bulk copy per array (TMA,
-// on a barrier of the warp's own, outside the LSU pipe).
+// on a barrier of the warp's own, outside the LSU pipe).  A lane holds one or two 16-byte pieces of its row's part of the slice (PIECES): two halve
+// the reads of A and the address instructions per product.
 // Rows longer than kLongRow are left to spmm_long_row_kernel.
 template <typename T, int ROW_BYTES>
 __global__ void __launch_bounds__(256)
 spmm_bstage_prep_kernel(int slots, int gpw, const int* __restrict__ quad_row, const int* __restrict__ quad_pos,
                         const int* __restrict__ row_ptr, const int* __restrict__ col_idx, const T* __restrict__ vals,
-                        unsigned short* __restrict__ qoff, T* __restrict__ qval) {
+                        unsigned short* __restrict__ qoff, T* __restrict__ qval, int reorder, int* __restrict__ slot_row, int* __restrict__ slot_len) {
   constexpr int G = 128 / ROW_BYTES;
+  constexpr int SLOTS = 32;                   // of a CTA of 256 threads: whole blocks of gpw = 8, 16 or 32
+  __shared__ int excess[SLOTS];
   constexpr unsigned FULL = 0xFFFFFFFFu;
   grid_dependency_wait();
   const int lane = threadIdx.x & 31, sub = lane & 7, first = lane & ~7;   // eight lanes per row, four rows per warp
   const long long slot = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
-  int rs = 0, re = 0, g = 0;
-  long long base = 0;       // entry index of quad 0 of this row
+  const int b = (int)(slot / gpw);
+  int rs = 0, re = 0, g = (int)(slot - (long long)b * gpw), row = -1;   // g also past the last slot: `excess` is indexed with it
   if (slot < slots) {
-    const int row = __ldg(quad_row + slot);
-    const int b = (int)(slot / gpw);
-    g = (int)(slot - (long long)b * gpw);
+    row = __ldg(quad_row + slot);
     if (row >= 0) { rs = __ldg(row_ptr + row); re = __ldg(row_ptr + row + 1); }
-    base = ((long long)__ldg(quad_pos + b) + g) * 4;
   }
   const int len = re - rs;
+  int even = 0;    // entries in even columns
+  if constexpr (G == 2) {
+    for (int p = rs + sub; p < re; p += 8) even += !(__ldg(col_idx + p) & 1);
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) even += __shfl_xor_sync(FULL, even, d);
+  }
+  if (G == 2 && reorder) {
+    // Neighbouring slots read the same banks in every step in which one of their rows is in its even columns and the other as well, which
+    // is as often as the even columns of the one differ in number from the odd ones of the other.  So the row with the largest excess
+    // of even columns is put next to the one with the smallest, and so on inward: the rows of a block change places.
+    const int mine = (int)(threadIdx.x >> 3), block0 = mine - g, ex = 2 * even - len;
+    if (sub == 0) excess[mine] = ex;
+    __syncthreads();
+    int rank = 0;
+    for (int j = sub; j < gpw; j += 8) rank += excess[block0 + j] < ex || (excess[block0 + j] == ex && j < g);
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) rank += __shfl_xor_sync(FULL, rank, d);
+    g = 2 * rank < gpw ? 2 * rank : 2 * (gpw - 1 - rank) + 1;
+    if (slot < slots && sub == 0) { slot_row[(long long)b * gpw + g] = row; slot_len[(long long)b * gpw + g] = len; }
+  }
+  const long long base = slot < slots ? ((long long)__ldg(quad_pos + b) + g) * 4 : 0;       // entry index of quad 0 of this row
   const int stride = gpw * 4;                 // entries from one quad of the row to the next
   const int gc = g & (G - 1);
   int start[G];    // where class j begins inside the row
@@ -233,7 +256,9 @@ spmm_bstage_prep_kernel(int slots, int gpw, const int* __restrict__ quad_row, co
     int cnt[G];
 #pragma unroll
     for (int j = 0; j < G; ++j) cnt[j] = 0;
-    if (G > 1) {
+    if constexpr (G == 2) {
+      cnt[0] = gc ? len - even : even;
+    } else if (G > 1) {
       for (int p = rs + sub; p < re; p += 8) {
         const int cls = (__ldg(col_idx + p) - gc) & (G - 1);
 #pragma unroll
@@ -302,12 +327,12 @@ template <bool SHARED> struct QuadLoad<bf16_t, SHARED> {
   }
 };
 
-// acc += the products of one row's quads 0 .. (len + 3) / 4 - 1 with this lane's columns of the slice (whose piece of row 0
-// is at shared address bs).  SHARED: the quads sit in shared memory at addresses so / sv, else in global memory at qo / qv;
-// consecutive quads of the row are qstride quads apart.
-template <typename T, int VEC, bool SHARED>
+// acc += the products of one row's quads 0 .. (len + 3) / 4 - 1 with this lane's columns of the slice: PIECES pieces of 16 bytes, the first one of
+// row 0 at shared address bs, the second `other` bytes from it.  SHARED: the quads sit in shared memory at addresses so / sv, else in global
+// memory at qo / qv; consecutive quads of the row are qstride quads apart.
+template <typename T, int VEC, int PIECES, bool SHARED>
 __device__ __forceinline__ void bstage_row_quads(const uint2* __restrict__ qo, const T* __restrict__ qv, unsigned so, unsigned sv, int qstride,
-                                                 int len, unsigned bs, float (&acc)[VEC], float (&tot)[VEC]) {
+                                                 int len, unsigned bs, int other, float (&acc)[PIECES][VEC], float (&tot)[PIECES][VEC]) {
   typedef typename RawVec<T, VEC>::type raw_t;
   const int full = len >> 2, rem = len & 3;
   int fold = 0;
@@ -315,39 +340,55 @@ __device__ __forceinline__ void bstage_row_quads(const uint2* __restrict__ qo, c
     if (++fold > kChainBlock / 4) {
       fold = 1;
 #pragma unroll
-      for (int j = 0; j < VEC; ++j) { tot[j] += acc[j]; acc[j] = 0.0f; }
+      for (int e = 0; e < PIECES; ++e)
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) { tot[e][j] += acc[e][j]; acc[e][j] = 0.0f; }
     }
     unsigned a[4];
     float v[4];
     QuadLoad<T, SHARED>::ld(qo, qv, so, sv, bs, a, v);
     so += 8u * qstride; sv += 4u * (unsigned)sizeof(T) * qstride; qo += qstride; qv += 4 * qstride;
-    raw_t b[4];
+    constexpr int U = PIECES == 2 && sizeof(T) == 2 ? 2 : 4;   // loads in flight: two entries' worth where 16 columns a lane leave no registers
 #pragma unroll
-    for (int u = 0; u < 4; ++u) b[u] = lds128(a[u], (const raw_t*)nullptr);
+    for (int u0 = 0; u0 < 4; u0 += U) {
+      raw_t b[U][PIECES];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) RawVec<T, VEC>::fma_mixed(b[u], v[u], acc);
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int e = 0; e < PIECES; ++e) b[u][e] = lds128(a[u0 + u] + (e ? other : 0), (const raw_t*)nullptr);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int e = 0; e < PIECES; ++e) RawVec<T, VEC>::fma_mixed(b[u][e], v[u0 + u], acc[e]);
+    }
   }
   if (rem) {   // the padded last quad: its padding is never multiplied (0 * inf would be NaN)
     unsigned a[4];
     float v[4];
     QuadLoad<T, SHARED>::ld(qo, qv, so, sv, bs, a, v);
-    RawVec<T, VEC>::fma_mixed(lds128(a[0], (const raw_t*)nullptr), v[0], acc);
-    if (rem > 1) RawVec<T, VEC>::fma_mixed(lds128(a[1], (const raw_t*)nullptr), v[1], acc);
-    if (rem > 2) RawVec<T, VEC>::fma_mixed(lds128(a[2], (const raw_t*)nullptr), v[2], acc);
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      if (u < rem)
+#pragma unroll
+        for (int e = 0; e < PIECES; ++e) RawVec<T, VEC>::fma_mixed(lds128(a[u] + (e ? other : 0), (const raw_t*)nullptr), v[u], acc[e]);
   }
 }
 
+// Bound by the L1 data pipe (85 % busy on 2^14 rows of 20 x 4096 FP32, n = 2048), whose wavefronts are the reads of B (43 M of 61.8 M, 128 bytes
+// each), the stores of Y (7.2 M), the reads of A (4.4 M; 8.7 M with one piece per lane), conflicts (4.5 M; 10.2 M without the re-ordered blocks) and
+// the bulk copies' writes (2.8 M).  With 128-byte slices there are no conflicts and the issue slots bind (81 %).  2^16 rows: 941 us; one piece
+// per lane and blocks as sorted 1092 us.
 // Dynamic shared memory: [ slice of B: bslice_bytes | per warp: capq offset quads (8 B each), capq value quads (4 values each) ]; capq is even.
 // CTA `chunk` of a slice takes the blocks chunk, chunk + row_chunks, ... of the sorted list, its warps in turn, so that
 // every CTA gets the same mix of long and short rows.  A block of more than capq quads is read from global memory.
 // (Fetching the next block's quads a step ahead into a second half of the buffer was measured: no gain.)
-template <typename T, int VEC, int LANES, int THREADS>
+template <typename T, int VEC, int LANES, int PIECES, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 spmm_bstage_quads_kernel(const __grid_constant__ CUtensorMap tmapB, int n, int k, int row_chunks, int blocks, int box_rows, int bslice_bytes,
                          int capq, const int* __restrict__ quad_row, const int* __restrict__ quad_len, const int* __restrict__ quad_pos,
                          const unsigned short* __restrict__ qoff, const T* __restrict__ qval, T* __restrict__ Y, float alpha, float beta,
                          int* __restrict__ err, int spin_limit, int no_copies) {
-  constexpr int KS = LANES * VEC, ROW_BYTES = LANES * 16, GPW = 32 / LANES, WARPS = THREADS / 32;
+  constexpr int KS = LANES * PIECES * VEC, ROW_BYTES = LANES * PIECES * 16, GPW = 32 / LANES, WARPS = THREADS / 32;
   constexpr unsigned FULL = 0xFFFFFFFFu;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) unsigned long long bar;
@@ -367,9 +408,10 @@ spmm_bstage_quads_kernel(const __grid_constant__ CUtensorMap tmapB, int n, int k
       tma_load_2d(smem_addr(smem + (size_t)b * box_rows * ROW_BYTES), &tmapB, col_base, b * box_rows, smem_addr(&bar));
   }
   const int gl = lane / LANES, l = lane % LANES;     // group inside the warp, lane inside the group
-  const int col0 = col_base + l * VEC;
-  const bool active = col0 < k;
-  const unsigned bs = smem_addr(smem) + l * 16;
+  // a lane's first piece is in the one half of the slice or in the other, so that the rows a quarter warp reads at once spread over the banks
+  const int first = PIECES == 2 ? gl / (128 / ROW_BYTES) & 1 : 0, other = first ? -LANES * 16 : LANES * 16;
+  const int col0 = col_base + (first * LANES + l) * VEC;
+  const unsigned bs = smem_addr(smem) + (first * LANES + l) * 16;
   constexpr unsigned VQ = 4u * (unsigned)sizeof(T);                          // bytes of a quad's values
   const unsigned woff = smem_addr(smem) + bslice_bytes + warp * capq * (8u + VQ);   // the warp's buffer: capq quads of offsets, then of values
   const unsigned wval = woff + capq * 8u;
@@ -419,29 +461,31 @@ spmm_bstage_quads_kernel(const __grid_constant__ CUtensorMap tmapB, int n, int k
       phase ^= 1u;
     }
     const int row = __shfl_sync(FULL, row_cur, gl), len = __shfl_sync(FULL, len_cur, gl);
-    float acc[VEC], tot[VEC];   // acc: the current block of at most kChainBlock products; tot: the sum of the completed blocks
+    float acc[PIECES][VEC], tot[PIECES][VEC];   // acc: the current block of at most kChainBlock products; tot: the sum of the completed blocks
 #pragma unroll
-    for (int j = 0; j < VEC; ++j) { acc[j] = 0.0f; tot[j] = 0.0f; }
+    for (int e = 0; e < PIECES; ++e)
+#pragma unroll
+      for (int j = 0; j < VEC; ++j) { acc[e][j] = 0.0f; tot[e][j] = 0.0f; }
     if (staged) {
-      bstage_row_quads<T, VEC, true>(nullptr, nullptr, woff + 8u * gl, wval + VQ * gl, GPW, len, bs, acc, tot);
+      bstage_row_quads<T, VEC, PIECES, true>(nullptr, nullptr, woff + 8u * gl, wval + VQ * gl, GPW, len, bs, other, acc, tot);
     } else {
-      bstage_row_quads<T, VEC, false>((const uint2*)qoff + q0_cur + gl, qval + 4LL * (q0_cur + gl), 0u, 0u, GPW, len, bs, acc, tot);
+      bstage_row_quads<T, VEC, PIECES, false>((const uint2*)qoff + q0_cur + gl, qval + 4LL * (q0_cur + gl), 0u, 0u, GPW, len, bs, other, acc, tot);
     }
     __syncwarp();                       // every lane is done with the buffer: the next block's quads may land in it
     issue(q0_next, nq_next);            // (past the last block nq_next is 0)
-    if (active && row >= 0) {
-      T* yp = Y + (long long)row * k + col0;
+#pragma unroll
+    for (int e = 0; e < PIECES; ++e) {
+      const int col = col0 + (e ? other / 16 * VEC : 0);
+      if (row < 0 || col >= k) continue;
+      T* yp = Y + (long long)row * k + col;
       float out[VEC];
 #pragma unroll
-      for (int j = 0; j < VEC; ++j) acc[j] += tot[j];
+      for (int j = 0; j < VEC; ++j) out[j] = alpha * (acc[e][j] + tot[e][j]);
       if (beta != 0.0f) {
         float old[VEC];
         VecLoad<T, VEC>::ld_plain(yp, old);
 #pragma unroll
-        for (int j = 0; j < VEC; ++j) out[j] = alpha * acc[j] + beta * old[j];
-      } else {
-#pragma unroll
-        for (int j = 0; j < VEC; ++j) out[j] = alpha * acc[j];
+        for (int j = 0; j < VEC; ++j) out[j] += beta * old[j];
       }
       VecLoad<T, VEC>::st(yp, out);
     }

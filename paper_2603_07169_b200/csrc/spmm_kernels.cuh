@@ -146,7 +146,15 @@ template <> struct RawVec<float, 4> {
   static __device__ __forceinline__ void fma(const float4& b, float v, float (&acc)[4]) {
     acc[0] = fmaf(v, b.x, acc[0]); acc[1] = fmaf(v, b.y, acc[1]); acc[2] = fmaf(v, b.z, acc[2]); acc[3] = fmaf(v, b.w, acc[3]);
   }
-  static __device__ __forceinline__ void fma_mixed(const float4& b, float v, float (&acc)[4]) { fma(b, v, acc); }
+  // Same values, two products to an instruction: 1017 against 1027 us in the kernel that keeps B in shared memory (2^16 rows of 20 x 4096).
+  static __device__ __forceinline__ void fma_mixed(const float4& b, float v, float (&acc)[4]) {
+    asm("{ .reg .b64 vv, b0, b1, a0, a1;\n\t"
+        "mov.b64 vv, {%4, %4};\n\tmov.b64 b0, {%5, %6};\n\tmov.b64 b1, {%7, %8};\n\t"
+        "mov.b64 a0, {%0, %1};\n\tmov.b64 a1, {%2, %3};\n\t"
+        "fma.rn.f32x2 a0, vv, b0, a0;\n\tfma.rn.f32x2 a1, vv, b1, a1;\n\t"
+        "mov.b64 {%0, %1}, a0;\n\tmov.b64 {%2, %3}, a1; }"
+        : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3]) : "f"(v), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w));
+  }
 };
 template <> struct RawVec<bf16_t, 8> {
   typedef uint4 type;
