@@ -169,7 +169,7 @@ int plan_quad_order(b200sp_plan* p, int gpw, b200sp_plan::QuadOrder** out, cudaS
 
 // The same with the rows in the plan's sorted order and A re-laid once per call into padded quads (spmm_bstage_prep_kernel),
 // which the main kernel's warps fetch with bulk copies; rows longer than kLongRow by spmm_long_row_kernel.
-template <typename T, int VEC, int SLICE_LANES, int PIECES, int THREADS>
+template <typename T, int VEC, int SLICE_LANES, int PIECES, bool OLD, int THREADS>
 int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
                              cudaStream_t stream, DeviceInfo* dev, EncodeTiledFn encode) {
   const b200sp_plan_info_t& I = p->info;
@@ -202,7 +202,7 @@ int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, c
   int rc = plan_quad_order(p, GPW, &Q, stream, dev);
   if (rc == B200SP_OK) rc = plan_row_lists(p, stream, dev);
   if (rc != B200SP_OK) return rc;
-  auto kernel = spmm_bstage_quads_kernel<T, VEC, LANES, PIECES, THREADS>;
+  auto kernel = spmm_bstage_quads_kernel<T, VEC, LANES, PIECES, OLD, THREADS>;
   static bool configured[64] = {};
   if (!configured[p->device]) {
     CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerSm - 2048));
@@ -238,9 +238,10 @@ int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, c
   const size_t entries = (((size_t)((I.nnz + 3 * I.m) / 4) + (size_t)(kLongRow / 4 + 2) * GPW) * 4 + 15) & ~(size_t)7;
   void* scratch = nullptr;
   const long long slots = (long long)blocks * GPW;
-  // 64-byte rows of the slice: the copy of A changes the order of a block's rows to have fewer bank conflicts, if there are slices enough to pay
-  // for it (2^14 rows of 20: 8 slices 18.5 us without, 19.5 us with; 16 slices 27.5 / 27.7; 32 slices, 2^15 rows 85.1 / 83.0; 256 slices 276 / 258)
-  const bool reorder = ROW_BYTES == 64 && slices >= 24;
+  // 64-byte rows of the slice: the copy of A changes the order of a block's rows to have fewer bank conflicts, if there are slices and rows enough
+  // to pay for it (2^14 rows of 20: 8 slices 18.5 us without, 19.5 us with; 16 slices 27.5 / 27.7; 256 slices 276 / 258; 2^15 rows, 32 slices
+  // 85.1 / 83.0; 2^11 rows, 32 slices 12.1 / 12.6; 11,782 rows, 33 slices 46.0 / 46.7)
+  const bool reorder = ROW_BYTES == 64 && slices >= 24 && (long long)slices * I.m >= (1 << 19);
   rc = pool_alloc(dev, &scratch, entries * (2 + sizeof(T)) + (reorder ? (size_t)slots * 8 : 0), stream);
   if (rc != B200SP_OK) return rc;
   unsigned short* qoff = (unsigned short*)scratch;       // entries 16-bit offsets, then entries values (16-byte aligned: entries is a multiple of 8)
@@ -271,16 +272,20 @@ int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, c
 // Pieces of 16 bytes per lane and row: two where the slice has at least 64 bytes a row and the warps of all SMs get a step at least (half as
 // many reads of A and half as many address instructions per product).  2^16 rows of 20 x 4096 FP32 1017 us with two, 1092 us with one; 2^14 rows
 // of 10 (128-byte slices) 156 / 203 us; but 2^10 rows x 256 columns, 1024 steps, 12.1 / 10.8 us.  BF16 with 16 columns a lane wants
-// 80 registers: 768 threads (512 threads 285 us, 768 threads 270 us on 2^16 rows x 2048 columns, one piece 308 us).
+// 80 registers: 768 threads (512 threads 285 us, 768 threads 270 us on 2^16 rows x 2048 columns, one piece 308 us).  With beta != 0 the old
+// values of Y take registers too and the CTAs are smaller (640 threads BF16: 186 us, 704 197, 768 203, one piece 197, 2^14 rows x 4096), which
+// pays from some ten steps a warp on (2^14 rows of 20 x 1024 BF16 56.4 / 60.2 us; 11,782 x 1048, eight steps, 46.7 / 45.6 us).
 template <typename T, int VEC, int SLICE_LANES, int THREADS>
 int launch_spmm_bstage_quads(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
                              cudaStream_t stream, DeviceInfo* dev, EncodeTiledFn encode) {
   if constexpr (SLICE_LANES >= 4 && THREADS == 1024) {
     const long long slices = (k + SLICE_LANES * VEC - 1) / (SLICE_LANES * VEC), steps = (p->info.m * SLICE_LANES / 64 + 1) * slices;
-    if (steps >= 32LL * dev->sms)
-      return launch_spmm_bstage_quads_as<T, VEC, SLICE_LANES, 2, sizeof(T) == 2 ? 768 : 1024>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev, encode);
+    if (beta == 0.0f && steps >= 32LL * dev->sms)
+      return launch_spmm_bstage_quads_as<T, VEC, SLICE_LANES, 2, false, sizeof(T) == 2 ? 768 : 1024>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev, encode);
+    if (beta != 0.0f && steps >= 192LL * dev->sms)
+      return launch_spmm_bstage_quads_as<T, VEC, SLICE_LANES, 2, true, sizeof(T) == 2 ? 640 : 768>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev, encode);
   }
-  return launch_spmm_bstage_quads_as<T, VEC, SLICE_LANES, 1, THREADS>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev, encode);
+  return launch_spmm_bstage_quads_as<T, VEC, SLICE_LANES, 1, false, THREADS>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev, encode);
 }
 
 // Column ranges for the k-sliced kernel: how many, and the per-row cut positions (computed once per col_idx; one small

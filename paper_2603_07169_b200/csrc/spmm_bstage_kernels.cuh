@@ -382,7 +382,9 @@ __device__ __forceinline__ void bstage_row_quads(const uint2* __restrict__ qo, c
 // CTA `chunk` of a slice takes the blocks chunk, chunk + row_chunks, ... of the sorted list, its warps in turn, so that
 // every CTA gets the same mix of long and short rows.  A block of more than capq quads is read from global memory.
 // (Fetching the next block's quads a step ahead into a second half of the buffer was measured: no gain.)
-template <typename T, int VEC, int LANES, int PIECES, int THREADS>
+// OLD (beta != 0 and two pieces): the old values of Y are asked for before the products, into registers that make the CTA smaller; asked for after
+// them, every step of a warp waits for HBM (2^14 rows of 20 x 4096 FP32 314 / 423 us, one piece per lane 346 us; BF16 186 / 261 / 197 us).
+template <typename T, int VEC, int LANES, int PIECES, bool OLD, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 spmm_bstage_quads_kernel(const __grid_constant__ CUtensorMap tmapB, int n, int k, int row_chunks, int blocks, int box_rows, int bslice_bytes,
                          int capq, const int* __restrict__ quad_row, const int* __restrict__ quad_len, const int* __restrict__ quad_pos,
@@ -461,6 +463,14 @@ spmm_bstage_quads_kernel(const __grid_constant__ CUtensorMap tmapB, int n, int k
       phase ^= 1u;
     }
     const int row = __shfl_sync(FULL, row_cur, gl), len = __shfl_sync(FULL, len_cur, gl);
+    uint4 held[PIECES];
+    if constexpr (OLD) {
+#pragma unroll
+      for (int e = 0; e < PIECES; ++e) {
+        const int col = col0 + (e ? other / 16 * VEC : 0);
+        held[e] = row >= 0 && col < k ? *(const uint4*)(Y + (long long)row * k + col) : make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
     float acc[PIECES][VEC], tot[PIECES][VEC];   // acc: the current block of at most kChainBlock products; tot: the sum of the completed blocks
 #pragma unroll
     for (int e = 0; e < PIECES; ++e)
@@ -481,9 +491,10 @@ spmm_bstage_quads_kernel(const __grid_constant__ CUtensorMap tmapB, int n, int k
       float out[VEC];
 #pragma unroll
       for (int j = 0; j < VEC; ++j) out[j] = alpha * (acc[e][j] + tot[e][j]);
-      if (beta != 0.0f) {
+      if (OLD || beta != 0.0f) {
         float old[VEC];
-        VecLoad<T, VEC>::ld_plain(yp, old);
+        if constexpr (OLD) VecLoad<T, VEC>::unpack(held[e], old);
+        else VecLoad<T, VEC>::ld_plain(yp, old);
 #pragma unroll
         for (int j = 0; j < VEC; ++j) out[j] += beta * old[j];
       }

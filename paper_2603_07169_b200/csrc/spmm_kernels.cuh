@@ -11,6 +11,9 @@ namespace b200sp {
 
 template <typename T, int VEC> struct VecLoad;
 template <> struct VecLoad<float, 4> {
+  static __device__ __forceinline__ void unpack(const uint4 t, float (&v)[4]) {
+    v[0] = __uint_as_float(t.x); v[1] = __uint_as_float(t.y); v[2] = __uint_as_float(t.z); v[3] = __uint_as_float(t.w);
+  }
   static __device__ __forceinline__ void ld(const float* p, float (&v)[4]) { const float4 t = __ldg((const float4*)p); v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w; }
   static __device__ __forceinline__ void ld_plain(const float* p, float (&v)[4]) { const float4 t = *(const float4*)p; v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w; }
   static __device__ __forceinline__ void st(float* p, const float (&v)[4]) { *(float4*)p = make_float4(v[0], v[1], v[2], v[3]); }

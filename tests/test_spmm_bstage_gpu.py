@@ -20,7 +20,8 @@ def lengths(m, n, seed):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
-@pytest.mark.parametrize("n,m,k", [(2048, 3001, 900), (2048, 3008, 1032), (2048, 3024, 904), (1700, 2003, 520), (1700, 2000, 1048), (3300, 3015, 888), (300, 1999, 1024)])
+@pytest.mark.parametrize("n,m,k", [(2048, 3001, 900), (2048, 3008, 1032), (2048, 3024, 904), (1700, 2003, 520), (1700, 2000, 1048), (3300, 3015, 888), (300, 1999, 1024),
+                                   (2048, 9999, 1000), (2048, 10003, 904)])       # the last two: blocks re-ordered
 def test_against_oracle(n, m, k, dtype):
     rng = np.random.default_rng(m + k)
     if dtype == "bf16":
@@ -37,10 +38,24 @@ def test_against_oracle(n, m, k, dtype):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("n,m,k", [(2048, 9001, 904), (2048, 9999, 1000), (1700, 9003, 1048)])
+def test_old_values_of_y_with_two_pieces(n, m, k, dtype):
+    """beta != 0 with steps enough for two pieces per lane: the old values are loaded ahead, past the last column and row as zeros."""
+    rng = np.random.default_rng(m)
+    if dtype == "bf16":
+        k *= 2
+    A = gen.random_csr(m, n, lengths(m, n, m) // 3, seed=n, sort_cols=False)
+    B, Y0 = rng.standard_normal(n * k).astype(np.float32), rng.standard_normal(m * k).astype(np.float32)
+    Y, Y_ref, S = run_spmm(A, B, k, Y0, -0.5, 1.25, dtype)
+    y0f = Y0 if dtype == "f32" else gen.bf16_to_f32(gen.to_bf16(Y0))
+    assert_within(Y, Y_ref, S, dtype, 1.0, np.abs(1.25 * y0f.astype(np.float64)).reshape(m, k), what="n=%d m=%d k=%d" % (n, m, k))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_rows_in_columns_of_one_parity(dtype):
     """All of a row's columns even, or all odd, in every mixture inside a block: the re-ordering at its extremes."""
     rng = np.random.default_rng(4)
-    m, n, k = 3003, 2048, 928 if dtype == "f32" else 1856
+    m, n, k = 10003, 2048, 928 if dtype == "f32" else 1856
     A = gen.random_csr(m, n, rng.integers(10, 14, m), seed=9, sort_cols=False, allow_dup=True)
     rows = np.repeat(np.arange(m), np.diff(A.row_ptr))
     A.col_idx[:] = (A.col_idx & ~1) | (rng.random(m) < 0.3)[rows]
