@@ -145,12 +145,14 @@ int b200sp_spmm(b200sp_plan* plan, int64_t k, const int32_t* col_idx, const void
  * out-of-range row indices return B200SP_ERR_UNSUPPORTED.  b200sp_cache_clear drops the cached offsets.
  *
  * CSC (tasks 10 / 11: values, row_indices, col_offsets of cols + 1 entries): the first call for a given
- * (device, col_ptr, row_idx, m, n, nnz) builds the row-major order of the entries on the device (row counts, an
- * exclusive scan, placement, and a sort of every row's entries by their CSC position, so that a row's entries are
- * added in ascending column order on every run) and caches it together with a scratch array of nnz values; it
- * synchronises the stream twice.  Every call then permutes vals into that order with one kernel and runs the
- * CSR kernels.  Inconsistent col_ptr / row_idx return B200SP_ERR_BAD_CSR.  Calls that share a cached pattern
- * must not overlap on the GPU.
+ * (device, col_ptr, row_idx, m, n, nnz) checks the pattern and counts the rows on the device, and caches what the calls derive from the
+ * pattern.  spmv_csc computes the products in column order, writes them sorted by buckets of rows into a scratch array and adds the rows
+ * up from there (up to 2^26 nonzeros in rows of at most 1024); its places, 6 bytes per nonzero, are built on the first spmv_csc
+ * call.  Otherwise, and for spmm_csc, the row-major order of the entries (a sort of every row's entries by their CSC position)
+ * and a scratch array of nnz values are built on the first call that needs them, and every call permutes vals into that order with one
+ * kernel and runs the CSR kernels.  Either way a row's entries are added in ascending column order on every run.  The calls that
+ * build something synchronise the stream, others do not.  Inconsistent col_ptr / row_idx return B200SP_ERR_BAD_CSR.  Calls that share a
+ * cached pattern must not overlap on the GPU.
  *
  * ELL: row-major, row i occupies entries [i*width, (i+1)*width) of col_ids and vals; an entry is padding
  * when its col_id is negative (its value is ignored, whatever it holds).  m * width < 2^31.  No plan, no
