@@ -89,6 +89,10 @@ int b200sp_get_option(const char* name, int* value);
 /* Environment, read once when the library is loaded: B200SP_OPTIONS="name=value,name=value" sets switches as
  * b200sp_set_option would (an entry that is not accepted is reported on stderr and skipped); B200SP_LOG=1 sets "log". */
 
+/* 1 if SpMM with k columns on a matrix with these row statistics (b200sp_plan_info) goes by equal shares of rows + nonzeros per warp
+ * under the present switches, 0 if not; B kept in shared memory (few columns of A) comes before it.  A rule of the host: no device needed. */
+int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, int dtype);
+
 /* ---- measurement probes (no counterpart in the paper's operations) ----------------------------------------------
  * Each enqueues one kernel that does nothing but the access pattern named, so that the caller, timing it with events,
  * gets the hardware rate that bounds the corresponding library kernel.  All pointers are device pointers; `sink` is

@@ -21,7 +21,7 @@ EXPORTS = (
     "spmv_csr", "spmm_csr", "b200sp_plan_create", "b200sp_plan_destroy", "b200sp_plan_info", "b200sp_spmv",
     "b200sp_spmm", "spmv_csr_host", "spmm_csr_host", "b200sp_validate_csr", "b200sp_cache_clear",
     "b200sp_status_string", "b200sp_last_cuda_error", "b200sp_version", "b200sp_checked_build", "b200sp_launch_count", "b200sp_set_option", "b200sp_get_option",
-    "b200sp_check", "b200sp_cache_drop", "spmv_csr_noalloc", "b200sp_noalloc_max_items", "b200sp_probe_gather", "b200sp_probe_gather_ex", "b200sp_probe_stream", "b200sp_probe_lines", "b200sp_probe_spmv_gather", "b200sp_spmv_naive", "b200sp_spmm_naive", "spmv_coo", "spmm_coo", "spmv_ell", "spmm_ell", "spmv_csc", "spmm_csc", "spmv_csr_vec_host",
+    "b200sp_check", "b200sp_cache_drop", "spmv_csr_noalloc", "b200sp_noalloc_max_items", "b200sp_probe_gather", "b200sp_probe_gather_ex", "b200sp_probe_stream", "b200sp_probe_lines", "b200sp_probe_spmv_gather", "b200sp_spmv_naive", "b200sp_spmm_naive", "spmv_coo", "spmm_coo", "spmv_ell", "spmm_ell", "spmv_csc", "spmm_csc", "spmv_csr_vec_host", "b200sp_spmm_by_shares",
 )
 
 
@@ -110,6 +110,8 @@ def lib() -> ctypes.CDLL:
         L.b200sp_set_option.argtypes = [ctypes.c_char_p, i32]
         L.b200sp_get_option.argtypes = [ctypes.c_char_p, ctypes.POINTER(ctypes.c_int)]
         L.b200sp_get_option.restype = i32
+        L.b200sp_spmm_by_shares.argtypes = [ctypes.POINTER(PlanInfo), i64, i32]
+        L.b200sp_spmm_by_shares.restype = i32
         L.b200sp_check.argtypes = [p]
         L.b200sp_check.restype = i32
         for name in ("spmv_csr", "spmm_csr", "spmv_csr_host", "spmm_csr_host", "b200sp_plan_create", "b200sp_plan_destroy",
@@ -466,6 +468,12 @@ def b200sp_plan_info(plan) -> dict:
     info = PlanInfo()
     _ck(lib().b200sp_plan_info(plan, ctypes.byref(info)), "b200sp_plan_info")
     return info.as_dict()
+
+
+def b200sp_spmm_by_shares(info: dict, k, dtype) -> bool:
+    """Whether SpMM with k columns on a matrix with these row statistics (b200sp_plan_info) takes the nnz-balanced kernel."""
+    I = PlanInfo(**{name: (ctypes.c_int64 * 6)(*info[name]) if name.startswith("bin_") else info[name] for name, _ in PlanInfo._fields_ if name in info})
+    return bool(lib().b200sp_spmm_by_shares(ctypes.byref(I), k, _dt(dtype)))
 
 
 def b200sp_spmv(plan, col_idx, vals, x, y, alpha, beta, dtype, stream=None):

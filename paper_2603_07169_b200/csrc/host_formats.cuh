@@ -349,7 +349,7 @@ static int run_ell_spmm(int64_t m, int width, int k, const int32_t* col_ids, con
   if (alpha == 0.0f || width == 0) return run_scale<T>((long long)m * k, Y, beta, stream, dev);
   if (k % VEC == 0) {
     constexpr int KS = 8 * VEC, GROUPS = kSpmmThreads / 8;
-    const int slices = (k + KS - 1) / KS;
+    const int slices = (k - 1) / KS + 1;
     const int row_blocks = (int)((m + GROUPS - 1) / GROUPS);
     if ((long long)slices * row_blocks >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
     return launch(spmm_ell_slice_kernel<T, VEC, kSpmmThreads>, dim3((unsigned)(slices * row_blocks)), dim3(kSpmmThreads), stream, nullptr, 0, dev,

@@ -22,7 +22,7 @@ int launch_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, co
   rc = launch(spmm_row_group_kernel<T, VEC, LANES, NCH, kSpmmThreads>, dim3(grid), dim3(kSpmmThreads), stream, B,
                   (size_t)I.n * k * sizeof(T), dev, (int)I.m, k, p->row_ptr, col_idx, vals, B, Y, alpha, beta, kLongRow);
   if (rc != B200SP_OK || p->num_long == 0) return rc;
-  const long long ctas = (long long)((k + 8 * VEC - 1) / (8 * VEC)) * p->num_long;
+  const long long ctas = (long long)((k - 1) / (8 * VEC) + 1) * p->num_long;
   if (ctas >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
   tl_pdl_kernel = true;
   return launch(spmm_long_row_kernel<T, VEC, kSpmmThreads>, dim3((unsigned)ctas), dim3(kSpmmThreads), stream, nullptr, 0, dev, k, p->num_long,
@@ -81,7 +81,7 @@ int launch_spmm_bstage(b200sp_plan* p, int k, const int32_t* col_idx, const T* v
     CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerSm - 2048));
     configured[p->device] = true;
   }
-  const int slices = (k + KS - 1) / KS;
+  const int slices = (k - 1) / KS + 1;
   const int per_cta = g_opt.bstage_nnz > 0 ? g_opt.bstage_nnz : 131072;
   long long chunks = (I.nnz + per_cta - 1) / per_cta;   // a given number of nonzeros per CTA ...
   const long long fill = (2LL * dev->sms + slices - 1) / slices;   // ... but at least two CTAs per SM over the grid
@@ -208,7 +208,7 @@ int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, c
     CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerSm - 2048));
     configured[p->device] = true;
   }
-  const int slices = (k + KS - 1) / KS;
+  const int slices = (k - 1) / KS + 1;
   const int blocks = Q->blocks;
   const long long most = (blocks + WARPS - 1) / WARPS;   // a block per warp at least
   long long chunks;
@@ -260,7 +260,7 @@ int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, c
   const cudaError_t e = cudaFreeAsync(scratch, stream);
   if (e != cudaSuccess && rc == B200SP_OK) rc = cuda_fail(e, "cudaFreeAsync");
   if (rc == B200SP_OK && p->num_long > 0) {
-    const long long ctas = (long long)((k + 8 * VEC - 1) / (8 * VEC)) * p->num_long;
+    const long long ctas = (long long)((k - 1) / (8 * VEC) + 1) * p->num_long;
     if (ctas >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
     tl_pdl_kernel = true;
     rc = launch(spmm_long_row_kernel<T, VEC, kSpmmThreads>, dim3((unsigned)ctas), dim3(kSpmmThreads), stream, nullptr, 0, dev, k, p->num_long,
@@ -279,7 +279,7 @@ template <typename T, int VEC, int SLICE_LANES, int THREADS>
 int launch_spmm_bstage_quads(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
                              cudaStream_t stream, DeviceInfo* dev, EncodeTiledFn encode) {
   if constexpr (SLICE_LANES >= 4 && THREADS == 1024) {
-    const long long slices = (k + SLICE_LANES * VEC - 1) / (SLICE_LANES * VEC), steps = (p->info.m * SLICE_LANES / 64 + 1) * slices;
+    const long long slices = (k - 1) / (SLICE_LANES * VEC) + 1, steps = (p->info.m * SLICE_LANES / 64 + 1) * slices;
     if (beta == 0.0f && steps >= 32LL * dev->sms)
       return launch_spmm_bstage_quads_as<T, VEC, SLICE_LANES, 2, false, sizeof(T) == 2 ? 768 : 1024>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev, encode);
     if (beta != 0.0f && steps >= 192LL * dev->sms)
@@ -337,6 +337,15 @@ bool spmm_rows_are_uneven(const b200sp_plan_info_t& I) {
          || (double)I.max_row_len > 4.0 * mean + 8.0;       // or the longest row is far above the mean
 }
 
+// Whether SpMM goes by equal shares (spmm_merge_kernel): uneven rows, and k that is no multiple of 16 bytes unless it is so narrow that a
+// lane per column and a group of lanes per row lose little (100,000 rows of 13: k = 13 18 us by rows, 27 us by shares; k = 23 35 / 27 us;
+// k = 50 47 / 35 us FP32, 42 / 34 us BF16).  The kernel counts the bytes of a row of B, and columns past k up to a slice, in 32 bits.
+bool spmm_by_shares(const b200sp_plan_info_t& I, int64_t k, int elem_bytes) {
+  if (k > (INT32_MAX - 2048) / elem_bytes) return false;
+  const int vec = 16 / elem_bytes;
+  return g_opt.spmm_sliced && (g_opt.spmm_flat == 1 || (g_opt.spmm_flat == 2 && (spmm_rows_are_uneven(I) || (k % vec != 0 && k > 16))));
+}
+
 template <typename T, int V, int J, bool LIST>
 int launch_spmm_merge_as(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
                       cudaStream_t stream, DeviceInfo* dev) {
@@ -365,7 +374,7 @@ int launch_spmm_merge_as(b200sp_plan* p, int k, const int32_t* col_idx, const T*
   }
   const long long per_tile = (long long)witems * shares * kMergeWarps;
   const int tiles = (int)((I.m + I.nnz + per_tile - 1) / per_tile);
-  const int slices = (k + KS - 1) / KS;
+  const int slices = (k - 1) / KS + 1;
   if ((long long)slices * tiles >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
   // per-call scratch: what each tile leaves unfinished and what it finishes for an earlier tile, KS floats per (slice, tile)
   float* scratch = nullptr;
@@ -416,7 +425,7 @@ int run_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals,
     p->spmm_split = (int32_t*)p->split_block;
     p->spmm_witems = w;
   }
-  const int loads = (k + 32 * v - 1) / (32 * v);
+  const int loads = (k - 1) / (32 * v) + 1;
 #define B200SP_MERGE_J(V)                                                                                                   \
   do {                                                                                                                      \
     if (loads == 1) return launch_spmm_merge<T, V, 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);                 \
@@ -467,9 +476,7 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
       if (rc != B200SP_ERR_UNSUPPORTED) return rc;   // unsupported shape for the tensor map: fall through to the sliced kernel
     }
   }
-  // Uneven rows, and k that is no multiple of 16 bytes unless it is so narrow that a lane per column and a group of lanes per row lose
-  // little (100,000 rows of 13: k = 13 18 us by rows, 27 us by shares; k = 23 35 / 27 us; k = 50 47 / 35 us FP32, 42 / 34 us BF16)
-  if (g_opt.spmm_sliced && (g_opt.spmm_flat == 1 || (g_opt.spmm_flat == 2 && (spmm_rows_are_uneven(I) || (k % VEC != 0 && k > 16))))) {
+  if (spmm_by_shares(I, k, (int)sizeof(T))) {
     const int rc = run_spmm_merge<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
     if (rc != B200SP_ERR_UNSUPPORTED) return rc;
   }
@@ -478,7 +485,7 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     const int vecs_k = k / VEC;
     const int lanes = vecs_k >= 8 ? 8 : (vecs_k > 2 ? 4 : vecs_k);
     const int KS = lanes * VEC, GROUPS = kSpmmThreads / lanes;
-    const int slices = (k + KS - 1) / KS;
+    const int slices = (k - 1) / KS + 1;
     const int row_blocks = (int)((I.m + GROUPS - 1) / GROUPS);
     if ((long long)slices * row_blocks >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
     int rc = plan_row_lists(p, stream, dev);
@@ -531,7 +538,7 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     else { B200SP_SLICE_LAUNCH(1); }
 #undef B200SP_SLICE_LAUNCH
     if (rc != B200SP_OK || p->num_long == 0) return rc;
-    const long long ctas = (long long)((k + 8 * VEC - 1) / (8 * VEC)) * p->num_long;
+    const long long ctas = (long long)((k - 1) / (8 * VEC) + 1) * p->num_long;
     if (ctas >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
     tl_pdl_kernel = true;
     return launch(spmm_long_row_kernel<T, VEC, kSpmmThreads>, dim3((unsigned)ctas), dim3(kSpmmThreads), stream, nullptr, 0,

@@ -65,7 +65,7 @@ spmm_row_group_kernel(int m, int k, const int* __restrict__ row_ptr, const int* 
   const int rs = row_ptr[row], re = row_ptr[row + 1];
   if (re - rs > long_thresh) return;
   constexpr int SPAN = LANES * VEC;  // columns covered by one chunk
-  for (int c0 = 0; c0 < k; c0 += SPAN * NCH) {
+  for (unsigned c0 = 0; c0 < (unsigned)k; c0 += SPAN * NCH) {   // (unsigned: c0 may pass k when k is close to 2^31)
     float acc[NCH][VEC], tot[NCH][VEC];
 #pragma unroll
     for (int h = 0; h < NCH; ++h)
@@ -89,8 +89,8 @@ spmm_row_group_kernel(int m, int k, const int* __restrict__ row_ptr, const int* 
       for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int h = 0; h < NCH; ++h) {
-          const int col = c0 + h * SPAN + lane * VEC;
-          if (col < k) VecLoad<T, VEC>::ld(B + (long long)cc[u] * k + col, b[u][h]);
+          const unsigned col = c0 + h * SPAN + lane * VEC;
+          if (col < (unsigned)k) VecLoad<T, VEC>::ld(B + (long long)cc[u] * k + col, b[u][h]);
           else {
 #pragma unroll
             for (int j = 0; j < VEC; ++j) b[u][h][j] = 0.0f;
@@ -108,8 +108,8 @@ spmm_row_group_kernel(int m, int k, const int* __restrict__ row_ptr, const int* 
       const float vv = to_f32(__ldg(vals + p));
 #pragma unroll
       for (int h = 0; h < NCH; ++h) {
-        const int col = c0 + h * SPAN + lane * VEC;
-        if (col < k) {
+        const unsigned col = c0 + h * SPAN + lane * VEC;
+        if (col < (unsigned)k) {
           float b[VEC];
           VecLoad<T, VEC>::ld(B + (long long)cc * k + col, b);
 #pragma unroll
@@ -119,8 +119,8 @@ spmm_row_group_kernel(int m, int k, const int* __restrict__ row_ptr, const int* 
     }
 #pragma unroll
     for (int h = 0; h < NCH; ++h) {
-      const int col = c0 + h * SPAN + lane * VEC;
-      if (col < k) {
+      const unsigned col = c0 + h * SPAN + lane * VEC;
+      if (col < (unsigned)k) {
         float out[VEC];
         T* yp = Y + row * k + col;
 #pragma unroll
