@@ -167,12 +167,16 @@ __global__ void __launch_bounds__(256) csc_bucket_rows_plan(const int* __restric
   bucket_start[b] = row_ptr[lo];
 }
 
-// Largest bucket -> stat[0]; widest range of columns of a tile -> stat[1]; tile_col[t]: the column of the tile's first entry.
+// Most nonzeros of a bucket -> stat[0]; widest range of columns of a tile -> stat[1]; most rows of a bucket -> stat[2]; tile_col[t]: the column
+// of the tile's first entry.
 __global__ void __launch_bounds__(256) csc_extents_plan(const int* __restrict__ row_ptr, const int* __restrict__ bucket_row, int buckets,
                                                         const int* __restrict__ col_ptr, int n, int nnz, int tile, int tiles,
                                                         int* __restrict__ tile_col, int* __restrict__ stat) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < buckets) atomicMax(stat, row_ptr[bucket_row[i + 1]] - row_ptr[bucket_row[i]]);
+  if (i < buckets) {
+    atomicMax(stat, row_ptr[bucket_row[i + 1]] - row_ptr[bucket_row[i]]);
+    atomicMax(stat + 2, bucket_row[i + 1] - bucket_row[i]);
+  }
   if (i < tiles) {
     auto column = [&](int p) {                   // the last j with col_ptr[j] <= p
       int lo = 0, hi = n;

@@ -60,6 +60,7 @@ struct CscEntry {
   void* vals_t = nullptr;
   void* prod_block = nullptr;
   bool prod_tried = false;
+  int bucket_rows = 0;                // most rows of a bucket, once counted
   int tile = 0, tiles = 0, buckets = 0, cap = 0;
   int *bucket_row = nullptr, *bucket_start = nullptr, *tile_col = nullptr, *run_shift = nullptr;
   unsigned short *src = nullptr, *dst = nullptr, *dcol = nullptr, *run_before = nullptr;
@@ -157,16 +158,28 @@ static int csc_csr_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, const in
   return B200SP_OK;
 }
 
+// Most rows of one bucket for which the products pay.  Buckets are cut by nonzeros, so one may hold any number of empty rows, and its CTA
+// walks them 512 at a time, 0.28 us a step (0.43 us where y is read), while the CSR kernels spread them over the GPU.  Where both take
+// the same time, FP32 and BF16 alike (beta = 0 / beta != 0): 262,144 nonzeros 12,000 / 8,600 rows, 2^20 16,500 / 9,700, 2^22 36,000 / 24,000,
+// 6.2 M (R-MAT) 33,000 / 20,000, 2^24 110,000 / 66,000, 27 M (R-MAT) more than 49,000 / 65,000; 2000 nonzeros in 2^22 rows 2278 us by products,
+// 27 us by the CSR kernels.
+static int64_t csc_most_bucket_rows(int64_t nnz, float beta) {
+  const int64_t rows = std::min(4096 + nnz / 16, 12000 + nnz / 300);
+  return beta == 0.0f ? rows : rows * 2 / 3;
+}
+
+
 // The places of the products of csc_kernels.cuh; leaves e->prod_block null where they do not apply.  Synchronises the stream once.
 // Sizes: below 4.8 M nonzeros tiles and buckets of 2048 or 4096, so that every SM gets several; else one tile of 24576 .. 32768 entries
 // per SM and round (96 .. 128 KB of products), the size that leaves the least of the last round idle, and buckets of 8192 nonzeros,
 // 16384 above 2^25.  A run (a tile's products for one bucket) then averages tile * C / nnz = 3.5 .. 55 words: 2^24 nonzeros take 78 us,
 // 81 us with tiles of 32768, 84 us with two tiles of 16384 per SM.  Above 2^26
-// nonzeros, with a row of more than kCscSlack nonzeros or a tile over more than 65536 columns, SpMV takes the CSR kernels.
-static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr, const int32_t* row_idx, cudaStream_t stream,
-                            DeviceInfo* dev) {
+// nonzeros, with a row of more than kCscSlack nonzeros, a tile over more than 65536 columns or a bucket of too many rows (most_rows), SpMV takes
+// the CSR kernels.
+static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr, const int32_t* row_idx, int64_t most_rows,
+                            cudaStream_t stream, DeviceInfo* dev) {
   std::lock_guard<std::mutex> lock(g_csc_build);
-  if (e->prod_tried) return B200SP_OK;
+  if (e->prod_tried || e->bucket_rows > most_rows) return B200SP_OK;
   if (nnz <= 0 || nnz > ((int64_t)1 << 26)) { e->prod_tried = true; return B200SP_OK; }
   const int64_t sms = dev->sms;
   int tile = nnz < sms * 4 * 2048 ? 2048 : 4096;
@@ -195,8 +208,8 @@ static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, cons
   int* place = (int*)(blk + o_prod);             // the products' CSC positions; the products come later
   int* brow = (int*)(blk + o_brow);
   int* tcol = (int*)(blk + o_tcol);
-  int h[2] = {0, 0};
-  CUP(cudaMemsetAsync(stat, 0, 2 * sizeof(int), stream));
+  int h[3] = {0, 0, 0};
+  CUP(cudaMemsetAsync(stat, 0, sizeof h, stream));
   csc_bucket_rows_plan<<<(buckets + 1 + 255) / 256, 256, 0, stream>>>(e->row_ptr, (int)m, buckets, shift, brow, (int*)(blk + o_bstart));
   const int wider = buckets > tiles ? buckets : tiles;
   csc_extents_plan<<<(wider + 255) / 256, 256, 0, stream>>>(e->row_ptr, brow, buckets, col_ptr, (int)n, (int)nnz, tile, tiles, tcol, stat);
@@ -204,7 +217,9 @@ static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, cons
   CUP(cudaGetLastError());
   CUP(cudaMemcpyAsync(h, stat, sizeof h, cudaMemcpyDeviceToHost, stream));
   CUP(cudaStreamSynchronize(stream));
-  if (h[0] > cap || h[1] > 65535) { e->prod_tried = true; return fail(B200SP_OK); }
+  e->bucket_rows = h[2];
+  e->prod_tried = h[0] > cap || h[1] > 65535;
+  if (e->prod_tried || e->bucket_rows > most_rows) return fail(B200SP_OK);
   const size_t slots_smem = (size_t)buckets * 12 + (size_t)tile * 2;
   CUP(cudaFuncSetAttribute(csc_tile_slots_plan, cudaFuncAttributeMaxDynamicSharedMemorySize, kCscMaxBuckets * 12 + kCscMaxTile * 2));
   csc_tile_counts_plan<<<tiles, 512, (size_t)buckets * 4, stream>>>(row_idx, e->row_ptr, (int)nnz, tile, shift, buckets, count);
@@ -276,9 +291,10 @@ static int csc_call(bool is_mm, int64_t m, int64_t n, int64_t nnz, int64_t k, co
   rc = csc_plan(&entry, m, n, nnz, col_ptr, row_idx, stream);
   if (rc != B200SP_OK) return rc;
   if (!is_mm && nnz > 0 && alpha != 0.0f && in && out && aligned16(vals) && aligned16(in) && aligned16(out)) {
-    rc = csc_product_part(entry, m, n, nnz, col_ptr, row_idx, stream, dev);
+    const int64_t most_rows = csc_most_bucket_rows(nnz, beta);
+    rc = csc_product_part(entry, m, n, nnz, col_ptr, row_idx, most_rows, stream, dev);
     if (rc != B200SP_OK) return rc;
-    if (entry->prod_block)
+    if (entry->prod_block && entry->bucket_rows <= most_rows)
       return dtype == B200SP_F32 ? run_csc_products<float>(entry, nnz, (const float*)vals, (const float*)in, (float*)out, alpha, beta, stream, dev)
                                  : run_csc_products<bf16_t>(entry, nnz, (const bf16_t*)vals, (const bf16_t*)in, (bf16_t*)out, alpha, beta, stream, dev);
   }

@@ -27,6 +27,10 @@ def matrices():
         "wide_tile": (np.full(3000, 2), 900_000),                 # a tile spans more than 65536 columns: CSR kernels
         "trailing_empty_rows": (tail, 100),
         "more_rows_than_a_bucket": (np.concatenate([tail, np.zeros(4000, np.int64), tail]), 100),
+        # one bucket of 2048 nonzeros and as many rows as the products take (beta = 0 / beta != 0), and one more
+        "bucket_rows_at_the_limit": (np.resize(np.repeat([32, 0], 64), 4224) * (np.arange(4224) < 128), 300),
+        "bucket_rows_over_the_limit": (np.resize(np.repeat([32, 0], 64), 4225) * (np.arange(4225) < 128), 300),
+        "bucket_rows_at_the_limit_of_beta": (np.resize(np.repeat([32, 0], 64), 2816) * (np.arange(2816) < 128), 300),
         "power_law": ((rng.pareto(1.5, 30_000) * 2).astype(np.int64).clip(0, 900), 20_000),
         "tile_4096": (rng.integers(0, 30, 100_000), 50_000),
         "tile_24576": (16, 328_000),                              # 5.2 M nonzeros (equal rows: drawn by the fast generator)
@@ -79,6 +83,34 @@ def test_csc_products_around_the_largest_bucket_size(per_row):
     ref = torch.zeros(m, dtype=torch.float64, device="cuda").index_add_(0, row.long(), p)
     S = torch.zeros(m, dtype=torch.float64, device="cuda").index_add_(0, row.long(), p.abs())
     assert float(((y.double() - ref).abs() / (1e-5 * S + 1e-30)).max()) <= 1.0
+    b200sp.b200sp_cache_clear()
+
+
+@pytest.mark.parametrize("beta", [0.0, 0.5])
+def test_a_few_entries_in_many_rows(beta):
+    """2000 entries in 2^22 rows are one bucket of products: one CTA would walk all rows (2.3 ms, 3.5 ms with beta != 0; 27 us by the CSR kernels)."""
+    m, n, nnz = 1 << 22, 4096, 2000
+    rng = np.random.default_rng(6)
+    key = np.sort(rng.integers(0, n, nnz) * m + rng.integers(0, m, nnz))
+    col, row = key // m, (key % m).astype(np.int32)
+    cp = np.searchsorted(col, np.arange(n + 1)).astype(np.int32)
+    va, x = rng.standard_normal(nnz).astype(np.float32), rng.standard_normal(n).astype(np.float32)
+    d = [to_dev(a) for a in (cp, row, va, x)]
+    y = torch.ones(m, device="cuda")
+    call = lambda: b200sp.spmv_csc(m, n, nnz, d[0], d[1], d[2], d[3], y, 1.0, beta, "f32")  # noqa: E731
+    call()
+    p, at = va.astype(np.float64) * x[col], row.astype(np.int64)
+    ref, S = beta + np.bincount(at, p, m), beta + np.bincount(at, np.abs(p), m)
+    assert np.all(np.abs(y.cpu().numpy() - ref) <= 1e-5 * S + 1e-30)
+    start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    best = 1e9
+    for _ in range(5):
+        start.record()
+        call()
+        end.record()
+        torch.cuda.synchronize()
+        best = min(best, start.elapsed_time(end))
+    assert best < 0.5, "%.3f ms" % best
     b200sp.b200sp_cache_clear()
 
 
