@@ -25,7 +25,8 @@ extern "C" {
  *   "spmm_sliced"    1 = SpMM walks k in 128-byte slices so that a slice of B can stay in L2 (default), 0 = one pass
  *   "spmm_flat"      SpMM by equal shares of rows + nonzeros per warp instead of by rows (nnz-balanced, with carries between warps and
  *                    CTAs): 1 = always, 0 = never, 2 = when the rows are uneven (5 % or more of the nonzeros in rows longer than
- *                    128, a quarter or more of the rows empty, or a longest row far above the mean) or k > 16 is no multiple of 16 bytes (default)
+ *                    128, a quarter or more of the rows empty, or a longest row far above the mean; with few columns only where the
+ *                    rows differ enough, b200sp_spmm_by_shares) or k > 16 is no multiple of 16 bytes (default)
  *   "spmm_stage_a"   the k-sliced SpMM kernel's warps first copy their rows' (col, val) pairs into shared memory: 1 = yes, 0 = no,
  *                    2 = for BF16 storage only (default: measured 5-6 % faster there and 2-3 % slower for FP32)
  *   "spmm_ranges"    k-sliced SpMM on rows with ascending columns, one launch per column range so that the rows of B a
@@ -91,7 +92,7 @@ int b200sp_get_option(const char* name, int* value);
 
 /* 1 if SpMM with k columns on a matrix with these row statistics (b200sp_plan_info) goes by equal shares of rows + nonzeros per warp
  * under the present switches, 0 if not; B kept in shared memory (few columns of A) comes before it.  A rule of the host: no device needed. */
-int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, int dtype);
+int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, float beta, int dtype);
 
 /* ---- measurement probes (no counterpart in the paper's operations) ----------------------------------------------
  * Each enqueues one kernel that does nothing but the access pattern named, so that the caller, timing it with events,

@@ -110,7 +110,7 @@ def lib() -> ctypes.CDLL:
         L.b200sp_set_option.argtypes = [ctypes.c_char_p, i32]
         L.b200sp_get_option.argtypes = [ctypes.c_char_p, ctypes.POINTER(ctypes.c_int)]
         L.b200sp_get_option.restype = i32
-        L.b200sp_spmm_by_shares.argtypes = [ctypes.POINTER(PlanInfo), i64, i32]
+        L.b200sp_spmm_by_shares.argtypes = [ctypes.POINTER(PlanInfo), i64, f32, i32]
         L.b200sp_spmm_by_shares.restype = i32
         L.b200sp_check.argtypes = [p]
         L.b200sp_check.restype = i32
@@ -470,10 +470,10 @@ def b200sp_plan_info(plan) -> dict:
     return info.as_dict()
 
 
-def b200sp_spmm_by_shares(info: dict, k, dtype) -> bool:
+def b200sp_spmm_by_shares(info: dict, k, beta, dtype) -> bool:
     """Whether SpMM with k columns on a matrix with these row statistics (b200sp_plan_info) takes the nnz-balanced kernel."""
     I = PlanInfo(**{name: (ctypes.c_int64 * 6)(*info[name]) if name.startswith("bin_") else info[name] for name, _ in PlanInfo._fields_ if name in info})
-    return bool(lib().b200sp_spmm_by_shares(ctypes.byref(I), k, _dt(dtype)))
+    return bool(lib().b200sp_spmm_by_shares(ctypes.byref(I), k, beta, _dt(dtype)))
 
 
 def b200sp_spmv(plan, col_idx, vals, x, y, alpha, beta, dtype, stream=None):

@@ -129,8 +129,8 @@ int b200sp_spmm(b200sp_plan* plan, int64_t k, const int32_t* col_idx, const void
   return run_spmm<bf16_t, 8>(plan, (int)k, col_idx, (const bf16_t*)vals, (const bf16_t*)B, (bf16_t*)Y, alpha, beta, (cudaStream_t)stream, dev);
 }
 
-int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, int dtype) {
-  return info && spmm_by_shares(*info, k, dtype == B200SP_F32 ? 4 : 2);
+int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, float beta, int dtype) {
+  return info && spmm_by_shares(*info, k, dtype == B200SP_F32 ? 4 : 2, beta);
 }
 
 int spmv_csr(int64_t m, int64_t n, int64_t nnz, const int32_t* row_ptr, const int32_t* col_idx, const void* vals, const void* x,

@@ -337,13 +337,47 @@ bool spmm_rows_are_uneven(const b200sp_plan_info_t& I) {
          || (double)I.max_row_len > 4.0 * mean + 8.0;       // or the longest row is far above the mean
 }
 
-// Whether SpMM goes by equal shares (spmm_merge_kernel): uneven rows, and k that is no multiple of 16 bytes unless it is so narrow that a
-// lane per column and a group of lanes per row lose little (100,000 rows of 13: k = 13 18 us by rows, 27 us by shares; k = 23 35 / 27 us;
-// k = 50 47 / 35 us FP32, 42 / 34 us BF16).  The kernel counts the bytes of a row of B, and columns past k up to a slice, in 32 bits.
-bool spmm_by_shares(const b200sp_plan_info_t& I, int64_t k, int elem_bytes) {
-  if (k > (INT32_MAX - 2048) / elem_bytes) return false;
+// Uneven rows and few columns: whether the kernels by rows are faster than shares, by a model of both times in us.  A warp of the nnz-balanced
+// kernel takes a nonzero at a time however few columns there are, so its time is that of the rows + nonzeros.  By rows a nonzero costs less
+// the fewer lanes hold its row, more where the rows of a warp differ (spread: mean length over the nonzeros, by length bins, over the mean
+// length), and the longest row walked by one lane group is a chain; rows of 129-1024 nonzeros (aligned k) and longer ones are launches apart.
+// Constants: least squares over log-normal rows (means 4 .. 40, sigma 0.7 .. 1.2, 5000 .. 2 M rows) and even rows with a few long ones, both
+// dtypes, beta = 0 and 1, 1268 points (rms error 0.2 in the logarithm).  Of the 444 that go by rows 8 are slower by 5 % than by shares, by 10 % at
+// most; of those that go by shares 104 are slower by 5 % than by rows.  By rows / shares in us: 600,000 log-normal rows of 12, FP32 k = 2
+// 76 / 116, k = 3 91 / 117, k = 8 155 / 117, BF16 k = 2 89 / 135, k = 16 142 / 136; 20,011 rows of 10, k = 2 21.5 / 10.6; 600,000 rows of 8 and one of
+// 3000, k = 2 41 / 89, k = 8 49 / 90; R-MAT 2^20 (spread above 30) k = 2 359 / 140, k = 16 465 / 146.
+bool spmm_uneven_by_rows(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, float beta) {
   const int vec = 16 / elem_bytes;
-  return g_opt.spmm_sliced && (g_opt.spmm_flat == 1 || (g_opt.spmm_flat == 2 && (spmm_rows_are_uneven(I) || (k % vec != 0 && k > 16))));
+  if (k > (k % vec == 0 ? 4 * vec : 16) || I.bin_rows[0] * 4 >= I.m) return false;
+  const double m = 1e-6 * (double)I.m, nnz = 1e-6 * (double)I.nnz;
+  double squares = 0.0;
+  for (int j = 1; j < B200SP_NUM_BINS; ++j)
+    if (I.bin_rows[j] > 0) squares += (double)I.bin_nnz[j] * (double)I.bin_nnz[j] / (double)I.bin_rows[j];
+  const double spread = squares * (double)I.m / ((double)I.nnz * (double)I.nnz);
+  if (spread > (k % vec == 0 && k > 2 * vec ? 1.5 : 2.6) || (I.bin_rows[4] > 0 && I.bin_rows[5] > 0)) return false;
+  const int longest = I.max_row_len, medium = I.bin_rows[4] > 0 ? longest : 0;
+  const int shortest = longest <= 128 ? longest : 128;
+  double rows;
+  if (k % vec == 0) {
+    rows = std::max(nnz * (4.4 + 3.2 * (double)(k / vec)) * (1.0 + 0.34 * (spread - 1.0)), 0.09 * shortest) + 0.09 * medium;
+  } else {
+    int lanes = 2;
+    while (lanes < k) lanes *= 2;
+    rows = std::max(nnz * (3.9 + 1.15 * lanes) * (1.0 + 0.77 * (spread - 1.0)), 0.088 * std::max(shortest, medium)) * (elem_bytes == 4 ? 1.0 : 1.2);
+  }
+  rows += 5.0 + (longest > 1024 ? 0.005 * longest : 0.0);
+  const double shares = 8.6 + nnz * (elem_bytes == 4 ? 11.8 : 14.3) + m * (beta != 0.0f ? 75.0 : 40.0);
+  return 1.05 * rows < shares;
+}
+
+// Whether SpMM goes by equal shares (spmm_merge_kernel): uneven rows (see above), and k that is no multiple of 16 bytes unless it is so narrow
+// that a lane per column and a group of lanes per row lose little (100,000 rows of 13: k = 13 18 us by rows, 27 us by shares; k = 23 35 / 27 us;
+// k = 50 47 / 35 us FP32, 42 / 34 us BF16).  The kernel counts the bytes of a row of B, and columns past k up to a slice, in 32 bits.
+bool spmm_by_shares(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, float beta) {
+  if (k > (INT32_MAX - 2048) / elem_bytes || !g_opt.spmm_sliced) return false;
+  if (g_opt.spmm_flat != 2) return g_opt.spmm_flat == 1;
+  if (k % (16 / elem_bytes) != 0 && k > 16) return true;
+  return spmm_rows_are_uneven(I) && !spmm_uneven_by_rows(I, k, elem_bytes, beta);
 }
 
 template <typename T, int V, int J, bool LIST>
@@ -476,7 +510,7 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
       if (rc != B200SP_ERR_UNSUPPORTED) return rc;   // unsupported shape for the tensor map: fall through to the sliced kernel
     }
   }
-  if (spmm_by_shares(I, k, (int)sizeof(T))) {
+  if (spmm_by_shares(I, k, (int)sizeof(T), beta)) {
     const int rc = run_spmm_merge<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
     if (rc != B200SP_ERR_UNSUPPORTED) return rc;
   }

@@ -4,7 +4,7 @@ import pytest
 
 import gen
 import paper_2603_07169_b200 as b200sp
-from gpu_util import assert_within, run_spmm
+from gpu_util import assert_within, run_spmm, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -55,6 +55,27 @@ def test_even_rows_of_ragged_width_on_both_sides_of_the_rule(dtype):
         B = rng.standard_normal(A.n * k).astype(np.float32)
         Y, Y_ref, S = run_spmm(A, B, k, None, 1.0, 0.0, dtype)
         assert_within(Y, Y_ref, S, dtype, what="k=%d" % k)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_uneven_rows_and_few_columns_by_rows(dtype):
+    """Nearly even rows and a few longer ones: a lane or a few per row, rows of more than 128 by a launch of their own (aligned k)."""
+    rng = np.random.default_rng(3)
+    lens = rng.integers(6, 11, 200_000)
+    lens[17], lens[160_000], lens[-1] = 60, 129, 140
+    A = gen.random_csr(len(lens), 50_000, lens, seed=9)
+    plan = b200sp.b200sp_plan_create(A.m, A.n, A.nnz, to_dev(A.row_ptr))
+    stats = b200sp.b200sp_plan_info(plan)
+    b200sp.b200sp_plan_destroy(plan)
+    for k in (2, 3, 4, 8, 16):
+        assert k > 3 or not b200sp.b200sp_spmm_by_shares(stats, k, 0.0, dtype)
+        B = rng.standard_normal(A.n * k).astype(np.float32)
+        Y0 = rng.standard_normal(A.m * k).astype(np.float32)
+        Y, Y_ref, S = run_spmm(A, B, k, None, 1.0, 0.0, dtype)
+        assert_within(Y, Y_ref, S, dtype, what="k=%d" % k)
+        Y, Y_ref, S = run_spmm(A, B, k, Y0, -0.5, 1.25, dtype)
+        y0f = Y0 if dtype == "f32" else gen.bf16_to_f32(gen.to_bf16(Y0))
+        assert_within(Y, Y_ref, S, dtype, 1.0, np.abs(1.25 * y0f.astype(np.float64)).reshape(A.m, k), what="k=%d ab" % k)
 
 
 def test_non_finite_rows_of_b_touch_only_the_rows_that_use_them():
