@@ -21,8 +21,8 @@ constexpr size_t kCacheCap = 1024;
 int plan_free(b200sp_plan* p, bool stream_ordered = false, cudaStream_t stream = nullptr) {
   if (!p) return B200SP_OK;
   int rc = B200SP_OK;
-  void* const blocks[] = {p->block, p->cuts_block, p->compact_block, p->split_block, p->quad[0].block, p->quad[1].block, p->quad[2].block,
-                          p->quad[3].block, p->lists_block};
+  void* const blocks[] = {p->block, p->cuts_block, p->compact_block, p->shares.block, p->quad[0].block, p->quad[1].block, p->quad[2].block,
+                          p->quad[3].block, p->lists.block};
   bool any = false;
   for (void* b : blocks) any |= b != nullptr;
   if (any) {
@@ -108,24 +108,46 @@ int spmm_share_items(const b200sp_plan_info_t& I, const DeviceInfo* dev) {
 
 // The lists of rows of kMediumRow + 1 .. kLongRow and of more than kLongRow nonzeros, built on the device in stream order on the
 // first SpMM call that needs them; their lengths are known from the plan pass.
-int plan_row_lists(b200sp_plan* p, cudaStream_t stream, DeviceInfo* dev) {
-  if (p->lists_block || p->num_medium + p->num_long == 0) return B200SP_OK;
-  const size_t n_mid = (size_t)p->num_medium, n_long = (size_t)p->num_long;
-  int* blk = nullptr;
-  int rc = pool_alloc(dev, (void**)&blk, (4 + n_mid + n_long) * sizeof(int32_t), stream);
-  if (rc != B200SP_OK) return rc;
-  cudaError_t e = cudaMemsetAsync(blk, 0, 2 * sizeof(int), stream);
-  if (e == cudaSuccess) {
-    const int blocks = (int)((p->info.m + 255) / 256);
-    plan_row_lists_kernel<<<blocks < dev->sms * 8 ? blocks : dev->sms * 8, 256, 0, stream>>>(
-        p->row_ptr, (int)p->info.m, kMediumRow, kLongRow, (int)n_mid, (int)n_long, blk + 4, blk + 4 + n_mid, blk);
-    g_launches++;
-    e = cudaGetLastError();
+int plan_row_lists(b200sp_plan* p, b200sp_plan::RowLists* out, cudaStream_t stream, DeviceInfo* dev) {
+  if (p->num_medium + p->num_long == 0) return B200SP_OK;
+  std::lock_guard<std::mutex> lock(p->build);
+  if (!p->lists.block) {
+    const size_t n_mid = (size_t)p->num_medium, n_long = (size_t)p->num_long;
+    int* blk = nullptr;
+    const int rc = pool_alloc(dev, (void**)&blk, (4 + n_mid + n_long) * sizeof(int32_t), stream);
+    if (rc != B200SP_OK) return rc;
+    cudaError_t e = cudaMemsetAsync(blk, 0, 2 * sizeof(int), stream);
+    if (e == cudaSuccess) {
+      const int blocks = (int)((p->info.m + 255) / 256);
+      plan_row_lists_kernel<<<blocks < dev->sms * 8 ? blocks : dev->sms * 8, 256, 0, stream>>>(
+          p->row_ptr, (int)p->info.m, kMediumRow, kLongRow, (int)n_mid, (int)n_long, blk + 4, blk + 4 + n_mid, blk);
+      g_launches++;
+      e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) { cudaFreeAsync(blk, stream); return cuda_fail(e, "lists of medium and long rows"); }
+    p->lists = {blk, blk + 4, blk + 4 + n_mid};
   }
-  if (e != cudaSuccess) { cudaFreeAsync(blk, stream); return cuda_fail(e, "lists of medium and long rows"); }
-  p->lists_block = blk;
-  p->medium_rows = blk + 4;
-  p->long_rows = blk + 4 + n_mid;
+  *out = p->lists;
+  return B200SP_OK;
+}
+
+// The shares of the nnz-balanced SpMM kernel: with the plan pass for small matrices, else by a small kernel in stream order on the first
+// SpMM call that needs them.
+int plan_shares(b200sp_plan* p, b200sp_plan::Shares* out, cudaStream_t stream, DeviceInfo* dev) {
+  std::lock_guard<std::mutex> lock(p->build);
+  if (!p->shares.split) {
+    const b200sp_plan_info_t& I = p->info;
+    const int w = spmm_share_items(I, dev);
+    const long long shares = (I.m + I.nnz + w - 1) / w;
+    int* blk = nullptr;
+    int rc = pool_alloc(dev, (void**)&blk, (size_t)(shares + 1) * sizeof(int32_t), stream);
+    if (rc != B200SP_OK) return rc;
+    rc = launch(plan_merge_split_kernel, dim3((unsigned)((shares + 1 + 255) / 256)), dim3(256), stream, nullptr, 0, dev, p->row_ptr, (int)I.m,
+                (int)I.nnz, w, (int)shares, blk);
+    if (rc != B200SP_OK) { cudaFreeAsync(blk, stream); return rc; }
+    p->shares = {blk, blk, w};
+  }
+  *out = p->shares;
   return B200SP_OK;
 }
 
@@ -173,7 +195,8 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
   p->split_row = (int32_t*)(base + o_split);
   p->carry = (float*)(base + o_carry);
   p->tail = (float*)(base + o_tail);
-  if (with_shares) { p->spmm_split = (int32_t*)(base + o_share); p->spmm_witems = witems; }
+  int32_t* const share_split = (int32_t*)(base + o_share);
+  if (with_shares) p->shares = {nullptr, share_split, witems};
   I.scratch_bytes = (int64_t)total;
   int slot = 0;
   rc = plan_slot_take(&slot);
@@ -184,7 +207,7 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
     const long long blocks = (work + 256 * 4 - 1) / (256 * 4);   // four rows and at most one search per thread
     const int grid = (int)(blocks < dev->sms * 8 ? blocks : dev->sms * 8);
     plan_pass_kernel<<<grid, 256, 0, stream>>>(row_ptr, (int)m, (int)nnz, slot, g_slots.host + slot, items, (int)nt, p->split_row,
-                                               with_shares ? witems : 0, (int)shares, p->spmm_split);
+                                               with_shares ? witems : 0, (int)shares, share_split);
     g_launches++;
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);

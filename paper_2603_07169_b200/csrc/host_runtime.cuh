@@ -244,15 +244,22 @@ struct b200sp_plan {
   int32_t* split_row = nullptr;       // spmv tiles + 1
   float* carry = nullptr;             // spmv tiles
   float* tail = nullptr;              // spmv tiles
-  void* lists_block = nullptr;        // one pool block for the two lists below, built on the first SpMM call that needs them
-  int32_t* medium_rows = nullptr;     // rows of kMediumRow + 1 .. kLongRow nonzeros, in any order
-  int32_t* long_rows = nullptr;       // rows longer than kLongRow, in any order
   unsigned long long* probe_out = nullptr;  // two counters for the column-locality probe
   int num_medium = 0, num_long = 0;
   const void* probed_col_idx = nullptr;   // col_idx the column-locality probe last ran on
-  int32_t* spmm_split = nullptr;          // warp shares of the nnz-balanced SpMM kernel (part of `block` for small matrices, else a pool block of its own, built on first use)
-  void* split_block = nullptr;            // that block
-  int spmm_witems = 0;                    // merge items per share
+  // Parts that only some SpMM kernels need, built on first use under `build` and complete when it is released: calls from other threads
+  // either find them or wait (the work that fills them is ahead of theirs in the stream).
+  std::mutex build;
+  struct RowLists {
+    void* block = nullptr;                // one pool block for both
+    const int* medium = nullptr;          // rows of kMediumRow + 1 .. kLongRow nonzeros, in any order
+    const int* longer = nullptr;          // rows longer than kLongRow, in any order
+  } lists;
+  struct Shares {                         // warp shares of the nnz-balanced SpMM kernel
+    void* block = nullptr;                // their pool block (null: part of the plan's block, for small matrices)
+    const int* split = nullptr;           // row ends before each share
+    int witems = 0;                       // merge items per share
+  } shares;
   // merge list over the rows that have nonzeros (matrices with many empty rows)
   void* compact_block = nullptr;          // one pool block: row ids, their offsets, block counts
   int compact_rows = 0;                   // number of rows that have nonzeros (0 = the list has not been built)
@@ -264,12 +271,12 @@ struct b200sp_plan {
   const void* cuts_col_idx = nullptr;     // col_idx they were computed from
   int cuts_ranges = 0;                    // number of ranges they describe (0 = none computed)
   bool cols_sorted = false;               // every row's columns ascend
-  // processing order of the SpMM kernel with B in shared memory: rows of at most kLongRow nonzeros sorted by length, in blocks of quad_gpw
+  // processing order of the SpMM kernel with B in shared memory: rows of at most kLongRow nonzeros sorted by length, in blocks of as many rows as a warp takes
   struct QuadOrder {
-    void* block = nullptr;                // one pool block: row numbers, row lengths, block offsets (built on first use)
-    int32_t* row = nullptr;               // blocks * gpw row numbers (-1 = unused slot)
-    int32_t* len = nullptr;               // their lengths
-    int32_t* pos = nullptr;               // blocks + 1: where each block's quads start in the per-call copy of A
+    void* block = nullptr;                // one pool block: row numbers, row lengths, block offsets
+    const int* row = nullptr;             // blocks * gpw row numbers (-1 = unused slot)
+    const int* len = nullptr;             // their lengths
+    const int* pos = nullptr;             // blocks + 1: where each block's quads start in the per-call copy of A
     int blocks = 0;
   } quad[4];                              // for 4, 8, 16 and 32 rows per warp
   const void* probed_key = nullptr;       // host entry points: the HOST col_idx that verdict belongs to

@@ -16,7 +16,8 @@ int launch_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, co
   const b200sp_plan_info_t& I = p->info;
   constexpr int GROUPS = kSpmmThreads / LANES;
   const unsigned grid = (unsigned)((I.m + GROUPS - 1) / GROUPS);
-  int rc = plan_row_lists(p, stream, dev);
+  b200sp_plan::RowLists lists;
+  int rc = plan_row_lists(p, &lists, stream, dev);
   if (rc != B200SP_OK) return rc;
   tl_pdl_kernel = true;
   rc = launch(spmm_row_group_kernel<T, VEC, LANES, NCH, kSpmmThreads>, dim3(grid), dim3(kSpmmThreads), stream, B,
@@ -26,7 +27,7 @@ int launch_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, co
   if (ctas >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
   tl_pdl_kernel = true;
   return launch(spmm_long_row_kernel<T, VEC, kSpmmThreads>, dim3((unsigned)ctas), dim3(kSpmmThreads), stream, nullptr, 0, dev, k, p->num_long,
-                (const int*)p->long_rows, p->row_ptr, col_idx, vals, B, Y, alpha, beta);
+                lists.longer, p->row_ptr, col_idx, vals, B, Y, alpha, beta);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
@@ -113,11 +114,11 @@ int device_scan_in_place(int* data, long long count, int* bsum, cudaStream_t str
 
 // The processing order of spmm_bstage_quads_kernel (see plan_kernels.cuh), built once per plan and lane-group width, on the
 // device and in stream order: no synchronisation.  B200SP_ERR_UNSUPPORTED when the positions would not fit 32 bits.
-int plan_quad_order(b200sp_plan* p, int gpw, b200sp_plan::QuadOrder** out, cudaStream_t stream, DeviceInfo* dev) {
+int plan_quad_order(b200sp_plan* p, int gpw, b200sp_plan::QuadOrder* out, cudaStream_t stream, DeviceInfo* dev) {
   static_assert(kLongRow == 1024, "quad_key() assumes rows of at most 1024 nonzeros");
   b200sp_plan::QuadOrder& Q = p->quad[gpw == 4 ? 0 : gpw == 8 ? 1 : gpw == 16 ? 2 : 3];
-  *out = &Q;
-  if (Q.block) return B200SP_OK;
+  std::lock_guard<std::mutex> lock(p->build);
+  if (Q.block) { *out = Q; return B200SP_OK; }
   const b200sp_plan_info_t& I = p->info;
   const long long listed = I.m - p->num_long;
   const long long blocks = (listed + gpw - 1) / gpw;
@@ -159,11 +160,8 @@ int plan_quad_order(b200sp_plan* p, int gpw, b200sp_plan::QuadOrder** out, cudaS
   if (rc != B200SP_OK) return fail(rc);
   CUQ(cudaFreeAsync(tmp, stream));
 #undef CUQ
-  Q.block = blk;
-  Q.row = row_of;
-  Q.len = len_of;
-  Q.pos = pos;
-  Q.blocks = (int)blocks;
+  Q = {blk, row_of, len_of, pos, (int)blocks};
+  *out = Q;
   return B200SP_OK;
 }
 
@@ -198,9 +196,10 @@ int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, c
                              gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS) return B200SP_ERR_UNSUPPORTED;
-  b200sp_plan::QuadOrder* Q = nullptr;
+  b200sp_plan::QuadOrder Q;
+  b200sp_plan::RowLists lists;
   int rc = plan_quad_order(p, GPW, &Q, stream, dev);
-  if (rc == B200SP_OK) rc = plan_row_lists(p, stream, dev);
+  if (rc == B200SP_OK) rc = plan_row_lists(p, &lists, stream, dev);
   if (rc != B200SP_OK) return rc;
   auto kernel = spmm_bstage_quads_kernel<T, VEC, LANES, PIECES, OLD, THREADS>;
   static bool configured[64] = {};
@@ -209,7 +208,7 @@ int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, c
     configured[p->device] = true;
   }
   const int slices = (k - 1) / KS + 1;
-  const int blocks = Q->blocks;
+  const int blocks = Q.blocks;
   const long long most = (blocks + WARPS - 1) / WARPS;   // a block per warp at least
   long long chunks;
   if (g_opt.bstage_nnz > 0) {
@@ -246,15 +245,15 @@ int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, c
   if (rc != B200SP_OK) return rc;
   unsigned short* qoff = (unsigned short*)scratch;       // entries 16-bit offsets, then entries values (16-byte aligned: entries is a multiple of 8)
   T* qval = (T*)((char*)scratch + entries * 2);
-  int* slot_row = reorder ? (int*)((char*)scratch + entries * (2 + sizeof(T))) : Q->row;
-  int* slot_len = reorder ? slot_row + slots : Q->len;
+  int* const new_row = reorder ? (int*)((char*)scratch + entries * (2 + sizeof(T))) : nullptr;
+  int* const new_len = reorder ? new_row + slots : nullptr;
   tl_pdl_kernel = true;
   rc = launch(spmm_bstage_prep_kernel<T, ROW_BYTES>, dim3((unsigned)((slots * 8 + 255) / 256)), dim3(256), stream, nullptr, 0, dev, (int)slots, GPW,
-              (const int*)Q->row, (const int*)Q->pos, p->row_ptr, col_idx, vals, qoff, qval, (int)reorder, slot_row, slot_len);
+              Q.row, Q.pos, p->row_ptr, col_idx, vals, qoff, qval, (int)reorder, new_row, new_len);
   if (rc == B200SP_OK) {
     tl_pdl_kernel = true;
     rc = launch_smem(kernel, dim3((unsigned)(slices * row_chunks)), dim3(THREADS), smem, stream, nullptr, 0, dev, map, (int)I.n, k, row_chunks,
-                     blocks, box_rows, (int)bslice, capq, (const int*)slot_row, (const int*)slot_len, (const int*)Q->pos,
+                     blocks, box_rows, (int)bslice, capq, (const int*)(reorder ? new_row : Q.row), (const int*)(reorder ? new_len : Q.len), Q.pos,
                      (const unsigned short*)qoff, (const T*)qval, Y, alpha, beta, dev->err_flag, g_opt.spin_limit, g_opt.debug_no_copies);
   }
   const cudaError_t e = cudaFreeAsync(scratch, stream);
@@ -264,7 +263,7 @@ int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, c
     if (ctas >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
     tl_pdl_kernel = true;
     rc = launch(spmm_long_row_kernel<T, VEC, kSpmmThreads>, dim3((unsigned)ctas), dim3(kSpmmThreads), stream, nullptr, 0, dev, k, p->num_long,
-                (const int*)p->long_rows, p->row_ptr, col_idx, vals, B, Y, alpha, beta);
+                lists.longer, p->row_ptr, col_idx, vals, B, Y, alpha, beta);
   }
   return rc;
 }
@@ -381,11 +380,11 @@ bool spmm_by_shares(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, floa
 }
 
 template <typename T, int V, int J, bool LIST>
-int launch_spmm_merge_as(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
+int launch_spmm_merge_as(b200sp_plan* p, const b200sp_plan::Shares& work, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
                       cudaStream_t stream, DeviceInfo* dev) {
   const b200sp_plan_info_t& I = p->info;
   constexpr int KS = 32 * V * J;
-  const int witems = p->spmm_witems;
+  const int witems = work.witems;
   auto kernel = spmm_merge_kernel<T, V, J, LIST>;
   static int per_sm[64] = {};   // per instantiation and device: resident CTAs
   if (!per_sm[p->device]) {
@@ -418,7 +417,7 @@ int launch_spmm_merge_as(b200sp_plan* p, int k, const int32_t* col_idx, const T*
   if (rc != B200SP_OK) return rc;
   tl_pdl_kernel = true;
   rc = launch(kernel, dim3((unsigned)(slices * tiles)), dim3(kMergeWarps * 32), stream, B, (size_t)I.n * k * sizeof(T), dev,
-              (int)I.m, (int)I.nnz, k, tiles, witems, shares, (const int*)p->spmm_split, p->row_ptr, col_idx, vals, B, Y, scratch, scratch + per, tile_row, alpha, beta);
+              (int)I.m, (int)I.nnz, k, tiles, witems, shares, work.split, p->row_ptr, col_idx, vals, B, Y, scratch, scratch + per, tile_row, alpha, beta);
   if (rc == B200SP_OK && tiles > 1) {
     tl_pdl_kernel = true;
     const int lanes = KS >= 128 ? 128 : KS;      // a power of two
@@ -433,11 +432,11 @@ int launch_spmm_merge_as(b200sp_plan* p, int k, const int32_t* col_idx, const T*
 // beta != 0 and one row in sixteen or more without nonzeros: these are listed and scaled apart (R-MAT 2^21, k = 64 BF16, 61 % empty: 458 us
 // against 657 us; with beta == 0 the listing costs as much as it saves).
 template <typename T, int V, int J>
-int launch_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
+int launch_spmm_merge(b200sp_plan* p, const b200sp_plan::Shares& work, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
                       cudaStream_t stream, DeviceInfo* dev) {
   return beta != 0.0f && p->info.bin_rows[0] * 16 >= p->info.m
-             ? launch_spmm_merge_as<T, V, J, true>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev)
-             : launch_spmm_merge_as<T, V, J, false>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
+             ? launch_spmm_merge_as<T, V, J, true>(p, work, k, col_idx, vals, B, Y, alpha, beta, stream, dev)
+             : launch_spmm_merge_as<T, V, J, false>(p, work, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
 }
 
 // nnz-balanced SpMM (spmm_merge_kernel), any k.  The widest pieces (16 bytes per lane at most) that k allows, narrowed while half as
@@ -445,26 +444,17 @@ int launch_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* va
 template <typename T, int VMAX>
 int run_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
                    cudaStream_t stream, DeviceInfo* dev) {
-  const b200sp_plan_info_t& I = p->info;
   int v = 1;
   while (v < VMAX && k % (2 * v) == 0 && 32 * v < k) v *= 2;
-  if (!p->spmm_split) {   // shares: once per plan, a small kernel in stream order
-    const int w = spmm_share_items(I, dev);
-    const long long shares = (I.m + I.nnz + w - 1) / w;
-    int rc = pool_alloc(dev, &p->split_block, (size_t)(shares + 1) * sizeof(int32_t), stream);
-    if (rc != B200SP_OK) return rc;
-    rc = launch(plan_merge_split_kernel, dim3((unsigned)((shares + 1 + 255) / 256)), dim3(256), stream, nullptr, 0, dev, p->row_ptr, (int)I.m,
-                (int)I.nnz, w, (int)shares, (int*)p->split_block);
-    if (rc != B200SP_OK) return rc;
-    p->spmm_split = (int32_t*)p->split_block;
-    p->spmm_witems = w;
-  }
+  b200sp_plan::Shares work;
+  const int rc = plan_shares(p, &work, stream, dev);
+  if (rc != B200SP_OK) return rc;
   const int loads = (k - 1) / (32 * v) + 1;
 #define B200SP_MERGE_J(V)                                                                                                   \
   do {                                                                                                                      \
-    if (loads == 1) return launch_spmm_merge<T, V, 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);                 \
-    if (loads == 2) return launch_spmm_merge<T, V, 2>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);                 \
-    return launch_spmm_merge<T, V, (V * sizeof(T) >= 16 ? 2 : 4)>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);     \
+    if (loads == 1) return launch_spmm_merge<T, V, 1>(p, work, k, col_idx, vals, B, Y, alpha, beta, stream, dev);                 \
+    if (loads == 2) return launch_spmm_merge<T, V, 2>(p, work, k, col_idx, vals, B, Y, alpha, beta, stream, dev);                 \
+    return launch_spmm_merge<T, V, (V * sizeof(T) >= 16 ? 2 : 4)>(p, work, k, col_idx, vals, B, Y, alpha, beta, stream, dev);     \
   } while (0)
   if (v == 1) B200SP_MERGE_J(1);
   if (v == 2) B200SP_MERGE_J(2);
@@ -522,7 +512,8 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     const int slices = (k - 1) / KS + 1;
     const int row_blocks = (int)((I.m + GROUPS - 1) / GROUPS);
     if ((long long)slices * row_blocks >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
-    int rc = plan_row_lists(p, stream, dev);
+    b200sp_plan::RowLists lists;
+    int rc = plan_row_lists(p, &lists, stream, dev);
     if (rc != B200SP_OK) return rc;
     const int mid_blocks = (p->num_medium + GROUPS - 1) / GROUPS;
     int ranges = 1;
@@ -547,7 +538,7 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
       if (rc == B200SP_OK && p->num_medium > 0) {
         tl_pdl_kernel = true;
         rc = launch(spmm_medium_row_kernel<T, VEC, kSpmmThreads, 8>, dim3((unsigned)(slices * mid_blocks)), dim3(kSpmmThreads), stream,
-                    nullptr, 0, dev, p->num_medium, (const int*)p->medium_rows, k, mid_blocks, p->row_ptr, col_idx, vals, B, Y, alpha, beta);
+                    nullptr, 0, dev, p->num_medium, lists.medium, k, mid_blocks, p->row_ptr, col_idx, vals, B, Y, alpha, beta);
       }
     } else
     // rows of at most kMediumRow nonzeros: the register-capped kernel; kMediumRow + 1 .. kLongRow: the same scheme with
@@ -564,7 +555,7 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     if (rc == B200SP_OK && p->num_medium > 0) {                                                                                     \
       tl_pdl_kernel = true;                                                                                                         \
       rc = launch(spmm_medium_row_kernel<T, VEC, kSpmmThreads, L>, dim3((unsigned)(slices * mid_blocks)), dim3(kSpmmThreads), stream, \
-                  nullptr, 0, dev, p->num_medium, (const int*)p->medium_rows, k, mid_blocks, p->row_ptr, col_idx, vals, B, Y, alpha, beta); \
+                  nullptr, 0, dev, p->num_medium, lists.medium, k, mid_blocks, p->row_ptr, col_idx, vals, B, Y, alpha, beta); \
     }
     if (lanes == 8) { B200SP_SLICE_LAUNCH(8); }
     else if (lanes == 4) { B200SP_SLICE_LAUNCH(4); }
@@ -576,7 +567,7 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     if (ctas >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
     tl_pdl_kernel = true;
     return launch(spmm_long_row_kernel<T, VEC, kSpmmThreads>, dim3((unsigned)ctas), dim3(kSpmmThreads), stream, nullptr, 0,
-                  dev, k, p->num_long, (const int*)p->long_rows, p->row_ptr, col_idx, vals, B, Y, alpha, beta);
+                  dev, k, p->num_long, lists.longer, p->row_ptr, col_idx, vals, B, Y, alpha, beta);
   }
   if (k % VEC != 0) {  // ragged k: scalar lanes
     if (k <= 2) return launch_spmm<T, 1, 2, 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
