@@ -117,6 +117,7 @@ int spmm_csr(int64_t m, int64_t n, int64_t nnz, int64_t k, const int32_t* row_pt
  * built on the first SpMM call that uses them, in stream order: the lists of rows of 129-1024 and of more than 1024 nonzeros,
  * the shares of large matrices, and the order of the rows by length that SpMM uses when A has so few columns that a slice
  * of B is kept in shared memory.
+ * A first call that is captured into a graph builds them inside the graph, for that call alone, and leaves the plan as it was.
  * When the row statistics select the row-direct SpMV kernel, the first b200sp_spmv / spmv_csr call with a given
  * col_idx additionally samples how local the columns are (one small kernel and one synchronisation of the stream)
  * and falls back to the merge-tile kernel for matrices with scattered columns.

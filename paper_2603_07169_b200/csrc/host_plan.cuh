@@ -108,7 +108,7 @@ int spmm_share_items(const b200sp_plan_info_t& I, const DeviceInfo* dev) {
 
 // The lists of rows of kMediumRow + 1 .. kLongRow and of more than kLongRow nonzeros, built on the device in stream order on the
 // first SpMM call that needs them; their lengths are known from the plan pass.
-int plan_row_lists(b200sp_plan* p, b200sp_plan::RowLists* out, cudaStream_t stream, DeviceInfo* dev) {
+int plan_row_lists(b200sp_plan* p, b200sp_plan::RowLists* out, CallBlock* own, cudaStream_t stream, DeviceInfo* dev) {
   if (p->num_medium + p->num_long == 0) return B200SP_OK;
   std::lock_guard<std::mutex> lock(p->build);
   if (!p->lists.block) {
@@ -125,7 +125,9 @@ int plan_row_lists(b200sp_plan* p, b200sp_plan::RowLists* out, cudaStream_t stre
       e = cudaGetLastError();
     }
     if (e != cudaSuccess) { cudaFreeAsync(blk, stream); return cuda_fail(e, "lists of medium and long rows"); }
-    p->lists = {blk, blk + 4, blk + 4 + n_mid};
+    *out = {blk, blk + 4, blk + 4 + n_mid};
+    if (stream_captures(stream)) { own->take(blk, stream); return B200SP_OK; }
+    p->lists = *out;
   }
   *out = p->lists;
   return B200SP_OK;
@@ -133,7 +135,7 @@ int plan_row_lists(b200sp_plan* p, b200sp_plan::RowLists* out, cudaStream_t stre
 
 // The shares of the nnz-balanced SpMM kernel: with the plan pass for small matrices, else by a small kernel in stream order on the first
 // SpMM call that needs them.
-int plan_shares(b200sp_plan* p, b200sp_plan::Shares* out, cudaStream_t stream, DeviceInfo* dev) {
+int plan_shares(b200sp_plan* p, b200sp_plan::Shares* out, CallBlock* own, cudaStream_t stream, DeviceInfo* dev) {
   std::lock_guard<std::mutex> lock(p->build);
   if (!p->shares.split) {
     const b200sp_plan_info_t& I = p->info;
@@ -145,7 +147,9 @@ int plan_shares(b200sp_plan* p, b200sp_plan::Shares* out, cudaStream_t stream, D
     rc = launch(plan_merge_split_kernel, dim3((unsigned)((shares + 1 + 255) / 256)), dim3(256), stream, nullptr, 0, dev, p->row_ptr, (int)I.m,
                 (int)I.nnz, w, (int)shares, blk);
     if (rc != B200SP_OK) { cudaFreeAsync(blk, stream); return rc; }
-    p->shares = {blk, blk, w};
+    *out = {blk, blk, w};
+    if (stream_captures(stream)) { own->take(blk, stream); return B200SP_OK; }
+    p->shares = *out;
   }
   *out = p->shares;
   return B200SP_OK;

@@ -158,6 +158,25 @@ int pool_alloc(DeviceInfo* d, void** ptr, size_t bytes, cudaStream_t stream) {
   return B200SP_OK;
 }
 
+// Whether work put on `stream` is recorded into a graph instead of run.
+bool stream_captures(cudaStream_t stream) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &status) != cudaSuccess) (void)cudaGetLastError();
+  return status != cudaStreamCaptureStatusNone;
+}
+
+// A pool block that lives as long as one call.  What is built while the stream is captured must not outlive the call: its memory belongs to
+// the graph, and nothing is in it until the graph runs.
+struct CallBlock {
+  void* block = nullptr;
+  cudaStream_t stream = nullptr;
+  CallBlock() = default;
+  CallBlock(const CallBlock&) = delete;
+  CallBlock& operator=(const CallBlock&) = delete;
+  ~CallBlock() { if (block) cudaFreeAsync(block, stream); }
+  void take(void* b, cudaStream_t s) { block = b; stream = s; }
+};
+
 // The flag that kernels with bounded waits raise: one int in the library image per device (zero when the module is
 // loaded), so finding it neither allocates nor synchronises.
 __device__ int g_timeout_flag;
@@ -248,7 +267,7 @@ struct b200sp_plan {
   int num_medium = 0, num_long = 0;
   const void* probed_col_idx = nullptr;   // col_idx the column-locality probe last ran on
   // Parts that only some SpMM kernels need, built on first use under `build` and complete when it is released: calls from other threads
-  // either find them or wait (the work that fills them is ahead of theirs in the stream).
+  // either find them or wait (the work that fills them is ahead of theirs in the stream).  Built for the one call when the stream is captured.
   std::mutex build;
   struct RowLists {
     void* block = nullptr;                // one pool block for both

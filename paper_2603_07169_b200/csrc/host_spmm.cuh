@@ -17,7 +17,8 @@ int launch_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, co
   constexpr int GROUPS = kSpmmThreads / LANES;
   const unsigned grid = (unsigned)((I.m + GROUPS - 1) / GROUPS);
   b200sp_plan::RowLists lists;
-  int rc = plan_row_lists(p, &lists, stream, dev);
+  CallBlock own_lists;
+  int rc = plan_row_lists(p, &lists, &own_lists, stream, dev);
   if (rc != B200SP_OK) return rc;
   tl_pdl_kernel = true;
   rc = launch(spmm_row_group_kernel<T, VEC, LANES, NCH, kSpmmThreads>, dim3(grid), dim3(kSpmmThreads), stream, B,
@@ -114,7 +115,7 @@ int device_scan_in_place(int* data, long long count, int* bsum, cudaStream_t str
 
 // The processing order of spmm_bstage_quads_kernel (see plan_kernels.cuh), built once per plan and lane-group width, on the
 // device and in stream order: no synchronisation.  B200SP_ERR_UNSUPPORTED when the positions would not fit 32 bits.
-int plan_quad_order(b200sp_plan* p, int gpw, b200sp_plan::QuadOrder* out, cudaStream_t stream, DeviceInfo* dev) {
+int plan_quad_order(b200sp_plan* p, int gpw, b200sp_plan::QuadOrder* out, CallBlock* own, cudaStream_t stream, DeviceInfo* dev) {
   static_assert(kLongRow == 1024, "quad_key() assumes rows of at most 1024 nonzeros");
   b200sp_plan::QuadOrder& Q = p->quad[gpw == 4 ? 0 : gpw == 8 ? 1 : gpw == 16 ? 2 : 3];
   std::lock_guard<std::mutex> lock(p->build);
@@ -160,8 +161,9 @@ int plan_quad_order(b200sp_plan* p, int gpw, b200sp_plan::QuadOrder* out, cudaSt
   if (rc != B200SP_OK) return fail(rc);
   CUQ(cudaFreeAsync(tmp, stream));
 #undef CUQ
-  Q = {blk, row_of, len_of, pos, (int)blocks};
-  *out = Q;
+  *out = {blk, row_of, len_of, pos, (int)blocks};
+  if (stream_captures(stream)) own->take(blk, stream);
+  else Q = *out;
   return B200SP_OK;
 }
 
@@ -197,9 +199,11 @@ int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, c
                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS) return B200SP_ERR_UNSUPPORTED;
   b200sp_plan::QuadOrder Q;
+  CallBlock own_order;
   b200sp_plan::RowLists lists;
-  int rc = plan_quad_order(p, GPW, &Q, stream, dev);
-  if (rc == B200SP_OK) rc = plan_row_lists(p, &lists, stream, dev);
+  CallBlock own_lists;
+  int rc = plan_quad_order(p, GPW, &Q, &own_order, stream, dev);
+  if (rc == B200SP_OK) rc = plan_row_lists(p, &lists, &own_lists, stream, dev);
   if (rc != B200SP_OK) return rc;
   auto kernel = spmm_bstage_quads_kernel<T, VEC, LANES, PIECES, OLD, THREADS>;
   static bool configured[64] = {};
@@ -447,7 +451,8 @@ int run_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals,
   int v = 1;
   while (v < VMAX && k % (2 * v) == 0 && 32 * v < k) v *= 2;
   b200sp_plan::Shares work;
-  const int rc = plan_shares(p, &work, stream, dev);
+  CallBlock own_work;
+  const int rc = plan_shares(p, &work, &own_work, stream, dev);
   if (rc != B200SP_OK) return rc;
   const int loads = (k - 1) / (32 * v) + 1;
 #define B200SP_MERGE_J(V)                                                                                                   \
@@ -513,7 +518,8 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     const int row_blocks = (int)((I.m + GROUPS - 1) / GROUPS);
     if ((long long)slices * row_blocks >= (1LL << 31)) return B200SP_ERR_UNSUPPORTED;
     b200sp_plan::RowLists lists;
-    int rc = plan_row_lists(p, &lists, stream, dev);
+    CallBlock own_lists;
+    int rc = plan_row_lists(p, &lists, &own_lists, stream, dev);
     if (rc != B200SP_OK) return rc;
     const int mid_blocks = (p->num_medium + GROUPS - 1) / GROUPS;
     int ranges = 1;

@@ -1,4 +1,5 @@
-"""Parts of a plan that are built by the first SpMM call that needs them: first calls from several host threads on one stream."""
+"""Parts of a plan that are built by the first SpMM call that needs them: first calls from several host threads on one stream, and
+a first call that is captured into a graph."""
 import threading
 
 import numpy as np
@@ -89,5 +90,37 @@ def test_first_calls_from_several_threads(case):
             for Y in outs[1:]:
                 assert torch.equal(Y, outs[0])
             b200sp.b200sp_plan_destroy(plan)
+    finally:
+        P.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("case", sorted(CASES))
+def test_first_call_captured(case, dtype):
+    """What the captured call builds belongs to its graph: calls outside it, before it has run and after it is gone, build their own."""
+    P = Problem(case, dtype)
+    try:
+        warm, Y = P.plan(), P.out()
+        P.call(warm, Y)                         # kernels loaded, attributes set
+        torch.cuda.synchronize()
+        P.check(Y, "eager")
+        b200sp.b200sp_plan_destroy(warm)
+        plan, captured, before, after = P.plan(), P.out(), P.out(), P.out()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            P.call(plan, captured)
+        P.call(plan, before)
+        torch.cuda.synchronize()
+        P.check(before, "outside the graph, before it has run")
+        for _ in range(2):
+            captured.fill_(0)
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(captured, before)
+        del graph
+        P.call(plan, after)
+        torch.cuda.synchronize()
+        assert torch.equal(after, before)
+        b200sp.b200sp_plan_destroy(plan)
     finally:
         P.close()
