@@ -122,7 +122,7 @@ int spmm_csr(int64_t m, int64_t n, int64_t nnz, int64_t k, const int32_t* row_pt
  * col_idx additionally samples how local the columns are (one small kernel and one synchronisation of the stream)
  * and falls back to the merge-tile kernel for matrices with scattered columns.
  * It takes one block of a few bytes per tile from the library's pool, in the order of `stream`, and
- * synchronises `stream` once.  A plan may be used from one stream at a time.  b200sp_plan_destroy
+ * synchronises `stream` once, so a capturing stream is refused (B200SP_ERR_UNSUPPORTED; the capture stays valid).  A plan may be used from one stream at a time.  b200sp_plan_destroy
  * synchronises the plan's device before it returns the block. */
 int b200sp_plan_create(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32_t* row_ptr, void* stream);
 int b200sp_plan_destroy(b200sp_plan* plan);

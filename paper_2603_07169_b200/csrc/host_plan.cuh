@@ -180,6 +180,7 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
   I.spmv_tiles = (int32_t)((m + nnz + items - 1) / items);
   I.spmv_kernel = g_opt.spmv_kernel >= 0 ? g_opt.spmv_kernel : 0;
   if (m == 0) { *out = p; return B200SP_OK; }
+  if (stream_captures(stream)) { delete p; return B200SP_ERR_UNSUPPORTED; }   // the statistics are read back
 
   // one block from the pool: the probe's counters, split points, carries, tails; for small matrices also the shares of the
   // nnz-balanced SpMM kernel, which then cost no launch of their own (large ones search them on first use)
@@ -210,13 +211,12 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
     const long long searches = (long long)nt + 1 + (with_shares ? shares + 1 : 0), work = m > searches * 4 ? m : searches * 4;
     const long long blocks = (work + 256 * 4 - 1) / (256 * 4);   // four rows and at most one search per thread
     const int grid = (int)(blocks < dev->sms * 8 ? blocks : dev->sms * 8);
-    plan_pass_kernel<<<grid, 256, 0, stream>>>(row_ptr, (int)m, (int)nnz, slot, g_slots.host + slot, items, (int)nt, p->split_row,
-                                               with_shares ? witems : 0, (int)shares, share_split);
-    g_launches++;
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    rc = launch(plan_pass_kernel, dim3((unsigned)grid), dim3(256), stream, nullptr, 0, dev, row_ptr, (int)m, (int)nnz, slot, g_slots.host + slot, items, (int)nt,
+                p->split_row, with_shares ? witems : 0, (int)shares, share_split);
+    const cudaError_t e = cudaStreamSynchronize(stream);
     h = g_slots.host[slot];
-    plan_slot_give(slot);
+    if (e == cudaSuccess) plan_slot_give(slot);   // only a finished pass (or none) has left its slot to the next; an error here means a lost device
+    if (rc != B200SP_OK) return fail(rc);
     if (e != cudaSuccess) return fail(cuda_fail(e, "plan pass"));
   }
   if (!h.bad) { p->num_medium = (int)h.bin_rows[4]; p->num_long = (int)h.bin_rows[5]; }

@@ -56,3 +56,21 @@ def test_passes_from_several_threads():
     for t in threads:
         t.join()
     assert not failures, failures[0]
+
+
+def test_a_capturing_stream_is_refused():
+    """No pass is recorded and no accumulator lost (there are 64): the capture goes on, and later passes count from zero."""
+    lens = lengths(5000, 1)
+    row_ptr = torch.from_numpy(np.concatenate([[0], lens.cumsum()]).astype(np.int32)).to("cuda:0")
+    x, graph = torch.zeros(8, device="cuda:0"), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(70):
+            with pytest.raises(b200sp.B200spError) as e:
+                b200sp.b200sp_plan_create(len(lens), 1 << 20, int(lens.sum()), row_ptr)
+            assert e.value.status == 2      # B200SP_ERR_UNSUPPORTED
+        x += 1
+    graph.replay()
+    torch.cuda.synchronize()
+    assert x.sum().item() == 8
+    for seed in range(70):
+        check(lengths(3000, seed))
