@@ -33,7 +33,8 @@ extern "C" {
  *                    launch gathers from stay in L2: 1 = no ranges (default: measured slower, see the benchmarks' record),
  *                    0 = as many as make a range of B fit L2, 2, 3, 4 or 8 = that many
  *  merge-tile SpMV kernel
- *   "merge_items"    merge items per tile: 1024, 2048 (default; 1024 below 12 million rows + nonzeros) or 4096
+ *   "merge_items"    merge items per tile: 1024, 2048 or 4096; until it is set, and after it is set to 0, 1024 below 12 million
+ *                    rows + nonzeros and 2048 above (and the switch reads as 2048)
  *   "merge_threads"  threads per CTA: 64, 128 (default) or 256
  *   "merge_carve"    shared-memory carveout in percent requested for it: 0, 25, 45 (default), 60, 75, 100 or -1 = leave to the driver
  *   "merge_short"    rows of up to this many products are added by one thread: 8, 16, 32 (default) or 64

@@ -592,7 +592,8 @@ int64_t b200sp_launch_count(void) { return g_launches.load(); }
 // One row per switch: where it lives and which values it accepts (exactly those listed in b200sp_tuning.h; the test suite
 // runs every one of them).  Called with g_mutex held.
 static int option_access(const char* name, int* get, const int* set) {
-  struct Entry { const char* name; int* slot; bool boolean; std::initializer_list<int> values; int lo, hi; };
+  // set_by_caller: a switch that is a rule of the library until it is set, and again when it is set to 0 (it then reads as by_rule)
+  struct Entry { const char* name; int* slot; bool boolean; std::initializer_list<int> values; int lo, hi; bool* set_by_caller = nullptr; int by_rule = 0; };
   const Entry table[] = {
       {"spmv_kernel", &g_opt.spmv_kernel, false, {-1, 0, 1, 2, 3}, 0, 0},
       {"spmm_bstage", &g_opt.spmm_bstage, true, {}, 0, 0},
@@ -600,7 +601,7 @@ static int option_access(const char* name, int* get, const int* set) {
       {"spmm_stage_a", &g_opt.spmm_stage_a, false, {0, 1, 2}, 0, 0},
       {"spmm_flat", &g_opt.spmm_flat, false, {0, 1, 2}, 0, 0},
       {"spmm_ranges", &g_opt.spmm_ranges, false, {0, 1, 2, 3, 4, 8}, 0, 0},
-      {"merge_items", &g_opt.merge_items, false, {1024, 2048, 4096}, 0, 0},
+      {"merge_items", &g_opt.merge_items, false, {1024, 2048, 4096}, 0, 0, &g_opt.merge_items_set, 2048},
       {"merge_threads", &g_opt.merge_threads, false, {64, 128, 256}, 0, 0},
       {"merge_carve", &g_opt.merge_carve, false, {-1, 0, 25, 45, 60, 75, 100}, 0, 0},
       {"merge_short", &g_opt.merge_short, false, {8, 16, 32, 64}, 0, 0},
@@ -629,9 +630,10 @@ static int option_access(const char* name, int* get, const int* set) {
     if (strcmp(name, e.name)) continue;
     if (get) { *get = *e.slot; return B200SP_OK; }
     const int value = *set;
+    if (e.set_by_caller && value == 0) { *e.slot = e.by_rule; *e.set_by_caller = false; return B200SP_OK; }
     if (e.boolean) { *e.slot = value ? 1 : 0; return B200SP_OK; }
     if (e.values.size()) {
-      for (int v : e.values) if (v == value) { *e.slot = value; return B200SP_OK; }
+      for (int v : e.values) if (v == value) { *e.slot = value; if (e.set_by_caller) *e.set_by_caller = true; return B200SP_OK; }
       return B200SP_ERR_INVALID_ARG;
     }
     if (value < e.lo || value > e.hi) return B200SP_ERR_INVALID_ARG;

@@ -175,7 +175,7 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
   I.m = m; I.n = n; I.nnz = nnz;
   // SpMV tiles of 1024 items instead of 2048 below 12 M: more CTAs (R-MAT 2^17 10.4 / 11.5 us, 2^18 15.9 / 16.5 us, 2^19 23.7 / 25.4 us,
   // 2^20 40.6 / 42.2 us; equal from 2^21 on)
-  const int items = g_opt.merge_items == 2048 && m + nnz < 12000000 ? 1024 : g_opt.merge_items;
+  const int items = !g_opt.merge_items_set && m + nnz < 12000000 ? 1024 : g_opt.merge_items;
   I.spmv_tile_items = items;
   I.spmv_tiles = (int32_t)((m + nnz + items - 1) / items);
   I.spmv_kernel = g_opt.spmv_kernel >= 0 ? g_opt.spmv_kernel : 0;

@@ -54,6 +54,7 @@ struct Options {
   int uni_unroll = 0;     // groups of four nonzeros in flight per thread of the uniform-row kernel (1, 2 or 4); 0 = 1 (32 registers, full occupancy)
   int uni_ctas = 0;       // CTAs per SM for the uniform-row kernel (0 = as many as fit)
   int merge_items = 2048; // merge items per tile (1024, 2048 or 4096)
+  bool merge_items_set = false;   // set by the caller; else 1024 below 12 M items (see plan_build)
   int merge_threads = 128; // threads per CTA of the one-tile-per-CTA merge kernel (128 or 256)
   int bstage_threads = 1024; // threads per CTA of that kernel (256, 512 or 1024)
   int bstage_nnz = 0;        // nonzeros per CTA it aims for; 0 = chosen so that the grid fills whole rounds of one CTA per SM (the kernel on the caller's CSR arrays: 131072)

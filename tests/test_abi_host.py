@@ -88,7 +88,8 @@ def test_switches_read_back_and_environment_at_load():
     try:
         assert b200sp.b200sp_get_option("merge_items") == 4096
     finally:
-        b200sp.b200sp_set_option("merge_items", 2048)
+        b200sp.b200sp_set_option("merge_items", 0)       # by the library's rule again
+    assert b200sp.b200sp_get_option("merge_items") == 2048
     with pytest.raises(b200sp.B200spError):
         b200sp.b200sp_get_option("no_such_option")
     code = ("import sys; sys.path.insert(0, %r); import paper_2603_07169_b200 as b; "

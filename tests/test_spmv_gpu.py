@@ -157,6 +157,9 @@ def test_merge_kernel_tile_sizes(items, empty, dtype):
         for name, lens in (("power_law", (rng.pareto(1.1, 40000) * 2).astype(np.int64).clip(0, 60000)),
                            ("every_length", np.arange(300)), ("empty_run", np.concatenate([np.zeros(20000, np.int64), [5000, 1, 0, 7]]))):
             A = gen.random_csr(len(lens), 3001, lens, seed=7)
+            plan = b200sp.b200sp_plan_create(A.m, A.n, A.nnz, to_dev(A.row_ptr))
+            assert b200sp.b200sp_plan_info(plan)["spmv_tile_items"] == items
+            b200sp.b200sp_plan_destroy(plan)
             x = rng.standard_normal(3001).astype(np.float32)
             y0 = rng.standard_normal(len(lens)).astype(np.float32)
             y, y_ref, S = run_spmv(A, x, None, 1.0, 0.0, dtype)
@@ -166,7 +169,7 @@ def test_merge_kernel_tile_sizes(items, empty, dtype):
             assert_within(y, y_ref, S, dtype, 2.0, np.abs(0.5 * y0f.astype(np.float64)), what="%s items=%d ab" % (name, items))
         b200sp.b200sp_check()
     finally:
-        for k, v in (("spmv_kernel", -1), ("merge_items", 2048), ("merge_empty", 0)):
+        for k, v in (("spmv_kernel", -1), ("merge_items", 0), ("merge_empty", 0)):
             b200sp.b200sp_set_option(k, v)
 
 

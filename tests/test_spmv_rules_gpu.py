@@ -32,6 +32,27 @@ def test_sub_warps_only_while_no_lane_has_a_long_chain(longest, kernel, dtype):
     check(A, dtype, "longest=%d" % longest)
 
 
+def test_tile_size_by_the_rule_and_as_set():
+    """1024 items below 12 million, 2048 from there on, unless the caller sets a size; 0 gives the choice back."""
+    def items(m, nnz):
+        row_ptr = torch.clamp(torch.arange(m + 1, device="cuda") * 8, max=nnz).int()
+        plan = b200sp.b200sp_plan_create(m, 1000, nnz, row_ptr)
+        found = b200sp.b200sp_plan_info(plan)["spmv_tile_items"]
+        b200sp.b200sp_plan_destroy(plan)
+        return found
+
+    below, above = (1_500_000, 10_499_999), (1_500_000, 10_500_000)
+    b200sp.b200sp_set_option("merge_items", 0)
+    try:
+        assert (items(*below), items(*above)) == (1024, 2048)
+        for size in (2048, 4096, 1024):
+            b200sp.b200sp_set_option("merge_items", size)
+            assert (items(*below), items(*above)) == (size, size)
+    finally:
+        b200sp.b200sp_set_option("merge_items", 0)
+    assert (items(*below), items(*above)) == (1024, 2048)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("tiles", [1, 2, 15, 16, 17, 32, 33, 40])
 def test_rows_cut_by_tile_boundaries(tiles, dtype):
