@@ -37,7 +37,7 @@ extern "C" {
  *                    rows + nonzeros and 2048 above (and the switch reads as 2048)
  *   "merge_threads"  threads per CTA: 64, 128 (default) or 256
  *   "merge_carve"    shared-memory carveout in percent requested for it: 0, 25, 45 (default), 60, 75, 100 or -1 = leave to the driver
- *   "merge_short"    rows of up to this many products are added by one thread: 8, 16, 32 (default) or 64
+ *   "merge_short"    rows of up to this many products are added by one thread: 8, 16, 32 (default) or 64; tiles of 1024 and 2048 items
  *   "merge_empty"    1 = when a quarter or more of the rows have no nonzeros the merge list holds only the other rows, and y
  *                    of the empty rows is written by a pass of its own, 0 = every row is a merge item (default: the list
  *                    measured 3 % slower on the power-law workload with 61 % empty rows)

@@ -259,20 +259,25 @@ int run_spmv_subwarp(b200sp_plan* p, const int32_t* col_idx, const T* vals, cons
   }
 }
 
-// The merge-tile kernel by tile size and by the length up to which one thread adds a row.
+// The merge-tile kernel by tile size and, for tiles of 1024 and 2048, by the length up to which one thread adds a row.
+template <typename T, int ITEMS>
+int run_spmv_merge_short(b200sp_plan* p, const int32_t* col_idx, const T* vals, const T* x, T* y, float alpha, float beta,
+                         cudaStream_t stream, DeviceInfo* dev) {
+  switch (g_opt.merge_short) {
+    case 8: return run_spmv_merge<T, ITEMS, 8>(p, col_idx, vals, x, y, alpha, beta, stream, dev);
+    case 16: return run_spmv_merge<T, ITEMS, 16>(p, col_idx, vals, x, y, alpha, beta, stream, dev);
+    case 64: return run_spmv_merge<T, ITEMS, 64>(p, col_idx, vals, x, y, alpha, beta, stream, dev);
+    default: return run_spmv_merge<T, ITEMS, 32>(p, col_idx, vals, x, y, alpha, beta, stream, dev);
+  }
+}
+
 template <typename T>
 int run_spmv_merge_any(b200sp_plan* p, const int32_t* col_idx, const T* vals, const T* x, T* y, float alpha, float beta,
                        cudaStream_t stream, DeviceInfo* dev) {
-  const int items = p->info.spmv_tile_items, sh = g_opt.merge_short;
-#define B200SP_MERGE_BY_SHORT(FN, ITEMS)                                                      \
-  if (sh == 8) return FN<T, ITEMS, 8>(p, col_idx, vals, x, y, alpha, beta, stream, dev);      \
-  if (sh == 16) return FN<T, ITEMS, 16>(p, col_idx, vals, x, y, alpha, beta, stream, dev);    \
-  if (sh == 64) return FN<T, ITEMS, 64>(p, col_idx, vals, x, y, alpha, beta, stream, dev);    \
-  return FN<T, ITEMS, 32>(p, col_idx, vals, x, y, alpha, beta, stream, dev)
+  const int items = p->info.spmv_tile_items;
   if (items == 4096) return run_spmv_merge<T, 4096>(p, col_idx, vals, x, y, alpha, beta, stream, dev);
-  if (items == 1024) return run_spmv_merge<T, 1024>(p, col_idx, vals, x, y, alpha, beta, stream, dev);
-  B200SP_MERGE_BY_SHORT(run_spmv_merge, 2048);
-#undef B200SP_MERGE_BY_SHORT
+  if (items == 1024) return run_spmv_merge_short<T, 1024>(p, col_idx, vals, x, y, alpha, beta, stream, dev);
+  return run_spmv_merge_short<T, 2048>(p, col_idx, vals, x, y, alpha, beta, stream, dev);
 }
 
 // The row-direct kernel gives its shared memory to stages and leaves little L1; that pays only when the gather of x is

@@ -4,10 +4,11 @@ is run here against the CPU oracle, element by element, on three small matrices 
 The kernel a switch belongs to is forced where the plan would not pick it, so that the switch is really exercised."""
 import numpy as np
 import pytest
+import torch
 
 import gen
 import paper_2603_07169_b200 as b200sp
-from gpu_util import assert_within, run_spmm, run_spmv
+from gpu_util import assert_within, run_spmm, run_spmv, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -82,6 +83,35 @@ def test_spmv_switch_value_against_oracle(switch, value, force, dtype):
             y0f = y0 if dtype == "f32" else gen.bf16_to_f32(gen.to_bf16(y0))
             assert_within(y, y_ref, S, dtype, 1.0, np.abs(0.5 * y0f.astype(np.float64)), what="%s=%d %s %s ab" % (switch, value, name, dtype))
         b200sp.b200sp_check()
+    finally:
+        reset_all()
+
+
+@pytest.mark.parametrize("items", [1024, 2048])
+def test_merge_short_reaches_the_kernel(items):
+    """A row of up to merge_short products is one chain of one thread, a longer one 32 chains and a tree: values that cancel show which it was."""
+    lens = np.repeat([8, 16, 32, 64, 65], 400)
+    A = gen.random_csr(len(lens), 200, lens, seed=5)
+    starts = np.asarray(A.row_ptr[:-1], np.int64)
+    A.vals[:] = np.random.default_rng(3).uniform(0.5, 1.0, A.nnz).astype(np.float32)
+    A.vals[starts], A.vals[starts + 1] = 2.0**25, -2.0**25       # apart in different chains: the products added to either lose their low bits
+    d = [to_dev(a) for a in (A.row_ptr, A.col_idx, A.vals, np.ones(A.n, np.float32))]
+    try:
+        b200sp.b200sp_set_option("spmv_kernel", 0)
+        b200sp.b200sp_set_option("merge_items", items)
+        for short in (8, 16, 32, 64):
+            b200sp.b200sp_set_option("merge_short", short)
+            y = torch.empty(A.m, device="cuda")
+            b200sp.spmv_csr(A.m, A.n, A.nnz, d[0], d[1], d[2], d[3], y, 1.0, 0.0, "f32")
+            y = y.cpu().numpy()
+            b200sp.b200sp_cache_clear()
+            for length in (8, 16, 32, 64, 65):
+                rows = np.flatnonzero(lens == length)
+                chain = np.zeros(len(rows), np.float32)
+                for j in range(length):
+                    chain = chain + A.vals[starts[rows] + j]
+                in_one_chain = (y[rows] == chain).mean()         # (rows cut by a tile boundary are not)
+                assert in_one_chain > 0.8 if length <= short else in_one_chain < 0.2, (short, length, in_one_chain)
     finally:
         reset_all()
 
