@@ -43,7 +43,8 @@ extern "C" {
  *                    measured 3 % slower on the power-law workload with 61 % empty rows)
  *  row-direct SpMV kernel
  *   "row_stages"     shared-memory stages per CTA, 2 (default) .. 4
- *   "row_ctas"       CTAs per SM the tiles are sized for, 1..4, default 3 (3 and 4 are raised to 5 at most where short rows leave room)
+ *   "row_ctas"       CTAs per SM the tiles are sized for, 1..4; until it is set, and after it is set to 0, 3, or up to 5 where
+ *                    short rows leave room (and the switch reads as 3)
  *   "row_smem_kb"    shared memory per SM it may use for stages: 48, 96, 160, 220 (default) or 227 (what is left stays L1)
  *   "row_threads"    threads per CTA, 128 or 256 (default)
  *   "row_unroll"     gathers in flight per thread, 8 (default) or 16

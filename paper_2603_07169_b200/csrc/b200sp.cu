@@ -607,7 +607,7 @@ static int option_access(const char* name, int* get, const int* set) {
       {"merge_short", &g_opt.merge_short, false, {8, 16, 32, 64}, 0, 0},
       {"merge_empty", &g_opt.merge_empty, true, {}, 0, 0},
       {"row_stages", &g_opt.row_stages, false, {2, 3, 4}, 0, 0},
-      {"row_ctas", &g_opt.row_ctas, false, {1, 2, 3, 4}, 0, 0},
+      {"row_ctas", &g_opt.row_ctas, false, {1, 2, 3, 4}, 0, 0, &g_opt.row_ctas_set, 3},
       {"row_smem_kb", &g_opt.row_smem_kb, false, {48, 96, 160, 220, 227}, 0, 0},
       {"row_threads", &g_opt.row_threads, false, {128, 256}, 0, 0},
       {"row_unroll", &g_opt.row_unroll, false, {8, 16}, 0, 0},

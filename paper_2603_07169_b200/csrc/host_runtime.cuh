@@ -48,6 +48,7 @@ struct Options {
   int x_l2_window = 0;   // measured: no gain on the large workloads (x stays in L2 anyway), +1.4 us per launch on tiny ones
   int row_stages = 2;   // shared-memory stages per CTA of the row-direct kernel (2..4)
   int row_ctas = 3;     // CTAs per SM the row-direct kernel is sized for (1..4)
+  bool row_ctas_set = false;   // set by the caller; else up to 5 where rows are short (see row_ctas_for)
   int row_unroll = 8;   // gathers in flight per thread (8 or 16)
   int row_smem_kb = 220;  // shared memory per SM the row-direct kernel may use for its stages (the rest stays L1)
   int row_threads = 256;  // threads per CTA of the row-direct kernel (128 or 256)

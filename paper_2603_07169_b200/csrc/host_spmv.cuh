@@ -20,13 +20,14 @@ int run_scale(long long count, T* y, float beta, cudaStream_t stream, DeviceInfo
 
 int gcd_int(int a, int b) { while (b) { const int t = a % b; a = b; b = t; } return a; }
 
-// CTAs per SM that the row-direct kernel's tiles are sized for: the switch, raised to at most 5 (what the registers allow) where rows are so short
-// that tiles of a row per thread leave shared memory unused: 5-point Laplacian 1000^2 FP32 13.5 us with 5, 17.2 us with 3.
+// CTAs per SM that the row-direct kernel's tiles are sized for: the switch where it is set, else 3, raised to at most 5 (what the registers allow)
+// where rows are so short that tiles of a row per thread leave shared memory unused: 5-point Laplacian 1000^2 FP32 13.5 us with 5, 17.2 us with 3.
 template <typename T>
 int row_ctas_for(int threads, int max_len, int stages, int sm_budget) {
   int ctas = g_opt.row_ctas;
+  if (g_opt.row_ctas_set) return ctas;
   const int full = stages * row_tile_stage_bytes<T>(threads, (threads * max_len + 16 + 7) & ~7) + 1024 + 256 + 128;
-  while (ctas >= 3 && ctas < 5 && (ctas + 1) * full <= sm_budget) ++ctas;
+  while (ctas < 5 && (ctas + 1) * full <= sm_budget) ++ctas;
   return ctas;
 }
 

@@ -49,7 +49,7 @@ def spmv_matrices():
     }
 
 
-BY_RULE = ("merge_items",)      # 0: chosen by the library again (the switch then reads as its default)
+BY_RULE = ("merge_items", "row_ctas")      # 0: chosen by the library again (the switch then reads as its default)
 
 
 def reset_all():
@@ -85,6 +85,47 @@ def test_spmv_switch_value_against_oracle(switch, value, force, dtype):
         b200sp.b200sp_check()
     finally:
         reset_all()
+
+
+def captured_grids(call):
+    """Grid sizes of the kernels that `call` launches, from a graph that is never run."""
+    from cuda.bindings import driver
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    err, nodes, count = driver.cuGraphGetNodes(raw)
+    err, nodes, count = driver.cuGraphGetNodes(raw, count)
+    assert int(err) == 0
+    kernels = [n for n in nodes[:count] if driver.cuGraphNodeGetType(n)[1] == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL]
+    return [driver.cuGraphKernelNodeGetParams(n)[1].gridDimX for n in kernels]
+
+
+@pytest.mark.parametrize("ell", [False, True])
+def test_row_ctas_as_set_and_by_the_rule(ell):
+    """Rows of five FP32 entries leave room for five CTAs of 256 rows per SM: these by the rule, what the caller sets otherwise."""
+    m = 300_000
+    A = gen.uniform_rows(m, m, 5, 3)
+    d = [to_dev(a) for a in (A.row_ptr, A.col_idx, A.vals, np.ones(m, np.float32))]
+    y = torch.empty(m, device="cuda")
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+
+    def call():
+        if ell:
+            b200sp.spmv_ell(m, m, 5, d[1], d[2], d[3], y, 1.0, 0.0, "f32")
+        else:
+            b200sp.spmv_csr(m, m, A.nnz, d[0], d[1], d[2], d[3], y, 1.0, 0.0, "f32")
+
+    try:
+        b200sp.b200sp_set_option("spmv_kernel", 1)
+        for value in (0, 1, 2, 3, 4, 0):
+            b200sp.b200sp_set_option("row_ctas", value)
+            call()
+            torch.cuda.synchronize()
+            assert captured_grids(call) == [(value or 5) * sms]
+    finally:
+        reset_all()
+        b200sp.b200sp_cache_clear()
 
 
 @pytest.mark.parametrize("items", [1024, 2048])
