@@ -315,7 +315,7 @@ static int csc_call(bool is_mm, int64_t m, int64_t n, int64_t nnz, int64_t k, co
 
 // ---- ELL front end ----
 static int check_ell(int64_t m, int64_t n, int64_t width, const void* col_ids, const void* vals, const void* in, const void* out, int dtype) {
-  if (m < 0 || n < 0 || width < 0 || n >= ((int64_t)1 << 31) || m >= ((int64_t)1 << 31) - 1) return B200SP_ERR_INVALID_ARG;
+  if (m < 0 || n < 0 || width < 0 || n >= ((int64_t)1 << 31) || m >= ((int64_t)1 << 31) - 1 || width >= ((int64_t)1 << 31)) return B200SP_ERR_INVALID_ARG;
   if (m * width >= ((int64_t)1 << 31)) return B200SP_ERR_INVALID_ARG;
   if (dtype != B200SP_F32 && dtype != B200SP_BF16) return B200SP_ERR_INVALID_ARG;
   if (m > 0 && !out) return B200SP_ERR_INVALID_ARG;

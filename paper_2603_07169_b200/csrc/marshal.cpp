@@ -51,6 +51,16 @@ struct Reader {
     ok = false;
     return 0;
   }
+  // The product of two sizes; one that 64 bits do not hold is left to Python, whose integers do.
+  int64_t times(int64_t a, int64_t b) {
+    int64_t v = 0;
+    if (__builtin_mul_overflow(a, b, &v)) ok = false;
+    return v;
+  }
+  int64_t plus1(int64_t a) {
+    if (a == INT64_MAX) ok = false;
+    return ok ? a + 1 : a;
+  }
   // Address of a device operand of at least `elems` elements of `esize` bytes; None stays NULL.
   void* operand(PyObject* o, int64_t elems, int64_t esize) {
     if (!ok || o == Py_None) return nullptr;
@@ -103,12 +113,12 @@ PyObject* product(PyObject*, PyObject* const* v, Py_ssize_t argc) {
     const int dtype = r.dtype(v[13]);
     if (!r.ok || k < 0) return -1;
     const int64_t e = dtype == B200SP_F32 ? 4 : 2, kk = k > 1 ? k : 1;
-    const int64_t na = layout == 0 ? (m > 0 ? m + 1 : 0) : layout == 1 ? nnz : n + 1;
+    const int64_t na = layout == 0 ? (m > 0 ? r.plus1(m) : 0) : layout == 1 ? nnz : r.plus1(n);
     const int32_t* a = (const int32_t*)r.operand(v[6], na, 4);
     const int32_t* b = (const int32_t*)r.operand(v[7], nnz, 4);
     void* const vals = r.operand(v[8], nnz, e);
-    void* const in = r.operand(v[9], nnz > 0 ? n * kk : 0, e);
-    void* const out = r.operand(v[10], atleast0(m) * kk, e);
+    void* const in = r.operand(v[9], nnz > 0 ? r.times(n, kk) : 0, e);
+    void* const out = r.operand(v[10], r.times(atleast0(m), kk), e);
     void* const stream = r.stream(v[14]);
     if (!r.ok) return -1;
     int status;
@@ -130,11 +140,11 @@ PyObject* ell_product(PyObject*, PyObject* const* v, Py_ssize_t argc) {
     const float alpha = r.scalar(v[9]), beta = r.scalar(v[10]);
     const int dtype = r.dtype(v[11]);
     if (!r.ok || k < 0) return -1;
-    const int64_t e = dtype == B200SP_F32 ? 4 : 2, kk = k > 1 ? k : 1, slots = m * width;
+    const int64_t e = dtype == B200SP_F32 ? 4 : 2, kk = k > 1 ? k : 1, slots = r.times(m, width);
     const int32_t* cols = (const int32_t*)r.operand(v[5], slots, 4);
     void* const vals = r.operand(v[6], slots, e);
-    void* const in = r.operand(v[7], slots > 0 ? n * kk : 0, e);
-    void* const out = r.operand(v[8], m * kk, e);
+    void* const in = r.operand(v[7], slots > 0 ? r.times(n, kk) : 0, e);
+    void* const out = r.operand(v[8], r.times(m, kk), e);
     void* const stream = r.stream(v[12]);
     if (!r.ok) return -1;
     int status;
@@ -164,8 +174,8 @@ PyObject* plan_product(PyObject*, PyObject* const* v, Py_ssize_t argc) {
     const int64_t e = dtype == B200SP_F32 ? 4 : 2, kk = k > 1 ? k : 1;
     const int32_t* col = (const int32_t*)r.operand(v[4], I.nnz, 4);
     void* const vals = r.operand(v[5], I.nnz, e);
-    void* const in = r.operand(v[6], I.nnz > 0 ? I.n * kk : 0, e);
-    void* const out = r.operand(v[7], I.m * kk, e);
+    void* const in = r.operand(v[6], I.nnz > 0 ? r.times(I.n, kk) : 0, e);
+    void* const out = r.operand(v[7], r.times(I.m, kk), e);
     void* const stream = r.stream(v[11]);
     if (!r.ok) return -1;
     int status;
@@ -185,7 +195,7 @@ PyObject* plan_create(PyObject*, PyObject* const* v, Py_ssize_t argc) {
       Reader r;
       void* const fn = r.address(v[0]);
       const int64_t m = r.size(v[1]), n = r.size(v[2]), nnz = r.size(v[3]);
-      const int32_t* row_ptr = (const int32_t*)r.operand(v[4], m > 0 ? m + 1 : 0, 4);
+      const int32_t* row_ptr = (const int32_t*)r.operand(v[4], m > 0 ? r.plus1(m) : 0, 4);
       void* const stream = r.stream(v[5]);
       if (r.ok) {
         b200sp_plan* plan = nullptr;

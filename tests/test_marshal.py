@@ -31,6 +31,21 @@ def test_unusual_arguments_are_left_to_python():
     assert native()(1, 2, 3) == -1
 
 
+def test_sizes_whose_products_64_bits_do_not_hold():
+    """A wrapped product would let a short operand pass.  Left to Python, which counts exactly; the library refuses such sizes as well."""
+    mm = binding._address if native() else None
+    for m, n, nnz, k in ((4, 4, 4, 1 << 62), (4, 1 << 32, 4, 1 << 32), (1 << 32, 4, 4, 1 << 32), ((1 << 63) - 1, 4, 4, 1)):
+        assert native()(mm["spmm_csr"], 0, m, n, nnz, k, None, None, None, None, None, 1.0, 0.0, "f32", 1) == -1
+    assert native()(mm["spmv_csc"], 2, 4, (1 << 63) - 1, 4, 0, None, None, None, None, None, 1.0, 0.0, "f32", 1) == -1
+    for m, n, width, k in ((1 << 30, 4, 1 << 34, 0), (1 << 30, 4, 1 << 34, 2), (4, 1 << 40, 4, 1 << 40)):
+        assert binding._ell_product(mm["spmm_ell" if k else "spmv_ell"], m, n, width, k, None, None, None, None, 1.0, 0.0, "f32", 1) == -1
+    assert binding._plan_create(mm["b200sp_plan_create"], (1 << 63) - 1, 4, 4, None, 1) == -1
+    L, y = b200sp.lib(), np.zeros(16, np.float32)
+    for width in (1 << 34, 1 << 62):                                  # m * width = 0 modulo 2^64
+        assert L.spmv_ell(1 << 30, 4, width, None, None, None, y.ctypes.data, 1.0, 0.0, 0, None) == 1
+        assert L.spmm_ell(1 << 30, 4, width, 2, None, None, None, y.ctypes.data, 1.0, 0.0, 0, None) == 1
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_every_entry_point_through_it(dtype):
