@@ -11,6 +11,9 @@
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <new>
+#include <stdexcept>
+
 #include "../../include/b200sp.h"
 
 namespace {
@@ -99,6 +102,23 @@ PyObject* guarded(Body body) {
   return PyLong_FromLong(status);
 }
 
+// A call of the library without the interpreter lock.  An exception that leaves it (out of host memory) becomes a status, and the lock is
+// held again whichever way the call ends.
+template <typename Call>
+int unlocked(Call call) {
+  struct Released {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Released() { PyEval_RestoreThread(state); }
+  } released;
+  try {
+    return call();
+  } catch (const std::bad_alloc&) {
+    return B200SP_ERR_ALLOC;
+  } catch (const std::exception&) {
+    return B200SP_ERR_CUDA;
+  }
+}
+
 int64_t atleast0(int64_t v) { return v > 0 ? v : 0; }
 
 // (fn, layout, m, n, nnz, k, a, b, vals, in, out, alpha, beta, dtype, stream); k == 0: SpMV.  layout 0: CSR (a = row_ptr, b = col_idx),
@@ -121,12 +141,10 @@ PyObject* product(PyObject*, PyObject* const* v, Py_ssize_t argc) {
     void* const out = r.operand(v[10], r.times(atleast0(m), kk), e);
     void* const stream = r.stream(v[14]);
     if (!r.ok) return -1;
-    int status;
-    Py_BEGIN_ALLOW_THREADS
-    status = k == 0 ? ((decltype(&spmv_csr))fn)(m, n, nnz, a, b, vals, in, out, alpha, beta, dtype, stream)
+    return unlocked([&]() -> int {
+      return k == 0 ? ((decltype(&spmv_csr))fn)(m, n, nnz, a, b, vals, in, out, alpha, beta, dtype, stream)
                     : ((decltype(&spmm_csr))fn)(m, n, nnz, k, a, b, vals, in, out, alpha, beta, dtype, stream);
-    Py_END_ALLOW_THREADS
-    return status;
+    });
   });
 }
 
@@ -147,12 +165,10 @@ PyObject* ell_product(PyObject*, PyObject* const* v, Py_ssize_t argc) {
     void* const out = r.operand(v[8], r.times(m, kk), e);
     void* const stream = r.stream(v[12]);
     if (!r.ok) return -1;
-    int status;
-    Py_BEGIN_ALLOW_THREADS
-    status = k == 0 ? ((decltype(&spmv_ell))fn)(m, n, width, cols, vals, in, out, alpha, beta, dtype, stream)
+    return unlocked([&]() -> int {
+      return k == 0 ? ((decltype(&spmv_ell))fn)(m, n, width, cols, vals, in, out, alpha, beta, dtype, stream)
                     : ((decltype(&spmm_ell))fn)(m, n, width, k, cols, vals, in, out, alpha, beta, dtype, stream);
-    Py_END_ALLOW_THREADS
-    return status;
+    });
   });
 }
 
@@ -178,12 +194,10 @@ PyObject* plan_product(PyObject*, PyObject* const* v, Py_ssize_t argc) {
     void* const out = r.operand(v[7], r.times(I.m, kk), e);
     void* const stream = r.stream(v[11]);
     if (!r.ok) return -1;
-    int status;
-    Py_BEGIN_ALLOW_THREADS
-    status = k == 0 ? ((decltype(&b200sp_spmv))fn)(plan, col, vals, in, out, alpha, beta, dtype, stream)
+    return unlocked([&]() -> int {
+      return k == 0 ? ((decltype(&b200sp_spmv))fn)(plan, col, vals, in, out, alpha, beta, dtype, stream)
                     : ((decltype(&b200sp_spmm))fn)(plan, k, col, vals, in, out, alpha, beta, dtype, stream);
-    Py_END_ALLOW_THREADS
-    return status;
+    });
   });
 }
 
@@ -199,10 +213,7 @@ PyObject* plan_create(PyObject*, PyObject* const* v, Py_ssize_t argc) {
       void* const stream = r.stream(v[5]);
       if (r.ok) {
         b200sp_plan* plan = nullptr;
-        int status;
-        Py_BEGIN_ALLOW_THREADS
-        status = ((decltype(&b200sp_plan_create))fn)(&plan, m, n, nnz, row_ptr, stream);
-        Py_END_ALLOW_THREADS
+        const int status = unlocked([&]() -> int { return ((decltype(&b200sp_plan_create))fn)(&plan, m, n, nnz, row_ptr, stream); });
         result = status == B200SP_OK ? (long long)(intptr_t)plan : -2 - status;
       }
     }

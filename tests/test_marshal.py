@@ -1,5 +1,8 @@
 """The native marshalling of the binding (csrc/marshal.cpp): what it does not take as it stands comes back as -1 and is refused, or handled,
 by the Python path, exactly as before; what it takes reaches the library."""
+import ctypes
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -44,6 +47,24 @@ def test_sizes_whose_products_64_bits_do_not_hold():
     for width in (1 << 34, 1 << 62):                                  # m * width = 0 modulo 2^64
         assert L.spmv_ell(1 << 30, 4, width, None, None, None, y.ctypes.data, 1.0, 0.0, 0, None) == 1
         assert L.spmm_ell(1 << 30, 4, width, 2, None, None, None, y.ctypes.data, 1.0, 0.0, 0, None) == 1
+
+
+def test_an_exception_out_of_the_call_becomes_a_status(tmp_path):
+    """In place of the library: functions that run out of host memory.  The interpreter lock is held again afterwards."""
+    (tmp_path / "throws.cpp").write_text("#include <new>\nextern \"C\" int f() { throw std::bad_alloc(); }\n"
+                                         "extern \"C\" int info(const void*, void* out) { for (int i = 0; i < 144; ++i) ((char*)out)[i] = 0; return 0; }\n")
+    lib = str(tmp_path / "throws.so")
+    subprocess.check_call(["g++", "-shared", "-fPIC", "-o", lib, str(tmp_path / "throws.cpp")])
+    L = ctypes.CDLL(lib)
+    f, info = (ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in ("f", "info"))
+    nothing = [None] * 5
+    native()
+    for _ in range(3):
+        assert binding._product(f, 0, 0, 0, 0, 0, *nothing, 1.0, 0.0, "f32", 1) == 4      # B200SP_ERR_ALLOC
+        assert binding._ell_product(f, 0, 0, 0, 0, *nothing[1:], 1.0, 0.0, "f32", 1) == 4
+        assert binding._plan_product(info, f, 16, 0, *nothing[1:], 1.0, 0.0, "f32", 1) == 4
+        assert binding._plan_create(f, 0, 0, 0, None, 1) == -2 - 4
+        assert sum(range(1000)) == 499500
 
 
 @pytest.mark.gpu
