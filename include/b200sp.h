@@ -151,9 +151,11 @@ int b200sp_spmm(b200sp_plan* plan, int64_t k, const int32_t* col_idx, const void
  * up from there (up to 2^26 nonzeros in rows of at most 1024); its places, 6 bytes per nonzero, are built on the first spmv_csc
  * call.  Otherwise, and for spmm_csc, the row-major order of the entries (a sort of every row's entries by their CSC position)
  * and a scratch array of nnz values are built on the first call that needs them, and every call permutes vals into that order with one
- * kernel and runs the CSR kernels.  Either way a row's entries are added in ascending column order on every run.  The calls that
- * build something synchronise the stream, others do not.  Inconsistent col_ptr / row_idx return B200SP_ERR_BAD_CSR.  Calls that share a
- * cached pattern must not overlap on the GPU.
+ * kernel and runs the CSR kernels.  Either way a row's entries are added in ascending column order on every run.  The first call of a pattern
+ * and the first spmv_csc synchronise the stream; what a call builds is complete in the order of its stream, not when it returns.  The first
+ * call of a pattern is refused on a capturing stream (B200SP_ERR_UNSUPPORTED; the capture stays valid); later ones are not: what they
+ * lack is built inside the graph for that call, and spmv_csc then takes the CSR kernels.  Inconsistent col_ptr / row_idx return
+ * B200SP_ERR_BAD_CSR.  Calls that share a cached pattern must not overlap on the GPU.
  *
  * ELL: row-major, row i occupies entries [i*width, (i+1)*width) of col_ids and vals; an entry is padding
  * when its col_id is negative (its value is ignored, whatever it holds).  m * width < 2^31.  No plan, no

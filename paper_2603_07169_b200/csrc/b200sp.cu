@@ -506,7 +506,7 @@ int b200sp_cache_drop(const void* key_ptr) {
     }
     for (auto it = g_csc_cache.begin(); it != g_csc_cache.end();) {
       if (std::get<0>(it->first) == dev && std::get<1>(it->first) == key_ptr) {
-        for (void* q : {it->second.block, it->second.csr_block, it->second.prod_block}) blocks.push_back(q);
+        for (void* q : {it->second.block, it->second.csr.block, it->second.prod_block}) blocks.push_back(q);
         row_ptrs.push_back(it->second.row_ptr);
         it = g_csc_cache.erase(it);
       } else ++it;

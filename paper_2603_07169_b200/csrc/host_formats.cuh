@@ -54,10 +54,7 @@ struct CscEntry {
   void* block = nullptr;
   int32_t* row_ptr = nullptr;
   int32_t* fill = nullptr;            // m + 2 counters, for building the parts below
-  void* csr_block = nullptr;
-  int32_t* perm = nullptr;
-  int32_t* col = nullptr;
-  void* vals_t = nullptr;
+  struct Csr { void* block = nullptr; int32_t* perm = nullptr; int32_t* col = nullptr; void* vals_t = nullptr; } csr;
   void* prod_block = nullptr;
   bool prod_tried = false;
   int bucket_rows = 0;                // most rows of a bucket, once counted
@@ -70,7 +67,7 @@ static std::map<std::tuple<int, const void*, const void*, int64_t, int64_t, int6
 static std::mutex g_csc_build;      // one thread at a time adds parts to an entry
 
 static void csc_free(CscEntry& e) {
-  for (void* b : {e.block, e.csr_block, e.prod_block}) if (b) cudaFree(b);
+  for (void* b : {e.block, e.csr.block, e.prod_block}) if (b) cudaFree(b);
   e = CscEntry();
 }
 
@@ -86,6 +83,7 @@ static int csc_plan(CscEntry** out, int64_t m, int64_t n, int64_t nnz, const int
     auto it = g_csc_cache.find(key);
     if (it != g_csc_cache.end()) { *out = &it->second; return B200SP_OK; }
   }
+  if (stream_captures(stream)) return B200SP_ERR_UNSUPPORTED;    // the check of the pattern is read back
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
   const size_t blocks = (size_t)((m + 1 + kScanBlock - 1) / kScanBlock);
   const size_t o_rp = 0, o_fill = o_rp + up(((size_t)m + 2) * 4), o_bs = o_fill + up(((size_t)m + 2) * 4), o_bad = o_bs + up((blocks + 1) * 4), total = o_bad + 256;
@@ -127,11 +125,12 @@ static int csc_plan(CscEntry** out, int64_t m, int64_t n, int64_t nnz, const int
   return B200SP_OK;
 }
 
-// CSC positions and columns in row-major order and room for the permuted values: what the CSR kernels need.
-static int csc_csr_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr, const int32_t* row_idx, cudaStream_t stream,
-                        DeviceInfo* dev) {
+// CSC positions and columns in row-major order and room for the permuted values: what the CSR kernels need.  Built for the one call when the
+// stream is captured.
+static int csc_csr_part(CscEntry* e, CscEntry::Csr* out, CallBlock* own, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr,
+                        const int32_t* row_idx, cudaStream_t stream, DeviceInfo* dev) {
   std::lock_guard<std::mutex> lock(g_csc_build);
-  if (e->csr_block) return B200SP_OK;
+  if (e->csr.block) { *out = e->csr; return B200SP_OK; }
   const size_t bytes = ((size_t)(nnz > 0 ? nnz : 1) * 4 + 255) & ~(size_t)255;
   char* blk = nullptr;
   const int rc = pool_alloc(dev, (void**)&blk, 3 * bytes, stream);
@@ -151,10 +150,9 @@ static int csc_csr_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, const in
     }
     if (err != cudaSuccess) { cudaFreeAsync(blk, stream); return cuda_fail(err, "CSC row-major order"); }
   }
-  e->perm = perm;
-  e->col = col;
-  e->vals_t = blk + 2 * bytes;
-  e->csr_block = blk;
+  *out = {blk, perm, col, blk + 2 * bytes};
+  if (stream_captures(stream)) own->take(blk, stream);
+  else e->csr = *out;
   return B200SP_OK;
 }
 
@@ -169,7 +167,8 @@ static int64_t csc_most_bucket_rows(int64_t nnz, float beta) {
 }
 
 
-// The places of the products of csc_kernels.cuh; leaves e->prod_block null where they do not apply.  Synchronises the stream once.
+// The places of the products of csc_kernels.cuh; leaves e->prod_block null where they do not apply, and while the stream is captured
+// (their limits are read back).  Synchronises the stream.
 // Sizes: below 4.8 M nonzeros tiles and buckets of 2048 or 4096, so that every SM gets several; else one tile of 24576 .. 32768 entries
 // per SM and round (96 .. 128 KB of products), the size that leaves the least of the last round idle, and buckets of 8192 nonzeros,
 // 16384 above 2^25.  A run (a tile's products for one bucket) then averages tile * C / nnz = 3.5 .. 55 words: 2^24 nonzeros take 78 us,
@@ -179,7 +178,7 @@ static int64_t csc_most_bucket_rows(int64_t nnz, float beta) {
 static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr, const int32_t* row_idx, int64_t most_rows,
                             cudaStream_t stream, DeviceInfo* dev) {
   std::lock_guard<std::mutex> lock(g_csc_build);
-  if (e->prod_tried || e->bucket_rows > most_rows) return B200SP_OK;
+  if (e->prod_tried || e->bucket_rows > most_rows || stream_captures(stream)) return B200SP_OK;
   if (nnz <= 0 || nnz > ((int64_t)1 << 26)) { e->prod_tried = true; return B200SP_OK; }
   const int64_t sms = dev->sms;
   int tile = nnz < sms * 4 * 2048 ? 2048 : 4096;
@@ -234,6 +233,9 @@ static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, cons
   g_launches += 4;
   CUP(cudaGetLastError());
 #undef CUP
+  b200sp_plan* plan = nullptr;       // of the row offsets: made now, because the first call of the CSR kernels may be a captured one
+  rc = get_cached_plan(&plan, m, n, nnz, e->row_ptr, stream);
+  if (rc != B200SP_OK) return fail(rc);
   e->tile = tile; e->tiles = tiles; e->buckets = buckets; e->cap = cap;
   e->bucket_row = brow; e->bucket_start = (int*)(blk + o_bstart); e->tile_col = tcol; e->run_shift = (int*)(blk + o_shift);
   e->src = (unsigned short*)(blk + o_src); e->dst = (unsigned short*)(blk + o_dst); e->dcol = (unsigned short*)(blk + o_dcol);
@@ -294,13 +296,14 @@ static int csc_call(bool is_mm, int64_t m, int64_t n, int64_t nnz, int64_t k, co
     const int64_t most_rows = csc_most_bucket_rows(nnz, beta);
     rc = csc_product_part(entry, m, n, nnz, col_ptr, row_idx, most_rows, stream, dev);
     if (rc != B200SP_OK) return rc;
-    if (entry->prod_block && entry->bucket_rows <= most_rows)
+    if (entry->prod_block && (entry->bucket_rows <= most_rows || (!entry->csr.block && stream_captures(stream))))
       return dtype == B200SP_F32 ? run_csc_products<float>(entry, nnz, (const float*)vals, (const float*)in, (float*)out, alpha, beta, stream, dev)
                                  : run_csc_products<bf16_t>(entry, nnz, (const bf16_t*)vals, (const bf16_t*)in, (bf16_t*)out, alpha, beta, stream, dev);
   }
-  rc = csc_csr_part(entry, m, n, nnz, col_ptr, row_idx, stream, dev);
+  CscEntry::Csr e;
+  CallBlock own;
+  rc = csc_csr_part(entry, &e, &own, m, n, nnz, col_ptr, row_idx, stream, dev);
   if (rc != B200SP_OK) return rc;
-  const CscEntry& e = *entry;
   if (nnz > 0) {
     long long blocks = (nnz + 255) / 256;
     if (blocks > (long long)dev->sms * 16) blocks = (long long)dev->sms * 16;
@@ -309,8 +312,8 @@ static int csc_call(bool is_mm, int64_t m, int64_t n, int64_t nnz, int64_t k, co
              : launch(csc_permute_vals_kernel<bf16_t>, dim3((unsigned)blocks), dim3(256), stream, nullptr, 0, dev, (long long)nnz, (const int*)e.perm, (const bf16_t*)vals, (bf16_t*)e.vals_t);
     if (rc != B200SP_OK) return rc;
   }
-  return is_mm ? spmm_csr(m, n, nnz, k, e.row_ptr, e.col, e.vals_t, in, out, alpha, beta, dtype, stream_v)
-               : spmv_csr(m, n, nnz, e.row_ptr, e.col, e.vals_t, in, out, alpha, beta, dtype, stream_v);
+  return is_mm ? spmm_csr(m, n, nnz, k, entry->row_ptr, e.col, e.vals_t, in, out, alpha, beta, dtype, stream_v)
+               : spmv_csr(m, n, nnz, entry->row_ptr, e.col, e.vals_t, in, out, alpha, beta, dtype, stream_v);
 }
 
 // ---- ELL front end ----

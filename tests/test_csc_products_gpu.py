@@ -136,3 +136,51 @@ def test_dropping_a_csc_pattern_drops_the_plans_of_its_row_offsets():
         assert_within(to_host(y, "f32"), y_ref[:, 0], S[:, 0], "f32")
         b200sp.b200sp_cache_drop(ptr)
     b200sp.b200sp_cache_clear()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("first", ["spmv", "spmm"])
+def test_the_other_operation_captured(first, dtype):
+    """After one eager call, of SpMV or of SpMM, both can be captured.  What only the captured call needed goes with its graph."""
+    rng = np.random.default_rng(5)
+    m, n, k = 6000, 5000, 24
+    A = gen.random_csr(m, n, rng.integers(2, 30, m), seed=4, sort_cols=True)
+    cp, ri, va = gen.csr_to_csc(A)
+    v_s, x_s, B_s = (store(a, dtype) for a in (va, rng.standard_normal(n).astype(np.float32), rng.standard_normal(n * k).astype(np.float32)))
+    d = [to_dev(a) for a in (cp, ri, v_s, x_s, B_s)]
+    calls = {"spmv": lambda y: b200sp.spmv_csc(m, n, A.nnz, d[0], d[1], d[2], d[3], y, 1.0, 0.0, dtype),
+             "spmm": lambda y: b200sp.spmm_csc(m, n, A.nnz, k, d[0], d[1], d[2], d[4], y, 1.0, 0.0, dtype)}
+    refs = {"spmv": oracle.spmm_csc(m, n, 1, cp, ri, v_s, x_s, None, 1.0, 0.0, dtype), "spmm": oracle.spmm_csc(m, n, k, cp, ri, v_s, B_s, None, 1.0, 0.0, dtype)}
+    sizes = {"spmv": m, "spmm": m * k}
+
+    def check(y, op, what):
+        assert_within(to_host(y, dtype).reshape(refs[op][0].shape), *refs[op], dtype, what="%s %s" % (op, what))
+
+    outs = {op: [empty_out(sizes[op], dtype) for _ in range(4)] for op in calls}
+    for op, call in calls.items():                                # kernels loaded
+        call(outs[op][3])
+        check(outs[op][3], op, "eager")
+    b200sp.b200sp_cache_clear()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for op, call in calls.items():                            # nothing is known of the pattern
+            with pytest.raises(b200sp.B200spError) as e:
+                call(outs[op][0])
+            assert e.value.status == 2      # B200SP_ERR_UNSUPPORTED
+    calls[first](outs[first][3])
+    check(outs[first][3], first, "first")
+    for op in (first, "spmm" if first == "spmv" else "spmv"):
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            calls[op](outs[op][0])
+        calls[op](outs[op][1])                                    # before the graph has run
+        torch.cuda.synchronize()
+        check(outs[op][1], op, "outside the graph")
+        graph.replay()
+        torch.cuda.synchronize()
+        check(outs[op][0], op, "replayed")
+        del graph
+        calls[op](outs[op][2])
+        torch.cuda.synchronize()
+        assert torch.equal(outs[op][1], outs[op][2])
+    b200sp.b200sp_cache_clear()
