@@ -246,6 +246,16 @@ static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, cons
   return B200SP_OK;
 }
 
+// Gives back the memory of the places, in stream order (the calls of a pattern do not overlap); the next SpMV builds them again.
+static bool csc_drop_products(CscEntry* e, cudaStream_t stream) {
+  std::lock_guard<std::mutex> lock(g_csc_build);
+  if (!e->prod_block || stream_captures(stream)) return false;
+  if (cudaFreeAsync(e->prod_block, stream) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+  e->prod_block = nullptr;
+  e->prod_tried = false;
+  return true;
+}
+
 template <typename T, int TILE, int THREADS>
 static int launch_csc_products(const CscEntry* e, int64_t nnz, const T* vals, const T* x, cudaStream_t stream, DeviceInfo* dev) {
   auto kernel = csc_products_kernel<T, TILE, THREADS>;
@@ -295,7 +305,7 @@ static int csc_call(bool is_mm, int64_t m, int64_t n, int64_t nnz, int64_t k, co
   if (!is_mm && nnz > 0 && alpha != 0.0f && in && out && aligned16(vals) && aligned16(in) && aligned16(out)) {
     const int64_t most_rows = csc_most_bucket_rows(nnz, beta);
     rc = csc_product_part(entry, m, n, nnz, col_ptr, row_idx, most_rows, stream, dev);
-    if (rc != B200SP_OK) return rc;
+    if (rc != B200SP_OK && rc != B200SP_ERR_ALLOC) return rc;   // without memory for the places: the CSR kernels
     if (entry->prod_block && (entry->bucket_rows <= most_rows || (!entry->csr.block && stream_captures(stream))))
       return dtype == B200SP_F32 ? run_csc_products<float>(entry, nnz, (const float*)vals, (const float*)in, (float*)out, alpha, beta, stream, dev)
                                  : run_csc_products<bf16_t>(entry, nnz, (const bf16_t*)vals, (const bf16_t*)in, (bf16_t*)out, alpha, beta, stream, dev);
@@ -303,6 +313,7 @@ static int csc_call(bool is_mm, int64_t m, int64_t n, int64_t nnz, int64_t k, co
   CscEntry::Csr e;
   CallBlock own;
   rc = csc_csr_part(entry, &e, &own, m, n, nnz, col_ptr, row_idx, stream, dev);
+  if (rc == B200SP_ERR_ALLOC && csc_drop_products(entry, stream)) rc = csc_csr_part(entry, &e, &own, m, n, nnz, col_ptr, row_idx, stream, dev);
   if (rc != B200SP_OK) return rc;
   if (nnz > 0) {
     long long blocks = (nnz + 255) / 256;

@@ -507,7 +507,7 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
   }
   if (spmm_by_shares(I, k, (int)sizeof(T), beta)) {
     const int rc = run_spmm_merge<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
-    if (rc != B200SP_ERR_UNSUPPORTED) return rc;
+    if (rc != B200SP_ERR_UNSUPPORTED && rc != B200SP_ERR_ALLOC) return rc;   // without its scratch (nothing is launched then) by rows, which need none
   }
   if (k % VEC == 0 && g_opt.spmm_sliced) {
     // lanes per row: eight (a 128-byte slice) unless k is narrower than that

@@ -122,6 +122,63 @@ def test_injected_allocation_failure_in_the_plan_pass_and_the_host_entry_points(
     b200sp.b200sp_cache_clear()
 
 
+def failing(nth, fn):
+    b200sp.b200sp_set_option("fail_alloc_after", nth)
+    try:
+        fn()
+        assert b200sp.b200sp_get_option("fail_alloc_after") == 0, "the call made fewer than %d allocations" % nth
+    finally:
+        b200sp.b200sp_set_option("fail_alloc_after", 0)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_spmm_by_shares_without_its_scratch_goes_by_rows(dtype):
+    """Columns that are no multiple of 16 bytes on even rows took no memory before they went by shares; uneven rows go by rows as well then."""
+    rng = np.random.default_rng(2)
+    for lens, k in ((np.full(4000, 11), 50), (np.full(4000, 11), 17), (rng.integers(0, 4, 4000) * rng.integers(0, 100, 4000), 40)):
+        A = gen.random_csr(len(lens), 9000, lens, seed=k, sort_cols=True)
+        B, vals = store(rng.standard_normal(A.n * k).astype(np.float32), dtype), store(A.vals, dtype)
+        d = [to_dev(a) for a in (A.row_ptr, A.col_idx, vals, B)]
+        plan = b200sp.b200sp_plan_create(A.m, A.n, A.nnz, d[0])
+        assert b200sp.b200sp_spmm_by_shares(b200sp.b200sp_plan_info(plan), k, 0.0, dtype)
+        Y = empty_out(A.m * k, dtype)
+        failing(1, lambda: b200sp.b200sp_spmm(plan, k, d[1], d[2], d[3], Y, 1.0, 0.0, dtype))
+        ref, S = oracle.spmm_csr(A.m, A.n, k, A.row_ptr, A.col_idx, vals, B, None, 1.0, 0.0, dtype)
+        assert_within(to_host(Y, dtype).reshape(A.m, k), ref, S, dtype, what="k=%d" % k)
+        b200sp.b200sp_plan_destroy(plan)
+
+
+def test_csc_without_memory_for_one_of_its_parts():
+    """12 bytes per nonzero were enough for both operations: SpMV does without its places, SpMM takes their memory back."""
+    rng = np.random.default_rng(7)
+    m, n, k = 5000, 4000, 16
+    A = gen.random_csr(m, n, rng.integers(0, 30, m), seed=2, sort_cols=True)
+    cp, ri, va = gen.csr_to_csc(A)
+    x, B = rng.standard_normal(n).astype(np.float32), rng.standard_normal(n * k).astype(np.float32)
+    d = [to_dev(a) for a in (cp, ri, va, x, B)]
+    y, Y = empty_out(m, "f32"), empty_out(m * k, "f32")
+    spmv = lambda: b200sp.spmv_csc(m, n, A.nnz, d[0], d[1], d[2], d[3], y, 1.0, 0.0, "f32")
+    spmm = lambda: b200sp.spmm_csc(m, n, A.nnz, k, d[0], d[1], d[2], d[4], Y, 1.0, 0.0, "f32")
+    refs = {"y": oracle.spmm_csc(m, n, 1, cp, ri, va, x, None, 1.0, 0.0, "f32"), "Y": oracle.spmm_csc(m, n, k, cp, ri, va, B, None, 1.0, 0.0, "f32")}
+
+    def check():
+        for out, (ref, S) in ((y, refs["y"]), (Y, refs["Y"])):
+            assert_within(to_host(out, "f32").reshape(ref.shape), ref, S, "f32")
+            out.fill_(float("nan"))
+
+    failing(2, spmv)                 # 1: the pattern's counts, 2: the places
+    spmm()
+    check()
+    b200sp.b200sp_cache_clear()
+    spmv()
+    failing(1, spmm)                 # the row-major order: built in the memory of the places
+    check()
+    for f in (spmv, spmm):           # both parts again
+        f()
+    check()
+    b200sp.b200sp_cache_clear()
+
+
 def test_plan_used_with_arguments_that_do_not_fit_it():
     A = gen.random_csr(500, 300, np.full(500, 6), 3)
     d_rp, d_ci, d_va, d_x = to_dev(A.row_ptr), to_dev(A.col_idx), to_dev(A.vals), to_dev(np.ones(300, np.float32))
