@@ -252,7 +252,7 @@ __device__ __forceinline__ int block_exclusive_sum(int v, int* s, int* total) {
 // Dynamic shared memory: 3 * buckets ints, then tile 16-bit words.
 __global__ void __launch_bounds__(1024) csc_tile_slots_plan(const int* __restrict__ row_idx, const int* __restrict__ row_ptr, const int* __restrict__ col_ptr,
                                                             const int* __restrict__ tile_col, int n, int nnz, int tile, int shift, int buckets,
-                                                            int unsigned short* __restrict__ src, unsigned short* __restrict__ run_before, int* start,
+                                                            unsigned short* __restrict__ src, unsigned short* __restrict__ run_before, int* start,
                                                             unsigned short* __restrict__ dcol, int* __restrict__ position) {
   extern __shared__ int csc_slots_smem[];
   __shared__ int s_scan[33];

@@ -22,7 +22,7 @@ int plan_free(b200sp_plan* p, bool stream_ordered = false, cudaStream_t stream =
   if (!p) return B200SP_OK;
   int rc = B200SP_OK;
   void* const blocks[] = {p->block, p->cuts_block, p->compact_block, p->shares.block, p->quad[0].block, p->quad[1].block, p->quad[2].block,
-                          p->quad[3].block, p->lists.block};
+                          p->lists.block};
   bool any = false;
   for (void* b : blocks) any |= b != nullptr;
   if (any) {

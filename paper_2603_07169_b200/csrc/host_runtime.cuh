@@ -299,7 +299,7 @@ struct b200sp_plan {
     const int* len = nullptr;             // their lengths
     const int* pos = nullptr;             // blocks + 1: where each block's quads start in the per-call copy of A
     int blocks = 0;
-  } quad[4];                              // for 4, 8, 16 and 32 rows per warp
+  } quad[3];                              // for 4, 8 and 16 rows per warp
   const void* probed_key = nullptr;       // host entry points: the HOST col_idx that verdict belongs to
   bool cols_local = true;                 // its verdict: adjacent rows share most of their lines of x
 };

@@ -117,7 +117,7 @@ int device_scan_in_place(int* data, long long count, int* bsum, cudaStream_t str
 // device and in stream order: no synchronisation.  B200SP_ERR_UNSUPPORTED when the positions would not fit 32 bits.
 int plan_quad_order(b200sp_plan* p, int gpw, b200sp_plan::QuadOrder* out, CallBlock* own, cudaStream_t stream, DeviceInfo* dev) {
   static_assert(kLongRow == 1024, "quad_key() assumes rows of at most 1024 nonzeros");
-  b200sp_plan::QuadOrder& Q = p->quad[gpw == 4 ? 0 : gpw == 8 ? 1 : gpw == 16 ? 2 : 3];
+  b200sp_plan::QuadOrder& Q = p->quad[gpw == 4 ? 0 : gpw == 8 ? 1 : 2];   // rows per warp: 4, 8 or 16
   std::lock_guard<std::mutex> lock(p->build);
   if (Q.block) { *out = Q; return B200SP_OK; }
   const b200sp_plan_info_t& I = p->info;
@@ -174,6 +174,7 @@ int launch_spmm_bstage_quads_as(b200sp_plan* p, int k, const int32_t* col_idx, c
                              cudaStream_t stream, DeviceInfo* dev, EncodeTiledFn encode) {
   const b200sp_plan_info_t& I = p->info;
   constexpr int LANES = SLICE_LANES / PIECES;
+  static_assert(LANES == 2 || LANES == 4 || LANES == 8, "one order of the rows for each");
   constexpr int KS = SLICE_LANES * VEC, ROW_BYTES = SLICE_LANES * 16, GPW = 32 / LANES, WARPS = THREADS / 32;
   const int box_rows = I.n < 256 ? (int)I.n : 256;
   const int boxes = (int)((I.n + box_rows - 1) / box_rows);

@@ -215,7 +215,7 @@ spmm_bstage_prep_kernel(int slots, int gpw, const int* __restrict__ quad_row, co
                         const int* __restrict__ row_ptr, const int* __restrict__ col_idx, const T* __restrict__ vals,
                         unsigned short* __restrict__ qoff, T* __restrict__ qval, int reorder, int* __restrict__ slot_row, int* __restrict__ slot_len) {
   constexpr int G = 128 / ROW_BYTES;
-  constexpr int SLOTS = 32;                   // of a CTA of 256 threads: whole blocks of gpw = 8, 16 or 32
+  constexpr int SLOTS = 32;                   // of a CTA of 256 threads: whole blocks of gpw = 4, 8 or 16
   __shared__ int excess[SLOTS];
   constexpr unsigned FULL = 0xFFFFFFFFu;
   grid_dependency_wait();
