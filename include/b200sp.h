@@ -39,8 +39,9 @@
  *    nothing; a device that is not compute capability 10.x returns B200SP_ERR_ARCH; a failing CUDA
  *    call returns B200SP_ERR_CUDA and its message is kept for b200sp_last_cuda_error().
  *  - Device memory the library needs (plan scratch, the staging buffers of the "host" entry
- *    points, and per-call scratch for SpMM, taken and returned in the order of `stream`: on matrices
- *    with very uneven rows a few bytes per 1024 nonzeros and dense column; on matrices with so few
+ *    points, and per-call scratch for SpMM, taken and returned in the order of `stream`: where SpMM goes by
+ *    equal shares (uneven rows, or k > 16 that is no multiple of 16 bytes) 8 bytes per dense column and
+ *    256 .. 4096 rows + nonzeros, the fewer the smaller the matrix (without that memory it goes by rows); on matrices with so few
  *    columns that a slice of B is kept in shared memory a re-laid copy of A, about (2 + bytes per
  *    value) * (nnz + 3 m) bytes, plus 8 m bytes kept with the plan) comes from a
  *    stream-ordered memory pool of its own, one per device, created at first use.  The pool keeps up to 1 GiB of freed memory for the next call (option "pool_keep_mb",
@@ -113,14 +114,16 @@ int spmm_csr(int64_t m, int64_t n, int64_t nnz, int64_t k, const int32_t* row_pt
  * row-length statistics and bins, chooses the kernels, and computes the nnz-balanced split points
  * (a merge-path search over rows + nonzeros), all on the device and in one launch.  From the same statistics it decides
  * whether SpMM gives every row to a group of eight lanes (even rows) or cuts rows + nonzeros into equal shares per warp
- * (uneven rows: many empty rows, or a share of the nonzeros in rows of more than 128).  What only some SpMM kernels need is
+ * (uneven rows: many empty rows, a share of the nonzeros in rows of more than 128, or a longest row far above the mean; with few
+ * columns only where the rows differ enough for it to pay).  What only some SpMM kernels need is
  * built on the first SpMM call that uses them, in stream order: the lists of rows of 129-1024 and of more than 1024 nonzeros,
  * the shares of large matrices, and the order of the rows by length that SpMM uses when A has so few columns that a slice
  * of B is kept in shared memory.
  * A first call that is captured into a graph builds them inside the graph, for that call alone, and leaves the plan as it was.
  * When the row statistics select the row-direct SpMV kernel, the first b200sp_spmv / spmv_csr call with a given
  * col_idx additionally samples how local the columns are (one small kernel and one synchronisation of the stream)
- * and falls back to the merge-tile kernel for matrices with scattered columns.
+ * and, for matrices with scattered columns, takes another kernel: the equal-rows kernel where all rows have one length of
+ * 3 .. 64, else the merge-tile kernel.  That first call must not be captured.
  * It takes one block of a few bytes per tile from the library's pool, in the order of `stream`, and
  * synchronises `stream` once, so a capturing stream is refused (B200SP_ERR_UNSUPPORTED; the capture stays valid).  A plan may be used from one stream at a time.  b200sp_plan_destroy
  * synchronises the plan's device before it returns the block. */
