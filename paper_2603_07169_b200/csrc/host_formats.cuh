@@ -233,9 +233,6 @@ static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, cons
   g_launches += 4;
   CUP(cudaGetLastError());
 #undef CUP
-  b200sp_plan* plan = nullptr;       // of the row offsets: made now, because the first call of the CSR kernels may be a captured one
-  rc = get_cached_plan(&plan, m, n, nnz, e->row_ptr, stream);
-  if (rc != B200SP_OK) return fail(rc);
   e->tile = tile; e->tiles = tiles; e->buckets = buckets; e->cap = cap;
   e->bucket_row = brow; e->bucket_start = (int*)(blk + o_bstart); e->tile_col = tcol; e->run_shift = (int*)(blk + o_shift);
   e->src = (unsigned short*)(blk + o_src); e->dst = (unsigned short*)(blk + o_dst); e->dcol = (unsigned short*)(blk + o_dcol);
@@ -287,6 +284,23 @@ static int run_csc_products(const CscEntry* e, int64_t nnz, const T* vals, const
                      (const int*)e->bucket_start, (const int*)e->row_ptr, (const float*)e->prod, (const unsigned short*)e->dst, y, alpha, beta);
 }
 
+// SpMM in a capture before any plan of the row offsets exists (the pattern has only been used for SpMV): the statistics cannot be read back,
+// and the nnz-balanced kernel needs none.
+template <typename T, int VEC>
+static int csc_spmm_without_plan(int64_t m, int64_t n, int64_t nnz, int64_t k, const int32_t* row_ptr, const int32_t* col, const T* vals, const void* B,
+                                 void* Y, float alpha, float beta, int dtype, cudaStream_t stream, DeviceInfo* dev) {
+  b200sp_plan p;
+  CU(cudaGetDevice(&p.device));
+  p.row_ptr = row_ptr;
+  p.info.m = m; p.info.n = n; p.info.nnz = nnz;
+  const int rc = check_common(&p, col, vals, B, Y, dtype);
+  if (rc != B200SP_OK) return rc;
+  if (k >= ((int64_t)1 << 31) || m * k >= ((int64_t)1 << 40)) return B200SP_ERR_INVALID_ARG;
+  if (alpha == 0.0f || nnz == 0) return run_scale<T>((long long)m * k, (T*)Y, beta, stream, dev);
+  if (!spmm_offsets_fit(k, (int)sizeof(T))) return B200SP_ERR_UNSUPPORTED;
+  return run_spmm_merge<T, VEC>(&p, (int)k, col, vals, (const T*)B, (T*)Y, alpha, beta, stream, dev);
+}
+
 static int csc_call(bool is_mm, int64_t m, int64_t n, int64_t nnz, int64_t k, const int32_t* col_ptr, const int32_t* row_idx, const void* vals,
                     const void* in, void* out, float alpha, float beta, int dtype, void* stream_v) {
   int rc = check_sizes(m, n, nnz);
@@ -323,6 +337,11 @@ static int csc_call(bool is_mm, int64_t m, int64_t n, int64_t nnz, int64_t k, co
              : launch(csc_permute_vals_kernel<bf16_t>, dim3((unsigned)blocks), dim3(256), stream, nullptr, 0, dev, (long long)nnz, (const int*)e.perm, (const bf16_t*)vals, (bf16_t*)e.vals_t);
     if (rc != B200SP_OK) return rc;
   }
+  int d = 0;
+  CU(cudaGetDevice(&d));
+  if (is_mm && own.block && !cache_find(std::make_tuple(d, (const void*)entry->row_ptr, m, n, nnz)))
+    return dtype == B200SP_F32 ? csc_spmm_without_plan<float, 4>(m, n, nnz, k, entry->row_ptr, e.col, (const float*)e.vals_t, in, out, alpha, beta, dtype, stream, dev)
+                               : csc_spmm_without_plan<bf16_t, 8>(m, n, nnz, k, entry->row_ptr, e.col, (const bf16_t*)e.vals_t, in, out, alpha, beta, dtype, stream, dev);
   return is_mm ? spmm_csr(m, n, nnz, k, entry->row_ptr, e.col, e.vals_t, in, out, alpha, beta, dtype, stream_v)
                : spmv_csr(m, n, nnz, entry->row_ptr, e.col, e.vals_t, in, out, alpha, beta, dtype, stream_v);
 }

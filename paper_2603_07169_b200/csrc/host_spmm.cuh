@@ -374,11 +374,14 @@ bool spmm_uneven_by_rows(const b200sp_plan_info_t& I, int64_t k, int elem_bytes,
   return 1.05 * rows < shares;
 }
 
+// The nnz-balanced kernel counts the bytes of a row of B, and columns past k up to a slice, in 32 bits.
+bool spmm_offsets_fit(int64_t k, int elem_bytes) { return k <= (INT32_MAX - 2048) / elem_bytes; }
+
 // Whether SpMM goes by equal shares (spmm_merge_kernel): uneven rows (see above), and k that is no multiple of 16 bytes unless it is so narrow
 // that a lane per column and a group of lanes per row lose little (100,000 rows of 13: k = 13 18 us by rows, 27 us by shares; k = 23 35 / 27 us;
-// k = 50 47 / 35 us FP32, 42 / 34 us BF16).  The kernel counts the bytes of a row of B, and columns past k up to a slice, in 32 bits.
+// k = 50 47 / 35 us FP32, 42 / 34 us BF16).
 bool spmm_by_shares(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, float beta) {
-  if (k > (INT32_MAX - 2048) / elem_bytes || !g_opt.spmm_sliced) return false;
+  if (!spmm_offsets_fit(k, elem_bytes) || !g_opt.spmm_sliced) return false;
   if (g_opt.spmm_flat != 2) return g_opt.spmm_flat == 1;
   if (k % (16 / elem_bytes) != 0 && k > 16) return true;
   return spmm_rows_are_uneven(I) && !spmm_uneven_by_rows(I, k, elem_bytes, beta);
