@@ -1,6 +1,7 @@
 """Helpers for the GPU parity tests: upload a workload, call the C ABI through the binding, compare
 with the CPU oracle under the acceptance bounds (FP32: 1e-5 * S + 1e-30; BF16: 8e-3 * |y_ref| + 1e-5 * S)."""
 import numpy as np
+import pytest
 import torch
 
 import gen
@@ -8,6 +9,8 @@ import oracle
 import paper_2603_07169_b200 as b200sp
 
 DEV = "cuda:0"
+# the checked build validates every call on the device: one more allocation, and a synchronisation that a capture does not allow
+needs_plain_build = pytest.mark.skipif(b200sp.b200sp_checked_build() != 0, reason="the checked build validates every call on the device")
 
 
 def to_dev(a):

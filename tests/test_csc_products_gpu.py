@@ -7,7 +7,7 @@ import torch
 import gen
 import oracle
 import paper_2603_07169_b200 as b200sp
-from gpu_util import assert_within, empty_out, store, to_dev, to_host
+from gpu_util import assert_within, empty_out, needs_plain_build, store, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -138,6 +138,7 @@ def test_dropping_a_csc_pattern_drops_the_plans_of_its_row_offsets():
     b200sp.b200sp_cache_clear()
 
 
+@needs_plain_build
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("first", ["spmv", "spmm"])
 def test_the_other_operation_captured(first, dtype):

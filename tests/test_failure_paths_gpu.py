@@ -11,7 +11,7 @@ import torch
 import gen
 import oracle
 import paper_2603_07169_b200 as b200sp
-from gpu_util import assert_within, empty_out, run_spmm, run_spmv, store, to_dev, to_host
+from gpu_util import assert_within, empty_out, needs_plain_build, run_spmm, run_spmv, store, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 TIMEOUT, ALLOC, INVALID = 7, 4, 1
@@ -131,6 +131,7 @@ def failing(nth, fn):
         b200sp.b200sp_set_option("fail_alloc_after", 0)
 
 
+@needs_plain_build
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_spmm_by_shares_without_its_scratch_goes_by_rows(dtype):
     """Columns that are no multiple of 16 bytes on even rows took no memory before they went by shares; uneven rows go by rows as well then."""
@@ -148,6 +149,7 @@ def test_spmm_by_shares_without_its_scratch_goes_by_rows(dtype):
         b200sp.b200sp_plan_destroy(plan)
 
 
+@needs_plain_build
 def test_csc_without_memory_for_one_of_its_parts():
     """12 bytes per nonzero were enough for both operations: SpMV does without its places, SpMM takes their memory back."""
     rng = np.random.default_rng(7)

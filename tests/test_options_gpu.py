@@ -8,7 +8,7 @@ import torch
 
 import gen
 import paper_2603_07169_b200 as b200sp
-from gpu_util import assert_within, run_spmm, run_spmv, to_dev
+from gpu_util import assert_within, needs_plain_build, run_spmm, run_spmv, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -101,6 +101,7 @@ def captured_grids(call):
     return [driver.cuGraphKernelNodeGetParams(n)[1].gridDimX for n in kernels]
 
 
+@needs_plain_build
 @pytest.mark.parametrize("ell", [False, True])
 def test_row_ctas_as_set_and_by_the_rule(ell):
     """Rows of five FP32 entries leave room for five CTAs of 256 rows per SM: these by the rule, what the caller sets otherwise."""

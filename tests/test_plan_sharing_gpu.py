@@ -9,7 +9,7 @@ import torch
 import gen
 import oracle
 import paper_2603_07169_b200 as b200sp
-from gpu_util import assert_within, empty_out, store, to_dev, to_host
+from gpu_util import assert_within, empty_out, needs_plain_build, store, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -94,6 +94,7 @@ def test_first_calls_from_several_threads(case):
         P.close()
 
 
+@needs_plain_build
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("case", sorted(CASES))
 def test_first_call_captured(case, dtype):
