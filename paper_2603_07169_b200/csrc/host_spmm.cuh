@@ -387,13 +387,13 @@ bool spmm_by_shares(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, floa
   return spmm_rows_are_uneven(I) && !spmm_uneven_by_rows(I, k, elem_bytes, beta);
 }
 
-template <typename T, int V, int J, bool LIST>
+template <typename T, int V, int J, int MODE>
 int launch_spmm_merge_as(b200sp_plan* p, const b200sp_plan::Shares& work, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
                       cudaStream_t stream, DeviceInfo* dev) {
   const b200sp_plan_info_t& I = p->info;
   constexpr int KS = 32 * V * J;
   const int witems = work.witems;
-  auto kernel = spmm_merge_kernel<T, V, J, LIST>;
+  auto kernel = spmm_merge_kernel<T, V, J, MODE>;
   static int per_sm[64] = {};   // per instantiation and device: resident CTAs
   if (!per_sm[p->device]) {
     int nb = 0;
@@ -438,13 +438,13 @@ int launch_spmm_merge_as(b200sp_plan* p, const b200sp_plan::Shares& work, int k,
 }
 
 // beta != 0 and one row in sixteen or more without nonzeros: these are listed and scaled apart (R-MAT 2^21, k = 64 BF16, 61 % empty: 458 us
-// against 657 us; with beta == 0 the listing costs as much as it saves).
+// against 657 us; with beta == 0 the listing costs as much as it saves).  Otherwise Y's old values are asked for a row ahead.
 template <typename T, int V, int J>
 int launch_spmm_merge(b200sp_plan* p, const b200sp_plan::Shares& work, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
                       cudaStream_t stream, DeviceInfo* dev) {
-  return beta != 0.0f && p->info.bin_rows[0] * 16 >= p->info.m
-             ? launch_spmm_merge_as<T, V, J, true>(p, work, k, col_idx, vals, B, Y, alpha, beta, stream, dev)
-             : launch_spmm_merge_as<T, V, J, false>(p, work, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
+  if (beta == 0.0f) return launch_spmm_merge_as<T, V, J, 0>(p, work, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
+  return p->info.bin_rows[0] * 16 >= p->info.m ? launch_spmm_merge_as<T, V, J, 2>(p, work, k, col_idx, vals, B, Y, alpha, beta, stream, dev)
+                                               : launch_spmm_merge_as<T, V, J, 1>(p, work, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
 }
 
 // nnz-balanced SpMM (spmm_merge_kernel), any k.  The widest pieces (16 bytes per lane at most) that k allows, narrowed while half as

@@ -103,6 +103,16 @@ __device__ __forceinline__ void piece_store(T* yp, const float (&acc)[V], float 
   *(raw*)yp = Piece<T, V>::pack(out);
 }
 
+// The same with Y's old values already here.
+template <typename T, int V>
+__device__ __forceinline__ void piece_store(T* yp, const float (&acc)[V], float alpha, float beta, const typename Piece<T, V>::raw& old) {
+  float out[V];
+  Piece<T, V>::widen(old, out);
+#pragma unroll
+  for (int j = 0; j < V; ++j) out[j] = alpha * acc[j] + beta * out[j];
+  *(typename Piece<T, V>::raw*)yp = Piece<T, V>::pack(out);
+}
+
 // N consecutive words of shared memory (N 2, 4 or 8; aligned to 4 N or 16 bytes) with vector loads
 template <int N, typename W>
 __device__ __forceinline__ void lds_group(const W* p, W (&o)[N]) {
@@ -167,13 +177,18 @@ template <> struct MergeStage<bf16_t> {
 // order, and what crosses the CTA's own ends goes to tile_tail / tile_carry and is finished by spmm_merge_fixup_kernel.  No
 // chain is longer than kMergeWarpItems products + kMergeShares + kMergeWarps partial sums + the tiles' terms.
 // split[i]: row ends before item i * witems.
-// LIST: for matrices with empty rows and beta != 0 (see below); the listing costs 2-5 % where there are none.
-template <typename T, int V, int J, bool LIST>
+// MODE 0: beta == 0.  1: beta != 0; Y's old values of a row are asked for when the row before it ends, not when it ends itself (50,000 uneven
+// rows of 11, k = 128 FP32: 37.1 -> 34.0 us; 30,000 of 12, k = 256 48.8 -> 41.8 us; two rows ahead, in a second set of registers: 41.2 us for the
+// former).  Not with four 2- or 4-byte loads a nonzero, where the registers spill (k = 127 BF16 89 / 104 us).
+// 2: beta != 0 and empty rows, which are listed apart (see below); the listing costs 2-5 % where there are none, and old values asked for
+// ahead cost it more than they save (R-MAT 2^20, k = 64 FP32 303 / 442 us).
+template <typename T, int V, int J, int MODE>
 __global__ void __launch_bounds__(kMergeWarps * 32, (merge_ctas<T, V, J>()))
 spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, const int* __restrict__ split, const int* __restrict__ row_ptr,
                   const int* __restrict__ col_idx, const T* __restrict__ vals, const T* __restrict__ B, T* __restrict__ Y,
                   float* __restrict__ tile_carry, float* __restrict__ tile_tail, int2* __restrict__ tile_row, float alpha, float beta) {
   constexpr int U = kMergeUnroll<V, J>, KS = 32 * V * J;
+  constexpr bool LIST = MODE == 2, AHEAD = MODE == 1 && !(V == 1 && J == 4);
   typedef typename Piece<T, V>::raw raw;
   __shared__ __align__(16) MergeStage<T> stage_s[kMergeWarps][2];
   __shared__ __align__(16) float wide_s[sizeof(T) == 2 ? kMergeWarps : 1][sizeof(T) == 2 ? kMergeWarpItems + 8 : 4];   // BF16: the current share's values widened
@@ -228,6 +243,12 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
   const int row_bytes = k * (int)sizeof(T);
   T* yrow = Y + (long long)r_first * k + col0;
   int begin = start0;                                        // start of the current row
+  raw old[AHEAD ? J : 1];                                    // Y's old values of the current row
+  auto ask_old = [&]() {
+#pragma unroll
+    for (int j = 0; j < (AHEAD ? J : 0); ++j) if (on[j]) old[j] = *(const raw*)(yrow + 32 * V * j);
+  };
+  if (AHEAD && r_first < m) ask_old();
   // rows empty_s[warp][0 .. count) of the share whose first row is at ys: y = beta * y over the slice's columns
   auto scale_rows = [&](T* ys, int count) {
     const int width = min(KS, k - slice * KS);
@@ -321,7 +342,11 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
       } else {
         T* const yp = LIST ? ys + (long long)(row >> 8) * k + col0 : yrow;
 #pragma unroll
-        for (int j = 0; j < J; ++j) if (on[j]) piece_store<T, V>(yp + 32 * V * j, acc[j], alpha, beta);
+        for (int j = 0; j < J; ++j)
+          if (on[j]) {
+            if constexpr (AHEAD) piece_store<T, V>(yp + 32 * V * j, acc[j], alpha, beta, old[j]);
+            else piece_store<T, V>(yp + 32 * V * j, acc[j], alpha, MODE ? beta : 0.0f);
+          }
       }
 #pragma unroll
       for (int j = 0; j < J; ++j)
@@ -330,6 +355,7 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
       row = share_end(++j_row);
       end = LIST ? row & 0xFF : row;
       if constexpr (!LIST) yrow += k;
+      if (AHEAD && r_lo + j_row < m) ask_old();
     };
     for (int q = 0; q < cnt; q += U) {
       int c[U];

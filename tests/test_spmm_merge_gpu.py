@@ -78,6 +78,26 @@ def test_uneven_rows_and_few_columns_by_rows(dtype):
         assert_within(Y, Y_ref, S, dtype, 1.0, np.abs(1.25 * y0f.astype(np.float64)).reshape(A.m, k), what="k=%d ab" % k)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_old_values_asked_for_ahead_belong_to_their_rows(dtype):
+    """beta != 0 and no empty rows: Y's old values of a row are read when the row before it ends.  Old values that differ from row to row by
+    more than the products, rows that end at the first and the last nonzero of a group of 8 and of a share, several to a group, and every
+    number of loads per nonzero (k up to 256 and a second slice)."""
+    lens = np.concatenate([np.arange(1, 41), np.full(200, 1), np.full(64, 8), np.full(33, 31), [700], np.full(60, 7), [1]])
+    n = 30_000
+    A = gen.random_csr(len(lens), n, lens, seed=17, sort_cols=False)
+    rng = np.random.default_rng(4)
+    b200sp.b200sp_set_option("spmm_flat", 1)
+    try:
+        for k in (2, 17, 33, 50, 63, 64, 100, 127, 128, 130, 256, 320):
+            B = rng.standard_normal(n * k).astype(np.float32)
+            Y0 = np.repeat((64 + 64 * (np.arange(A.m) % 4)).astype(np.float32), k)
+            Y, Y_ref, S = run_spmm(A, B, k, Y0, 0.5, -1.0, dtype)
+            assert_within(Y, Y_ref, S, dtype, 0.5, np.abs(Y0.astype(np.float64)).reshape(A.m, k), what="k=%d" % k)
+    finally:
+        b200sp.b200sp_set_option("spmm_flat", 2)
+
+
 def test_non_finite_rows_of_b_touch_only_the_rows_that_use_them():
     """What a warp reads ahead of its last nonzero (row 0 of B) is never multiplied."""
     n, k = 9000, 64
