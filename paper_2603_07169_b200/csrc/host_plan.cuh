@@ -187,7 +187,7 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
   const size_t nt = (size_t)I.spmv_tiles;
   const int witems = spmm_share_items(I, dev);
   const long long shares = (m + nnz + witems - 1) / witems;
-  const bool with_shares = shares <= 65536;
+  const bool with_shares = shares <= 65536 && m + nnz <= (1 << 23);   // (65536 shares of 128; the pass divides item numbers below 2^23)
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
   const size_t o_split = 256, o_carry = o_split + up((nt + 1) * 4), o_tail = o_carry + up((nt + 1) * 4), o_share = o_tail + up((nt + 1) * 4),
                total = o_share + (with_shares ? up((size_t)(shares + 1) * 4) : 0);
@@ -208,11 +208,12 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
   if (rc != B200SP_OK) return fail(rc);
   PlanStats h;
   {
-    const long long searches = (long long)nt + 1 + (with_shares ? shares + 1 : 0), work = m > searches * 4 ? m : searches * 4;
-    const long long blocks = (work + 256 * 4 - 1) / (256 * 4);   // four rows and at most one search per thread
-    const int grid = (int)(blocks < dev->sms * 8 ? blocks : dev->sms * 8);
-    rc = launch(plan_pass_kernel, dim3((unsigned)grid), dim3(256), stream, nullptr, 0, dev, row_ptr, (int)m, (int)nnz, slot, g_slots.host + slot, items, (int)nt,
-                p->split_row, with_shares ? witems : 0, (int)shares, share_split);
+    int tile_shift = 0;
+    while ((1 << tile_shift) < items) ++tile_shift;   // (1024, 2048 or 4096)
+    const long long blocks = (m + 255) / 256;   // a row per thread, up to 8 blocks per SM
+    const unsigned long long inverse = ((1ULL << 40) + witems - 1) / witems;
+    rc = launch(m > (1 << 17) ? plan_pass_kernel<true> : plan_pass_kernel<false>, dim3((unsigned)(blocks < dev->sms * 8 ? blocks : dev->sms * 8)), dim3(256), stream, nullptr, 0, dev, row_ptr, (int)m,
+                (int)nnz, slot, g_slots.host + slot, tile_shift, (int)nt, p->split_row, with_shares ? witems : 0, inverse, (int)shares, share_split);
     const cudaError_t e = cudaStreamSynchronize(stream);
     h = g_slots.host[slot];
     if (e == cudaSuccess) plan_slot_give(slot);   // only a finished pass (or none) has left its slot to the next; an error here means a lost device

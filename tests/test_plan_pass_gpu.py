@@ -39,6 +39,35 @@ def test_statistics_match_numpy(m):
     check(np.full(m, 7, np.int64))       # nothing left over from the passes before
 
 
+@pytest.mark.parametrize("case", ["mixed", "longest_first", "longest_last", "one_row", "all_empty_but_one", "rows_of_a_share", "rows_of_a_tile", "several_rows_a_thread", "most_rows_without_a_search"])
+def test_split_points_from_the_rows(case):
+    """Tiles of SpMV and shares of SpMM cut where the pass says: sums of ones, which are the row lengths.  Rows that hold no split point, one,
+    and more than the sixteen that a lane writes alone; the split points behind the last row; more rows than one turn of the grid."""
+    lens = {"mixed": lengths(3001, 5), "longest_first": np.concatenate([[150_000], np.full(999, 3)]), "longest_last": np.concatenate([np.full(999, 3), [150_000]]),
+            "one_row": np.array([70_000]), "all_empty_but_one": np.concatenate([np.zeros(40_000), [5], np.zeros(9_000)]), "rows_of_a_share": np.full(500, 31),
+            "rows_of_a_tile": np.full(64, 1023), "several_rows_a_thread": np.random.default_rng(1).integers(0, 6, 1_300_000), "most_rows_without_a_search": np.random.default_rng(2).integers(0, 9, 1 << 17)}[case].astype(np.int64)
+    m, nnz, k = len(lens), int(lens.sum()), 4
+    row_ptr = torch.from_numpy(np.concatenate([[0], lens.cumsum()]).astype(np.int32)).to("cuda:0")
+    col = torch.randint(0, 1000, (nnz,), dtype=torch.int32, device="cuda:0")
+    ones, x = torch.ones(nnz, device="cuda:0"), torch.ones(1000 * k, device="cuda:0")
+    want = torch.from_numpy(lens).to("cuda:0").float()
+    b200sp.b200sp_set_option("spmv_kernel", 0)
+    b200sp.b200sp_set_option("spmm_flat", 1)
+    b200sp.b200sp_set_option("spmm_bstage", 0)
+    try:
+        for items in (0, 1024, 4096):
+            b200sp.b200sp_set_option("merge_items", items)
+            plan = b200sp.b200sp_plan_create(m, 1000, nnz, row_ptr)
+            y, Y = torch.full((m,), float("nan"), device="cuda:0"), torch.full((m * k,), float("nan"), device="cuda:0")
+            b200sp.b200sp_spmv(plan, col, ones, x, y, 1.0, 0.0, "f32")
+            b200sp.b200sp_spmm(plan, k, col, ones, x, Y, 1.0, 0.0, "f32")
+            b200sp.b200sp_plan_destroy(plan)
+            assert torch.equal(y, want) and torch.equal(Y.view(m, k), want[:, None].expand(m, k))
+    finally:
+        for name, value in (("spmv_kernel", -1), ("spmm_flat", 2), ("spmm_bstage", 1), ("merge_items", 0)):
+            b200sp.b200sp_set_option(name, value)
+
+
 def test_passes_from_several_threads():
     failures = []
 
