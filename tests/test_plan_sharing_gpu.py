@@ -125,3 +125,29 @@ def test_first_call_captured(case, dtype):
         b200sp.b200sp_plan_destroy(plan)
     finally:
         P.close()
+
+
+@pytest.mark.parametrize("side_stream", [False, True])
+def test_a_plan_destroyed_behind_its_product(side_stream):
+    """A new pattern in every step, nothing waited for: the memory that a plan gives back is the next plan's at once, and each product is done
+    with it by then.  With a plan also used on another stream, destroying it waits for the device."""
+    P, side = Problem("lists"), torch.cuda.Stream()
+    others = [gen.random_csr(20_000 + 100 * i, 20_000, np.random.default_rng(i).integers(0, 30, 20_000 + 100 * i), seed=i) for i in range(3)]
+    try:
+        work = [(A, [to_dev(a) for a in (A.row_ptr, A.col_idx, A.vals)], empty_out(A.m * P.k, "f32")) for A in [P.A] + others]
+        torch.cuda.synchronize()
+        first = None
+        for step in range(40):
+            outs = []
+            for A, d, Y in work:
+                plan = b200sp.b200sp_plan_create(A.m, A.n, A.nnz, d[0])
+                b200sp.b200sp_spmm(plan, P.k, d[1], d[2], P.d[3], Y, 1.0, 0.0, "f32", side if side_stream and step % 2 else None)
+                b200sp.b200sp_plan_destroy(plan)
+                outs.append(Y.clone() if step in (0, 39) else None)
+            if step == 0:
+                first = outs
+        torch.cuda.synchronize()
+        P.check(work[0][2], "last step")
+        assert all(torch.equal(a, b) for a, b in zip(first, outs))
+    finally:
+        P.close()
