@@ -28,7 +28,8 @@ extern "C" {
  *                    128, a quarter or more of the rows empty, or a longest row far above the mean; with few columns only where the
  *                    rows differ enough, b200sp_spmm_by_shares) or k > 16 is no multiple of 16 bytes (default)
  *   "spmm_stage_a"   the k-sliced SpMM kernel's warps first copy their rows' (col, val) pairs into shared memory: 1 = yes, 0 = no,
- *                    2 = for BF16 storage only (default: measured 5-6 % faster there and 2-3 % slower for FP32)
+ *                    2 = for BF16 storage only (default: measured 5-6 % faster there and 2-3 % slower for FP32), and not where
+ *                    rows of B come in whole pieces of 32 bytes and are at least 128 wide: there four lanes share a row
  *   "spmm_ranges"    k-sliced SpMM on rows with ascending columns, one launch per column range so that the rows of B a
  *                    launch gathers from stay in L2: 1 = no ranges (default: measured slower, see the benchmarks' record),
  *                    0 = as many as make a range of B fit L2, 2, 3, 4 or 8 = that many

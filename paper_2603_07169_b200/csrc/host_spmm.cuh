@@ -526,6 +526,12 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     int rc = plan_row_lists(p, &lists, &own_lists, stream, dev);
     if (rc != B200SP_OK) return rc;
     const int mid_blocks = (p->num_medium + GROUPS - 1) / GROUPS;
+    // BF16 rows of B in whole 32-byte pieces: 32 bytes a lane from 64 columns on (narrower slices, 16 / 32 bytes a lane on 2^18 rows: k = 32 31.8 /
+    // 33.6 us, k = 16 24.1 / 26.6 us), while a slice of B is about as large as half of L2 at most: beyond that the loads wait for memory, and the
+    // single steps at the ends of rows, with half as many warps, cost more than the loads save (2^20 rows of 13, 134 MB a slice, k = 64 286 / 303 us,
+    // rows of 16 k = 128 514 / 491 us; 2^19 rows of 32, 67 MB, k = 64 179 / 158 us; 2^18 rows of 13, 34 MB, k = 256 225 / 208 us).
+    const bool wide = sizeof(T) == 2 && lanes == 8 && g_opt.spmm_stage_a == 2 && k % 16 == 0 && ((uintptr_t)B & 31) == 0 &&
+                      (double)I.n * 128.0 <= 0.55 * (double)dev->l2_bytes;
     int ranges = 1;
     if (lanes == 8) {
       rc = spmm_column_ranges(p, col_idx, 8 * 16, stream, dev, &ranges);
@@ -549,6 +555,19 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
         tl_pdl_kernel = true;
         rc = launch(spmm_medium_row_kernel<T, VEC, kSpmmThreads, 8>, dim3((unsigned)(slices * mid_blocks)), dim3(kSpmmThreads), stream,
                     nullptr, 0, dev, p->num_medium, lists.medium, k, mid_blocks, p->row_ptr, col_idx, vals, B, Y, alpha, beta);
+      }
+    } else if (wide) {
+      if constexpr (sizeof(T) == 2) {
+        constexpr int THREADS = 128;
+        static_assert(THREADS / 4 == kSpmmThreads / 8, "the same rows per block as the kernels with eight lanes a row");
+        tl_pdl_kernel = true;
+        rc = launch(spmm_slice_wide_kernel<THREADS>, dim3((unsigned)(slices * row_blocks)), dim3(THREADS), stream, B, (size_t)I.n * k * sizeof(T), dev, (int)I.m,
+                    k, row_blocks, p->row_ptr, col_idx, vals, B, Y, alpha, beta, kMediumRow);
+        if (rc == B200SP_OK && p->num_medium > 0) {
+          tl_pdl_kernel = true;
+          rc = launch(spmm_medium_row_kernel<T, VEC, kSpmmThreads, 8>, dim3((unsigned)(slices * mid_blocks)), dim3(kSpmmThreads), stream, nullptr, 0, dev,
+                      p->num_medium, lists.medium, k, mid_blocks, p->row_ptr, col_idx, vals, B, Y, alpha, beta);
+        }
       }
     } else
     // rows of at most kMediumRow nonzeros: the register-capped kernel; kMediumRow + 1 .. kLongRow: the same scheme with

@@ -397,6 +397,68 @@ spmm_slice_kernel(int m, int k, int row_blocks, const int* __restrict__ row_ptr,
   VecLoad<T, VEC>::st(yp, out);
 }
 
+// 32 bytes of a row of B as one load: sixteen BF16 columns
+struct __align__(32) Wide { unsigned w[8]; };
+__device__ __forceinline__ Wide ld_wide(const void* p) {
+  Wide r;
+  asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+      : "=r"(r.w[0]), "=r"(r.w[1]), "=r"(r.w[2]), "=r"(r.w[3]), "=r"(r.w[4]), "=r"(r.w[5]), "=r"(r.w[6]), "=r"(r.w[7]) : "l"(p));
+  return r;
+}
+__device__ __forceinline__ void wide_fma(const Wide& b, float v, float (&acc)[16]) {      // v is a widened BF16 value
+#pragma unroll
+  for (int i = 0; i < 8; ++i) RawVec<bf16_t, 8>::fma2((unsigned short)(__float_as_uint(v) >> 16), b.w[i], acc[2 * i], acc[2 * i + 1]);
+}
+
+// k-sliced kernel for BF16 with 32 bytes of a row of B per load: four lanes own a row of A and a line of every row of B, so that a load of a warp
+// takes eight lines instead of four, and a nonzero costs its (col, val) pair, its address and its loop to four lanes instead of eight.  What
+// bounds the kernels with 16 bytes a lane is the issue rate (74-79 % busy) and the instructions that L1 takes (about 4 cycles each and 1.5 per
+// line).  64 registers: four lines in flight per lane, 32 warps per SM.  The products are added in the order of spmm_slice_kernel, so the
+// results are the same bit for bit.  us, 16 bytes a lane with staged pairs / this: 2^17 rows of
+// 16, k = 128 49.0 / 42.8, k = 80 48.5 / 38.8; 2^14 rows of 32, k = 64 9.0 / 7.2; 2^16 rows of 8, k = 256 33.5 / 30.2; 2^19 rows of 32, k = 64 179 /
+// 158, k = 256 679 / 670.
+// (FP32 has half the columns per load and is not bound by issue: k = 64 317 / 302-325, k = 256 249 / 266; it stays with 16 bytes.)
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS)
+spmm_slice_wide_kernel(int m, int k, int row_blocks, const int* __restrict__ row_ptr, const int* __restrict__ col_idx, const bf16_t* __restrict__ vals,
+                       const bf16_t* __restrict__ B, bf16_t* __restrict__ Y, float alpha, float beta, int long_thresh) {
+  constexpr int LANES = 4, VEC = 16, GROUPS = THREADS / LANES, KS = LANES * VEC;
+  grid_dependency_wait();
+  const int slice = blockIdx.x / row_blocks, rb = blockIdx.x - slice * row_blocks;
+  const int g = threadIdx.x / LANES, l = threadIdx.x % LANES;
+  const long long row = (long long)rb * GROUPS + g;
+  if (row >= m) return;
+  const int rs = __ldg(row_ptr + row), re = __ldg(row_ptr + row + 1);
+  if (re - rs > long_thresh) return;
+  const int col0 = slice * KS + l * VEC;
+  if (col0 >= k) return;
+  const char* const Bc = (const char*)(B + col0);
+  const long long row_bytes = 2LL * k;
+  float acc[VEC];
+#pragma unroll
+  for (int j = 0; j < VEC; ++j) acc[j] = 0.0f;
+  int p = rs;
+  for (; p < re && (p & 3); ++p) wide_fma(ld_wide(Bc + __ldg(col_idx + p) * row_bytes), to_f32(__ldg(vals + p)), acc);   // up to the first multiple of four
+  for (; p + 4 <= re; p += 4) {
+    int c[4]; float v[4];
+    ld_a4(col_idx, vals, p, c, v);
+    Wide b[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) b[u] = ld_wide(Bc + c[u] * row_bytes);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) wide_fma(b[u], v[u], acc);
+  }
+  for (; p < re; ++p) wide_fma(ld_wide(Bc + __ldg(col_idx + p) * row_bytes), to_f32(__ldg(vals + p)), acc);
+  bf16_t* const yp = Y + row * k + col0;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float half[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) half[j] = acc[8 * h + j];
+    slice_store<bf16_t, 8>(yp + 8 * h, half, alpha, beta);
+  }
+}
+
 // Column-range variant of the k-sliced kernel, for matrices whose rows hold their columns in ascending order.  When the
 // part of B that one slice touches (n rows x 128 bytes) is larger than what L2 keeps, the columns are cut into `ranges`
 // equal ranges and the kernel is launched once per range: launch r walks, in every row, only the nonzeros whose column lies

@@ -105,6 +105,40 @@ def test_b_slice_in_shared_memory(n, k, dtype):
     b200sp.b200sp_check()
 
 
+@pytest.mark.parametrize("k", [64, 80, 128, 256, 272])
+@pytest.mark.parametrize("case", ["even", "few_rows", "some_long"])
+def test_bf16_rows_of_b_in_pieces_of_32_bytes(case, k):
+    """Four lanes per row and 32 bytes of B per load where B and its rows are aligned to 32 bytes: the same sums in the same order as the kernel
+    with 16 bytes a lane, which also takes a B that is only aligned to 16 bytes; so the results are equal bit for bit.  Row lengths of every
+    remainder modulo four, a last block that is not full, a last slice that is not full, rows of more than 128 nonzeros, beta != 0."""
+    import torch
+    from gpu_util import to_dev
+    rng = np.random.default_rng(k)
+    lens = {"even": rng.integers(9, 17, 3001), "few_rows": np.array([5, 6, 7]), "some_long": np.concatenate([rng.integers(30, 40, 2000), [129, 140]])}[case]
+    m, n = len(lens), 20_000
+    A = gen.random_csr(m, n, lens, seed=k, sort_cols=False)
+    B, Y0, vals = rng.standard_normal(n * k).astype(np.float32), rng.standard_normal(m * k).astype(np.float32), gen.to_bf16(A.vals)
+    d = [to_dev(a) for a in (A.row_ptr, A.col_idx, vals)]
+    odd = torch.zeros(n * k + 8, dtype=torch.int16, device="cuda:0")[8:]
+    assert odd.data_ptr() % 32 == 16
+    odd.copy_(to_dev(gen.to_bf16(B)))
+    for alpha, beta in ((1.0, 0.0), (0.5, -2.0)):
+        outs = []
+        for d_B, stage_a in ((odd.clone(), 2), (odd, 2), (odd.clone(), 1)):
+            b200sp.b200sp_set_option("spmm_stage_a", stage_a)
+            try:
+                d_Y = to_dev(gen.to_bf16(Y0)).clone()
+                b200sp.spmm_csr(m, n, A.nnz, k, d[0], d[1], d[2], d_B, d_Y, alpha, beta, "bf16")
+                outs.append(d_Y)
+            finally:
+                b200sp.b200sp_set_option("spmm_stage_a", 2)
+        assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+        Y_ref, S = oracle.spmm_csr(m, n, k, A.row_ptr, A.col_idx, vals, gen.to_bf16(B), gen.to_bf16(Y0), alpha, beta, "bf16")
+        assert_within(outs[0].cpu().numpy().view(np.uint16).reshape(m, k), Y_ref, S, "bf16", abs(alpha),
+                      np.abs(beta * gen.bf16_to_f32(gen.to_bf16(Y0)).astype(np.float64)).reshape(m, k), what="%s k=%d" % (case, k))
+    b200sp.b200sp_cache_clear()
+
+
 @pytest.mark.parametrize("dtype", DTYPES)
 def test_spmm_column_equals_spmv(dtype):
     from gpu_util import run_spmv
