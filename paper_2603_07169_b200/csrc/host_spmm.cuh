@@ -527,11 +527,12 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     if (rc != B200SP_OK) return rc;
     const int mid_blocks = (p->num_medium + GROUPS - 1) / GROUPS;
     // BF16 rows of B in whole 32-byte pieces: 32 bytes a lane from 64 columns on (narrower slices, 16 / 32 bytes a lane on 2^18 rows: k = 32 31.8 /
-    // 33.6 us, k = 16 24.1 / 26.6 us), while a slice of B is about as large as half of L2 at most: beyond that the loads wait for memory, and the
-    // single steps at the ends of rows, with half as many warps, cost more than the loads save (2^20 rows of 13, 134 MB a slice, k = 64 286 / 303 us,
-    // rows of 16 k = 128 514 / 491 us; 2^19 rows of 32, 67 MB, k = 64 179 / 158 us; 2^18 rows of 13, 34 MB, k = 256 225 / 208 us).
+    // 33.6 us, k = 16 24.1 / 26.6 us).  Rows that do not all begin and end on a multiple of four nonzeros take single steps there, which with half
+    // as many warps cost more than the loads save once the loads wait for memory: they go this way while a slice of B takes less than half of L2
+    // (rows of 13, k = 64: 350,000 of them 78.1 / 74.5 us, 450,000 102.9 / 100.6, 550,000 130 / 132, 2^20 286 / 303; rows of 6, 550,000 86.0 / 88.4;
+    // but 2^20 rows of 16, k = 128 514 / 491).
     const bool wide = sizeof(T) == 2 && lanes == 8 && g_opt.spmm_stage_a == 2 && k % 16 == 0 && ((uintptr_t)B & 31) == 0 &&
-                      (double)I.n * 128.0 <= 0.55 * (double)dev->l2_bytes;
+                      ((double)I.n * 128.0 <= 0.45 * (double)dev->l2_bytes || (I.min_row_len == I.max_row_len && I.max_row_len % 4 == 0));
     int ranges = 1;
     if (lanes == 8) {
       rc = spmm_column_ranges(p, col_idx, 8 * 16, stream, dev, &ranges);
