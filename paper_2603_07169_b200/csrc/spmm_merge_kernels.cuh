@@ -156,6 +156,13 @@ constexpr int merge_ctas() {
   return need <= 20 ? 6 : need <= 24 ? 5 : need <= 40 ? 4 : 3;
 }
 
+// Forms whose registers are full without Y's old values asked for ahead (bytes spilled, and us on 150,000 uneven rows of 11, without / with them):
+// four loads of one column (FP32 0 / 68 bytes, k = 127 187 / 248 us; BF16 42 / 86 bytes, 168 / 218 us) and two of eight BF16 columns
+// (52 / 300 bytes, k = 264 190 / 306 us, k = 512 285 / 410 us).  Where two loads of one or two BF16 columns spill some 40 bytes for them the wait
+// saved is still worth more (k = 63 83.5 / 80.1 us, k = 66 86.5 / 83.8 us).
+template <typename T, int V, int J>
+constexpr bool kMergeNoRoom = (V == 1 && J == 4) || (sizeof(T) == 2 && V == 8 && J == 2);
+
 // What a warp keeps in shared memory of one share: its columns, its values and the ends of its rows, and room to read a group ahead.
 template <typename T> struct MergeStage;
 template <> struct MergeStage<float> {
@@ -179,7 +186,7 @@ template <> struct MergeStage<bf16_t> {
 // split[i]: row ends before item i * witems.
 // MODE 0: beta == 0.  1: beta != 0; Y's old values of a row are asked for when the row before it ends, not when it ends itself (50,000 uneven
 // rows of 11, k = 128 FP32: 37.1 -> 34.0 us; 30,000 of 12, k = 256 48.8 -> 41.8 us; two rows ahead, in a second set of registers: 41.2 us for the
-// former).  Not with four 2- or 4-byte loads a nonzero, where the registers spill (k = 127 BF16 89 / 104 us).
+// former).  Not in kMergeNoRoom's forms, which have no registers left for them.
 // 2: beta != 0 and empty rows, which are listed apart (see below); the listing costs 2-5 % where there are none, and old values asked for
 // ahead cost it more than they save (R-MAT 2^20, k = 64 FP32 303 / 442 us).
 template <typename T, int V, int J, int MODE>
@@ -188,7 +195,7 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
                   const int* __restrict__ col_idx, const T* __restrict__ vals, const T* __restrict__ B, T* __restrict__ Y,
                   float* __restrict__ tile_carry, float* __restrict__ tile_tail, int2* __restrict__ tile_row, float alpha, float beta) {
   constexpr int U = kMergeUnroll<V, J>, KS = 32 * V * J;
-  constexpr bool LIST = MODE == 2, AHEAD = MODE == 1 && !(V == 1 && J == 4);
+  constexpr bool LIST = MODE == 2, AHEAD = MODE == 1 && !kMergeNoRoom<T, V, J>;
   typedef typename Piece<T, V>::raw raw;
   __shared__ __align__(16) MergeStage<T> stage_s[kMergeWarps][2];
   __shared__ __align__(16) float wide_s[sizeof(T) == 2 ? kMergeWarps : 1][sizeof(T) == 2 ? kMergeWarpItems + 8 : 4];   // BF16: the current share's values widened
