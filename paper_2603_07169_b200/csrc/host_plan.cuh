@@ -187,7 +187,7 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
   const size_t nt = (size_t)I.spmv_tiles;
   const int witems = spmm_share_items(I, dev);
   const long long shares = (m + nnz + witems - 1) / witems;
-  const bool with_shares = shares <= 65536 && m + nnz <= (1 << 23);   // (65536 shares of 128; the pass divides item numbers below 2^23)
+  const bool with_shares = shares <= 65536;   // (m + nnz <= 2^23)
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
   const size_t o_split = 256, o_carry = o_split + up((nt + 1) * 4), o_tail = o_carry + up((nt + 1) * 4), o_share = o_tail + up((nt + 1) * 4),
                total = o_share + (with_shares ? up((size_t)(shares + 1) * 4) : 0);
@@ -208,12 +208,15 @@ int plan_build(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32
   if (rc != B200SP_OK) return fail(rc);
   PlanStats h;
   {
-    int tile_shift = 0;
-    while ((1 << tile_shift) < items) ++tile_shift;   // (1024, 2048 or 4096)
-    const long long blocks = (m + 255) / 256;   // a row per thread, up to 8 blocks per SM
-    const unsigned long long inverse = ((1ULL << 40) + witems - 1) / witems;
-    rc = launch(m > (1 << 17) ? plan_pass_kernel<true> : plan_pass_kernel<false>, dim3((unsigned)(blocks < dev->sms * 8 ? blocks : dev->sms * 8)), dim3(256), stream, nullptr, 0, dev, row_ptr, (int)m,
-                (int)nnz, slot, g_slots.host + slot, tile_shift, (int)nt, p->split_row, with_shares ? witems : 0, inverse, (int)shares, share_split);
+    const SplitRule tile_rule = split_rule(items, (unsigned)nt + 1), share_rule = split_rule(witems, with_shares ? (unsigned)shares + 1 : 0);
+    // The rows write their split points themselves, or every split point is searched.  Rows: up to 2^17 of them (plan_pass_kernel), while a block's
+    // 256 rows hold few, which it writes alone however many blocks there are (creating a plan, search / rows, us: 8 rows of 2 x 10^8 nonzeros
+    // 22 / 204, 200 of 30,000 17 / 33, 500 of 2000 18 / 19; but 2^17 of 16,000, 8 to a row, 38 / 24, 30,000 of 50,000, 24 to a row, 30 / 24).
+    const long long splits = (long long)tile_rule.count + share_rule.count;
+    const bool by_rows = m <= (1 << 17) && splits <= (m >= (1 << 14) ? 32 : 8) * m;
+    const long long work = by_rows || m > splits ? m : splits, blocks = (work + 255) / 256;
+    rc = launch(by_rows ? plan_pass_kernel<false> : plan_pass_kernel<true>, dim3((unsigned)(by_rows || blocks < dev->sms * 8 ? blocks : dev->sms * 8)), dim3(256),
+                stream, nullptr, 0, dev, row_ptr, (int)m, (int)nnz, slot, g_slots.host + slot, tile_rule, p->split_row, share_rule, share_split);
     const cudaError_t e = cudaStreamSynchronize(stream);
     h = g_slots.host[slot];
     if (e == cudaSuccess) plan_slot_give(slot);   // only a finished pass (or none) has left its slot to the next; an error here means a lost device

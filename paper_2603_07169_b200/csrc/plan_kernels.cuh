@@ -42,86 +42,106 @@ __device__ __forceinline__ int merge_split(const int* __restrict__ row_ptr, int 
   return lo;
 }
 
-// Row `row` holds the merge items [u, w): its nonzeros' and its end.  Every split point that lies there has `row` row ends before it: the entries
-// [lo, hi) of `split` get the number of the row.  All lanes of the warp call it; long ranges (rows of many shares) are written by all of them.
-__device__ __forceinline__ void write_splits(int* __restrict__ split, unsigned lo, unsigned hi, int row) {
-  constexpr unsigned FULL = 0xFFFFFFFFu, LONG = 16;
-  if (!__any_sync(FULL, hi > lo)) return;
-  const bool many = hi > lo && hi - lo > LONG;
-  if (!many) for (unsigned t = lo; t < hi; ++t) split[t] = row;
-  for (unsigned left = __ballot_sync(FULL, many); left; left &= left - 1) {
-    const int src = __ffs(left) - 1, r = __shfl_sync(FULL, row, src);
-    const unsigned l = __shfl_sync(FULL, lo, src), h = __shfl_sync(FULL, hi, src);
-    for (unsigned t = l + (threadIdx.x & 31); t < h; t += 32) split[t] = r;
-  }
+// Split points lie before the merge items 0, items, 2 items, ..., the last one behind all of them.
+struct SplitRule {
+  int items;
+  unsigned count;               // number of split points (0: none)
+  unsigned long long inverse;   // ceil(2^40 / items)
+};
+inline SplitRule split_rule(int items, unsigned count) { return {items, count, ((1ULL << 40) + items - 1) / items}; }
+
+// Split points before merge item `item`; those at the items of a row, that is its nonzeros and its end, have the row's number of row ends before
+// them.  Item numbers are divided by a product: exact for powers of two below 2^32 and for 32 .. 128 below 2^29 (shares: m + nnz <= 2^23).
+__device__ __forceinline__ unsigned splits_before(const SplitRule& rule, unsigned item) {
+  const unsigned n = item == 0 ? 0u : (unsigned)(((item - 1u) * rule.inverse) >> 40) + 1u;
+  return n < rule.count ? n : rule.count;
 }
 
 // The plan pass, one launch: min / max row length and the six length bins (rows, nnz per bin), and two sets of merge-path
-// splits (SpMV tiles of 1 << tile_shift items; SpMM shares where share_items > 0).  Every lane adds up its rows, a warp combines its counts with
+// splits (SpMV tiles; SpMM shares where share_rule.count > 0).  Every lane adds up its rows, a warp combines its counts with
 // redux and its first lane adds them to the block's (integer atomics only: the result does not depend on scheduling); the last block to
 // finish writes the statistics to `out`, which is pinned host memory, so that no copy follows.  Latency-bound.
-// SEARCH: a search per split point, a chain of log2(m) loads.  Otherwise the splits fall out of the rows as they are read: the row that holds a
-// split point writes it, which costs every row some arithmetic: up to 2^17 rows.  Cold, search / rows: 4,011 rows 9.9 / 8.2 us, 20,011
+// SEARCH: a search per split point, a chain of log2(m) loads, and four rows in flight per thread.  Otherwise a row per thread (the grid covers
+// them), and the splits fall out of the rows as they are read: the row that holds a split point writes it, which costs every row some
+// arithmetic: up to 2^17 rows that hold few of them (plan_build).  Cold, search / rows: 4,011 rows 9.9 / 8.2 us, 20,011
 // 13.4 / 8.8, 131,072 13.5 / 10.4, 300,000 15.4 / 16.5, 4.2 M 26 / 33 (28.5 with a row at a time; rows with eight in flight per thread 38).
 // (20,011 rows in one block of 1024 threads, which need not meet others in global memory: 43.)
-// share_inverse: ceil(2^40 / share_items); item numbers below 2^23, which is where shares are asked for, are divided exactly by it.
+// Rows of more than 16 split points are left to the warps of the block, of more than 1024 to all of it.
 template <bool SEARCH>
-__global__ void __launch_bounds__(256) plan_pass_kernel(const int* __restrict__ row_ptr, int m, int nnz, int slot_index, PlanStats* out, int tile_shift,
-                                                        int tiles, int* __restrict__ split_row, int share_items, unsigned long long share_inverse, int shares, int* __restrict__ share_split) {
-  constexpr unsigned FULL = 0xFFFFFFFFu;
-  constexpr int R = 4;                           // rows in flight per thread
+__global__ void __launch_bounds__(256) plan_pass_kernel(const int* __restrict__ row_ptr, int m, int nnz, int slot_index, PlanStats* out, const SplitRule tile_rule,
+                                                        int* __restrict__ split_row, const SplitRule share_rule, int* __restrict__ share_split) {
+  constexpr unsigned FULL = 0xFFFFFFFFu, BY_WARP = 16, BY_BLOCK = 1024;
+  constexpr int RANGES = SEARCH ? 1 : 2 * (256 + 1);       // of each set one per row, and what lies behind the last row
   __shared__ unsigned s_rows[6], s_nnz[6];
-  __shared__ int s_short, s_max, s_bad, s_last;
+  __shared__ int s_short, s_max, s_bad, s_last, s_ranges, s_long;
+  __shared__ int4 range_s[RANGES];                         // (first split point, the one behind the last, row, set): by warps from the front, by the block from the back
   PlanSlot* const slot = &g_plan_slots[slot_index];
   if (threadIdx.x < 6) { s_rows[threadIdx.x] = 0; s_nnz[threadIdx.x] = 0; }
-  if (threadIdx.x == 0) { s_short = 0; s_max = 0; s_bad = 0; }
+  if (threadIdx.x == 0) { s_short = 0; s_max = 0; s_bad = 0; s_ranges = 0; s_long = 0; }
   __syncthreads();
   const int lane = threadIdx.x & 31;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  if constexpr (SEARCH) {
-    const long long first_tile = share_items > 0 ? (long long)shares + 1 : 0;      // one search per thread, whichever set it belongs to
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t <= first_tile + tiles; t += stride) {
-      if (t < first_tile) share_split[t] = merge_split(row_ptr, m, nnz, share_items, (int)t);
-      else split_row[t - first_tile] = merge_split(row_ptr, m, nnz, 1 << tile_shift, (int)(t - first_tile));
-    }
-  }
+  const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
   int lshort = 0, lmax = 0, bad = 0;
   unsigned rows[6] = {0, 0, 0, 0, 0, 0}, nz[6] = {0, 0, 0, 0, 0, 0};
-  for (long long base = (long long)blockIdx.x * blockDim.x + threadIdx.x - lane; base < m; base += R * stride) {   // the same turns for a whole warp
-    int from[R], to[R];
+  auto count_row = [&](int len) {
+    if (len < 0) { bad = 1; return; }
+    lshort = max(lshort, 0x7FFFFFFF - len); lmax = max(lmax, len);
+    const int b = length_bin(len);
 #pragma unroll
-    for (int x = 0; x < R; ++x) {
-      const long long i = base + x * stride + lane;
-      from[x] = i < m ? __ldg(row_ptr + i) : 0;
-      to[x] = i < m ? __ldg(row_ptr + i + 1) : 0;
+    for (int j = 0; j < 6; ++j) if (b == j) { rows[j]++; nz[j] += (unsigned)len; }
+  };
+  if constexpr (SEARCH) {
+    const long long first_tile = share_rule.count;           // one search per thread, whichever set it belongs to
+    for (long long t = i0; t < first_tile + tile_rule.count; t += stride) {
+      if (t < first_tile) share_split[t] = merge_split(row_ptr, m, nnz, share_rule.items, (int)t);
+      else split_row[t - first_tile] = merge_split(row_ptr, m, nnz, tile_rule.items, (int)(t - first_tile));
     }
+    constexpr int R = 4;
+    for (long long base = i0; base < m; base += R * stride) {
+      int from[R], to[R];
 #pragma unroll
-    for (int x = 0; x < R; ++x) {
-      const long long i = base + x * stride + lane;
-      if (i - lane >= m) break;
-      const int len = to[x] - from[x];
-      const bool ok = i < m && len >= 0;
-      if (i < m && len < 0) bad = 1;
-      if (ok) {
-        lshort = max(lshort, 0x7FFFFFFF - len); lmax = max(lmax, len);
-        const int b = length_bin(len);
-#pragma unroll
-        for (int j = 0; j < 6; ++j) if (b == j) { rows[j]++; nz[j] += (unsigned)len; }
+      for (int x = 0; x < R; ++x) {
+        const long long i = base + x * stride;
+        from[x] = i < m ? __ldg(row_ptr + i) : 0;
+        to[x] = i < m ? __ldg(row_ptr + i + 1) : 0;
       }
-      if constexpr (SEARCH) continue;
-      // Split t stands before item t * items: in row i if u <= t * items < w, items counted in 32 bits (m + nnz < 2^32).  Row 0 takes what lies
-      // before it and row m - 1 also writes m to what lies behind it, so that every entry is written and in range whatever row_ptr holds.
-      const unsigned u = (unsigned)from[x] + (unsigned)i, w = (unsigned)to[x] + (unsigned)i + 1u;
-      auto write = [&](int* split, unsigned count, auto behind) {      // behind(v): the first split point at or behind item v
-        const unsigned hi = min(behind(w), count);
-        unsigned lo = __shfl_up_sync(FULL, hi, 1);                     // (where the row before ends)
-        if (lane == 0) lo = min(behind(u), count);
-        if (i == 0) lo = 0;
-        write_splits(split, ok ? lo : 0u, ok ? hi : 0u, (int)i);
-        if (i - lane + 32 >= m) write_splits(split, i == m - 1 ? hi : 0u, i == m - 1 ? count : 0u, m);
-      };
-      write(split_row, (unsigned)tiles + 1u, [&](unsigned v) { return v == 0 ? 0u : ((v - 1u) >> tile_shift) + 1u; });
-      if (share_items > 0) write(share_split, (unsigned)shares + 1u, [&](unsigned v) { return v == 0 ? 0u : (unsigned)(((v - 1u) * share_inverse) >> 40) + 1u; });
+#pragma unroll
+      for (int x = 0; x < R; ++x) if (base + x * stride < m) count_row(to[x] - from[x]);
+    }
+  } else {
+    const int i = (int)i0;
+    const bool here = i < m;
+    const int from = here ? __ldg(row_ptr + i) : 0, to = here ? __ldg(row_ptr + i + 1) : 0;
+    if (here) count_row(to - from);
+    const bool ok = here && to >= from;
+    const unsigned u = (unsigned)from + (unsigned)i, w = (unsigned)to + (unsigned)i + 1u;   // the row's items, counted in 32 bits (m + nnz < 2^32)
+    auto put = [&](int* split, int set, unsigned lo, unsigned hi, int row) {
+      if (hi <= lo) return;
+      if (hi - lo <= BY_WARP) { for (unsigned t = lo; t < hi; ++t) split[t] = row; }
+      else range_s[hi - lo <= BY_BLOCK ? atomicAdd(&s_ranges, 1) : RANGES - 1 - atomicAdd(&s_long, 1)] = make_int4((int)lo, (int)hi, row, set);
+    };
+    auto write = [&](const SplitRule& rule, int* split, int set) {
+      const unsigned hi = splits_before(rule, w);
+      unsigned lo = __shfl_up_sync(FULL, hi, 1);             // (where the row before ends)
+      if (lane == 0) lo = splits_before(rule, u);
+      if (i == 0) lo = 0;
+      if (ok) put(split, set, lo, hi, i);
+      if (ok && i == m - 1) put(split, set, hi, rule.count, m);
+    };
+    write(tile_rule, split_row, 0);
+    if (share_rule.count) write(share_rule, share_split, 1);
+    __syncthreads();
+    const int ranges = s_ranges, longer = s_long;
+    for (int r = threadIdx.x >> 5; r < ranges; r += 8) {
+      const int4 e = range_s[r];
+      int* const split = e.w ? share_split : split_row;
+      for (unsigned t = (unsigned)e.x + lane; t < (unsigned)e.y; t += 32) split[t] = e.z;
+    }
+    for (int r = 0; r < longer; ++r) {
+      const int4 e = range_s[RANGES - 1 - r];
+      int* const split = e.w ? share_split : split_row;
+#pragma unroll 4
+      for (unsigned t = (unsigned)e.x + threadIdx.x; t < (unsigned)e.y; t += 256) split[t] = e.z;
     }
   }
   lshort = __reduce_max_sync(FULL, lshort); lmax = __reduce_max_sync(FULL, lmax); bad = __any_sync(FULL, bad);
