@@ -97,6 +97,11 @@ int b200sp_get_option(const char* name, int* value);
  * under the present switches, 0 if not; B kept in shared memory (few columns of A) comes before it.  A rule of the host: no device needed. */
 int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, float beta, int dtype);
 
+/* The plan pass's split points as it takes them from the rows: out[t] = row ends before merge item t * items of the merge of the m row ends with the
+ * nnz nonzeros, for t = 0 .. ceil((m + nnz) / items).  `items` a power of two from 32 on, or anything from 32 to 128 while m + nnz < 2^29; row_ptr (m + 1
+ * ascending entries) and out are host pointers.  Arithmetic of the host: no device needed. */
+int b200sp_split_points(int64_t m, int64_t nnz, const int32_t* row_ptr, int items, int32_t* out);
+
 /* ---- measurement probes (no counterpart in the paper's operations) ----------------------------------------------
  * Each enqueues one kernel that does nothing but the access pattern named, so that the caller, timing it with events,
  * gets the hardware rate that bounds the corresponding library kernel.  All pointers are device pointers; `sink` is

@@ -21,7 +21,7 @@ EXPORTS = (
     "spmv_csr", "spmm_csr", "b200sp_plan_create", "b200sp_plan_destroy", "b200sp_plan_info", "b200sp_spmv",
     "b200sp_spmm", "spmv_csr_host", "spmm_csr_host", "b200sp_validate_csr", "b200sp_cache_clear",
     "b200sp_status_string", "b200sp_last_cuda_error", "b200sp_version", "b200sp_checked_build", "b200sp_launch_count", "b200sp_set_option", "b200sp_get_option",
-    "b200sp_check", "b200sp_cache_drop", "spmv_csr_noalloc", "b200sp_noalloc_max_items", "b200sp_probe_gather", "b200sp_probe_gather_ex", "b200sp_probe_stream", "b200sp_probe_lines", "b200sp_probe_spmv_gather", "b200sp_spmv_naive", "b200sp_spmm_naive", "spmv_coo", "spmm_coo", "spmv_ell", "spmm_ell", "spmv_csc", "spmm_csc", "spmv_csr_vec_host", "b200sp_spmm_by_shares",
+    "b200sp_check", "b200sp_cache_drop", "spmv_csr_noalloc", "b200sp_noalloc_max_items", "b200sp_probe_gather", "b200sp_probe_gather_ex", "b200sp_probe_stream", "b200sp_probe_lines", "b200sp_probe_spmv_gather", "b200sp_spmv_naive", "b200sp_spmm_naive", "spmv_coo", "spmm_coo", "spmv_ell", "spmm_ell", "spmv_csc", "spmm_csc", "spmv_csr_vec_host", "b200sp_spmm_by_shares", "b200sp_split_points",
 )
 
 
@@ -112,6 +112,8 @@ def lib() -> ctypes.CDLL:
         L.b200sp_get_option.restype = i32
         L.b200sp_spmm_by_shares.argtypes = [ctypes.POINTER(PlanInfo), i64, f32, i32]
         L.b200sp_spmm_by_shares.restype = i32
+        L.b200sp_split_points.argtypes = [i64, i64, p, i32, p]
+        L.b200sp_split_points.restype = i32
         L.b200sp_check.argtypes = [p]
         L.b200sp_check.restype = i32
         for name in ("spmv_csr", "spmm_csr", "spmv_csr_host", "spmm_csr_host", "b200sp_plan_create", "b200sp_plan_destroy",
@@ -474,6 +476,13 @@ def b200sp_spmm_by_shares(info: dict, k, beta, dtype) -> bool:
     """Whether SpMM with k columns on a matrix with these row statistics (b200sp_plan_info) takes the nnz-balanced kernel."""
     I = PlanInfo(**{name: (ctypes.c_int64 * 6)(*info[name]) if name.startswith("bin_") else info[name] for name, _ in PlanInfo._fields_ if name in info})
     return bool(lib().b200sp_spmm_by_shares(ctypes.byref(I), k, beta, _dt(dtype)))
+
+
+def b200sp_split_points(m, nnz, row_ptr, items, out):
+    """Row ends before every `items`-th merge item, as the plan pass takes them from the rows (contiguous int32 numpy arrays on the host)."""
+    if row_ptr.dtype.str[1:] != "i4" or out.dtype.str[1:] != "i4" or row_ptr.size < m + 1 or out.size < (m + nnz + items - 1) // items + 1:
+        raise ValueError("row_ptr and out are int32 arrays of m + 1 and ceil((m + nnz) / items) + 1 entries")
+    _ck(lib().b200sp_split_points(m, nnz, row_ptr.ctypes.data, items, out.ctypes.data), "b200sp_split_points")
 
 
 def b200sp_spmv(plan, col_idx, vals, x, y, alpha, beta, dtype, stream=None):

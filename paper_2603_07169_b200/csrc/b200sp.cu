@@ -150,6 +150,18 @@ int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, float beta,
   return info && spmm_by_shares(*info, k, dtype == B200SP_F32 ? 4 : 2, beta);
 }
 
+int b200sp_split_points(int64_t m, int64_t nnz, const int32_t* row_ptr, int items, int32_t* out) {
+  if (check_sizes(m, m, nnz) != B200SP_OK || m == 0 || !row_ptr || !out || items < 32 || ((items & (items - 1)) != 0 && (items > 128 || m + nnz >= 1 << 29))) return B200SP_ERR_INVALID_ARG;
+  const SplitRule rule = split_rule(items, (unsigned)((m + nnz + items - 1) / items) + 1);
+  for (int64_t i = 0; i < m; ++i) {
+    unsigned lo, hi;
+    row_splits(rule, row_ptr[i], row_ptr[i + 1], (int)i, (int)nnz, &lo, &hi);
+    for (unsigned t = i == 0 ? 0 : lo; t < hi; ++t) out[t] = (int32_t)i;
+    for (unsigned t = hi; i == m - 1 && t < rule.count; ++t) out[t] = (int32_t)m;
+  }
+  return B200SP_OK;
+}
+
 int spmv_csr(int64_t m, int64_t n, int64_t nnz, const int32_t* row_ptr, const int32_t* col_idx, const void* vals, const void* x,
              void* y, float alpha, float beta, int dtype, void* stream) {
   int rc = check_sizes(m, n, nnz);

@@ -50,11 +50,19 @@ struct SplitRule {
 };
 inline SplitRule split_rule(int items, unsigned count) { return {items, count, ((1ULL << 40) + items - 1) / items}; }
 
-// Split points before merge item `item`; those at the items of a row, that is its nonzeros and its end, have the row's number of row ends before
-// them.  Item numbers are divided by a product: exact for powers of two below 2^32 and for 32 .. 128 below 2^29 (shares: m + nnz <= 2^23).
-__device__ __forceinline__ unsigned splits_before(const SplitRule& rule, unsigned item) {
+// The split points [*lo, *hi) lie at the merge items of row `row`, that is its nonzeros [from, to) and its end (those before row 0 too): they have
+// `row` row ends before them.  Offsets outside [0, nnz] are taken as the nearer end of that range, which is what the bounds of merge_split's
+// search amount to, so that a share's nonzeros stay within nnz whatever ascending row_ptr holds.
+// Item numbers are divided by a product: exact for powers of two below 2^32 and for 32 .. 128 below 2^29 (shares: m + nnz <= 2^23).
+__host__ __device__ __forceinline__ unsigned splits_before(const SplitRule& rule, unsigned item) {
   const unsigned n = item == 0 ? 0u : (unsigned)(((item - 1u) * rule.inverse) >> 40) + 1u;
   return n < rule.count ? n : rule.count;
+}
+__host__ __device__ __forceinline__ void row_splits(const SplitRule& rule, int from, int to, int row, int nnz, unsigned* lo, unsigned* hi) {
+  from = from < 0 ? 0 : from > nnz ? nnz : from;
+  to = to < 0 ? 0 : to > nnz ? nnz : to;
+  *lo = row == 0 ? 0u : splits_before(rule, (unsigned)from + (unsigned)row);
+  *hi = splits_before(rule, (unsigned)to + (unsigned)row + 1u);
 }
 
 // The plan pass, one launch: min / max row length and the six length bins (rows, nnz per bin), and two sets of merge-path
@@ -114,22 +122,21 @@ __global__ void __launch_bounds__(256) plan_pass_kernel(const int* __restrict__ 
     const int from = here ? __ldg(row_ptr + i) : 0, to = here ? __ldg(row_ptr + i + 1) : 0;
     if (here) count_row(to - from);
     const bool ok = here && to >= from;
-    const unsigned u = (unsigned)from + (unsigned)i, w = (unsigned)to + (unsigned)i + 1u;   // the row's items, counted in 32 bits (m + nnz < 2^32)
     auto put = [&](int* split, int set, unsigned lo, unsigned hi, int row) {
       if (hi <= lo) return;
       if (hi - lo <= BY_WARP) { for (unsigned t = lo; t < hi; ++t) split[t] = row; }
       else range_s[hi - lo <= BY_BLOCK ? atomicAdd(&s_ranges, 1) : RANGES - 1 - atomicAdd(&s_long, 1)] = make_int4((int)lo, (int)hi, row, set);
     };
     auto write = [&](const SplitRule& rule, int* split, int set) {
-      const unsigned hi = splits_before(rule, w);
-      unsigned lo = __shfl_up_sync(FULL, hi, 1);             // (where the row before ends)
-      if (lane == 0) lo = splits_before(rule, u);
-      if (i == 0) lo = 0;
-      if (ok) put(split, set, lo, hi, i);
-      if (ok && i == m - 1) put(split, set, hi, rule.count, m);
+      unsigned lo, hi;
+      row_splits(rule, from, to, i, nnz, &lo, &hi);
+      put(split, set, lo, hi, i);
+      if (i == m - 1) put(split, set, hi, rule.count, m);
     };
-    write(tile_rule, split_row, 0);
-    if (share_rule.count) write(share_rule, share_split, 1);
+    if (ok) {
+      write(tile_rule, split_row, 0);
+      if (share_rule.count) write(share_rule, share_split, 1);
+    }
     __syncthreads();
     const int ranges = s_ranges, longer = s_long;
     for (int r = threadIdx.x >> 5; r < ranges; r += 8) {
