@@ -28,8 +28,11 @@ extern "C" {
  *                    128, a quarter or more of the rows empty, or a longest row far above the mean; with few columns only where the
  *                    rows differ enough, b200sp_spmm_by_shares) or k > 16 is no multiple of 16 bytes (default)
  *   "spmm_stage_a"   the k-sliced SpMM kernel's warps first copy their rows' (col, val) pairs into shared memory: 1 = yes, 0 = no,
- *                    2 = for BF16 storage only (default: measured 5-6 % faster there and 2-3 % slower for FP32), and not where
- *                    rows of B come in whole pieces of 32 bytes and are at least 128 wide: there four lanes share a row
+ *                    2 = for BF16 storage only (default: measured 5-6 % faster there and 2-3 % slower for FP32), and there a kernel
+ *                    with four lanes a row and 32 bytes of B per load instead, without staging, where it is faster: k a multiple
+ *                    of 16 from 64 on, B aligned to 32 bytes, and row lengths and sizes as b200sp_spmm_wide_pieces has them
+ *                    (rows all of one length that is a multiple of four; others while a slice of B takes less than half of L2,
+ *                    but not very small calls; longer ones not where their blocks fill little more than one wave)
  *   "spmm_ranges"    k-sliced SpMM on rows with ascending columns, one launch per column range so that the rows of B a
  *                    launch gathers from stay in L2: 1 = no ranges (default: measured slower, see the benchmarks' record),
  *                    0 = as many as make a range of B fit L2, 2, 3, 4 or 8 = that many
@@ -96,6 +99,10 @@ int b200sp_get_option(const char* name, int* value);
 /* 1 if SpMM with k columns on a matrix with these row statistics (b200sp_plan_info) goes by equal shares of rows + nonzeros per warp
  * under the present switches, 0 if not; B kept in shared memory (few columns of A) comes before it.  A rule of the host: no device needed. */
 int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, float beta, int dtype);
+
+/* 1 if BF16 SpMM by rows with k columns and a B aligned to 32 bytes takes the kernel with 32 bytes of B per load and four lanes a row, on a device
+ * with that many SMs and bytes of L2, under the present switches, 0 if not ("spmm_stage_a").  A rule of the host: no device needed. */
+int b200sp_spmm_wide_pieces(const b200sp_plan_info_t* info, int64_t k, int sms, int64_t l2_bytes);
 
 /* The plan pass's split points as it takes them from the rows: out[t] = row ends before merge item t * items of the merge of the m row ends with the
  * nnz nonzeros, for t = 0 .. ceil((m + nnz) / items).  `items` a power of two from 32 on, or anything from 32 to 128 while m + nnz < 2^29; row_ptr (m + 1

@@ -150,6 +150,10 @@ int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, float beta,
   return info && spmm_by_shares(*info, k, dtype == B200SP_F32 ? 4 : 2, beta);
 }
 
+int b200sp_spmm_wide_pieces(const b200sp_plan_info_t* info, int64_t k, int sms, int64_t l2_bytes) {
+  return info && sms > 0 && k >= 64 && k % 16 == 0 && g_opt.spmm_stage_a == 2 && spmm_wide_pieces(*info, k, sms, l2_bytes);
+}
+
 int b200sp_split_points(int64_t m, int64_t nnz, const int32_t* row_ptr, int items, int32_t* out) {
   if (check_sizes(m, m, nnz) != B200SP_OK || m == 0 || !row_ptr || !out || items < 32 || ((items & (items - 1)) != 0 && (items > 128 || m + nnz >= 1 << 29))) return B200SP_ERR_INVALID_ARG;
   const SplitRule rule = split_rule(items, (unsigned)((m + nnz + items - 1) / items) + 1);

@@ -65,7 +65,7 @@ struct Options {
   int spmm_sliced = 1;     // 1 = k-sliced SpMM kernel (default), 0 = one pass over all of k
   int sub_lanes = 0;       // lanes per row of the sub-warp kernel (0 = from the mean row length)
   int merge_empty = 0;     // 1 = when a quarter or more of the rows have no nonzeros the merge list holds only the others, 0 = every row is a merge item (default: measured 3 % slower on the power-law workload, where the extra pass over y costs more than the skipped items save)
-  int spmm_stage_a = 2;    // the k-sliced SpMM kernel's warps stage their rows' (col, val) pairs in shared memory: 1 = yes, 0 = no (broadcast loads from global memory), 2 = for BF16 storage only, and 32 bytes of B per lane instead where it is aligned so (default)
+  int spmm_stage_a = 2;    // the k-sliced SpMM kernel's warps stage their rows' (col, val) pairs in shared memory: 1 = yes, 0 = no (broadcast loads from global memory), 2 = for BF16 storage only, or 32 bytes of B per lane instead where spmm_wide_pieces says so (default)
   int spmm_flat = 2;       // nnz-balanced SpMM kernel (equal shares of rows + nonzeros per warp): 1 = always, 0 = never, 2 = when the rows are uneven or a wide k is no multiple of 16 bytes (default)
   int spmm_ranges = 1;     // column ranges per slice of the k-sliced SpMM kernel with sorted columns: 1 = none (default), 0 = as many as make a range of B fit L2, 2, 3, 4, 8 = forced
   int merge_short = 32;    // rows up to this many products are added by one thread (8, 16, 32, 64)

@@ -387,6 +387,29 @@ bool spmm_by_shares(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, floa
   return spmm_rows_are_uneven(I) && !spmm_uneven_by_rows(I, k, elem_bytes, beta);
 }
 
+// Even rows of A, BF16, rows of B in whole 32-byte pieces and at least 64 columns of them (narrower slices, 16 / 32 bytes a lane on 2^18 rows: k = 32
+// 31.8 / 33.6 us, k = 16 24.1 / 26.6 us): whether four lanes a row with 32 bytes of B per load (spmm_slice_wide_kernel) are faster than eight with 16
+// and staged pairs.  Per nonzero they are; what they lose by are single steps, which rows take up to a multiple of four nonzeros at both ends
+// ("quads": no row does), and half as many warps where few blocks are left.  Times: 16 / 32 bytes a lane, us; waves: blocks over those resident.
+// - Other rows than quads only while a slice of B takes less than half of L2, where loads do not wait for memory (rows of 13, k = 64: 350,000 of them
+//   78.1 / 74.5, 450,000 102.9 / 100.6, 550,000 130 / 132, 2^20 286 / 303; rows of 6, 550,000 86.0 / 88.4; but 2^20 rows of 16, k = 128 514 / 491).
+// - Other rows than quads of up to 25 nonzeros: the shorter ones from a quarter of a wave on (8000 of 5 to 15, k = 64 5.1 / 5.2; 20,000 9.6 / 7.4),
+//   and those of less than 5 and mixed lengths up to three waves (100,000 of 2 to 6, k = 64 16.2 / 14.8, k = 128 31.3 / 32.2).
+// - Of 26 to 32: where the blocks are one wave or many (20,000 of 20 to 36, k = 64 16.5 / 14.3, k = 128 18.5 / 20.2; 100,000, k = 192 103 / 99).
+// - Rows of more than 32, whose pairs the staged kernel's warps read from memory as well: quads, and rows of clearly different lengths, except where
+//   blocks wait for a second or a third wave (k = 128, 26,000 rows of 64 32.1 / 36.8, 16,000 23.8 / 21.5, 54,000 59.4 / 53.8; 20,000 of 64 to 128,
+//   k = 192 65.4 / 71.5, 100,000 282 / 247); not others of one length (20,000 of 33, k = 256 31.5 / 35.3, of 65 53.9 / 61.5).
+bool spmm_wide_pieces(const b200sp_plan_info_t& I, int64_t k, int sms, int64_t l2_bytes) {
+  const bool equal = I.min_row_len == I.max_row_len, quads = equal && I.max_row_len % 4 == 0;
+  if (!quads && (double)I.n * 128.0 > 0.45 * (double)l2_bytes) return false;
+  const double mean = I.m > 0 ? (double)I.nnz / (double)I.m : 0.0;
+  const double waves = (double)((k + 63) / 64) * (double)((I.m + 31) / 32) / (8.0 * sms);      // 64 columns, 32 rows a block; eight of them per SM
+  if (quads && I.max_row_len <= 32) return true;
+  if (!quads && mean <= 25.0) return (waves >= 0.25 || mean >= 20.0) && (equal || mean >= 5.0 || waves <= 3.0);
+  if (!quads && mean <= 32.0) return waves <= 1.0 || waves >= 4.0;
+  return (quads || 2 * I.max_row_len >= 3 * I.min_row_len) && (waves <= 1.0 || waves >= 2.6);
+}
+
 template <typename T, int V, int J, int MODE>
 int launch_spmm_merge_as(b200sp_plan* p, const b200sp_plan::Shares& work, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
                       cudaStream_t stream, DeviceInfo* dev) {
@@ -526,13 +549,7 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     int rc = plan_row_lists(p, &lists, &own_lists, stream, dev);
     if (rc != B200SP_OK) return rc;
     const int mid_blocks = (p->num_medium + GROUPS - 1) / GROUPS;
-    // BF16 rows of B in whole 32-byte pieces: 32 bytes a lane from 64 columns on (narrower slices, 16 / 32 bytes a lane on 2^18 rows: k = 32 31.8 /
-    // 33.6 us, k = 16 24.1 / 26.6 us).  Rows that do not all begin and end on a multiple of four nonzeros take single steps there, which with half
-    // as many warps cost more than the loads save once the loads wait for memory: they go this way while a slice of B takes less than half of L2
-    // (rows of 13, k = 64: 350,000 of them 78.1 / 74.5 us, 450,000 102.9 / 100.6, 550,000 130 / 132, 2^20 286 / 303; rows of 6, 550,000 86.0 / 88.4;
-    // but 2^20 rows of 16, k = 128 514 / 491).
-    const bool wide = sizeof(T) == 2 && lanes == 8 && g_opt.spmm_stage_a == 2 && k % 16 == 0 && ((uintptr_t)B & 31) == 0 &&
-                      ((double)I.n * 128.0 <= 0.45 * (double)dev->l2_bytes || (I.min_row_len == I.max_row_len && I.max_row_len % 4 == 0));
+    const bool wide = sizeof(T) == 2 && lanes == 8 && g_opt.spmm_stage_a == 2 && k % 16 == 0 && ((uintptr_t)B & 31) == 0 && spmm_wide_pieces(I, k, dev->sms, dev->l2_bytes);
     int ranges = 1;
     if (lanes == 8) {
       rc = spmm_column_ranges(p, col_idx, 8 * 16, stream, dev, &ranges);

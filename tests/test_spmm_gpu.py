@@ -105,18 +105,31 @@ def test_b_slice_in_shared_memory(n, k, dtype):
     b200sp.b200sp_check()
 
 
+def takes_wide_pieces(A, k):
+    import torch
+    from gpu_util import to_dev
+    device = torch.cuda.get_device_properties(0)
+    plan = b200sp.b200sp_plan_create(A.m, A.n, A.nnz, to_dev(A.row_ptr))
+    stats = b200sp.b200sp_plan_info(plan)
+    b200sp.b200sp_plan_destroy(plan)
+    return not b200sp.b200sp_spmm_by_shares(stats, k, 0.0, "bf16") and b200sp.b200sp_spmm_wide_pieces(stats, k, device.multi_processor_count, device.L2_cache_size)
+
+
 @pytest.mark.parametrize("k", [64, 80, 128, 256, 272])
-@pytest.mark.parametrize("case", ["even", "few_rows", "some_long"])
+@pytest.mark.parametrize("case", ["even", "few_rows", "some_long", "many", "quads", "long_quads"])
 def test_bf16_rows_of_b_in_pieces_of_32_bytes(case, k):
     """Four lanes per row and 32 bytes of B per load where B and its rows are aligned to 32 bytes: the same sums in the same order as the kernel
     with 16 bytes a lane, which also takes a B that is only aligned to 16 bytes; so the results are equal bit for bit.  Row lengths of every
-    remainder modulo four, a last block that is not full, a last slice that is not full, rows of more than 128 nonzeros, beta != 0."""
+    remainder modulo four, a last block that is not full, a last slice that is not full, rows of more than 128 nonzeros, beta != 0; and two cases
+    too small for it (one of them up to 128 columns), where all calls take 16 bytes a lane."""
     import torch
     from gpu_util import to_dev
     rng = np.random.default_rng(k)
-    lens = {"even": rng.integers(9, 17, 3001), "few_rows": np.array([5, 6, 7]), "some_long": np.concatenate([rng.integers(30, 40, 2000), [129, 140]])}[case]
+    lens = {"even": rng.integers(9, 17, 3001), "few_rows": np.array([5, 6, 7]), "some_long": np.concatenate([rng.integers(30, 40, 2000), [129, 140]]),
+            "many": rng.integers(5, 17, 20_011), "quads": np.full(3001, 8), "long_quads": np.full(1001, 100)}[case]
     m, n = len(lens), 20_000
     A = gen.random_csr(m, n, lens, seed=k, sort_cols=False)
+    assert takes_wide_pieces(A, k) == (case not in ("even", "few_rows") or (case == "even" and k >= 256))
     B, Y0, vals = rng.standard_normal(n * k).astype(np.float32), rng.standard_normal(m * k).astype(np.float32), gen.to_bf16(A.vals)
     d = [to_dev(a) for a in (A.row_ptr, A.col_idx, vals)]
     odd = torch.zeros(n * k + 8, dtype=torch.int16, device="cuda:0")[8:]
@@ -136,6 +149,31 @@ def test_bf16_rows_of_b_in_pieces_of_32_bytes(case, k):
         Y_ref, S = oracle.spmm_csr(m, n, k, A.row_ptr, A.col_idx, vals, gen.to_bf16(B), gen.to_bf16(Y0), alpha, beta, "bf16")
         assert_within(outs[0].cpu().numpy().view(np.uint16).reshape(m, k), Y_ref, S, "bf16", abs(alpha),
                       np.abs(beta * gen.bf16_to_f32(gen.to_bf16(Y0)).astype(np.float64)).reshape(m, k), what="%s k=%d" % (case, k))
+    b200sp.b200sp_cache_clear()
+
+
+@pytest.mark.parametrize("length,wide", [(8, True), (7, False)])
+def test_bf16_rows_of_a_b_larger_than_l2_in_pieces_of_32_bytes(length, wide):
+    """A slice of B above 0.45 of L2: 32 bytes a lane only for rows of whole groups of four."""
+    import torch
+    from gpu_util import to_dev
+    m, n, k = 20_011, 500_000, 64
+    A = gen.random_csr(m, n, np.full(m, length), seed=length, sort_cols=False)
+    assert takes_wide_pieces(A, k) == wide
+    vals, B = gen.to_bf16(A.vals), gen.to_bf16(np.random.default_rng(0).standard_normal(n * k).astype(np.float32))
+    d = [to_dev(a) for a in (A.row_ptr, A.col_idx, vals, B)]
+    outs = []
+    for stage_a in (2, 1):
+        b200sp.b200sp_set_option("spmm_stage_a", stage_a)
+        try:
+            outs.append(torch.zeros(m * k, dtype=torch.int16, device="cuda:0"))
+            b200sp.spmm_csr(m, n, A.nnz, k, *d, outs[-1], 1.0, 0.0, "bf16")
+        finally:
+            b200sp.b200sp_set_option("spmm_stage_a", 2)
+    assert torch.equal(outs[0], outs[1])
+    rows = np.arange(0, m, 50)
+    Y_ref, S = oracle.spmm_csr(m, n, k, A.row_ptr, A.col_idx, vals, B, None, 1.0, 0.0, "bf16", rows=rows)
+    assert_within(outs[0].cpu().numpy().view(np.uint16).reshape(m, k)[rows], Y_ref, S, "bf16", what="rows of %d" % length)
     b200sp.b200sp_cache_clear()
 
 

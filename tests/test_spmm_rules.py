@@ -37,3 +37,35 @@ def test_uneven_rows_and_few_columns(stats, f32, bf16, beta):
             assert not b200sp.b200sp_spmm_by_shares(stats, k, beta, dtype), (dtype, k)
         for k in (17, 20, 23, 40, 64) if by_rows else (2, 3, 4, 5, 8, 12, 16, 17, 24, 32, 64):
             assert b200sp.b200sp_spmm_by_shares(stats, k, beta, dtype), (dtype, k)
+
+
+SMS, L2 = 148, 126 << 20
+
+
+@pytest.mark.parametrize("m,n,k,shortest,longest,mean,wide", [
+    # measured on both sides; rows all of one length that is a multiple of four, of any number and over a B of any size
+    (1 << 19, 1 << 19, 256, 32, 32, 32, True), (8000, 8192, 64, 4, 4, 4, True), (1 << 20, 1 << 20, 128, 16, 16, 16, True),
+    # other lengths: while a slice of B takes less than half of L2
+    (350_000, 350_000, 64, 13, 13, 13, True), (550_000, 550_000, 64, 13, 13, 13, False),
+    (464_000, 464_000, 64, 13, 13, 13, True), (465_000, 465_000, 64, 13, 13, 13, False),
+    # short ones: not in less than a quarter of a wave, nor of less than five nonzeros in more than three waves
+    (8000, 8192, 64, 5, 15, 10, False), (20_000, 20_000, 64, 5, 15, 10, True), (100_000, 100_000, 64, 2, 6, 4, True), (100_000, 100_000, 128, 2, 6, 4, False),
+    (8000, 8192, 64, 25, 25, 25, True),
+    (200_000, 200_000, 256, 1, 1, 1, True),
+    # of 26 to 32: in one wave or in many
+    (20_000, 20_000, 64, 20, 36, 28, True), (20_000, 20_000, 128, 20, 36, 28, False), (16_384, 16_384, 192, 30, 30, 30, False),
+    (100_000, 100_000, 192, 20, 36, 28, True), (20_000, 20_000, 128, 12, 30, 21, True),
+    # of more than 32: no odd ones of one length, others not in a second or third wave
+    (20_000, 20_000, 256, 65, 65, 65, False), (200_000, 200_000, 64, 33, 33, 33, False), (16_000, 16_000, 128, 64, 64, 64, True),
+    (26_000, 26_000, 128, 64, 64, 64, False), (54_000, 54_000, 128, 64, 64, 64, True), (20_000, 20_000, 192, 64, 128, 96, False),
+    (100_000, 100_000, 192, 64, 128, 96, True), (200_000, 200_000, 128, 32, 32, 32, True), (26_000, 26_000, 128, 32, 32, 32, True),
+    # widths that are no whole pieces, or too few of them
+    (50_000, 50_000, 72, 16, 16, 16, False), (50_000, 50_000, 48, 16, 16, 16, False), (50_000, 50_000, 80, 16, 16, 16, True)])
+def test_rows_of_b_in_pieces_of_32_bytes(m, n, k, shortest, longest, mean, wide):
+    stats = dict(info(m, n, [0, 0, m, 0, 0, 0], [0, 0, m * mean, 0, 0, 0], longest), min_row_len=shortest)
+    assert b200sp.b200sp_spmm_wide_pieces(stats, k, SMS, L2) == wide
+    b200sp.b200sp_set_option("spmm_stage_a", 1)
+    try:
+        assert not b200sp.b200sp_spmm_wide_pieces(stats, k, SMS, L2)
+    finally:
+        b200sp.b200sp_set_option("spmm_stage_a", 2)
