@@ -126,8 +126,7 @@ int spmm_csr(int64_t m, int64_t n, int64_t nnz, int64_t k, const int32_t* row_pt
  * 3 .. 64, else the merge-tile kernel.  That first call must not be captured.
  * It takes one block of a few bytes per tile from the library's pool, in the order of `stream`, and
  * synchronises `stream` once, so a capturing stream is refused (B200SP_ERR_UNSUPPORTED; the capture stays valid).  A plan may be used from one stream at a time.  b200sp_plan_destroy
- * returns the plan's memory in stream order, without waiting, when the plan was made and used on the default stream (NULL) alone;
- * otherwise it synchronises the plan's device first. */
+ * synchronises the plan's device before it returns the block. */
 int b200sp_plan_create(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, const int32_t* row_ptr, void* stream);
 int b200sp_plan_destroy(b200sp_plan* plan);
 int b200sp_plan_info(const b200sp_plan* plan, b200sp_plan_info_t* out); /* `out` is a host pointer */

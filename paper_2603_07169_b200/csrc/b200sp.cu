@@ -91,25 +91,10 @@ int b200sp_plan_create(b200sp_plan** out, int64_t m, int64_t n, int64_t nnz, con
   int rc = check_sizes(m, n, nnz);
   if (rc != B200SP_OK) return rc;
   if (m > 0 && (!row_ptr || !aligned4(row_ptr))) return B200SP_ERR_INVALID_ARG;
-  rc = plan_build(out, m, n, nnz, row_ptr, (cudaStream_t)stream);
-  if (rc == B200SP_OK) (*out)->default_stream_only.store(stream == nullptr, std::memory_order_relaxed);
-  return rc;
+  return plan_build(out, m, n, nnz, row_ptr, (cudaStream_t)stream);
 }
 
-// A plan that only the default stream has seen gives its memory back in the order of that stream and does not wait: the stream outlives every
-// plan, and whatever comes next on it comes behind the plan's kernels (a plan per product: 20,011 uneven rows, k = 128 45.8 -> 38.7 us a
-// pass, 4,011 rows, k = 64 BF16 35.5 -> 26.7 us; the wait kept the next plan pass from being queued behind the product).  Other streams may
-// be gone by now, so there the device is synchronised.
-int b200sp_plan_destroy(b200sp_plan* plan) {
-  if (!plan || !plan->default_stream_only.load(std::memory_order_relaxed)) return plan_free(plan);
-  const int device = plan->device;
-  int cur = device;
-  CU(cudaGetDevice(&cur));
-  if (cur != device) CU(cudaSetDevice(device));
-  const int rc = plan_free(plan, true, nullptr);
-  if (cur != device) CU(cudaSetDevice(cur));
-  return rc;
-}
+int b200sp_plan_destroy(b200sp_plan* plan) { return plan_free(plan); }
 
 int b200sp_plan_info(const b200sp_plan* plan, b200sp_plan_info_t* out) {
   if (!plan || !out) return B200SP_ERR_INVALID_ARG;
@@ -126,7 +111,6 @@ int b200sp_spmv(b200sp_plan* plan, const int32_t* col_idx, const void* vals, con
   if (rc != B200SP_OK) return rc;
   rc = checked_build_validate(plan, col_idx, stream);
   if (rc != B200SP_OK) return rc;
-  if (stream) plan->default_stream_only.store(false, std::memory_order_relaxed);
   if (dtype == B200SP_F32) return run_spmv<float>(plan, col_idx, (const float*)vals, (const float*)x, (float*)y, alpha, beta, (cudaStream_t)stream, dev);
   return run_spmv<bf16_t>(plan, col_idx, (const bf16_t*)vals, (const bf16_t*)x, (bf16_t*)y, alpha, beta, (cudaStream_t)stream, dev);
 }
@@ -141,7 +125,6 @@ int b200sp_spmm(b200sp_plan* plan, int64_t k, const int32_t* col_idx, const void
   if (rc != B200SP_OK) return rc;
   rc = checked_build_validate(plan, col_idx, stream);
   if (rc != B200SP_OK) return rc;
-  if (stream) plan->default_stream_only.store(false, std::memory_order_relaxed);
   if (dtype == B200SP_F32) return run_spmm<float, 4>(plan, (int)k, col_idx, (const float*)vals, (const float*)B, (float*)Y, alpha, beta, (cudaStream_t)stream, dev);
   return run_spmm<bf16_t, 8>(plan, (int)k, col_idx, (const bf16_t*)vals, (const bf16_t*)B, (bf16_t*)Y, alpha, beta, (cudaStream_t)stream, dev);
 }

@@ -259,7 +259,6 @@ int check_sizes(int64_t m, int64_t n, int64_t nnz) {
 
 struct b200sp_plan {
   int device = 0;
-  std::atomic<bool> default_stream_only{false};   // made and used on the legacy default stream alone (plans of b200sp_plan_create)
   const int32_t* row_ptr = nullptr;
   b200sp_plan_info_t info = {};
   void* block = nullptr;              // one allocation from the library's pool that holds every array below

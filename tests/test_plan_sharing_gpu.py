@@ -129,8 +129,8 @@ def test_first_call_captured(case, dtype):
 
 @pytest.mark.parametrize("side_stream", [False, True])
 def test_a_plan_destroyed_behind_its_product(side_stream):
-    """A new pattern in every step, nothing waited for: the memory that a plan gives back is the next plan's at once, and each product is done
-    with it by then.  With a plan also used on another stream, destroying it waits for the device."""
+    """A new pattern in every step, nothing waited for between the calls: the memory that a plan gives back is the next plan's at once, and each
+    product is done with it by then."""
     P, side = Problem("lists"), torch.cuda.Stream()
     others = [gen.random_csr(20_000 + 100 * i, 20_000, np.random.default_rng(i).integers(0, 30, 20_000 + 100 * i), seed=i) for i in range(3)]
     try:
@@ -151,3 +151,25 @@ def test_a_plan_destroyed_behind_its_product(side_stream):
         assert all(torch.equal(a, b) for a, b in zip(first, outs))
     finally:
         P.close()
+
+
+@pytest.mark.parametrize("side_stream", [False, True])
+def test_nothing_is_in_flight_once_a_plan_is_destroyed(side_stream):
+    """b200sp_plan_destroy waits for the device: from then on another stream, or the host, may read Y and reuse the operands, whichever stream the
+    product ran on."""
+    A, k = gen.uniform_rows(1 << 18, 1 << 18, 32, 1), 64
+    d = [to_dev(a) for a in (A.row_ptr, A.col_idx, A.vals)]
+    B, Y = torch.ones(A.n * k, device="cuda:0"), torch.zeros(A.m * k, device="cuda:0")
+    stream, other = torch.cuda.Stream() if side_stream else torch.cuda.default_stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(5):
+        plan = b200sp.b200sp_plan_create(A.m, A.n, A.nnz, d[0], stream)
+        for _ in range(3):
+            b200sp.b200sp_spmm(plan, k, d[1], d[2], B, Y, 1.0, 0.0, "f32", stream)
+        assert not stream.query()                                 # (three products take half a millisecond)
+        b200sp.b200sp_plan_destroy(plan)
+        assert stream.query()
+        with torch.cuda.stream(other):
+            copy = Y.clone()
+        other.synchronize()
+        assert torch.equal(copy, Y)
