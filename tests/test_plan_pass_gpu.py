@@ -40,13 +40,14 @@ def test_statistics_match_numpy(m):
     check(np.full(m, 7, np.int64))       # nothing left over from the passes before
 
 
-@pytest.mark.parametrize("case", ["mixed", "longest_first", "longest_last", "one_row", "all_empty_but_one", "rows_of_a_share", "rows_of_a_tile", "several_rows_a_thread", "most_rows_without_a_search"])
+@pytest.mark.parametrize("case", ["mixed", "longest_first", "longest_last", "several_long", "one_row", "all_empty_but_one", "rows_of_a_share", "rows_of_a_tile", "searched_four_rows_a_thread", "most_rows"])
 def test_split_points_from_the_rows(case):
     """Tiles of SpMV and shares of SpMM cut where the pass says: sums of ones, which are the row lengths.  Rows that hold no split point, one,
-    and more than the sixteen that a lane writes alone; the split points behind the last row; more rows than one turn of the grid."""
+    more than the sixteen that a lane writes alone and more than the 1024 that a warp does; the split points behind the last row.  Split points that
+    are searched: one_row and rows_of_a_tile, which hold many to a row, and more rows (1.3 million) than the rows' form takes (most_rows is its largest)."""
     lens = {"mixed": lengths(3001, 5), "longest_first": np.concatenate([[150_000], np.full(999, 3)]), "longest_last": np.concatenate([np.full(999, 3), [150_000]]),
-            "one_row": np.array([70_000]), "all_empty_but_one": np.concatenate([np.zeros(40_000), [5], np.zeros(9_000)]), "rows_of_a_share": np.full(500, 31),
-            "rows_of_a_tile": np.full(64, 1023), "several_rows_a_thread": np.random.default_rng(1).integers(0, 6, 1_300_000), "most_rows_without_a_search": np.random.default_rng(2).integers(0, 9, 1 << 17)}[case].astype(np.int64)
+            "several_long": np.concatenate([np.full(900, 3), np.full(5, 140_000), np.full(1100, 2)]), "one_row": np.array([70_000]), "all_empty_but_one": np.concatenate([np.zeros(40_000), [5], np.zeros(9_000)]), "rows_of_a_share": np.full(500, 31),
+            "rows_of_a_tile": np.full(64, 1023), "searched_four_rows_a_thread": np.random.default_rng(1).integers(0, 6, 1_300_000), "most_rows": np.random.default_rng(2).integers(0, 9, 1 << 17)}[case].astype(np.int64)
     m, nnz, k = len(lens), int(lens.sum()), 4
     row_ptr = torch.from_numpy(np.concatenate([[0], lens.cumsum()]).astype(np.int32)).to("cuda:0")
     col = torch.randint(0, 1000, (nnz,), dtype=torch.int32, device="cuda:0")
