@@ -414,9 +414,9 @@ __device__ __forceinline__ void wide_fma(const Wide& b, float v, float (&acc)[16
 // takes eight lines instead of four, and a nonzero costs its (col, val) pair, its address and its loop to four lanes instead of eight.  What
 // bounds the kernels with 16 bytes a lane is the issue rate (74-79 % busy) and the instructions that L1 takes (about 4 cycles each and 1.5 per
 // line).  64 registers: four lines in flight per lane, 32 warps per SM.  The products are added in the order of spmm_slice_kernel, so the
-// results are the same bit for bit.  us, 16 bytes a lane with staged pairs / this: 2^17 rows of
-// 16, k = 128 49.0 / 42.8, k = 80 48.5 / 38.8; 2^14 rows of 32, k = 64 9.0 / 7.2; 2^16 rows of 8, k = 256 33.5 / 30.2; 2^19 rows of 32, k = 64 179 /
-// 158, k = 256 679 / 670.
+// results are the same bit for bit.  Bound by the wait for lines of B (2^19 rows of 32, k = 64: issue slots 34 % busy, no pipe above 62 %).  us, 16
+// bytes a lane with staged pairs / this: 2^17 rows of 16, k = 128 49.0 / 42.8, k = 80 48.5 / 38.8; 2^14 rows of 32, k = 64 9.0 / 7.2; 2^16 rows of 8,
+// k = 256 33.5 / 30.2; 2^19 rows of 32, k = 64 171 / 158, k = 256 687 / 670.  Where it is taken: spmm_wide_pieces.
 // (FP32 has half the columns per load and is not bound by issue: k = 64 317 / 302-325, k = 256 249 / 266; it stays with 16 bytes.)
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
