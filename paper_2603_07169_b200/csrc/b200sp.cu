@@ -133,6 +133,10 @@ int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, float beta,
   return info && spmm_by_shares(*info, k, dtype == B200SP_F32 ? 4 : 2, beta);
 }
 
+int b200sp_spmm_by_bundles(const b200sp_plan_info_t* info, int64_t k, float beta, int dtype) {
+  return info && k > 1 && spmm_by_bundles(*info, k, dtype == B200SP_F32 ? 4 : 2, beta);
+}
+
 int b200sp_spmm_wide_pieces(const b200sp_plan_info_t* info, int64_t k, int sms, int64_t l2_bytes) {
   return info && sms > 0 && k >= 64 && k % 16 == 0 && g_opt.spmm_stage_a == 2 && spmm_wide_pieces(*info, k, sms, l2_bytes);
 }

@@ -5,6 +5,7 @@
 #include "spmm_kernels.cuh"
 #include "spmm_bstage_kernels.cuh"
 #include "spmm_merge_kernels.cuh"
+#include "spmm_bundle_kernels.cuh"
 #include "format_kernels.cuh"
 
 namespace {
@@ -496,6 +497,102 @@ int run_spmm_merge(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals,
 #undef B200SP_MERGE_J
 }
 
+// Merge items per warp of spmm_bundle_kernel: one wave of resident warps where that takes no more than `most`, else as few waves as that allows, all of them
+// full; small matrices fewer warps instead of very short regions.
+int bundle_region(int64_t items, int sms, int ctas, int most) {
+  const int64_t resident = (int64_t)ctas * kMergeWarps * sms, waves = (items + resident * most - 1) / (resident * most);
+  int64_t region = (items + resident * waves - 1) / (resident * waves);
+  if (region < most && region < 128) region = std::min((int64_t)std::min(most, 128), std::max((int64_t)24, items / (20 * sms)));
+  return (int)((region + 7) / 8 * 8);
+}
+
+template <typename T, int LANES, int YV, bool BETA>
+int launch_spmm_bundle_as(b200sp_plan* p, const b200sp_plan::Shares& work, int k, int row_bytes, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha,
+                          float beta, cudaStream_t stream, DeviceInfo* dev) {
+  const b200sp_plan_info_t& I = p->info;
+  constexpr int KS = LANES * (16 / (int)sizeof(T)), CTAS = kBundleCtas<T>;
+  const int region = bundle_region(I.m + I.nnz, dev->sms, CTAS, bundle_most(LANES));
+  const long long per_tile = (long long)region * kMergeWarps;
+  const int tiles = (int)((I.m + I.nnz + per_tile - 1) / per_tile);
+  float* scratch = nullptr;                      // what each tile leaves unfinished and what it finishes for an earlier tile
+  const size_t per = (size_t)tiles * KS;
+  int rc = pool_alloc(dev, (void**)&scratch, 2 * per * sizeof(float) + (size_t)tiles * sizeof(int2), stream);
+  if (rc != B200SP_OK) return rc;
+  int2* const tile_row = (int2*)(scratch + 2 * per);
+  tl_pdl_kernel = true;
+  rc = launch_smem(spmm_bundle_kernel<T, LANES, YV, BETA>, dim3((unsigned)tiles), dim3(kMergeWarps * 32), (size_t)kMergeWarps * bundle_bytes(region), stream, B,
+                   (size_t)I.n * row_bytes, dev, (int)I.m, (int)I.nnz, k, row_bytes, region, work.split, work.witems, p->row_ptr, col_idx, vals, B, Y, scratch,
+                   scratch + per, tile_row, alpha, beta);
+  if (rc == B200SP_OK && tiles > 1) {
+    tl_pdl_kernel = true;
+    const int lanes = KS >= 128 ? 128 : KS;      // a power of two
+    rc = launch(spmm_merge_fixup_kernel<T>, dim3((unsigned)(((long long)tiles * lanes + 255) / 256)), dim3(256), stream, nullptr, 0, dev, k, tiles, 1, KS, lanes,
+                (const int2*)tile_row, (const float*)scratch, (const float*)(scratch + per), Y, alpha, beta);
+  }
+  const cudaError_t e = cudaFreeAsync(scratch, stream);
+  if (e != cudaSuccess && rc == B200SP_OK) rc = cuda_fail(e, "cudaFreeAsync");
+  return rc;
+}
+
+// Columns of Y per store: all of a lane's where k is a multiple of 16 bytes; else B is copied into padded rows first (one kernel and n rows of memory from the
+// pool) and Y is written by pairs (even k) or one by one.
+template <typename T, int YV>
+int run_spmm_bundle(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta, cudaStream_t stream, DeviceInfo* dev) {
+  constexpr int VEC = 16 / (int)sizeof(T);
+  b200sp_plan::Shares work;
+  CallBlock own_work;
+  int rc = plan_shares(p, &work, &own_work, stream, dev);
+  if (rc != B200SP_OK) return rc;
+  T* padded = nullptr;
+  int row_bytes = k * (int)sizeof(T);
+  if (YV != VEC) {
+    row_bytes = (row_bytes + 127) / 128 * 128;   // whole lines (32-byte steps measured the same to 10 % more and less)
+    rc = pool_alloc(dev, (void**)&padded, (size_t)p->info.n * row_bytes, stream);
+    if (rc != B200SP_OK) return rc;
+    const long long blocks = (p->info.n + 31) / 32;
+    tl_pdl_kernel = true;
+    rc = launch(spmm_pad_rows_kernel<T>, dim3((unsigned)(blocks < dev->sms * 8 ? blocks : dev->sms * 8)), dim3(256), stream, nullptr, 0, dev, (int)p->info.n, k,
+                row_bytes / 4, B, (unsigned*)padded);
+    B = padded;
+  }
+  if (rc == B200SP_OK) {
+    const int pieces = (k + VEC - 1) / VEC;
+#define B200SP_BUNDLE(L)                                                                                                                       \
+    rc = beta == 0.0f ? launch_spmm_bundle_as<T, L, YV, false>(p, work, k, row_bytes, col_idx, vals, B, Y, alpha, beta, stream, dev)               \
+                      : launch_spmm_bundle_as<T, L, YV, true>(p, work, k, row_bytes, col_idx, vals, B, Y, alpha, beta, stream, dev)
+    if (pieces <= 4) B200SP_BUNDLE(4);
+    else if (pieces <= 8) B200SP_BUNDLE(8);
+    else if (pieces <= 16) B200SP_BUNDLE(16);
+    else if constexpr (sizeof(T) == 4 && YV == VEC) B200SP_BUNDLE(32);
+    else rc = B200SP_ERR_UNSUPPORTED;
+#undef B200SP_BUNDLE
+  }
+  if (padded) { const cudaError_t e = cudaFreeAsync(padded, stream); if (e != cudaSuccess && rc == B200SP_OK) rc = cuda_fail(e, "cudaFreeAsync"); }
+  return rc;
+}
+
+// Of the calls that go by shares, those whose rows of B are narrow for spmm_merge_kernel go to spmm_bundle_kernel.  Times: shares / bundles, us.
+// - k a multiple of 16 bytes, up to eight pieces of 16 bytes a row of B, four rows or more side by side, from 250,000 items on (four pieces) or 350,000 (BF16) or
+//   600,000 (FP32): 250,000 log-normal rows of 8, BF16 k = 64 46 / 35, FP32 k = 16 64 / 41; R-MAT 2^20, BF16 k = 64 162 / 106, FP32 k = 32 152 / 122.
+//   Below that the few regions are as long as before and start later (25,000 rows of 5, FP32 k = 32 9.0 / 10.7).
+// - Nine to sixteen pieces, two rows side by side: BF16 from 600,000 items on (80,000 rows of 9, k = 128 31 / 26; 400,000 items 16 / 20).  FP32 gains less
+//   from loads twice as wide than it loses at the ends of rows (R-MAT 2^22, k = 64 759 / 797), except
+// - where beta != 0 and a sixteenth of the rows is empty, which spmm_merge_kernel lists first: up to 32 pieces and from 60,000 items on (R-MAT 2^20,
+//   FP32 k = 64 303 / 240, 2^14 22 / 20; BF16 k = 64 248 / 182).
+// - Other k, with a padded copy of B: where spmm_merge_kernel loads single elements (odd k) or pairs of BF16, and B is read often enough to pay for the copy.
+//   BF16: odd k from 4.4 reads of a row of B on (100,001 rows of 11, k = 127 81 / 61, k = 33 47 / 33), k = 2 modulo 4 from 6 on (150,001 rows of 11,
+//   k = 50 beta = 1 48.2 / 40.4; but 80,000 of 9 and 4.5 reads 0.87x).  FP32: odd k up to 64 columns from 6 on (k = 33 51 / 43).
+bool spmm_by_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, float beta) {
+  const int64_t items = I.m + I.nnz, vec = 16 / elem_bytes, pieces = (k + vec - 1) / vec;
+  if (k % vec == 0) {
+    if (beta != 0.0f && I.bin_rows[0] * 16 >= I.m && items >= 60000) return pieces <= (elem_bytes == 2 ? 16 : 32);
+    return pieces <= 4 ? items >= 250000 : pieces <= 8 ? items >= (elem_bytes == 2 ? 350000 : 600000) : elem_bytes == 2 && pieces <= 16 && items >= 600000;
+  }
+  if (pieces > 16) return false;
+  if (elem_bytes == 2 && k % 2 != 0) return items >= 300000 && (double)I.nnz >= 4.4 * (double)I.n;
+  return k % (elem_bytes == 2 ? 4 : 2) == (elem_bytes == 2 ? 2 : 1) && items >= 450000 && I.nnz >= 6 * I.n;
+}
+
 template <typename T, int VEC>
 int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
              cudaStream_t stream, DeviceInfo* dev) {
@@ -533,6 +630,12 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     }
   }
   if (spmm_by_shares(I, k, (int)sizeof(T), beta)) {
+    if (spmm_by_bundles(I, k, (int)sizeof(T), beta)) {
+      const int rc = k % VEC == 0 ? run_spmm_bundle<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev)
+                     : sizeof(T) == 2 && k % 2 == 0 ? run_spmm_bundle<T, sizeof(T) == 2 ? 2 : 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev)
+                                  : run_spmm_bundle<T, 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
+      if (rc != B200SP_ERR_ALLOC) return rc;     // (nothing that writes Y is launched then)
+    }
     const int rc = run_spmm_merge<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
     if (rc != B200SP_ERR_UNSUPPORTED && rc != B200SP_ERR_ALLOC) return rc;   // without its scratch (nothing is launched then) by rows, which need none
   }

@@ -1,0 +1,81 @@
+"""SpMM with rows of about equal length side by side (spmm_bundle_kernel): every width and store, rows and empty rows at the ends of regions and tiles."""
+import numpy as np
+import pytest
+
+import gen
+import oracle
+import paper_2603_07169_b200 as b200sp
+from gpu_util import assert_within, empty_out, run_spmm, store, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+WIDTHS = {"f32": (4, 16, 20, 32, 36, 64, 100, 128, 17, 33, 63), "bf16": (8, 24, 32, 40, 64, 72, 128, 17, 33, 65, 127, 18, 50, 126)}
+
+
+def lengths(case):
+    rng = np.random.default_rng(6)
+    if case == "mixed":              # empty, short and cooperative rows (more than 32), rows over several warps and tiles, empty ends
+        lens = rng.integers(0, 45, 40_000) * (rng.random(40_000) < 0.8)
+        lens[rng.integers(0, 40_000, 40)] = rng.integers(200, 900, 40)
+        lens[12_345], lens[:300], lens[-7:] = 30_000, 0, 0
+        return lens
+    if case == "ones":               # as many pieces to a region as there can be
+        return np.ones(330_000, np.int64)
+    if case == "one_row":            # no region but the last holds the end of a row
+        return np.array([0, 700_000, 3])
+    return np.concatenate([np.tile([31, 32, 33, 1, 2, 3, 4, 5], 6000), [2500]])      # "edges": both sides of a step of four and of the cooperative rows
+
+
+def by_bundles(A, k, beta, dtype):
+    plan = b200sp.b200sp_plan_create(A.m, A.n, A.nnz, to_dev(A.row_ptr))
+    stats = b200sp.b200sp_plan_info(plan)
+    b200sp.b200sp_plan_destroy(plan)
+    return b200sp.b200sp_spmm_by_bundles(stats, k, beta, dtype)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("case", ["mixed", "ones", "one_row", "edges"])
+def test_bundles_against_oracle(case, dtype):
+    lens = lengths(case)
+    n = 30_000
+    A = gen.random_csr(len(lens), n, lens, seed=5, sort_cols=False)
+    rng = np.random.default_rng(7)
+    taken = 0
+    b200sp.b200sp_set_option("spmm_flat", 1)
+    try:
+        for k in WIDTHS[dtype] if case in ("mixed", "edges") else WIDTHS[dtype][::3]:
+            taken += by_bundles(A, k, 0.0, dtype) + by_bundles(A, k, 1.25, dtype)
+            B = rng.standard_normal(n * k).astype(np.float32)
+            Y0 = rng.standard_normal(A.m * k).astype(np.float32)
+            Y, Y_ref, S = run_spmm(A, B, k, None, 1.0, 0.0, dtype)
+            assert_within(Y, Y_ref, S, dtype, what="k=%d" % k)
+            Y, Y_ref, S = run_spmm(A, B, k, Y0, -0.5, 1.25, dtype)
+            y0f = Y0 if dtype == "f32" else gen.bf16_to_f32(gen.to_bf16(Y0))
+            assert_within(Y, Y_ref, S, dtype, 1.0, np.abs(1.25 * y0f.astype(np.float64)).reshape(A.m, k), what="k=%d ab" % k)
+    finally:
+        b200sp.b200sp_set_option("spmm_flat", 2)
+    assert taken >= 6, "the rule sends too few of these calls to the kernel"
+
+
+@pytest.mark.parametrize("dtype,k", [("f32", 32), ("f32", 33), ("bf16", 64), ("bf16", 50)])
+def test_infinities_stay_in_the_rows_that_hold_them(dtype, k):
+    """Loads that stand in for missing nonzeros read the last row of B again: an infinity there must not turn into 0 * inf."""
+    lens = np.tile([1, 2, 3, 5, 6, 7, 9, 40], 14_000)
+    n = 20_000
+    A = gen.random_csr(len(lens), n, lens, seed=9)
+    B = np.random.default_rng(3).standard_normal((n, k)).astype(np.float32)
+    B[::97] = np.inf
+    B[5::97, ::3] = np.nan
+    assert by_bundles(A, k, 0.0, dtype)
+    vals, Bs = store(A.vals, dtype), store(B.reshape(-1), dtype)
+    d = [to_dev(a) for a in (A.row_ptr, A.col_idx, vals, Bs)]
+    Y = empty_out(A.m * k, dtype)
+    b200sp.b200sp_set_option("spmm_flat", 1)
+    try:
+        b200sp.spmm_csr(A.m, n, A.nnz, k, d[0], d[1], d[2], d[3], Y, 1.0, 0.0, dtype)
+    finally:
+        b200sp.b200sp_set_option("spmm_flat", 2)
+    got = to_host(Y, dtype)
+    got = (got if dtype == "f32" else gen.bf16_to_f32(got)).reshape(A.m, k)
+    ref, _ = oracle.spmm_csr(A.m, n, k, A.row_ptr, A.col_idx, vals, Bs, None, 1.0, 0.0, dtype)
+    assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isposinf(got), np.isposinf(ref)) and np.array_equal(np.isneginf(got), np.isneginf(ref))

@@ -69,3 +69,23 @@ def test_rows_of_b_in_pieces_of_32_bytes(m, n, k, shortest, longest, mean, wide)
         assert not b200sp.b200sp_spmm_wide_pieces(stats, k, SMS, L2)
     finally:
         b200sp.b200sp_set_option("spmm_stage_a", 2)
+
+
+LARGE = info(150_001, 120_007, [175, 38_000, 103_000, 8_700, 126, 0], [0, 109_000, 1_250_000, 433_000, 20_000, 0], 400)
+EMPTY = info(1 << 17, 1 << 17, [80_000, 25_000, 18_000, 5_600, 2_200, 272], [0, 50_000, 210_000, 300_000, 290_000, 198_576], 6000)
+
+
+@pytest.mark.parametrize("stats,dtype,beta,taken,left", [
+    (LARGE, "f32", 0.0, (4, 8, 12, 16, 20, 32, 17, 33, 63), (36, 64, 128, 132, 18, 34, 50, 65, 127)),
+    (LARGE, "bf16", 1.0, (8, 32, 40, 64, 72, 128, 17, 33, 127, 18, 50, 126), (136, 256, 20, 36, 100, 129, 130)),
+    (EMPTY, "f32", 1.0, (4, 32, 64, 100, 128), (132, 50)),
+    (EMPTY, "bf16", 0.0, (8, 64, 128, 33, 50), (20, 136, 300)),
+    (LOG_NORMAL_20K, "f32", 0.0, (4, 16), (20, 32, 64, 33)),
+    (LOG_NORMAL_20K, "bf16", 1.0, (), (72, 128, 50)),
+], ids=["f32", "bf16", "empty_f32", "empty_bf16", "small_f32", "small_bf16"])
+def test_rows_side_by_side(stats, dtype, beta, taken, left):
+    """Narrow rows of B, by pieces of 16 bytes and by how often a padded copy would be read; larger matrices only."""
+    for k in taken:
+        assert b200sp.b200sp_spmm_by_bundles(stats, k, beta, dtype), k
+    for k in left:
+        assert not b200sp.b200sp_spmm_by_bundles(stats, k, beta, dtype), k
