@@ -169,11 +169,12 @@ static int64_t csc_most_bucket_rows(int64_t nnz, float beta) {
 
 // The places of the products of csc_kernels.cuh; leaves e->prod_block null where they do not apply, and while the stream is captured
 // (their limits are read back).  Synchronises the stream.
-// Sizes: below 4.8 M nonzeros tiles and buckets of 2048 or 4096, so that every SM gets several; else one tile of 24576 .. 32768 entries
-// per SM and round (96 .. 128 KB of products), the size that leaves the least of the last round idle, and buckets of 8192 nonzeros,
-// 16384 above 2^25.  A run (a tile's products for one bucket) then averages tile * C / nnz = 3.5 .. 55 words: 2^24 nonzeros take 78 us,
-// 81 us with tiles of 32768, 84 us with two tiles of 16384 per SM.  Above 2^26
-// nonzeros, with a row of more than kCscSlack nonzeros, a tile over more than 65536 columns or a bucket of too many rows (most_rows), SpMV takes
+// Sizes: below 7.3 M nonzeros tiles of 2048, 4096 or 8192 entries, so that every SM gets several that overlap, and buckets of as many nonzeros (8192 from 3.8 M
+// on: 4.3 M 24.0 / 21.5 us, 4.7 M 25.3 / 22.3 us); else one tile of 24576 .. 32768 entries per SM and round (96 .. 128 KB of products), the size that leaves
+// the least of the last round idle (4.9 M nonzeros in two rounds of 24576 31.3 us, in tiles of 8192 26.5 us; 6.9 M 40.9 / 35.6 us; but 8 M in two
+// rounds of 28672 38.9 us, in tiles of 8192 43.7 us), and buckets of 8192 nonzeros, 16384 above 2^25.  A run (a tile's products for one bucket) then averages
+// tile * C / nnz = 3.5 .. 55 words: 2^24 nonzeros take 78 us, 81 us with tiles of 32768, 84 us with two tiles of 16384 per SM, 90 us with buckets of 16384.
+// Above 2^26 nonzeros, with a row of more than kCscSlack nonzeros, a tile over more than 65536 columns or a bucket of too many rows (most_rows), SpMV takes
 // the CSR kernels.
 static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr, const int32_t* row_idx, int64_t most_rows,
                             cudaStream_t stream, DeviceInfo* dev) {
@@ -181,15 +182,15 @@ static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, cons
   if (e->prod_tried || e->bucket_rows > most_rows || stream_captures(stream)) return B200SP_OK;
   if (nnz <= 0 || nnz > ((int64_t)1 << 26)) { e->prod_tried = true; return B200SP_OK; }
   const int64_t sms = dev->sms;
-  int tile = nnz < sms * 4 * 2048 ? 2048 : 4096;
-  if (nnz >= sms * 8 * 4096) {
+  int tile = nnz < sms * 4 * 2048 ? 2048 : nnz < sms * 8 * 4096 ? 4096 : 8192;
+  if (nnz >= sms * 6 * 8192) {
     int64_t best = INT64_MAX;
     for (int t : {32768, 28672, 24576}) {
       const int64_t time = (((nnz + t - 1) / t + sms - 1) / sms) * t;     // rounds of one tile per SM
       if (time < best) { best = time; tile = t; }
     }
   }
-  const int shift = nnz < sms * 4 * 2048 ? 11 : nnz < sms * 8 * 4096 ? 12 : nnz <= ((int64_t)1 << 25) ? 13 : 14;
+  const int shift = nnz < sms * 4 * 2048 ? 11 : nnz < sms * 25 * 1024 ? 12 : nnz <= ((int64_t)1 << 25) ? 13 : 14;
   const int tiles = (int)((nnz + tile - 1) / tile), buckets = (int)(((nnz - 1) >> shift) + 1), cap = (1 << shift) + kCscSlack;
   if (buckets > kCscMaxBuckets) { e->prod_tried = true; return B200SP_OK; }
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
@@ -271,6 +272,7 @@ static int run_csc_products(const CscEntry* e, int64_t nnz, const T* vals, const
   switch (e->tile) {
     case 2048: rc = launch_csc_products<T, 2048, 512>(e, nnz, vals, x, stream, dev); break;
     case 4096: rc = launch_csc_products<T, 4096, 512>(e, nnz, vals, x, stream, dev); break;
+    case 8192: rc = launch_csc_products<T, 8192, 512>(e, nnz, vals, x, stream, dev); break;
     case 24576: rc = launch_csc_products<T, 24576, 1024>(e, nnz, vals, x, stream, dev); break;
     case 28672: rc = launch_csc_products<T, 28672, 1024>(e, nnz, vals, x, stream, dev); break;
     default: rc = launch_csc_products<T, 32768, 1024>(e, nnz, vals, x, stream, dev); break;

@@ -185,3 +185,17 @@ def test_the_other_operation_captured(first, dtype):
         torch.cuda.synchronize()
         assert torch.equal(outs[op][1], outs[op][2])
     b200sp.b200sp_cache_clear()
+
+
+@pytest.mark.parametrize("n", [245_001, 455_000, 640_000], ids=["tile_4096_bucket_8192", "tile_8192_ragged", "tile_24576"])
+def test_csc_products_of_the_sizes_between(n):
+    """Tiles of 4096 with buckets of 8192, the last size in tiles of 8192 (7.28 M nonzeros) and one in tiles of 24576."""
+    A = gen.uniform_rows(n, n, 16, 5)
+    x = np.random.default_rng(2).standard_normal(n).astype(np.float32)
+    cp, ri, va = gen.csr_to_csc(A)
+    d = [to_dev(a) for a in (cp, ri, va, x)]
+    y = empty_out(n, "f32")
+    b200sp.spmv_csc(n, n, A.nnz, d[0], d[1], d[2], d[3], y, 1.0, 0.0, "f32")
+    y_ref, S = oracle.spmm_csc(n, n, 1, cp, ri, va, x, None, 1.0, 0.0, "f32")
+    assert_within(to_host(y, "f32"), y_ref[:, 0], S[:, 0], "f32")
+    b200sp.b200sp_cache_clear()
