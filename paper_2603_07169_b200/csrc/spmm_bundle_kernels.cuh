@@ -65,7 +65,8 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
   unsigned char* const empty_rows = (unsigned char*)(list + region / 2 + 8);
 
   const long long total = (long long)m + nnz;
-  // row ends before item x: split[] has them for every `per` items, the rest is counted
+  // Row ends before item x: split[] has them for every `per` items, the rest is counted.  Within the bounds that the split points keep, and ends within the
+  // region below: whatever ascending row_ptr holds, a region's nonzeros lie in [0, nnz).
   auto row_ends = [&](long long x) {
     const int at = (int)((unsigned)x / (unsigned)per);
     const int r0 = __ldg(split + at);
@@ -74,13 +75,14 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
     int n = 0;
     for (int j = r0 + lane; __any_sync(0xFFFFFFFFu, j < r1); j += 32)
       n += __popc(__ballot_sync(0xFFFFFFFFu, j < r1 && (unsigned)__ldg(row_ptr + j + 1) + (unsigned)j < (unsigned)x));
-    return r0 + n;
+    return min(max(r0 + n, (int)max(x - nnz, 0LL)), (int)min(x, (long long)m));
   };
   const long long x0 = min(((long long)t * kMergeWarps + warp) * region, total), x1 = min(x0 + region, total);
   const int r_lo = uniform(row_ends(x0)), r_hi = uniform(row_ends(x1));
   const int p0 = (int)(x0 - r_lo), p1 = (int)(x1 - r_hi);
   const int cnt = p1 - p0, rows = r_hi - r_lo;
-  int e_next = lane < rows ? __ldg(row_ptr + r_lo + 1 + lane) - p0 : cnt;     // ends of 32 rows
+  auto row_end = [&](int i) { return i < rows ? min(max(__ldg(row_ptr + r_lo + 1 + i) - p0, 0), cnt) : cnt; };
+  int e_next = row_end(lane);                                // ends of 32 rows
   if constexpr (sizeof(T) == 4) {
     for (int i = lane; i < cnt; i += 32) {
       cp_async4(&pair[i].x, col_idx + p0 + i);
@@ -108,7 +110,7 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
   int listed = 0, before0 = 0;
   for (int i0 = 0; i0 <= rows; i0 += 32) {
     const int i = i0 + lane, e = e_next;
-    e_next = i + 32 < rows ? __ldg(row_ptr + r_lo + 33 + i) - p0 : cnt;
+    e_next = row_end(i + 32);
     int before = __shfl_up_sync(0xFFFFFFFFu, e, 1);
     if (lane == 0) before = before0;
     before0 = __shfl_sync(0xFFFFFFFFu, e, 31);
