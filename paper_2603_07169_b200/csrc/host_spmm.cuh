@@ -577,15 +577,15 @@ int run_spmm_bundle(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals
 //   Below that the few regions are as long as before and start later (25,000 rows of 5, FP32 k = 32 9.0 / 10.7).
 // - Nine to sixteen pieces, two rows side by side: BF16 from 600,000 items on (80,000 rows of 9, k = 128 31 / 26; 400,000 items 16 / 20).  FP32 gains less
 //   from loads twice as wide than it loses at the ends of rows (R-MAT 2^22, k = 64 759 / 797), except
-// - where beta != 0 and a sixteenth of the rows is empty, which spmm_merge_kernel lists first: up to 32 pieces and from 60,000 items on (R-MAT 2^20,
-//   FP32 k = 64 303 / 240, 2^14 22 / 20; BF16 k = 64 248 / 182).
+// - where beta != 0 and a sixteenth of the rows is empty, which spmm_merge_kernel lists first: from 60,000 items on (R-MAT 2^20,
+//   FP32 k = 64 303 / 240, 2^14 13.9 / 12.3; BF16 k = 64 248 / 182), and up to 32 pieces of FP32 from 250,000 on (R-MAT 2^15, k = 128 50 / 36; 2^14 17.4 / 19.7).
 // - Other k, with a padded copy of B: where spmm_merge_kernel loads single elements (odd k) or pairs of BF16, and B is read often enough to pay for the copy.
 //   BF16: odd k from 4.4 reads of a row of B on (100,001 rows of 11, k = 127 81 / 61, k = 33 47 / 33), k = 2 modulo 4 from 6 on (150,001 rows of 11,
 //   k = 50 beta = 1 48.2 / 40.4; but 80,000 of 9 and 4.5 reads 0.87x).  FP32: odd k up to 64 columns from 6 on (k = 33 51 / 43).
 bool spmm_by_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, float beta) {
   const int64_t items = I.m + I.nnz, vec = 16 / elem_bytes, pieces = (k + vec - 1) / vec;
   if (k % vec == 0) {
-    if (beta != 0.0f && I.bin_rows[0] * 16 >= I.m && items >= 60000) return pieces <= (elem_bytes == 2 ? 16 : 32);
+    if (beta != 0.0f && I.bin_rows[0] * 16 >= I.m) return pieces <= 16 ? items >= 60000 : elem_bytes == 4 && pieces <= 32 && items >= 250000;
     return pieces <= 4 ? items >= 250000 : pieces <= 8 ? items >= (elem_bytes == 2 ? 350000 : 600000) : elem_bytes == 2 && pieces <= 16 && items >= 600000;
   }
   if (pieces > 16) return false;
