@@ -100,9 +100,9 @@ int b200sp_get_option(const char* name, int* value);
  * under the present switches, 0 if not; B kept in shared memory (few columns of A) comes before it.  A rule of the host: no device needed. */
 int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, float beta, int dtype);
 
-/* 1 if an SpMM call that goes by shares has its warps walk several rows of about equal length side by side, 16 bytes of B per lane (k a multiple of
- * 16 bytes and narrow, or odd widths through a padded copy of B, which takes up to 128 n more bytes than B for the call), 0 if one nonzero after another.  A
- * rule of the host: no device needed. */
+/* 1 if SpMM has its warps walk several rows of about equal length side by side, 16 bytes of B per lane: of the calls that go by shares those with
+ * narrow rows of B (k a multiple of 16 bytes, or odd widths through a padded copy of B, which takes up to 128 n more bytes than B for the call), and rows all of
+ * one short length that is no multiple of four.  Larger matrices only.  A rule of the host: no device needed. */
 int b200sp_spmm_by_bundles(const b200sp_plan_info_t* info, int64_t k, float beta, int dtype);
 
 /* 1 if BF16 SpMM by rows with k columns and a B aligned to 32 bytes takes the kernel with 32 bytes of B per load and four lanes a row, on a device

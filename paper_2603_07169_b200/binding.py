@@ -486,7 +486,7 @@ def b200sp_spmm_by_shares(info: dict, k, beta, dtype) -> bool:
 
 
 def b200sp_spmm_by_bundles(info: dict, k, beta, dtype) -> bool:
-    """Whether an SpMM call that goes by shares walks rows of about equal length side by side (spmm_bundle_kernel)."""
+    """Whether SpMM on a matrix with these row statistics walks rows of about equal length side by side (spmm_bundle_kernel)."""
     return bool(lib().b200sp_spmm_by_bundles(ctypes.byref(_plan_info(info)), k, beta, _dt(dtype)))
 
 

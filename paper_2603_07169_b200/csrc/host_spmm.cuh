@@ -593,6 +593,18 @@ bool spmm_by_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, flo
   return k % (elem_bytes == 2 ? 4 : 2) == (elem_bytes == 2 ? 2 : 1) && items >= 450000 && I.nnz >= 6 * I.n;
 }
 
+// Rows all of one length of 5 to 13 that is no multiple of four, k a multiple of 16 bytes and five to sixteen pieces of them a row of B: by rows they take single
+// steps at both ends of nearly every row, side by side only at one.  From 1 M items on with up to eight pieces (BF16; 2 M for FP32, 5 M
+// there for rows of 11 and 13 and in both for rows of 10: 240,000 of them, beta = 1, BF16 k = 64 45.2 / 49.5), from 780,000 on with more.  By rows / side by side, us: 131,072 rows of 7, k = 64 BF16 23.5 / 18.2, k = 128 41.9 / 28.6, FP32 k = 64
+// 37.6 / 29.3; of 13, BF16 k = 128 52.2 / 48.1, FP32 k = 64 47.8 / 48.0; 8 M nonzeros in rows of 6, k = 64 FP32 466 / 373, BF16 243 / 194, in rows of 13 292 / 262
+// and 158 / 136.  Not rows of 21 (FP32 k = 64 192 / 201), fewer (70,000 rows of 6, BF16 k = 64 9.4 / 13.4) or wider (k = 128 FP32, rows of 13 241 / 254).
+bool spmm_even_by_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_bytes) {
+  const int64_t items = I.m + I.nnz, vec = 16 / elem_bytes, pieces = k / vec;
+  if (I.min_row_len != I.max_row_len || I.max_row_len % 4 == 0 || I.max_row_len < 5 || I.max_row_len > 13) return false;
+  const bool gains_less = I.max_row_len > 9 && (elem_bytes == 4 || I.max_row_len % 2 == 0);
+  return k % vec == 0 && pieces >= 5 && pieces <= 16 && items >= (pieces > 8 ? 780000 : gains_less ? 5000000 : elem_bytes == 2 ? 1000000 : 2000000);
+}
+
 template <typename T, int VEC>
 int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
              cudaStream_t stream, DeviceInfo* dev) {
@@ -638,6 +650,10 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
     }
     const int rc = run_spmm_merge<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
     if (rc != B200SP_ERR_UNSUPPORTED && rc != B200SP_ERR_ALLOC) return rc;   // without its scratch (nothing is launched then) by rows, which need none
+  }
+  if (g_opt.spmm_sliced && g_opt.spmm_flat == 2 && g_opt.spmm_stage_a == 2 && g_opt.spmm_ranges == 1 && spmm_even_by_bundles(I, k, (int)sizeof(T))) {
+    const int rc = run_spmm_bundle<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
+    if (rc != B200SP_ERR_ALLOC) return rc;
   }
   if (k % VEC == 0 && g_opt.spmm_sliced) {
     // lanes per row: eight (a 128-byte slice) unless k is narrower than that

@@ -66,12 +66,12 @@ def test_infinities_stay_in_the_rows_that_hold_them(dtype, k):
     B = np.random.default_rng(3).standard_normal((n, k)).astype(np.float32)
     B[::97] = np.inf
     B[5::97, ::3] = np.nan
-    assert by_bundles(A, k, 0.0, dtype)
     vals, Bs = store(A.vals, dtype), store(B.reshape(-1), dtype)
     d = [to_dev(a) for a in (A.row_ptr, A.col_idx, vals, Bs)]
     Y = empty_out(A.m * k, dtype)
     b200sp.b200sp_set_option("spmm_flat", 1)
     try:
+        assert by_bundles(A, k, 0.0, dtype)
         b200sp.spmm_csr(A.m, n, A.nnz, k, d[0], d[1], d[2], d[3], Y, 1.0, 0.0, dtype)
     finally:
         b200sp.b200sp_set_option("spmm_flat", 2)
@@ -79,3 +79,17 @@ def test_infinities_stay_in_the_rows_that_hold_them(dtype, k):
     got = (got if dtype == "f32" else gen.bf16_to_f32(got)).reshape(A.m, k)
     ref, _ = oracle.spmm_csr(A.m, n, k, A.row_ptr, A.col_idx, vals, Bs, None, 1.0, 0.0, dtype)
     assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isposinf(got), np.isposinf(ref)) and np.array_equal(np.isneginf(got), np.isneginf(ref))
+
+
+@pytest.mark.parametrize("dtype,k,length,rows", [("f32", 64, 7, 97_501), ("f32", 36, 5, 130_003), ("f32", 32, 9, 200_001), ("bf16", 72, 6, 111_500), ("bf16", 40, 11, 83_400)])
+def test_equal_rows_of_odd_length(dtype, k, length, rows):
+    """Just above the least number of items, in regions that cut rows at every place."""
+    A = gen.uniform_rows(rows, 40_000, length, 2)
+    assert by_bundles(A, k, 0.5, dtype)
+    rng = np.random.default_rng(5)
+    B, Y0 = rng.standard_normal(A.n * k).astype(np.float32), rng.standard_normal(A.m * k).astype(np.float32)
+    Y, Y_ref, S = run_spmm(A, B, k, None, 1.0, 0.0, dtype)
+    assert_within(Y, Y_ref, S, dtype)
+    Y, Y_ref, S = run_spmm(A, B, k, Y0, 1.5, 0.5, dtype)
+    y0f = Y0 if dtype == "f32" else gen.bf16_to_f32(gen.to_bf16(Y0))
+    assert_within(Y, Y_ref, S, dtype, 1.5, np.abs(0.5 * y0f.astype(np.float64)).reshape(A.m, k))

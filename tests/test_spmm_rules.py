@@ -89,3 +89,14 @@ def test_rows_side_by_side(stats, dtype, beta, taken, left):
         assert b200sp.b200sp_spmm_by_bundles(stats, k, beta, dtype), k
     for k in left:
         assert not b200sp.b200sp_spmm_by_bundles(stats, k, beta, dtype), k
+
+
+@pytest.mark.parametrize("dtype,k,length,rows,taken", [
+    ("f32", 64, 7, 97_500, True), ("f32", 64, 7, 97_499, False), ("f32", 64, 8, 1 << 20, False), ("f32", 64, 21, 1 << 20, False), ("f32", 68, 7, 1 << 20, False),
+    ("f32", 32, 13, 357_143, True), ("f32", 32, 13, 357_142, False), ("f32", 32, 9, 200_000, True), ("bf16", 64, 10, 454_545, False), ("f32", 16, 13, 1 << 20, False), ("bf16", 64, 6, 142_858, True), ("bf16", 64, 6, 142_857, False),
+    ("bf16", 128, 5, 130_000, True), ("bf16", 128, 4, 1 << 20, False), ("bf16", 136, 5, 1 << 20, False)])
+def test_equal_rows_side_by_side(dtype, k, length, rows, taken):
+    """Rows of one length of 5 to 13 that is no multiple of four, on both sides of each limit."""
+    stats = dict(info(rows, rows, [0, 0, rows, 0, 0, 0], [0, 0, rows * length, 0, 0, 0], length), min_row_len=length)
+    assert not b200sp.b200sp_spmm_by_shares(stats, k, 0.0, dtype)
+    assert b200sp.b200sp_spmm_by_bundles(stats, k, 0.0, dtype) == taken
