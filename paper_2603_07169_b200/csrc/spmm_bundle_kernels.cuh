@@ -57,8 +57,9 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
   extern __shared__ __align__(16) unsigned char bundle_smem[];
   __shared__ float head_s[kMergeWarps][KS], carry_s[kMergeWarps][KS];
   __shared__ int first_s[2];                                 // the tile's first row and where it starts, -1 when inside the tile
-  // Where B is a padded copy the kernel before this one made it, after everything before that had completed: only reads of B have to wait for it.
-  if (YV == VEC) grid_dependency_wait();
+  // Before anything is read, also where B is a padded copy and only B comes from the kernel before this one: that kernel has waited for the stream's earlier
+  // work, but what it then sees is promised to it alone, not to the kernel that it lets start.
+  grid_dependency_wait();
   const int t = blockIdx.x;
   const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31, g = lane / LANES, l = lane % LANES;
   unsigned char* const mine = bundle_smem + warp * bundle_bytes(region);
@@ -143,7 +144,6 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
       __syncwarp();
     }
   }
-  if (YV != VEC) grid_dependency_wait();                     // (the padded copy of B)
   if constexpr (sizeof(T) == 4) cp_async_wait<0>();
   __syncwarp();
   for (int j0 = 0; j0 < listed; j0 += 32) {
@@ -251,7 +251,7 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
 
 // Rows of B (k elements each) copied into rows of `pitch` 4-byte words (a multiple of 16 bytes), zeros behind column k, so that lanes can read 16 bytes of
 // any row.  A warp takes a row at a time, a word per lane, four rows in flight; pairs of 16-bit elements that no word of B holds (odd k) by two loads.
-// Latency-bound (120,007 rows of 50 BF16 6.9 us, half hidden behind the walk's set-up; 4, 8 or 16 consecutive pieces in flight 0.1 to 30 us slower or 0.5 faster).
+// Latency-bound (120,007 rows of 50 BF16 6.9 us; 4, 8 or 16 consecutive pieces in flight 0.1 to 30 us slower or 0.5 faster).
 template <typename T>
 __global__ void __launch_bounds__(256) spmm_pad_rows_kernel(int n, int k, int pitch, const T* __restrict__ B, unsigned* __restrict__ P) {
   grid_dependency_wait();

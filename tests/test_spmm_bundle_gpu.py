@@ -1,11 +1,12 @@
 """SpMM with rows of about equal length side by side (spmm_bundle_kernel): every width and store, rows and empty rows at the ends of regions and tiles."""
 import numpy as np
 import pytest
+import torch
 
 import gen
 import oracle
 import paper_2603_07169_b200 as b200sp
-from gpu_util import assert_within, empty_out, run_spmm, store, to_dev, to_host
+from gpu_util import assert_within, empty_out, needs_plain_build, run_spmm, store, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -93,3 +94,52 @@ def test_equal_rows_of_odd_length(dtype, k, length, rows):
     Y, Y_ref, S = run_spmm(A, B, k, Y0, 1.5, 0.5, dtype)
     y0f = Y0 if dtype == "f32" else gen.bf16_to_f32(gen.to_bf16(Y0))
     assert_within(Y, Y_ref, S, dtype, 1.5, np.abs(0.5 * y0f.astype(np.float64)).reshape(A.m, k))
+
+
+@needs_plain_build
+@pytest.mark.parametrize("pdl", [0, 1])
+@pytest.mark.parametrize("dtype,k", [("bf16", 50), ("bf16", 33), ("f32", 33)])
+def test_padded_calls_read_what_the_calls_just_before_them_wrote(dtype, k, pdl):
+    """The copy of B, the walk and the fix-up wait for the stream's earlier work before anything is read or written: the values of A, B and the old values
+    of Y all come from the calls just before, and a quarter of the rows are empty (Y of these is written first of all)."""
+    rng = np.random.default_rng(8)
+    m = 70_000
+    lens = rng.integers(4, 19, m) * (rng.random(m) < 0.75)
+    lens[5], lens[-1] = 3000, 0
+    A = gen.random_csr(m, m, lens, seed=4)
+    assert by_bundles(A, k, 0.5, dtype)
+    one_each = gen.uniform_rows(A.nnz, A.nnz, 1, 3)               # a product that writes the values of A
+    as_stored = torch.float32 if dtype == "f32" else torch.int16
+    d = [to_dev(a) for a in (A.row_ptr, A.col_idx, one_each.row_ptr, one_each.col_idx, store(np.full(A.nnz, 0.25, np.float32), dtype))]
+    x = [to_dev(store(rng.standard_normal(A.nnz).astype(np.float32), dtype)) for _ in range(2)]
+    start = [to_dev(store(rng.standard_normal(m * k).astype(np.float32), dtype)) for _ in range(2)]
+    plan = b200sp.b200sp_plan_create(A.m, A.n, A.nnz, d[0])
+    plan_of_values = b200sp.b200sp_plan_create(A.nnz, A.nnz, A.nnz, d[2])
+
+    def chain(wait):
+        vals = torch.zeros(A.nnz, dtype=as_stored, device="cuda")
+        P, Q = (t.clone() for t in start)
+        torch.cuda.synchronize()
+        for i in range(60):
+            b200sp.b200sp_spmv(plan_of_values, d[3], d[4], x[i % 2], vals, 1.0, 0.0, dtype)
+            wait()
+            b200sp.b200sp_spmm(plan, k, d[1], vals, P, Q, 0.5, -0.5, dtype)
+            wait()
+            b200sp.b200sp_spmm(plan, k, d[1], vals, Q, P, 0.5, 0.25 if i % 3 else 0.0, dtype)
+            wait()
+        torch.cuda.synchronize()
+        return P, Q
+
+    b200sp.b200sp_set_option("pdl", 0)
+    try:
+        expected = chain(torch.cuda.synchronize)
+        b200sp.b200sp_set_option("pdl", pdl)
+        for _ in range(3):
+            got = chain(lambda: None)
+            assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(got, expected))
+    finally:
+        b200sp.b200sp_set_option("pdl", 1)
+        b200sp.b200sp_plan_destroy(plan)
+        b200sp.b200sp_plan_destroy(plan_of_values)
+    values = expected[0] if dtype == "f32" else expected[0].view(torch.bfloat16)
+    assert bool(torch.isfinite(values).all()) and float(values.float().abs().max()) > 0.0
