@@ -97,16 +97,19 @@ int b200sp_get_option(const char* name, int* value);
  * b200sp_set_option would (an entry that is not accepted is reported on stderr and skipped); B200SP_LOG=1 sets "log". */
 
 /* 1 if SpMM with k columns on a matrix with these row statistics (b200sp_plan_info) goes by equal shares of rows + nonzeros per warp
- * under the present switches, 0 if not; B kept in shared memory (few columns of A) comes before it.  A rule of the host: no device needed. */
+ * under the present switches, 0 if not; B kept in shared memory (few columns of A) comes before it, and calls with narrow rows of B go side by side instead
+ * (b200sp_spmm_by_bundles).  A rule of the host: no device needed. */
 int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, float beta, int dtype);
 
 /* 1 if SpMM has its warps walk several rows of about equal length side by side, 16 bytes of B per lane: of the calls that go by shares those with
  * narrow rows of B (k a multiple of 16 bytes, or odd widths through a padded copy of B, which takes up to 128 n more bytes than B for the call), and rows all of
- * one short length that is no multiple of four.  Larger matrices only.  A rule of the host: no device needed. */
+ * one short length that is no multiple of four (these only while "spmm_sliced", "spmm_flat", "spmm_stage_a" and "spmm_ranges" have their default values).  Larger
+ * matrices only; B kept in shared memory comes before it.  0 if not, under the present switches.  A rule of the host: no device needed. */
 int b200sp_spmm_by_bundles(const b200sp_plan_info_t* info, int64_t k, float beta, int dtype);
 
 /* 1 if BF16 SpMM by rows with k columns and a B aligned to 32 bytes takes the kernel with 32 bytes of B per load and four lanes a row, on a device
- * with that many SMs and bytes of L2, under the present switches, 0 if not ("spmm_stage_a").  A rule of the host: no device needed. */
+ * with that many SMs and bytes of L2, under the present switches, 0 if not ("spmm_stage_a").  Says nothing of calls that do not go by rows: B kept in shared
+ * memory, b200sp_spmm_by_shares and b200sp_spmm_by_bundles come before it.  A rule of the host: no device needed. */
 int b200sp_spmm_wide_pieces(const b200sp_plan_info_t* info, int64_t k, int sms, int64_t l2_bytes);
 
 /* The plan pass's split points as it takes them from the rows: out[t] = row ends before merge item t * items of the merge of the m row ends with the

@@ -134,8 +134,7 @@ int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, float beta,
 }
 
 int b200sp_spmm_by_bundles(const b200sp_plan_info_t* info, int64_t k, float beta, int dtype) {
-  const int elem_bytes = dtype == B200SP_F32 ? 4 : 2;
-  return info && k > 1 && (spmm_by_shares(*info, k, elem_bytes, beta) ? spmm_by_bundles(*info, k, elem_bytes, beta) : spmm_even_by_bundles(*info, k, elem_bytes));
+  return info && k > 1 && spmm_side_by_side(*info, k, dtype == B200SP_F32 ? 4 : 2, beta);
 }
 
 int b200sp_spmm_wide_pieces(const b200sp_plan_info_t* info, int64_t k, int sms, int64_t l2_bytes) {

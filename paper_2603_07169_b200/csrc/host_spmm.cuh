@@ -598,11 +598,18 @@ bool spmm_by_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, flo
 // there for rows of 11 and 13 and in both for rows of 10: 240,000 of them, beta = 1, BF16 k = 64 45.2 / 49.5), from 780,000 on with more.  By rows / side by side, us: 131,072 rows of 7, k = 64 BF16 23.5 / 18.2, k = 128 41.9 / 28.6, FP32 k = 64
 // 37.6 / 29.3; of 13, BF16 k = 128 52.2 / 48.1, FP32 k = 64 47.8 / 48.0; 8 M nonzeros in rows of 6, k = 64 FP32 466 / 373, BF16 243 / 194, in rows of 13 292 / 262
 // and 158 / 136.  Not rows of 21 (FP32 k = 64 192 / 201), fewer (70,000 rows of 6, BF16 k = 64 9.4 / 13.4) or wider (k = 128 FP32, rows of 13 241 / 254).
+// Where a switch asks for one of the kernels by rows they stay by rows.
 bool spmm_even_by_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_bytes) {
   const int64_t items = I.m + I.nnz, vec = 16 / elem_bytes, pieces = k / vec;
+  if (!g_opt.spmm_sliced || g_opt.spmm_flat != 2 || g_opt.spmm_stage_a != 2 || g_opt.spmm_ranges != 1) return false;
   if (I.min_row_len != I.max_row_len || I.max_row_len % 4 == 0 || I.max_row_len < 5 || I.max_row_len > 13) return false;
   const bool gains_less = I.max_row_len > 9 && (elem_bytes == 4 || I.max_row_len % 2 == 0);
   return k % vec == 0 && pieces >= 5 && pieces <= 16 && items >= (pieces > 8 ? 780000 : gains_less ? 5000000 : elem_bytes == 2 ? 1000000 : 2000000);
+}
+
+// Whether spmm_bundle_kernel takes a call with k > 1 columns under the present switches.
+bool spmm_side_by_side(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, float beta) {
+  return spmm_by_shares(I, k, elem_bytes, beta) ? spmm_by_bundles(I, k, elem_bytes, beta) : spmm_even_by_bundles(I, k, elem_bytes);
 }
 
 template <typename T, int VEC>
@@ -641,19 +648,15 @@ int run_spmm(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals, const
       if (rc != B200SP_ERR_UNSUPPORTED) return rc;   // unsupported shape for the tensor map: fall through to the sliced kernel
     }
   }
+  if (spmm_side_by_side(I, k, (int)sizeof(T), beta)) {
+    const int rc = k % VEC == 0 ? run_spmm_bundle<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev)
+                   : sizeof(T) == 2 && k % 2 == 0 ? run_spmm_bundle<T, sizeof(T) == 2 ? 2 : 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev)
+                                : run_spmm_bundle<T, 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
+    if (rc != B200SP_ERR_ALLOC) return rc;       // (nothing that writes Y is launched then)
+  }
   if (spmm_by_shares(I, k, (int)sizeof(T), beta)) {
-    if (spmm_by_bundles(I, k, (int)sizeof(T), beta)) {
-      const int rc = k % VEC == 0 ? run_spmm_bundle<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev)
-                     : sizeof(T) == 2 && k % 2 == 0 ? run_spmm_bundle<T, sizeof(T) == 2 ? 2 : 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev)
-                                  : run_spmm_bundle<T, 1>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
-      if (rc != B200SP_ERR_ALLOC) return rc;     // (nothing that writes Y is launched then)
-    }
     const int rc = run_spmm_merge<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
     if (rc != B200SP_ERR_UNSUPPORTED && rc != B200SP_ERR_ALLOC) return rc;   // without its scratch (nothing is launched then) by rows, which need none
-  }
-  if (g_opt.spmm_sliced && g_opt.spmm_flat == 2 && g_opt.spmm_stage_a == 2 && g_opt.spmm_ranges == 1 && spmm_even_by_bundles(I, k, (int)sizeof(T))) {
-    const int rc = run_spmm_bundle<T, VEC>(p, k, col_idx, vals, B, Y, alpha, beta, stream, dev);
-    if (rc != B200SP_ERR_ALLOC) return rc;
   }
   if (k % VEC == 0 && g_opt.spmm_sliced) {
     // lanes per row: eight (a 128-byte slice) unless k is narrower than that

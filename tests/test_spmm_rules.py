@@ -100,3 +100,18 @@ def test_equal_rows_side_by_side(dtype, k, length, rows, taken):
     stats = dict(info(rows, rows, [0, 0, rows, 0, 0, 0], [0, 0, rows * length, 0, 0, 0], length), min_row_len=length)
     assert not b200sp.b200sp_spmm_by_shares(stats, k, 0.0, dtype)
     assert b200sp.b200sp_spmm_by_bundles(stats, k, 0.0, dtype) == taken
+
+
+@pytest.mark.parametrize("switch,values", [("spmm_sliced", [0]), ("spmm_flat", [0]), ("spmm_stage_a", [0, 1]), ("spmm_ranges", [0, 2, 3, 4, 8])])
+@pytest.mark.parametrize("dtype,k,rows", [("bf16", 64, 1 << 20), ("f32", 64, 1 << 20), ("bf16", 128, 130_000)])
+def test_equal_rows_stay_by_rows_where_a_switch_asks_for_it(dtype, k, rows, switch, values):
+    stats = dict(info(rows, rows, [0, 0, rows, 0, 0, 0], [0, 0, rows * 7, 0, 0, 0], 7), min_row_len=7)
+    default = b200sp.b200sp_get_option(switch)
+    assert b200sp.b200sp_spmm_by_bundles(stats, k, 0.0, dtype)
+    try:
+        for value in values:
+            b200sp.b200sp_set_option(switch, value)
+            assert not b200sp.b200sp_spmm_by_bundles(stats, k, 0.0, dtype), value
+    finally:
+        b200sp.b200sp_set_option(switch, default)
+    assert b200sp.b200sp_spmm_by_bundles(stats, k, 0.0, dtype)
