@@ -28,6 +28,7 @@
  *    hundred bytes, through pinned host memory that the library keeps, and synchronises the stream once).
  *  - beta == 0: y / Y is write-only (its old contents, NaN included, are ignored).  alpha == 0 or
  *    nnz == 0: y = beta * y without reading A.  m == 0: nothing is done.  x / B must not alias y / Y.
+ *    A row without nonzeros gets alpha * 0 + beta * y (alpha * 0 with beta == 0) like any other sum: NaN for an alpha that is not finite.
  *  - The compute kernels are launched with programmatic stream serialisation (option "pdl"): a kernel waits for the
  *    stream's earlier work (griddepcontrol.wait) before its first memory access, then lets the next kernel of the
  *    stream be scheduled behind it.  Ordinary launches that follow see ordinary stream order.  A caller that launches

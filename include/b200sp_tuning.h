@@ -43,8 +43,8 @@ extern "C" {
  *   "merge_carve"    shared-memory carveout in percent requested for it: 0, 25, 45 (default), 60, 75, 100 or -1 = leave to the driver
  *   "merge_short"    rows of up to this many products are added by one thread: 8, 16, 32 (default) or 64; tiles of 1024 and 2048 items
  *   "merge_empty"    1 = when a quarter or more of the rows have no nonzeros the merge list holds only the other rows, and y
- *                    of the empty rows is written by a pass of its own, 0 = every row is a merge item (default: the list
- *                    measured 3 % slower on the power-law workload with 61 % empty rows)
+ *                    of the empty rows is written by a pass of its own (beta * y, whatever alpha is), 0 = every row is a merge
+ *                    item (default: the list measured 3 % slower on the power-law workload with 61 % empty rows)
  *  row-direct SpMV kernel
  *   "row_stages"     shared-memory stages per CTA, 2 (default) .. 4
  *   "row_ctas"       CTAs per SM the tiles are sized for, 1..4; until it is set, and after it is set to 0, 3, or up to 5 where

@@ -139,7 +139,7 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
         for (int x = 0; x < VEC; ++x) zero[x] = 0.0f;
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-          if (j + u * G < empties && on) bundle_store<T, VEC, YV, BETA>(yp[u], left, zero, 0.0f, beta, old[u]);
+          if (j + u * G < empties && on) bundle_store<T, VEC, YV, BETA>(yp[u], left, zero, alpha, beta, old[u]);
       }
       __syncwarp();
     }

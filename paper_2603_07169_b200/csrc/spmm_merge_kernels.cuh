@@ -256,7 +256,7 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
     for (int j = 0; j < (AHEAD ? J : 0); ++j) if (on[j]) old[j] = *(const raw*)(yrow + 32 * V * j);
   };
   if (AHEAD && r_first < m) ask_old();
-  // rows empty_s[warp][0 .. count) of the share whose first row is at ys: y = beta * y over the slice's columns
+  // rows empty_s[warp][0 .. count) of the share whose first row is at ys: y = alpha * 0 + beta * y over the slice's columns
   auto scale_rows = [&](T* ys, int count) {
     const int width = min(KS, k - slice * KS);
     const bool wide = V * sizeof(T) < 16 && k * (int)sizeof(T) % 16 == 0;       // 16 bytes a lane where the rows allow it
@@ -273,12 +273,12 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
           float zero[16 / sizeof(T)];
 #pragma unroll
           for (int x = 0; x < 16 / (int)sizeof(T); ++x) zero[x] = 0.0f;
-          piece_store<T, 16 / (int)sizeof(T)>(y, zero, 0.0f, beta);
+          piece_store<T, 16 / (int)sizeof(T)>(y, zero, alpha, beta);
         } else {
           float zero[V];
 #pragma unroll
           for (int x = 0; x < V; ++x) zero[x] = 0.0f;
-          piece_store<T, V>(y, zero, 0.0f, beta);
+          piece_store<T, V>(y, zero, alpha, beta);
         }
       }
     }

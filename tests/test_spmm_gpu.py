@@ -5,7 +5,7 @@ import pytest
 import gen
 import oracle
 import paper_2603_07169_b200 as b200sp
-from gpu_util import assert_within, run_spmm, store
+from gpu_util import assert_within, run_spmm, store, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -420,3 +420,30 @@ def test_b_in_shared_memory_sorted_quads_reproducible_exact_and_nonfinite():
     rows_with_col0 = np.unique(np.repeat(np.arange(A.m), np.diff(A.row_ptr))[A.col_idx == 0])
     assert len(rows_with_col0) > 0 and not np.any(np.isfinite(Y2[rows_with_col0]))
     b200sp.b200sp_check()
+
+
+@pytest.mark.parametrize("alpha", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("beta", [0.0, 0.5])
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("m,empty", [(3000, 0.5), (3000, 0.02), (120_000, 0.5), (120_000, 0.02)])
+def test_empty_rows_under_an_alpha_that_is_not_finite(m, empty, dtype, beta, alpha):
+    """alpha * 0 + beta * y in every row without nonzeros, whichever kernel takes the call: few rows and many, few of them empty and half of them, by rows, by
+    shares and side by side."""
+    rng = np.random.default_rng(11)
+    lens = rng.integers(4, 12, m) * (rng.random(m) >= empty)
+    A = gen.random_csr(m, 30_000, lens, seed=2)
+    none = lens == 0
+    for flat, ks in ((0, (16, 33)), (1, (16, 33, 64, 132))):
+        b200sp.b200sp_set_option("spmm_flat", flat)
+        try:
+            for k in ks:
+                B, Y0 = rng.random(A.n * k).astype(np.float32) + 1.0, rng.standard_normal(m * k).astype(np.float32)
+                d = [to_dev(store(a, dtype)) if a.dtype == np.float32 else to_dev(a) for a in (A.row_ptr, A.col_idx, A.vals, B)]
+                out = to_dev(store(Y0, dtype)).clone()
+                b200sp.spmm_csr(m, A.n, A.nnz, k, d[0], d[1], d[2], d[3], out, float(alpha), beta, dtype)
+                Y = to_host(out, dtype)
+                Y = (Y if dtype == "f32" else gen.bf16_to_f32(Y)).reshape(m, k)
+                assert np.isnan(Y[none]).all(), "flat=%d k=%d" % (flat, k)
+        finally:
+            b200sp.b200sp_set_option("spmm_flat", 2)
+            b200sp.b200sp_cache_clear()
