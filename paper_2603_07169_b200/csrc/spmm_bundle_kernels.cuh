@@ -43,6 +43,34 @@ __device__ __forceinline__ void bundle_store(T* yp, int left, const float (&acc)
     }
 }
 
+// y = alpha * 0 + beta * y over `count` elements by a warp: whole rows, whatever their width, in pieces of 16 bytes but for what lies before the first boundary of
+// 16 bytes and after the last.  (40,000 rows of 20 and 100,000 empty ones, BF16 k = 127, beta = 0: 271 us with the columns of each row written one by one by the
+// lanes that hold its pieces.)
+template <typename T, bool BETA>
+__device__ __forceinline__ void bundle_scale_span(T* y, int count, int lane, float alpha, float beta) {
+  constexpr int VEC = 16 / sizeof(T);
+  typedef typename Piece<T, VEC>::raw raw;
+  const float zero[VEC] = {}, zero_1[1] = {};
+  const int before = min(count, (int)((16u - ((unsigned)(uintptr_t)y & 15u)) & 15u) / (int)sizeof(T));
+  const int pieces = (count - before) / VEC, after = count - before - pieces * VEC;
+  T* const body = y + before;
+  for (int p = lane; p < pieces; p += 4 * 32) {
+    raw old[4][1];
+    if constexpr (BETA) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) if (p + 32 * u < pieces) old[u][0] = *((const raw*)body + p + 32 * u);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) if (p + 32 * u < pieces) bundle_store<T, VEC, VEC, BETA>(body + (p + 32 * u) * VEC, VEC, zero, alpha, beta, old[u]);
+  }
+  T* const at = lane < before ? y + lane : body + pieces * VEC + (lane - before);
+  if (lane < before + after) {
+    typename Piece<T, 1>::raw old_1[1];
+    if constexpr (BETA) old_1[0] = *at;
+    bundle_store<T, 1, 1, BETA>(at, 1, zero_1, alpha, beta, old_1);
+  }
+}
+
 // A tile is kMergeWarps regions, one per warp.  What crosses the ends of a region goes to head_s / carry_s and is put together inside the tile after one
 // barrier; what crosses the ends of the tile goes to tile_carry / tile_tail and is finished by spmm_merge_fixup_kernel, as for spmm_merge_kernel: fixed order, no
 // atomics.  split[i]: row ends before item i * per.
@@ -122,24 +150,30 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
     if (full) list[listed + __popc(fulls & below)] = ((unsigned)(e - before) << 20) | (unsigned)(i << 10) | (unsigned)before;
     listed += __popc(fulls);
     if (none) {
-      if (empty) empty_rows[__popc(none & below)] = (unsigned char)lane;
-      __syncwarp();
-      const int empties = __popc(none);
-      T* const y0 = Yc + (long long)i0 * k;
-      for (int j = g; j < empties; j += 4 * G) {
-        yraw old[4][BETA ? NY : 1];
-        T* yp[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          yp[u] = y0 + (long long)empty_rows[min(j + u * G, empties - 1)] * k;
-          if constexpr (BETA) { if (j + u * G < empties && on) ask_old(yp[u], old[u]); }
+      if constexpr (YV != VEC) {
+        for (unsigned rest = none; rest;) {                    // runs of empty rows
+          const int first = __ffs(rest) - 1, run = __ffs(~(rest >> first)) - 1, count = run < 0 ? 32 : run;
+          rest &= ~((count == 32 ? ~0u : (1u << count) - 1u) << first);
+          bundle_scale_span<T, BETA>(Y + (long long)(r_lo + i0 + first) * k, count * k, lane, alpha, beta);
         }
-        float zero[VEC];
+      } else {
+        if (empty) empty_rows[__popc(none & below)] = (unsigned char)lane;
+        __syncwarp();
+        const int empties = __popc(none);
+        T* const y0 = Yc + (long long)i0 * k;
+        for (int j = g; j < empties; j += 4 * G) {
+          yraw old[4][BETA ? NY : 1];
+          T* yp[4];
 #pragma unroll
-        for (int x = 0; x < VEC; ++x) zero[x] = 0.0f;
+          for (int u = 0; u < 4; ++u) {
+            yp[u] = y0 + (long long)empty_rows[min(j + u * G, empties - 1)] * k;
+            if constexpr (BETA) { if (j + u * G < empties && on) ask_old(yp[u], old[u]); }
+          }
+          const float zero[VEC] = {};
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (j + u * G < empties && on) bundle_store<T, VEC, YV, BETA>(yp[u], left, zero, alpha, beta, old[u]);
+          for (int u = 0; u < 4; ++u)
+            if (j + u * G < empties && on) bundle_store<T, VEC, YV, BETA>(yp[u], left, zero, alpha, beta, old[u]);
+        }
       }
       __syncwarp();
     }

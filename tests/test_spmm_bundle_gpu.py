@@ -143,3 +143,30 @@ def test_padded_calls_read_what_the_calls_just_before_them_wrote(dtype, k, pdl):
         b200sp.b200sp_plan_destroy(plan_of_values)
     values = expected[0] if dtype == "f32" else expected[0].view(torch.bfloat16)
     assert bool(torch.isfinite(values).all()) and float(values.float().abs().max()) > 0.0
+
+
+@needs_plain_build
+@pytest.mark.parametrize("dtype,k", [("bf16", 63), ("bf16", 126), ("bf16", 127), ("f32", 63)])
+def test_empty_rows_of_ragged_width_cost_little_more_than_their_bytes(dtype, k):
+    """The same nonzeros with and without 100,000 empty rows behind them, whole regions of nothing else.  One column at a time by the lanes that hold a
+    piece of B, these took longer than the products."""
+    lens = np.random.default_rng(3).integers(2, 40, 40_000)
+    n = len(lens)
+    best = {}
+    for empties in (0, 100_000):
+        A = gen.random_csr(n + empties, n, np.concatenate([lens, np.zeros(empties, np.int64)]), seed=6, sort_cols=False)
+        assert by_bundles(A, k, 0.0, dtype)
+        d = [to_dev(a) for a in (A.row_ptr, A.col_idx, store(A.vals, dtype), store(np.ones(n * k, np.float32), dtype))]
+        Y = empty_out(A.m * k, dtype)
+        plan = b200sp.b200sp_plan_create(A.m, A.n, A.nnz, d[0])
+        best[empties] = 1e9
+        for _ in range(8):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            for _ in range(8):
+                b200sp.b200sp_spmm(plan, k, d[1], d[2], d[3], Y, 1.0, 0.0, dtype)
+            end.record()
+            torch.cuda.synchronize()
+            best[empties] = min(best[empties], start.elapsed_time(end) / 8)
+        b200sp.b200sp_plan_destroy(plan)
+    assert best[100_000] < 1.5 * best[0], "%.1f us, without the empty rows %.1f us" % (1e3 * best[100_000], 1e3 * best[0])
