@@ -71,6 +71,9 @@ __device__ __forceinline__ void bundle_scale_span(T* y, int count, int lane, flo
   }
 }
 
+// Empty rows of ragged width from this many bytes of Y on are written as one span.
+constexpr int kBundleSpan = 2048;
+
 // A tile is kMergeWarps regions, one per warp.  What crosses the ends of a region goes to head_s / carry_s and is put together inside the tile after one
 // barrier; what crosses the ends of the tile goes to tile_carry / tile_tail and is finished by spmm_merge_fixup_kernel, as for spmm_merge_kernel: fixed order, no
 // atomics.  split[i]: row ends before item i * per.
@@ -136,6 +139,8 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
 #pragma unroll
     for (int i = 0; i < (BETA ? NY : 0); ++i) if (YV == VEC || i * YV < left) old[i] = *((const yraw*)yp + i);
   };
+  int lanes_y = 32;                                          // lanes to a row of Y, one store each: a power of two
+  while (YV != VEC && lanes_y > 1 && (lanes_y / 2) * YV >= k) lanes_y /= 2;
   // Pieces of rows: length << 20 | row of the region << 10 | first nonzero.  Piece `rows`: of the row left unfinished.  Rows without nonzeros are
   // written on the way.
   int listed = 0, before0 = 0;
@@ -151,10 +156,39 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
     listed += __popc(fulls);
     if (none) {
       if constexpr (YV != VEC) {
-        for (unsigned rest = none; rest;) {                    // runs of empty rows
-          const int first = __ffs(rest) - 1, run = __ffs(~(rest >> first)) - 1, count = run < 0 ? 32 : run;
-          rest &= ~((count == 32 ? ~0u : (1u << count) - 1u) << first);
-          bundle_scale_span<T, BETA>(Y + (long long)(r_lo + i0 + first) * k, count * k, lane, alpha, beta);
+        // runs of 2 KB or more as one span, what is left by as many lanes to a row as it has stores, several rows in flight
+        unsigned apart = none;
+        if (__popc(none) * k >= kBundleSpan / (int)sizeof(T))
+          for (unsigned rest = none; rest;) {
+            const int first = __ffs(rest) - 1, run = __ffs(~(rest >> first)) - 1, count = run < 0 ? 32 : run;
+            const unsigned these = (count == 32 ? ~0u : (1u << count) - 1u) << first;
+            rest &= ~these;
+            if (count * k >= kBundleSpan / (int)sizeof(T)) {
+              apart &= ~these;
+              bundle_scale_span<T, BETA>(Y + (long long)(r_lo + i0 + first) * k, count * k, lane, alpha, beta);
+            }
+          }
+        if ((apart >> lane) & 1u) empty_rows[__popc(apart & below)] = (unsigned char)lane;
+        __syncwarp();
+        constexpr int NC = KS > 32 * YV ? KS / (32 * YV) : 1, R = LANES == 4 ? 4 : 8 / NC;
+        const int empties = __popc(apart), sub = lane / lanes_y, step = 32 / lanes_y, c0 = (lane & (lanes_y - 1)) * YV;
+        T* const y0 = Y + (long long)(r_lo + i0) * k + c0;
+        const float zero[YV] = {};
+        for (int j = sub; j < empties; j += R * step) {
+          yraw old[R][NC][1];
+          T* yp[R];
+#pragma unroll
+          for (int u = 0; u < R; ++u) {
+            yp[u] = y0 + (long long)empty_rows[min(j + u * step, empties - 1)] * k;
+#pragma unroll
+            for (int c = 0; c < (BETA ? NC : 0); ++c)
+              if (j + u * step < empties && c0 + 32 * YV * c < k) old[u][c][0] = *(const yraw*)(yp[u] + 32 * YV * c);
+          }
+#pragma unroll
+          for (int u = 0; u < R; ++u)
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+              if (j + u * step < empties && c0 + 32 * YV * c < k) bundle_store<T, YV, YV, BETA>(yp[u] + 32 * YV * c, YV, zero, alpha, beta, old[u][c]);
         }
       } else {
         if (empty) empty_rows[__popc(none & below)] = (unsigned char)lane;
