@@ -411,6 +411,9 @@ bool spmm_wide_pieces(const b200sp_plan_info_t& I, int64_t k, int sms, int64_t l
   return (quads || 2 * I.max_row_len >= 3 * I.min_row_len) && (waves <= 1.0 || waves >= 2.6);
 }
 
+// alpha * 0 + beta * y for rows without nonzeros as one number: the factor of y, or the value itself with beta == 0.
+float spmm_none(float alpha, float beta) { return beta == 0.0f ? alpha * 0.0f : std::isfinite(alpha) ? beta : std::numeric_limits<float>::quiet_NaN(); }
+
 template <typename T, int V, int J, int MODE>
 int launch_spmm_merge_as(b200sp_plan* p, const b200sp_plan::Shares& work, int k, const int32_t* col_idx, const T* vals, const T* B, T* Y, float alpha, float beta,
                       cudaStream_t stream, DeviceInfo* dev) {
@@ -449,7 +452,7 @@ int launch_spmm_merge_as(b200sp_plan* p, const b200sp_plan::Shares& work, int k,
   if (rc != B200SP_OK) return rc;
   tl_pdl_kernel = true;
   rc = launch(kernel, dim3((unsigned)(slices * tiles)), dim3(kMergeWarps * 32), stream, B, (size_t)I.n * k * sizeof(T), dev,
-              (int)I.m, (int)I.nnz, k, tiles, witems, shares, work.split, p->row_ptr, col_idx, vals, B, Y, scratch, scratch + per, tile_row, alpha, beta);
+              (int)I.m, (int)I.nnz, k, tiles, witems, shares, work.split, p->row_ptr, col_idx, vals, B, Y, scratch, scratch + per, tile_row, alpha, beta, spmm_none(alpha, beta));
   if (rc == B200SP_OK && tiles > 1) {
     tl_pdl_kernel = true;
     const int lanes = KS >= 128 ? 128 : KS;      // a power of two
@@ -522,7 +525,7 @@ int launch_spmm_bundle_as(b200sp_plan* p, const b200sp_plan::Shares& work, int k
   tl_pdl_kernel = true;
   rc = launch_smem(spmm_bundle_kernel<T, LANES, YV, BETA>, dim3((unsigned)tiles), dim3(kMergeWarps * 32), (size_t)kMergeWarps * bundle_bytes(region), stream, B,
                    (size_t)I.n * row_bytes, dev, (int)I.m, (int)I.nnz, k, row_bytes, region, work.split, work.witems, p->row_ptr, col_idx, vals, B, Y, scratch,
-                   scratch + per, tile_row, alpha, beta);
+                   scratch + per, tile_row, alpha, beta, spmm_none(alpha, beta));
   if (rc == B200SP_OK && tiles > 1) {
     tl_pdl_kernel = true;
     const int lanes = KS >= 128 ? 128 : KS;      // a power of two

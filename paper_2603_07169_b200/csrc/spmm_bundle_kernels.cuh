@@ -43,14 +43,22 @@ __device__ __forceinline__ void bundle_store(T* yp, int left, const float (&acc)
     }
 }
 
-// y = alpha * 0 + beta * y over `count` elements by a warp: whole rows, whatever their width, in pieces of 16 bytes but for what lies before the first boundary of
-// 16 bytes and after the last.  (40,000 rows of 20 and 100,000 empty ones, BF16 k = 127, beta = 0: 271 us with the columns of each row written one by one by the
-// lanes that hold its pieces.)
+// Y's VEC columns of a lane in a row without nonzeros.  none: the factor of its old values (BETA), or what it gets.  A parameter of the kernel, which takes no
+// register; alpha * 0 would (R-MAT 2^17, k = 63 FP32, beta = 1: 84 / 116 us).
+template <typename T, int VEC, int YV, bool BETA>
+__device__ __forceinline__ void bundle_store_empty(T* yp, int left, float none, const typename Piece<T, YV>::raw (&old)[BETA ? VEC / YV : 1]) {
+  float acc[VEC];
+#pragma unroll
+  for (int j = 0; j < VEC; ++j) acc[j] = BETA ? 0.0f : none;
+  bundle_store<T, VEC, YV, BETA>(yp, left, acc, BETA ? 0.0f : 1.0f, none, old);
+}
+
+// The same over `count` elements by a warp: whole rows, whatever their width, in pieces of 16 bytes but for what lies before the first boundary of
+// 16 bytes and after the last.
 template <typename T, bool BETA>
-__device__ __forceinline__ void bundle_scale_span(T* y, int count, int lane, float alpha, float beta) {
+__device__ __forceinline__ void bundle_empty_span(T* y, int count, int lane, float none) {
   constexpr int VEC = 16 / sizeof(T);
   typedef typename Piece<T, VEC>::raw raw;
-  const float zero[VEC] = {}, zero_1[1] = {};
   const int before = min(count, (int)((16u - ((unsigned)(uintptr_t)y & 15u)) & 15u) / (int)sizeof(T));
   const int pieces = (count - before) / VEC, after = count - before - pieces * VEC;
   T* const body = y + before;
@@ -61,18 +69,21 @@ __device__ __forceinline__ void bundle_scale_span(T* y, int count, int lane, flo
       for (int u = 0; u < 4; ++u) if (p + 32 * u < pieces) old[u][0] = *((const raw*)body + p + 32 * u);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) if (p + 32 * u < pieces) bundle_store<T, VEC, VEC, BETA>(body + (p + 32 * u) * VEC, VEC, zero, alpha, beta, old[u]);
+    for (int u = 0; u < 4; ++u) if (p + 32 * u < pieces) bundle_store_empty<T, VEC, VEC, BETA>(body + (p + 32 * u) * VEC, VEC, none, old[u]);
   }
   T* const at = lane < before ? y + lane : body + pieces * VEC + (lane - before);
   if (lane < before + after) {
     typename Piece<T, 1>::raw old_1[1];
     if constexpr (BETA) old_1[0] = *at;
-    bundle_store<T, 1, 1, BETA>(at, 1, zero_1, alpha, beta, old_1);
+    bundle_store_empty<T, 1, 1, BETA>(at, 1, none, old_1);
   }
 }
 
-// Empty rows of ragged width from this many bytes of Y on are written as one span.
-constexpr int kBundleSpan = 2048;
+// Rows without nonzeros are written as others are, by the lanes that hold a piece of B, several rows at a time; BF16 of ragged width above 32 columns apart, where
+// a lane has columns one or two at a time to store: consecutive empty rows of so many bytes of Y are one span, whatever k is, and with odd k a warp takes shorter runs
+// row by row.  40,000 rows of 20 and 100,000 empty ones, by lanes / so: k = 127 293 / 45 us, k = 63 146 / 26 us, k = 50 and beta = 1 56 / 35 us.  R-MAT 2^17, beta = 1: k = 63
+// 140 / 75 us, k = 50 56 / 54 us (61 us with k = 50 row by row).  FP32 spills for it (R-MAT 2^17, k = 63, beta = 1 84 / 95 us).
+constexpr int kBundleSpan = 512, kBundleSpanByLanes = 2048;
 
 // A tile is kMergeWarps regions, one per warp.  What crosses the ends of a region goes to head_s / carry_s and is put together inside the tile after one
 // barrier; what crosses the ends of the tile goes to tile_carry / tile_tail and is finished by spmm_merge_fixup_kernel, as for spmm_merge_kernel: fixed order, no
@@ -81,8 +92,9 @@ template <typename T, int LANES, int YV, bool BETA>
 __global__ void __launch_bounds__(kMergeWarps * 32, kBundleCtas<T>)
 spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* __restrict__ split, int per, const int* __restrict__ row_ptr,
                    const int* __restrict__ col_idx, const T* __restrict__ vals, const T* __restrict__ B, T* __restrict__ Y,
-                   float* __restrict__ tile_carry, float* __restrict__ tile_tail, int2* __restrict__ tile_row, float alpha, float beta) {
+                   float* __restrict__ tile_carry, float* __restrict__ tile_tail, int2* __restrict__ tile_row, float alpha, float beta, float none) {
   constexpr int VEC = 16 / sizeof(T), G = 32 / LANES, KS = LANES * VEC, NY = VEC / YV, U = 4;   // U: loads of B in flight per lane
+  constexpr bool BY_WARP = NY >= 8 && LANES >= 8;             // empty rows apart from others: see kBundleSpan
   typedef typename Piece<T, VEC>::raw raw;
   typedef typename Piece<T, YV>::raw yraw;
   extern __shared__ __align__(16) unsigned char bundle_smem[];
@@ -139,8 +151,6 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
 #pragma unroll
     for (int i = 0; i < (BETA ? NY : 0); ++i) if (YV == VEC || i * YV < left) old[i] = *((const yraw*)yp + i);
   };
-  int lanes_y = 32;                                          // lanes to a row of Y, one store each: a power of two
-  while (YV != VEC && lanes_y > 1 && (lanes_y / 2) * YV >= k) lanes_y /= 2;
   // Pieces of rows: length << 20 | row of the region << 10 | first nonzero.  Piece `rows`: of the row left unfinished.  Rows without nonzeros are
   // written on the way.
   int listed = 0, before0 = 0;
@@ -150,50 +160,48 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
     int before = __shfl_up_sync(0xFFFFFFFFu, e, 1);
     if (lane == 0) before = before0;
     before0 = __shfl_sync(0xFFFFFFFFu, e, 31);
-    const bool full = i <= rows && e > before, empty = i < rows && e == before && !(head && i == 0);
-    const unsigned fulls = __ballot_sync(0xFFFFFFFFu, full), none = __ballot_sync(0xFFFFFFFFu, empty), below = (1u << lane) - 1u;
+    const bool full = i <= rows && e > before, vacant = i < rows && e == before && !(head && i == 0);
+    const unsigned fulls = __ballot_sync(0xFFFFFFFFu, full), vacants = __ballot_sync(0xFFFFFFFFu, vacant), below = (1u << lane) - 1u;
     if (full) list[listed + __popc(fulls & below)] = ((unsigned)(e - before) << 20) | (unsigned)(i << 10) | (unsigned)before;
     listed += __popc(fulls);
-    if (none) {
-      if constexpr (YV != VEC) {
-        // runs of 2 KB or more as one span, what is left by as many lanes to a row as it has stores, several rows in flight
-        unsigned apart = none;
-        if (__popc(none) * k >= kBundleSpan / (int)sizeof(T))
-          for (unsigned rest = none; rest;) {
+    if (vacants) {
+      unsigned apart = vacants;                                   // without long runs of empty rows, which are written as one span
+      if constexpr (sizeof(T) == 2 && YV != VEC && LANES >= 8) {
+        constexpr int LEAST = (BY_WARP ? kBundleSpan : kBundleSpanByLanes) / (int)sizeof(T);
+        if (__popc(vacants) * k >= LEAST)
+          for (unsigned rest = vacants; rest;) {
             const int first = __ffs(rest) - 1, run = __ffs(~(rest >> first)) - 1, count = run < 0 ? 32 : run;
             const unsigned these = (count == 32 ? ~0u : (1u << count) - 1u) << first;
             rest &= ~these;
-            if (count * k >= kBundleSpan / (int)sizeof(T)) {
+            if (count * k >= LEAST) {
               apart &= ~these;
-              bundle_scale_span<T, BETA>(Y + (long long)(r_lo + i0 + first) * k, count * k, lane, alpha, beta);
+              bundle_empty_span<T, BETA>(Y + (long long)(r_lo + i0 + first) * k, count * k, lane, none);
             }
           }
-        if ((apart >> lane) & 1u) empty_rows[__popc(apart & below)] = (unsigned char)lane;
-        __syncwarp();
-        constexpr int NC = KS > 32 * YV ? KS / (32 * YV) : 1, R = LANES == 4 ? 4 : 8 / NC;
-        const int empties = __popc(apart), sub = lane / lanes_y, step = 32 / lanes_y, c0 = (lane & (lanes_y - 1)) * YV;
-        T* const y0 = Y + (long long)(r_lo + i0) * k + c0;
-        const float zero[YV] = {};
-        for (int j = sub; j < empties; j += R * step) {
+      }
+      if ((apart >> lane) & 1u) empty_rows[__popc(apart & below)] = (unsigned char)lane;
+      __syncwarp();
+      const int empties = __popc(apart);
+      if constexpr (BY_WARP) {
+        constexpr int NC = KS / 32, R = 8 / NC;
+        T* const y0 = Y + (long long)(r_lo + i0) * k + lane;
+        for (int j = 0; j < empties; j += R) {
           yraw old[R][NC][1];
           T* yp[R];
 #pragma unroll
           for (int u = 0; u < R; ++u) {
-            yp[u] = y0 + (long long)empty_rows[min(j + u * step, empties - 1)] * k;
+            yp[u] = y0 + (long long)empty_rows[min(j + u, empties - 1)] * k;
 #pragma unroll
             for (int c = 0; c < (BETA ? NC : 0); ++c)
-              if (j + u * step < empties && c0 + 32 * YV * c < k) old[u][c][0] = *(const yraw*)(yp[u] + 32 * YV * c);
+              if (j + u < empties && lane + 32 * c < k) old[u][c][0] = *(const yraw*)(yp[u] + 32 * c);
           }
 #pragma unroll
           for (int u = 0; u < R; ++u)
 #pragma unroll
             for (int c = 0; c < NC; ++c)
-              if (j + u * step < empties && c0 + 32 * YV * c < k) bundle_store<T, YV, YV, BETA>(yp[u] + 32 * YV * c, YV, zero, alpha, beta, old[u][c]);
+              if (j + u < empties && lane + 32 * c < k) bundle_store_empty<T, 1, 1, BETA>(yp[u] + 32 * c, 1, none, old[u][c]);
         }
       } else {
-        if (empty) empty_rows[__popc(none & below)] = (unsigned char)lane;
-        __syncwarp();
-        const int empties = __popc(none);
         T* const y0 = Yc + (long long)i0 * k;
         for (int j = g; j < empties; j += 4 * G) {
           yraw old[4][BETA ? NY : 1];
@@ -203,10 +211,9 @@ spmm_bundle_kernel(int m, int nnz, int k, int row_bytes, int region, const int* 
             yp[u] = y0 + (long long)empty_rows[min(j + u * G, empties - 1)] * k;
             if constexpr (BETA) { if (j + u * G < empties && on) ask_old(yp[u], old[u]); }
           }
-          const float zero[VEC] = {};
 #pragma unroll
           for (int u = 0; u < 4; ++u)
-            if (j + u * G < empties && on) bundle_store<T, VEC, YV, BETA>(yp[u], left, zero, alpha, beta, old[u]);
+            if (j + u * G < empties && on) bundle_store_empty<T, VEC, YV, BETA>(yp[u], left, none, old[u]);
         }
       }
       __syncwarp();

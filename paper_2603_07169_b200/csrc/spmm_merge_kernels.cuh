@@ -189,11 +189,12 @@ template <> struct MergeStage<bf16_t> {
 // former).  Not in kMergeNoRoom's forms, which have no registers left for them.
 // 2: beta != 0 and empty rows, which are listed apart (see below); the listing costs 2-5 % where there are none, and old values asked for
 // ahead cost it more than they save (R-MAT 2^20, k = 64 FP32 303 / 442 us).
+// none: what mode 2 multiplies the old values of an empty row by.
 template <typename T, int V, int J, int MODE>
 __global__ void __launch_bounds__(kMergeWarps * 32, (merge_ctas<T, V, J>()))
 spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, const int* __restrict__ split, const int* __restrict__ row_ptr,
                   const int* __restrict__ col_idx, const T* __restrict__ vals, const T* __restrict__ B, T* __restrict__ Y,
-                  float* __restrict__ tile_carry, float* __restrict__ tile_tail, int2* __restrict__ tile_row, float alpha, float beta) {
+                  float* __restrict__ tile_carry, float* __restrict__ tile_tail, int2* __restrict__ tile_row, float alpha, float beta, float none) {
   constexpr int U = kMergeUnroll<V, J>, KS = 32 * V * J;
   constexpr bool LIST = MODE == 2, AHEAD = MODE == 1 && !kMergeNoRoom<T, V, J>;
   typedef typename Piece<T, V>::raw raw;
@@ -256,7 +257,7 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
     for (int j = 0; j < (AHEAD ? J : 0); ++j) if (on[j]) old[j] = *(const raw*)(yrow + 32 * V * j);
   };
   if (AHEAD && r_first < m) ask_old();
-  // rows empty_s[warp][0 .. count) of the share whose first row is at ys: y = alpha * 0 + beta * y over the slice's columns
+  // rows empty_s[warp][0 .. count) of the share whose first row is at ys: y = none * y over the slice's columns
   auto scale_rows = [&](T* ys, int count) {
     const int width = min(KS, k - slice * KS);
     const bool wide = V * sizeof(T) < 16 && k * (int)sizeof(T) % 16 == 0;       // 16 bytes a lane where the rows allow it
@@ -273,12 +274,12 @@ spmm_merge_kernel(int m, int nnz, int k, int tiles, int witems, int shares, cons
           float zero[16 / sizeof(T)];
 #pragma unroll
           for (int x = 0; x < 16 / (int)sizeof(T); ++x) zero[x] = 0.0f;
-          piece_store<T, 16 / (int)sizeof(T)>(y, zero, alpha, beta);
+          piece_store<T, 16 / (int)sizeof(T)>(y, zero, 0.0f, none);
         } else {
           float zero[V];
 #pragma unroll
           for (int x = 0; x < V; ++x) zero[x] = 0.0f;
-          piece_store<T, V>(y, zero, alpha, beta);
+          piece_store<T, V>(y, zero, 0.0f, none);
         }
       }
     }

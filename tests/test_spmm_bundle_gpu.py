@@ -146,7 +146,7 @@ def test_padded_calls_read_what_the_calls_just_before_them_wrote(dtype, k, pdl):
 
 
 @needs_plain_build
-@pytest.mark.parametrize("dtype,k", [("bf16", 63), ("bf16", 126), ("bf16", 127), ("f32", 63)])
+@pytest.mark.parametrize("dtype,k", [("bf16", 50), ("bf16", 63), ("bf16", 126), ("bf16", 127)])
 def test_empty_rows_of_ragged_width_cost_little_more_than_their_bytes(dtype, k):
     """The same nonzeros with and without 100,000 empty rows behind them, whole regions of nothing else.  One column at a time by the lanes that hold a
     piece of B, these took longer than the products."""
