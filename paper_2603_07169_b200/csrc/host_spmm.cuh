@@ -537,6 +537,9 @@ int launch_spmm_bundle_as(b200sp_plan* p, const b200sp_plan::Shares& work, int k
   return rc;
 }
 
+// Bytes of a row of the padded copy of B: whole lines (32-byte steps measured the same to 10 % more and less).
+int64_t spmm_padded_row(int64_t k, int elem_bytes) { return (k * elem_bytes + 127) / 128 * 128; }
+
 // Columns of Y per store: all of a lane's where k is a multiple of 16 bytes; else B is copied into padded rows first (one kernel and n rows of memory from the
 // pool) and Y is written by pairs (even k) or one by one.
 template <typename T, int YV>
@@ -549,7 +552,7 @@ int run_spmm_bundle(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals
   T* padded = nullptr;
   int row_bytes = k * (int)sizeof(T);
   if (YV != VEC) {
-    row_bytes = (row_bytes + 127) / 128 * 128;   // whole lines (32-byte steps measured the same to 10 % more and less)
+    row_bytes = (int)spmm_padded_row(k, (int)sizeof(T));
     rc = pool_alloc(dev, (void**)&padded, (size_t)p->info.n * row_bytes, stream);
     if (rc != B200SP_OK) return rc;
     const long long blocks = (p->info.n + 31) / 32;
@@ -574,6 +577,34 @@ int run_spmm_bundle(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals
   return rc;
 }
 
+// Of the calls that go by shares with k no multiple of 16 bytes, those that spmm_bundle_kernel takes, with a padded copy of B: where spmm_merge_kernel loads single elements (odd k) or pairs of BF16, and B is read often enough, rows are long enough and the copy is small enough for it to pay:
+// a row of the copy takes 128 bytes at least, and one that does not fit L2 beside the rest is read from memory.  Lines drawn over 3027 calls that a laxer rule takes
+// (log-normal rows of 4 to 24, 25,000 to 800,000 of them, half to twice as many columns; the same with 12 % of the rows empty; R-MAT 2^16 to 2^21 with hubs packed and spread;
+// k = 2 .. 127): those taken are 1.34 times as fast as by shares, ten slower by more than 3 %, one of them by 12 %; those left would be 0.99.  By shares / side by side, us:
+// - BF16, odd k above 32, which by shares takes two loads of one element or more a nonzero: from 350,000 items, rows of seven and five reads of a row of B on, over copies of
+//   any size (50,000 rows of 14, n = 100,000, k = 33 24 / 14; 200,000 rows of 4, n = 100,000, k = 63 43 / 56: single stores of Y).
+// - beta != 0 and a sixteenth of the rows empty, which spmm_merge_kernel lists first: seven reads (R-MAT 2^18, k = 50 BF16 179 / 78; k = 17 FP32 138 / 66), up to 16 columns only
+//   while the copy takes less than a quarter of L2 (R-MAT 2^19, k = 3 BF16 95 / 106).
+// - beta == 0 and a quarter of the rows empty: BF16, eight reads, from 1 M items on, 2 M with more stores a row (R-MAT 2^18, k = 50 BF16 67 / 58, k = 127 153 / 138; 2^17 32 / 36 and
+//   79 / 92); not FP32 above 16 columns (R-MAT 2^17, k = 63 50 / 72), nor copies of more than a quarter of L2 (R-MAT 2^19, k = 50 95 / 102) but for odd k above 32.
+// - Odd k of 17 to 31, one load a nonzero by shares and up to eight stores a row here: with beta == 0 only small copies read 15 times (100,000 rows of 24, k = 17 FP32 44 / 38;
+//   100,000 of 14 26 / 28).
+// - The rest: ten reads (beta != 0: eight) while the copy takes less than a quarter of L2 (200,000 rows of 9, n = 200,000, k = 50 BF16 42.3 / 44.9; n = 100,000 43 / 39), beyond that 16,
+//   or 12 where a nonzero takes two loads by shares (400,000 rows of 14, k = 63 FP32 233 / 163); from 450,000, 600,000 or 900,000 items on.
+bool spmm_by_padded_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, float beta) {
+  const int64_t items = I.m + I.nnz, vec = 16 / elem_bytes, copy = I.n * spmm_padded_row(k, elem_bytes);
+  const bool bf16 = elem_bytes == 2, odd = k % 2 != 0, one_load = k <= (odd ? 32 : 64), small = copy <= 36000000;
+  if ((k + vec - 1) / vec > 16 || (!odd && (!bf16 || k % 4 != 2))) return false;
+  auto reads = [&](int64_t times) { return I.nnz >= times * I.n; };
+  const bool mostly = beta == 0.0f && I.bin_rows[0] * 4 >= I.m;             // a quarter of the rows or more are empty, and only written
+  if (bf16 && odd && k > 32) return mostly ? reads(8) && items >= (k > 40 ? 2000000 : 1000000) : reads(5) && I.nnz >= 7 * I.m && items >= 350000;
+  if (beta != 0.0f && I.bin_rows[0] * 16 >= I.m) return reads(7) && items >= 450000 && (k > 16 || !odd || small);
+  if (odd && k > 16 && k <= 32 && beta == 0.0f) return !mostly && reads(15) && copy <= 16000000 && items >= 1000000;
+  if (mostly) return reads(8) && small && items >= (odd || k > 64 ? 2000000 : 1000000) && (bf16 || k <= 16);
+  if (items < (!bf16 && one_load ? 900000 : !bf16 || one_load ? 600000 : 450000)) return false;
+  return reads(small ? (beta != 0.0f ? 8 : 10) : one_load || beta != 0.0f ? 16 : 12);
+}
+
 // Of the calls that go by shares, those whose rows of B are narrow for spmm_merge_kernel go to spmm_bundle_kernel.  Times: shares / bundles, us.
 // - k a multiple of 16 bytes, up to eight pieces of 16 bytes a row of B, four rows or more side by side, from 250,000 items on (four pieces) or 350,000 (BF16) or
 //   600,000 (FP32): 250,000 log-normal rows of 8, BF16 k = 64 46 / 35, FP32 k = 16 64 / 41; R-MAT 2^20, BF16 k = 64 162 / 106, FP32 k = 32 152 / 122.
@@ -582,18 +613,11 @@ int run_spmm_bundle(b200sp_plan* p, int k, const int32_t* col_idx, const T* vals
 //   from loads twice as wide than it loses at the ends of rows (R-MAT 2^22, k = 64 759 / 797), except
 // - where beta != 0 and a sixteenth of the rows is empty, which spmm_merge_kernel lists first: from 60,000 items on (R-MAT 2^20,
 //   FP32 k = 64 303 / 240, 2^14 13.9 / 12.3; BF16 k = 64 248 / 182), and up to 32 pieces of FP32 from 250,000 on (R-MAT 2^15, k = 128 50 / 36; 2^14 17.4 / 19.7).
-// - Other k, with a padded copy of B: where spmm_merge_kernel loads single elements (odd k) or pairs of BF16, and B is read often enough to pay for the copy.
-//   BF16: odd k from 4.4 reads of a row of B on (100,001 rows of 11, k = 127 81 / 61, k = 33 47 / 33), k = 2 modulo 4 from 6 on (150,001 rows of 11,
-//   k = 50 beta = 1 48.2 / 40.4; but 80,000 of 9 and 4.5 reads 0.87x).  FP32: odd k up to 64 columns from 6 on (k = 33 51 / 43).
 bool spmm_by_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, float beta) {
   const int64_t items = I.m + I.nnz, vec = 16 / elem_bytes, pieces = (k + vec - 1) / vec;
-  if (k % vec == 0) {
-    if (beta != 0.0f && I.bin_rows[0] * 16 >= I.m) return pieces <= 16 ? items >= 60000 : elem_bytes == 4 && pieces <= 32 && items >= 250000;
-    return pieces <= 4 ? items >= 250000 : pieces <= 8 ? items >= (elem_bytes == 2 ? 350000 : 600000) : elem_bytes == 2 && pieces <= 16 && items >= 600000;
-  }
-  if (pieces > 16) return false;
-  if (elem_bytes == 2 && k % 2 != 0) return items >= 300000 && (double)I.nnz >= 4.4 * (double)I.n;
-  return k % (elem_bytes == 2 ? 4 : 2) == (elem_bytes == 2 ? 2 : 1) && items >= 450000 && I.nnz >= 6 * I.n;
+  if (k % vec != 0) return spmm_by_padded_bundles(I, k, elem_bytes, beta);
+  if (beta != 0.0f && I.bin_rows[0] * 16 >= I.m) return pieces <= 16 ? items >= 60000 : elem_bytes == 4 && pieces <= 32 && items >= 250000;
+  return pieces <= 4 ? items >= 250000 : pieces <= 8 ? items >= (elem_bytes == 2 ? 350000 : 600000) : elem_bytes == 2 && pieces <= 16 && items >= 600000;
 }
 
 // Rows all of one length of 5 to 13 that is no multiple of four, k a multiple of 16 bytes and five to sixteen pieces of them a row of B: by rows they take single

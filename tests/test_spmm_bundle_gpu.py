@@ -148,12 +148,12 @@ def test_padded_calls_read_what_the_calls_just_before_them_wrote(dtype, k, pdl):
 @needs_plain_build
 @pytest.mark.parametrize("dtype,k", [("bf16", 50), ("bf16", 63), ("bf16", 126), ("bf16", 127)])
 def test_empty_rows_of_ragged_width_cost_little_more_than_their_bytes(dtype, k):
-    """The same nonzeros with and without 100,000 empty rows behind them, whole regions of nothing else.  One column at a time by the lanes that hold a
+    """The same nonzeros with and without 250,000 empty rows behind them, whole regions of nothing else.  One column at a time by the lanes that hold a
     piece of B, these took longer than the products."""
-    lens = np.random.default_rng(3).integers(2, 40, 40_000)
+    lens = np.random.default_rng(3).integers(2, 40, 100_000)
     n = len(lens)
     best = {}
-    for empties in (0, 100_000):
+    for empties in (0, 250_000):
         A = gen.random_csr(n + empties, n, np.concatenate([lens, np.zeros(empties, np.int64)]), seed=6, sort_cols=False)
         assert by_bundles(A, k, 0.0, dtype)
         d = [to_dev(a) for a in (A.row_ptr, A.col_idx, store(A.vals, dtype), store(np.ones(n * k, np.float32), dtype))]
@@ -169,4 +169,4 @@ def test_empty_rows_of_ragged_width_cost_little_more_than_their_bytes(dtype, k):
             torch.cuda.synchronize()
             best[empties] = min(best[empties], start.elapsed_time(end) / 8)
         b200sp.b200sp_plan_destroy(plan)
-    assert best[100_000] < 1.5 * best[0], "%.1f us, without the empty rows %.1f us" % (1e3 * best[100_000], 1e3 * best[0])
+    assert best[250_000] < 1.5 * best[0], "%.1f us, without the empty rows %.1f us" % (1e3 * best[250_000], 1e3 * best[0])

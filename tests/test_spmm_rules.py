@@ -115,3 +115,34 @@ def test_equal_rows_stay_by_rows_where_a_switch_asks_for_it(dtype, k, rows, swit
     finally:
         b200sp.b200sp_set_option(switch, default)
     assert b200sp.b200sp_spmm_by_bundles(stats, k, 0.0, dtype)
+
+
+def uneven(m, n, per_row, empty=0.0):
+    """per_row nonzeros a row on average, `empty` of the rows without any, and eleven long rows."""
+    none, nnz = int(m * empty), m * per_row
+    return info(m, n, [none, 0, m - none - 11, 0, 10, 1], [0, 0, nnz - 10_000, 0, 5000, 5000], 5000)
+
+
+@pytest.mark.parametrize("stats,dtype,k,beta,taken", [
+    # measured by shares and side by side; BF16 with odd k above 32: short rows are not
+    (uneven(50_000, 100_000, 14), "bf16", 33, 0.0, True), (uneven(200_000, 100_000, 4), "bf16", 63, 0.0, False), (uneven(800_000, 800_000, 9), "bf16", 127, 0.0, True),
+    (uneven(50_000, 50_000, 6), "bf16", 127, 1.0, False), (uneven(25_000, 12_500, 14), "bf16", 95, 0.0, True),
+    # many empty rows, old values of Y read: the copy may be large but for narrow rows
+    (uneven(1 << 18, 1 << 18, 8, 0.6), "bf16", 50, 1.0, True), (uneven(1 << 21, 1 << 21, 8, 0.6), "f32", 63, 1.0, True), (uneven(1 << 18, 1 << 18, 8, 0.6), "f32", 17, 1.0, True),
+    (uneven(1 << 18, 1 << 18, 8, 0.6), "bf16", 3, 1.0, True), (uneven(1 << 19, 1 << 19, 8, 0.6), "bf16", 3, 1.0, False), (uneven(1 << 18, 1 << 18, 6, 0.6), "bf16", 50, 1.0, False),
+    # many empty rows that are only written: BF16, in two waves or more, from copies that stay in L2
+    (uneven(1 << 18, 1 << 18, 8, 0.6), "bf16", 50, 0.0, True), (uneven(1 << 19, 1 << 19, 8, 0.6), "bf16", 50, 0.0, False), (uneven(1 << 17, 1 << 17, 8, 0.6), "bf16", 127, 0.0, False),
+    (uneven(1 << 18, 1 << 18, 8, 0.6), "bf16", 127, 0.0, True), (uneven(1 << 19, 1 << 19, 8, 0.6), "bf16", 33, 0.0, True), (uneven(1 << 18, 1 << 18, 8, 0.6), "bf16", 17, 0.0, False),
+    (uneven(1 << 18, 1 << 18, 8, 0.6), "f32", 63, 0.0, False), (uneven(1 << 18, 1 << 18, 8, 0.6), "f32", 9, 0.0, True), (uneven(1 << 17, 1 << 17, 8, 0.6), "bf16", 9, 0.0, False),
+    # odd k of 17 to 31 without old values: small copies, read often
+    (uneven(100_000, 100_000, 24), "f32", 17, 0.0, True), (uneven(100_000, 100_000, 14), "f32", 17, 0.0, False), (uneven(100_000, 100_000, 14), "f32", 17, 1.0, True),
+    (uneven(150_000, 150_000, 24), "bf16", 31, 0.0, False),
+    # the rest: how often a row of the copy is read, and whether it stays in L2
+    (uneven(200_000, 200_000, 9), "bf16", 50, 0.0, False), (uneven(200_000, 100_000, 9), "bf16", 50, 0.0, True), (uneven(200_000, 200_000, 9), "bf16", 50, 1.0, True),
+    (uneven(400_000, 400_000, 14), "f32", 63, 0.0, True), (uneven(400_000, 400_000, 14), "f32", 63, 1.0, False), (uneven(400_000, 400_000, 14), "bf16", 50, 0.0, False),
+    (uneven(400_000, 400_000, 16), "bf16", 50, 0.0, True), (uneven(1_000_000, 1_000_000, 10), "f32", 5, 0.0, False), (uneven(150_000, 150_000, 11), "f32", 5, 0.0, True),
+    (uneven(45_000, 45_000, 11), "f32", 5, 0.0, False), (uneven(1_000_000, 1_000_000, 10), "bf16", 2, 0.0, False), (uneven(45_000, 45_000, 11), "bf16", 10, 0.0, False),
+    (uneven(60_000, 60_000, 11), "bf16", 10, 0.0, True)])
+def test_a_padded_copy_of_b_only_where_it_pays(stats, dtype, k, beta, taken):
+    assert b200sp.b200sp_spmm_by_shares(stats, k, beta, dtype)
+    assert b200sp.b200sp_spmm_by_bundles(stats, k, beta, dtype) == taken
