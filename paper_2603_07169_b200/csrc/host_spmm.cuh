@@ -621,22 +621,32 @@ bool spmm_by_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, flo
 }
 
 // Rows all of one length of 5 to 13 that is no multiple of four, k a multiple of 16 bytes and five to sixteen pieces of them a row of B: by rows they take single
-// steps at both ends of nearly every row, side by side only at one.  From 1 M items on with up to eight pieces (BF16; 2 M for FP32, 5 M
-// there for rows of 11 and 13 and in both for rows of 10: 240,000 of them, beta = 1, BF16 k = 64 45.2 / 49.5), from 780,000 on with more.  By rows / side by side, us: 131,072 rows of 7, k = 64 BF16 23.5 / 18.2, k = 128 41.9 / 28.6, FP32 k = 64
-// 37.6 / 29.3; of 13, BF16 k = 128 52.2 / 48.1, FP32 k = 64 47.8 / 48.0; 8 M nonzeros in rows of 6, k = 64 FP32 466 / 373, BF16 243 / 194, in rows of 13 292 / 262
-// and 158 / 136.  Not rows of 21 (FP32 k = 64 192 / 201), fewer (70,000 rows of 6, BF16 k = 64 9.4 / 13.4) or wider (k = 128 FP32, rows of 13 241 / 254).
+// steps at both ends of nearly every row, side by side only at one.  What that gains goes with the last steps that the length leaves (5 and 7 most, 10 and 13 least), with the
+// number of items, and with what the call would take by rows: BF16 whose rows of B are whole pieces of 32 bytes has a faster kernel there (spmm_slice_wide_kernel).
+// 7 lengths, 10 widths, 0.8 to 9 M items, half to twice as many columns as rows, beta = 0 and 1; least number of items, and by rows / side by side in us on both sides of it:
+// - FP32, up to eight pieces: 2 M, 5 M for rows of 10 and more (k = 32: 190,000 rows of 10 56 / 56, 96,000 25 / 35); more pieces: 780,000 for rows of 5 and 7, 1.4 M for 6, 9 and 11, 3 M
+//   for 10 and 13 (k = 36: 57,000 rows of 13 20 / 27, 114,000 of 6 22 / 28; 8 M nonzeros in rows of 6, k = 64 466 / 373).
+// - BF16, k no multiple of 16, up to eight pieces: 1 M, 5 M for rows of 10 and 13; more: 780,000 (k = 72: 111,500 rows of 6 1.19 times as fast).
+// - BF16, k a multiple of 16, up to eight pieces: 1 M for rows of 5, 6 and 7, 3 M for 9 and 11, 8 M for 10 and 13 (k = 64: 150,000 rows of 13, beta = 1 31 / 37; 131,072 of 7 23.5 / 18.2; rows
+//   of 6 gain from 2 M on and lose up to 14 % at 1 M); more: 780,000 for 5 and 7, 1 M for 6, 9 and 11, 1.5 M for 10 and 13 and these with beta == 0 only (k = 128: 131,072 rows of 7 41.9 / 28.6,
+//   364,000 of 13 and beta = 1 163 / 172).
+// Not rows of 21 (FP32 k = 64 192 / 201), fewer (70,000 rows of 6, BF16 k = 64 9.4 / 13.4) or wider (k = 128 FP32, rows of 13 241 / 254).
 // Where a switch asks for one of the kernels by rows they stay by rows.
-bool spmm_even_by_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_bytes) {
+bool spmm_even_by_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, float beta) {
   const int64_t items = I.m + I.nnz, vec = 16 / elem_bytes, pieces = k / vec;
+  const int length = I.max_row_len;
   if (!g_opt.spmm_sliced || g_opt.spmm_flat != 2 || g_opt.spmm_stage_a != 2 || g_opt.spmm_ranges != 1) return false;
-  if (I.min_row_len != I.max_row_len || I.max_row_len % 4 == 0 || I.max_row_len < 5 || I.max_row_len > 13) return false;
-  const bool gains_less = I.max_row_len > 9 && (elem_bytes == 4 || I.max_row_len % 2 == 0);
-  return k % vec == 0 && pieces >= 5 && pieces <= 16 && items >= (pieces > 8 ? 780000 : gains_less ? 5000000 : elem_bytes == 2 ? 1000000 : 2000000);
+  if (I.min_row_len != length || length % 4 == 0 || length < 5 || length > 13 || k % vec != 0 || pieces < 5 || pieces > 16) return false;
+  const bool most = length == 5 || length == 7, least = length == 10 || length == 13, wide = elem_bytes == 2 && k % 16 == 0;
+  if (elem_bytes == 4) return items >= (pieces <= 8 ? (length < 10 ? 2000000 : 5000000) : most ? 780000 : least ? 3000000 : 1400000);
+  if (!wide) return items >= (pieces > 8 ? 780000 : least ? 5000000 : 1000000);
+  if (pieces <= 8) return items >= (length <= 7 ? 1000000 : least ? 8000000 : 3000000);
+  return items >= (most ? 780000 : least ? 1500000 : 1000000) && (!least || beta == 0.0f);
 }
 
 // Whether spmm_bundle_kernel takes a call with k > 1 columns under the present switches.
 bool spmm_side_by_side(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, float beta) {
-  return spmm_by_shares(I, k, elem_bytes, beta) ? spmm_by_bundles(I, k, elem_bytes, beta) : spmm_even_by_bundles(I, k, elem_bytes);
+  return spmm_by_shares(I, k, elem_bytes, beta) ? spmm_by_bundles(I, k, elem_bytes, beta) : spmm_even_by_bundles(I, k, elem_bytes, beta);
 }
 
 template <typename T, int VEC>

@@ -146,3 +146,17 @@ def uneven(m, n, per_row, empty=0.0):
 def test_a_padded_copy_of_b_only_where_it_pays(stats, dtype, k, beta, taken):
     assert b200sp.b200sp_spmm_by_shares(stats, k, beta, dtype)
     assert b200sp.b200sp_spmm_by_bundles(stats, k, beta, dtype) == taken
+
+
+@pytest.mark.parametrize("dtype,k,length,items,beta,taken", [
+    # measured on both sides: by what the length leaves over, the number of items and the kernel by rows that would take the call
+    ("f32", 36, 13, 800_000, 0.0, False), ("f32", 36, 6, 800_000, 0.0, False), ("f32", 36, 10, 2_100_000, 1.0, False), ("f32", 64, 10, 800_000, 0.0, False),
+    ("f32", 64, 9, 1_500_000, 0.0, True), ("f32", 48, 13, 3_200_000, 0.0, True), ("f32", 32, 11, 2_100_000, 0.0, False), ("f32", 20, 7, 2_100_000, 0.0, True),
+    ("bf16", 64, 13, 2_100_000, 1.0, False), ("bf16", 64, 9, 1_050_000, 0.0, False), ("bf16", 64, 9, 3_200_000, 0.0, True), ("bf16", 64, 10, 5_100_000, 1.0, False),
+    ("bf16", 64, 11, 2_100_000, 1.0, False), ("bf16", 40, 9, 1_050_000, 1.0, True), ("bf16", 40, 13, 1_050_000, 1.0, False), ("bf16", 72, 13, 800_000, 1.0, True),
+    ("bf16", 128, 13, 5_100_000, 1.0, False), ("bf16", 128, 13, 5_100_000, 0.0, True), ("bf16", 128, 10, 800_000, 0.0, False), ("bf16", 96, 6, 800_000, 1.0, False),
+    ("bf16", 128, 7, 800_000, 1.0, True)])
+def test_equal_rows_side_by_side_only_where_they_are_faster(dtype, k, length, items, beta, taken):
+    rows = -(-items // (length + 1))
+    stats = dict(info(rows, rows, [0, 0, rows, 0, 0, 0], [0, 0, rows * length, 0, 0, 0], length), min_row_len=length)
+    assert b200sp.b200sp_spmm_by_bundles(stats, k, beta, dtype) == taken
