@@ -609,15 +609,24 @@ bool spmm_by_padded_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_byt
 // - k a multiple of 16 bytes, up to eight pieces of 16 bytes a row of B, four rows or more side by side, from 250,000 items on (four pieces) or 350,000 (BF16) or
 //   600,000 (FP32): 250,000 log-normal rows of 8, BF16 k = 64 46 / 35, FP32 k = 16 64 / 41; R-MAT 2^20, BF16 k = 64 162 / 106, FP32 k = 32 152 / 122.
 //   Below that the few regions are as long as before and start later (25,000 rows of 5, FP32 k = 32 9.0 / 10.7).
-// - Nine to sixteen pieces, two rows side by side: BF16 from 600,000 items on (80,000 rows of 9, k = 128 31 / 26; 400,000 items 16 / 20).  FP32 gains less
-//   from loads twice as wide than it loses at the ends of rows (R-MAT 2^22, k = 64 759 / 797), except
-// - where beta != 0 and a sixteenth of the rows is empty, which spmm_merge_kernel lists first: from 60,000 items on (R-MAT 2^20,
-//   FP32 k = 64 303 / 240, 2^14 13.9 / 12.3; BF16 k = 64 248 / 182), and up to 32 pieces of FP32 from 250,000 on (R-MAT 2^15, k = 128 50 / 36; 2^14 17.4 / 19.7).
+// - Nine to sixteen pieces, two rows side by side: FP32 gains less from loads twice as wide than it loses at the ends of rows (R-MAT 2^22, k = 64 759 / 797).  BF16 gains by what is
+//   left of the last wave by shares, from 800,000 items on up to 1.4 M (beta != 0 2.5 M, a sixteenth of the rows empty 3 M; 100,000 rows of 8, k = 128 1.11 times as fast, beta = 1 1.21
+//   times; 124,000 rows of 4, k = 128 25.0 / 28.5, 320,000 57.3 / 61.3, 1,000,000 of 8 252 / 280), and where a quarter of the rows is empty from 1 M on (R-MAT 2^18 1.14 times).
+// - beta != 0 and a sixteenth of the rows empty, which spmm_merge_kernel lists first: up to eight pieces from 150,000 items on, 60,000 where it is a quarter (R-MAT 2^20, FP32 k = 32 1.56
+//   times as fast, 2^13 1.09 times; 7000 rows of 14, 12 % empty 0.94 times); up to 16 from 450,000, 60,000 (BF16 120,000) where it is a quarter (R-MAT 2^20, FP32 k = 64 303 / 240, 2^14 13.9 / 12.3,
+//   BF16 k = 128 1.19 times as fast; 20,000 rows of 14, 12 % empty, k = 48 0.87 times; 600,000, k = 72 BF16 310 / 337), and up to 32 pieces of FP32 only then, from 250,000 on (R-MAT 2^15, k = 128 50 / 36; 2^14 17.4 / 19.7).
 bool spmm_by_bundles(const b200sp_plan_info_t& I, int64_t k, int elem_bytes, float beta) {
   const int64_t items = I.m + I.nnz, vec = 16 / elem_bytes, pieces = (k + vec - 1) / vec;
   if (k % vec != 0) return spmm_by_padded_bundles(I, k, elem_bytes, beta);
-  if (beta != 0.0f && I.bin_rows[0] * 16 >= I.m) return pieces <= 16 ? items >= 60000 : elem_bytes == 4 && pieces <= 32 && items >= 250000;
-  return pieces <= 4 ? items >= 250000 : pieces <= 8 ? items >= (elem_bytes == 2 ? 350000 : 600000) : elem_bytes == 2 && pieces <= 16 && items >= 600000;
+  const bool bf16 = elem_bytes == 2, some = I.bin_rows[0] * 16 >= I.m, many = I.bin_rows[0] * 4 >= I.m;      // rows without nonzeros
+  if (beta != 0.0f && some) {
+    if (pieces <= 8) return items >= (many ? 60000 : 150000);
+    if (pieces <= 16) return items >= (!many ? 450000 : bf16 ? 120000 : 60000) && (many || !bf16 || items <= 6000000);
+    return !bf16 && pieces <= 32 && many && items >= 250000;
+  }
+  if (pieces <= 8) return items >= (pieces <= 4 ? 250000 : bf16 ? 350000 : 600000);
+  if (!bf16 || pieces > 16) return false;
+  return many ? items >= 1000000 : items >= 800000 && items <= (some ? 3000000 : beta != 0.0f ? 2500000 : 1400000);
 }
 
 // Rows all of one length of 5 to 13 that is no multiple of four, k a multiple of 16 bytes and five to sixteen pieces of them a row of B: by rows they take single

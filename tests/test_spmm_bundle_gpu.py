@@ -170,3 +170,23 @@ def test_empty_rows_of_ragged_width_cost_little_more_than_their_bytes(dtype, k):
             best[empties] = min(best[empties], start.elapsed_time(end) / 8)
         b200sp.b200sp_plan_destroy(plan)
     assert best[250_000] < 1.5 * best[0], "%.1f us, without the empty rows %.1f us" % (1e3 * best[250_000], 1e3 * best[0])
+
+
+@pytest.mark.parametrize("dtype,full,holes", [("f32", ((33, 0.0), (63, 1.25), (16, 0.0)), ((36, 1.25), (64, 1.25), (100, 1.25), (128, 1.25), (33, 1.25), (63, 1.25), (17, 1.25), (9, 1.25))),
+                                              ("bf16", ((72, 0.0), (120, 1.25), (128, 0.0), (127, 0.0), (65, 1.25), (126, 0.0), (50, 1.25)), ((72, 1.25), (128, 0.0), (128, 1.25), (33, 0.0), (127, 1.25), (50, 0.0), (34, 1.25)))])
+def test_every_form_that_the_rules_take(dtype, full, holes):
+    """Both matrices just large enough for the widest forms: rows of 1 to 40 and some longer than a region, without empty rows, and with 45 % of them, in long and short runs."""
+    rng = np.random.default_rng(12)
+    n = 30_000
+    lens = rng.integers(1, 40, 52_000)
+    lens[rng.integers(0, 52_000, 30)] = rng.integers(200, 1500, 30)
+    with_holes = rng.integers(1, 40, 100_000) * (rng.random(100_000) < 0.75)
+    with_holes[30_000:57_000] = 0
+    for rows, calls in ((lens, full), (with_holes, holes)):
+        A = gen.random_csr(len(rows), n, rows, seed=3, sort_cols=False)
+        for k, beta in calls:
+            assert by_bundles(A, k, beta, dtype), (k, beta)
+            B, Y0 = rng.standard_normal(n * k).astype(np.float32), rng.standard_normal(A.m * k).astype(np.float32)
+            Y, Y_ref, S = run_spmm(A, B, k, Y0 if beta else None, -0.5 if beta else 1.0, beta, dtype)
+            y0f = Y0 if dtype == "f32" else gen.bf16_to_f32(gen.to_bf16(Y0))
+            assert_within(Y, Y_ref, S, dtype, 1.0, np.abs(beta * y0f.astype(np.float64)).reshape(A.m, k), what="k=%d beta=%g" % (k, beta))

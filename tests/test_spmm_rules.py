@@ -160,3 +160,18 @@ def test_equal_rows_side_by_side_only_where_they_are_faster(dtype, k, length, it
     rows = -(-items // (length + 1))
     stats = dict(info(rows, rows, [0, 0, rows, 0, 0, 0], [0, 0, rows * length, 0, 0, 0], length), min_row_len=length)
     assert b200sp.b200sp_spmm_by_bundles(stats, k, beta, dtype) == taken
+
+
+@pytest.mark.parametrize("stats,dtype,k,beta,taken", [
+    # measured on both sides: BF16, nine to sixteen pieces of a row of B
+    (uneven(124_000, 62_000, 4), "bf16", 128, 0.0, False), (uneven(100_000, 100_000, 8), "bf16", 128, 0.0, True), (uneven(320_000, 160_000, 4), "bf16", 72, 0.0, False),
+    (uneven(320_000, 160_000, 4), "bf16", 72, 1.0, True), (uneven(1_000_000, 500_000, 8), "bf16", 72, 1.0, False), (uneven(60_000, 120_000, 9, 0.12), "bf16", 128, 0.0, False),
+    (uneven(200_000, 240_000, 9, 0.12), "bf16", 128, 0.0, True), (uneven(600_000, 720_000, 9, 0.12), "bf16", 128, 0.0, False), (uneven(1 << 20, 1 << 20, 8, 0.6), "bf16", 128, 0.0, True),
+    # old values of Y and empty rows
+    (uneven(7000, 9000, 14, 0.12), "f32", 32, 1.0, False), (uneven(20_000, 24_000, 9, 0.12), "f32", 32, 1.0, True), (uneven(1 << 13, 1 << 13, 8, 0.6), "f32", 32, 1.0, True),
+    (uneven(20_000, 24_000, 14, 0.12), "f32", 48, 1.0, False), (uneven(60_000, 72_000, 9, 0.12), "f32", 64, 1.0, True), (uneven(1 << 14, 1 << 14, 8, 0.6), "f32", 64, 1.0, True),
+    (uneven(1 << 13, 1 << 13, 8, 0.6), "bf16", 128, 1.0, False), (uneven(1 << 15, 1 << 15, 8, 0.6), "bf16", 128, 1.0, True), (uneven(60_000, 72_000, 9, 0.12), "f32", 128, 1.0, False), (uneven(600_000, 1_200_000, 14, 0.12), "bf16", 72, 1.0, False),
+    (uneven(1 << 15, 1 << 15, 8, 0.6), "f32", 128, 1.0, True), (uneven(1 << 14, 1 << 14, 8, 0.6), "f32", 128, 1.0, False)])
+def test_wide_rows_of_b_side_by_side_only_where_they_are_faster(stats, dtype, k, beta, taken):
+    assert b200sp.b200sp_spmm_by_shares(stats, k, beta, dtype)
+    assert b200sp.b200sp_spmm_by_bundles(stats, k, beta, dtype) == taken
