@@ -112,6 +112,10 @@ int b200sp_spmm_by_bundles(const b200sp_plan_info_t* info, int64_t k, float beta
  * memory, b200sp_spmm_by_shares and b200sp_spmm_by_bundles come before it.  A rule of the host: no device needed. */
 int b200sp_spmm_wide_pieces(const b200sp_plan_info_t* info, int64_t k, int sms, int64_t l2_bytes);
 
+/* The sizes with which SpMV of a CSC matrix by products first tries its places on a device with that many SMs: entries of a tile and nonzeros of a bucket (host
+ * pointers).  Between 25 * 1024 and 32 * 1024 nonzeros per SM buckets of 4096 take the place of larger ones that do not apply.  A rule of the host: no device needed. */
+int b200sp_csc_sizes(int64_t m, int64_t nnz, int sms, int* tile, int* bucket);
+
 /* The plan pass's split points as it takes them from the rows: out[t] = row ends before merge item t * items of the merge of the m row ends with the
  * nnz nonzeros, for t = 0 .. ceil((m + nnz) / items).  `items` a power of two from 32 on, or anything from 32 to 128 while m + nnz < 2^29; row_ptr (m + 1
  * ascending entries) and out are host pointers.  Arithmetic of the host: no device needed. */

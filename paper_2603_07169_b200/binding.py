@@ -21,7 +21,7 @@ EXPORTS = (
     "spmv_csr", "spmm_csr", "b200sp_plan_create", "b200sp_plan_destroy", "b200sp_plan_info", "b200sp_spmv",
     "b200sp_spmm", "spmv_csr_host", "spmm_csr_host", "b200sp_validate_csr", "b200sp_cache_clear",
     "b200sp_status_string", "b200sp_last_cuda_error", "b200sp_version", "b200sp_checked_build", "b200sp_launch_count", "b200sp_set_option", "b200sp_get_option",
-    "b200sp_check", "b200sp_cache_drop", "spmv_csr_noalloc", "b200sp_noalloc_max_items", "b200sp_probe_gather", "b200sp_probe_gather_ex", "b200sp_probe_stream", "b200sp_probe_lines", "b200sp_probe_spmv_gather", "b200sp_spmv_naive", "b200sp_spmm_naive", "spmv_coo", "spmm_coo", "spmv_ell", "spmm_ell", "spmv_csc", "spmm_csc", "spmv_csr_vec_host", "b200sp_spmm_by_shares", "b200sp_spmm_by_bundles", "b200sp_spmm_wide_pieces", "b200sp_split_points",
+    "b200sp_check", "b200sp_cache_drop", "spmv_csr_noalloc", "b200sp_noalloc_max_items", "b200sp_probe_gather", "b200sp_probe_gather_ex", "b200sp_probe_stream", "b200sp_probe_lines", "b200sp_probe_spmv_gather", "b200sp_spmv_naive", "b200sp_spmm_naive", "spmv_coo", "spmm_coo", "spmv_ell", "spmm_ell", "spmv_csc", "spmm_csc", "spmv_csr_vec_host", "b200sp_spmm_by_shares", "b200sp_spmm_by_bundles", "b200sp_spmm_wide_pieces", "b200sp_csc_sizes", "b200sp_split_points",
 )
 
 
@@ -116,6 +116,8 @@ def lib() -> ctypes.CDLL:
         L.b200sp_spmm_by_bundles.restype = i32
         L.b200sp_spmm_wide_pieces.argtypes = [ctypes.POINTER(PlanInfo), i64, i32, i64]
         L.b200sp_spmm_wide_pieces.restype = i32
+        L.b200sp_csc_sizes.argtypes = [i64, i64, i32, p, p]
+        L.b200sp_csc_sizes.restype = i32
         L.b200sp_split_points.argtypes = [i64, i64, p, i32, p]
         L.b200sp_split_points.restype = i32
         L.b200sp_check.argtypes = [p]
@@ -493,6 +495,13 @@ def b200sp_spmm_by_bundles(info: dict, k, beta, dtype) -> bool:
 def b200sp_spmm_wide_pieces(info: dict, k, sms, l2_bytes) -> bool:
     """Whether BF16 SpMM by rows on a matrix with these row statistics reads B, aligned to 32 bytes, in pieces of 32 bytes."""
     return bool(lib().b200sp_spmm_wide_pieces(ctypes.byref(_plan_info(info)), k, sms, l2_bytes))
+
+
+def b200sp_csc_sizes(m, nnz, sms):
+    """(entries of a tile, nonzeros of a bucket) of CSC SpMV by products."""
+    tile, bucket = ctypes.c_int(), ctypes.c_int()
+    _ck(lib().b200sp_csc_sizes(m, nnz, sms, ctypes.byref(tile), ctypes.byref(bucket)), "b200sp_csc_sizes")
+    return tile.value, bucket.value
 
 
 def b200sp_split_points(m, nnz, row_ptr, items, out):

@@ -137,6 +137,14 @@ int b200sp_spmm_by_bundles(const b200sp_plan_info_t* info, int64_t k, float beta
   return info && k > 1 && spmm_side_by_side(*info, k, dtype == B200SP_F32 ? 4 : 2, beta);
 }
 
+int b200sp_csc_sizes(int64_t m, int64_t nnz, int sms, int* tile, int* bucket) {
+  if (m < 0 || nnz < 0 || sms <= 0 || !tile || !bucket) return B200SP_ERR_INVALID_ARG;
+  const CscSizes s = csc_sizes(m, nnz, sms);
+  *tile = s.tile;
+  *bucket = 1 << s.shift;
+  return B200SP_OK;
+}
+
 int b200sp_spmm_wide_pieces(const b200sp_plan_info_t* info, int64_t k, int sms, int64_t l2_bytes) {
   return info && sms > 0 && k >= 64 && k % 16 == 0 && g_opt.spmm_stage_a == 2 && spmm_wide_pieces(*info, k, sms, l2_bytes);
 }

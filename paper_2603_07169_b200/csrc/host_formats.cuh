@@ -167,30 +167,34 @@ static int64_t csc_most_bucket_rows(int64_t nnz, float beta) {
 }
 
 
-// The places of the products of csc_kernels.cuh; leaves e->prod_block null where they do not apply, and while the stream is captured
-// (their limits are read back).  Synchronises the stream.
+// Entries of a tile and, as a power of two, nonzeros of a bucket of the products.
 // Sizes: below 7.3 M nonzeros tiles of 2048, 4096 or 8192 entries, so that every SM gets several that overlap, and buckets of as many nonzeros (8192 from 3.8 M
 // on: 4.3 M 24.0 / 21.5 us, 4.7 M 25.3 / 22.3 us); else one tile of 24576 .. 32768 entries per SM and round (96 .. 128 KB of products), the size that leaves
 // the least of the last round idle (4.9 M nonzeros in two rounds of 24576 31.3 us, in tiles of 8192 26.5 us; 6.9 M 40.9 / 35.6 us; but 8 M in two
 // rounds of 28672 38.9 us, in tiles of 8192 43.7 us), and buckets of 8192 nonzeros, 16384 above 2^25.  A run (a tile's products for one bucket) then averages
 // tile * C / nnz = 3.5 .. 55 words: 2^24 nonzeros take 78 us, 81 us with tiles of 32768, 84 us with two tiles of 16384 per SM, 90 us with buckets of 16384.
-// Above 2^26 nonzeros, with a row of more than kCscSlack nonzeros, a tile over more than 65536 columns or a bucket of too many rows (most_rows), SpMV takes
-// the CSR kernels.
-static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr, const int32_t* row_idx, int64_t most_rows,
-                            cudaStream_t stream, DeviceInfo* dev) {
-  std::lock_guard<std::mutex> lock(g_csc_build);
-  if (e->prod_tried || e->bucket_rows > most_rows || stream_captures(stream)) return B200SP_OK;
-  if (nnz <= 0 || nnz > ((int64_t)1 << 26)) { e->prod_tried = true; return B200SP_OK; }
-  const int64_t sms = dev->sms;
-  int tile = nnz < sms * 4 * 2048 ? 2048 : nnz < sms * 8 * 4096 ? 4096 : 8192;
+// Below 4.8 M buckets of 8192 only where a row has one nonzero or more on average, two below 4.2 M: what a CTA walks of empty rows doubles with its bucket (buckets of
+// 4096 / 8192: 3.9 M nonzeros in as many rows 31.9 / 33.9 us, in 7.8 M rows 45.8 / 49.4 us, 4.3 M in 8.6 M rows 50.1 / 51.1 us; but 4.8 M in as many rows 39.6 / 37.0 us).
+struct CscSizes { int tile, shift; };
+static CscSizes csc_sizes(int64_t m, int64_t nnz, int64_t sms) {
+  CscSizes s;
+  s.tile = nnz < sms * 4 * 2048 ? 2048 : nnz < sms * 8 * 4096 ? 4096 : 8192;
   if (nnz >= sms * 6 * 8192) {
     int64_t best = INT64_MAX;
     for (int t : {32768, 28672, 24576}) {
       const int64_t time = (((nnz + t - 1) / t + sms - 1) / sms) * t;     // rounds of one tile per SM
-      if (time < best) { best = time; tile = t; }
+      if (time < best) { best = time; s.tile = t; }
     }
   }
-  const int shift = nnz < sms * 4 * 2048 ? 11 : nnz < sms * 25 * 1024 ? 12 : nnz <= ((int64_t)1 << 25) ? 13 : 14;
+  const bool larger = nnz >= sms * 8 * 4096 || (nnz >= sms * 25 * 1024 && nnz >= (nnz >= sms * 28 * 1024 ? m : 2 * m));
+  s.shift = nnz < sms * 4 * 2048 ? 11 : !larger ? 12 : nnz <= ((int64_t)1 << 25) ? 13 : 14;
+  return s;
+}
+
+// The places of the products of csc_kernels.cuh with tiles and buckets of the given sizes; leaves e->prod_block null where they do not apply: a row of more than
+// kCscSlack nonzeros, a tile over more than 65536 columns or a bucket of more than most_rows rows.  Synchronises the stream.
+static int csc_places(CscEntry* e, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr, const int32_t* row_idx, int tile, int shift, int64_t most_rows,
+                      cudaStream_t stream, DeviceInfo* dev) {
   const int tiles = (int)((nnz + tile - 1) / tile), buckets = (int)(((nnz - 1) >> shift) + 1), cap = (1 << shift) + kCscSlack;
   if (buckets > kCscMaxBuckets) { e->prod_tried = true; return B200SP_OK; }
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
@@ -199,7 +203,7 @@ static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, cons
                o_brow = o_shift + up((size_t)tiles * buckets * 4), o_bstart = o_brow + up((size_t)(buckets + 1) * 4), o_tcol = o_bstart + up((size_t)(buckets + 1) * 4), o_prod = o_tcol + up((size_t)tiles * 4),
                total = o_prod + up(nz * 4);
   char* blk = nullptr;
-  int rc = pool_alloc(dev, (void**)&blk, total, stream);
+  const int rc = pool_alloc(dev, (void**)&blk, total, stream);
   if (rc != B200SP_OK) return rc;
   auto fail = [&](int code) { cudaFreeAsync(blk, stream); cudaStreamSynchronize(stream); return code; };
 #define CUP(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) return fail(cuda_fail(e_, #call)); } while (0)
@@ -242,6 +246,21 @@ static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, cons
   e->prod_block = blk;
   e->prod_tried = true;
   return B200SP_OK;
+}
+
+// The same with the sizes that csc_sizes names, and with buckets of 4096 below 4.8 M nonzeros where those of 8192 do not apply or hold more rows than pay with
+// beta != 0 (4.8 M nonzeros in 12 M rows, beta = 0.5 82 / 113 us by products / by the CSR kernels).  Nothing is done while the stream is captured (the limits are read
+// back).  Above 2^26 nonzeros, and where the places do not apply, SpMV takes the CSR kernels.
+static int csc_product_part(CscEntry* e, int64_t m, int64_t n, int64_t nnz, const int32_t* col_ptr, const int32_t* row_idx, int64_t most_rows,
+                            cudaStream_t stream, DeviceInfo* dev) {
+  std::lock_guard<std::mutex> lock(g_csc_build);
+  if (e->prod_tried || e->bucket_rows > most_rows || stream_captures(stream)) return B200SP_OK;
+  if (nnz <= 0 || nnz > ((int64_t)1 << 26)) { e->prod_tried = true; return B200SP_OK; }
+  const CscSizes sizes = csc_sizes(m, nnz, dev->sms);
+  const bool smaller = sizes.shift == 13 && nnz < (int64_t)dev->sms * 8 * 4096;
+  int rc = csc_places(e, m, n, nnz, col_ptr, row_idx, sizes.tile, sizes.shift, smaller ? csc_most_bucket_rows(nnz, 1.0f) : most_rows, stream, dev);
+  if (rc == B200SP_OK && smaller && !e->prod_block) rc = csc_places(e, m, n, nnz, col_ptr, row_idx, sizes.tile, 12, most_rows, stream, dev);
+  return rc;
 }
 
 // Gives back the memory of the places, in stream order (the calls of a pattern do not overlap); the next SpMV builds them again.

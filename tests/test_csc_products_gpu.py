@@ -199,3 +199,76 @@ def test_csc_products_of_the_sizes_between(n):
     y_ref, S = oracle.spmm_csc(n, n, 1, cp, ri, va, x, None, 1.0, 0.0, "f32")
     assert_within(to_host(y, "f32"), y_ref[:, 0], S[:, 0], "f32")
     b200sp.b200sp_cache_clear()
+
+
+def around_the_limits():
+    """(number of nonzeros over that of SMs, nonzeros a row, tile, bucket): the last and the first size of each pair of tile and bucket."""
+    return [(25 * 1024, 16, 4096, 8192), (8 * 4096 - 16, 16, 4096, 8192), (8 * 4096, 16, 8192, 8192), (6 * 8192 - 16, 16, 8192, 8192), (6 * 8192, 16, 24576, 8192), (6 * 8192 + 64, 16, 28672, 8192),
+            (69_000, 16, 24576, 8192), (25 * 1024 - 16, 16, 4096, 4096), (27_000, 1, 4096, 4096)]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("per_sm,per_row,tile,bucket", around_the_limits())
+def test_each_pair_of_tile_and_bucket_against_oracle(per_sm, per_row, tile, bucket, dtype):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    m = per_sm * sms // per_row
+    assert b200sp.b200sp_csc_sizes(m, m * per_row, sms) == (tile, bucket)
+    A = gen.uniform_rows(m, m, per_row, 7)
+    rng = np.random.default_rng(3)
+    cp, ri, va = gen.csr_to_csc(A)
+    v_s, x_s, y0_s = store(va, dtype), store(rng.standard_normal(m).astype(np.float32), dtype), store(rng.standard_normal(m).astype(np.float32), dtype)
+    d = [to_dev(a) for a in (cp, ri, v_s, x_s)]
+    outs = []
+    for _ in range(2):
+        y = to_dev(y0_s).clone()
+        b200sp.spmv_csc(m, m, A.nnz, d[0], d[1], d[2], d[3], y, -0.5, 1.25, dtype)
+        outs.append(to_host(y, dtype))
+        b200sp.b200sp_cache_drop(d[0])                            # planned again: the same sums in the same order
+    assert np.array_equal(outs[0], outs[1])
+    y_ref, S = oracle.spmm_csc(m, m, 1, cp, ri, v_s, x_s, y0_s, -0.5, 1.25, dtype)
+    y0f = y0_s if dtype == "f32" else gen.bf16_to_f32(y0_s)
+    assert_within(outs[0], y_ref[:, 0], S[:, 0], dtype, 1.0, np.abs(1.25 * y0f.astype(np.float64)))
+    b200sp.b200sp_cache_clear()
+
+
+@needs_plain_build
+@pytest.mark.parametrize("first,second", [(0.0, 0.5), (0.5, 0.0)])
+def test_larger_buckets_do_not_keep_a_pattern_from_its_products(first, second):
+    """4.4 M nonzeros in 200,000 rows and 20,000 empty ones in one run: whichever bucket holds the run has more rows than pay with beta != 0, so buckets of 4096 are
+    tried as well, and taken with beta == 0.  And 4 M in 9 M rows, where the smaller buckets are taken as before there were larger ones."""
+    rng = np.random.default_rng(9)
+    n = 300_000
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for lens in (np.repeat([22, 0, 22], [150_000, 20_000, 50_000]), (rng.random(9_000_000) < 0.45).astype(np.int64)):
+        A = gen.random_csr(len(lens), n, lens, seed=3, sort_cols=True)
+        assert sms * 25 * 1024 <= A.nnz < sms * 8 * 4096
+        cp, ri, va = gen.csr_to_csc(A)
+        x, y0 = rng.standard_normal(n).astype(np.float32), rng.standard_normal(A.m).astype(np.float32)
+        d = [to_dev(a) for a in (cp, ri, va, x)]
+        for beta in (first, second):
+            y = to_dev(y0).clone()
+            b200sp.spmv_csc(A.m, n, A.nnz, d[0], d[1], d[2], d[3], y, 1.0, beta, "f32")
+            y_ref, S = oracle.spmm_csc(A.m, n, 1, cp, ri, va, x, y0 if beta else None, 1.0, beta, "f32")
+            assert_within(to_host(y, "f32"), y_ref[:, 0], S[:, 0], "f32", 1.0, np.abs(beta * y0.astype(np.float64)))
+        b200sp.b200sp_cache_clear()
+
+
+@pytest.mark.parametrize("m", [12_000_000])
+def test_many_rows_and_few_nonzeros_keep_the_time_they_had(m):
+    """4.8 M nonzeros in 12 M rows, beta != 0: 82 us by products in buckets of 4096; with larger buckets alone the CSR kernels took the call, 113 us."""
+    nnz, n = 4_800_000, 1 << 20
+    g = torch.Generator("cuda").manual_seed(3)
+    key = (torch.randint(0, n, (nnz,), generator=g, device="cuda") * m + torch.randint(0, m, (nnz,), generator=g, device="cuda")).sort().values
+    col, row = key // m, (key % m).int()
+    cp = torch.searchsorted(col, torch.arange(n + 1, device="cuda")).int()
+    vals, x, y = (torch.randn(k, generator=g, device="cuda") for k in (nnz, n, m))
+    y0 = y.clone()
+    call = lambda: b200sp.spmv_csc(m, n, nnz, cp, row, vals, x, y, 1.0, 0.5, "f32")  # noqa: E731
+    call()
+    ref = (0.5 * y0.double()).index_add_(0, row.long(), vals.double() * x.double()[col])
+    S = (0.5 * y0.double()).abs().index_add_(0, row.long(), (vals.double() * x.double()[col]).abs())
+    assert float(((y.double() - ref).abs() / (1e-5 * S + 1e-30)).max()) <= 1.0
+    before = b200sp.b200sp_launch_count()
+    call()
+    assert b200sp.b200sp_checked_build() or b200sp.b200sp_launch_count() - before == 2      # the products and the sums
+    b200sp.b200sp_cache_clear()
