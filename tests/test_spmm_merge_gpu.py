@@ -146,3 +146,24 @@ def test_old_values_cost_no_more_than_their_bytes_and_a_wait(dtype, ks):
     finally:
         b200sp.b200sp_set_option("spmm_flat", 2)
         b200sp.b200sp_cache_clear()
+
+
+@pytest.mark.parametrize("dtype,k", [("bf16", 100), ("bf16", 130), ("bf16", 256), ("f32", 66), ("f32", 256)])
+def test_several_shares_to_a_warp(dtype, k):
+    """Shares of 128 items, several to a warp, at widths that stay by shares on a matrix of this size."""
+    lens = matrices()["large"]
+    rng = np.random.default_rng(k)
+    n = 40_000
+    A = gen.random_csr(len(lens), n, lens, seed=5, sort_cols=False)
+    stats = dict(m=A.m, n=n, nnz=A.nnz, min_row_len=0, max_row_len=59, bin_rows=[2000, 8000, 56_000, 54_000, 0, 0], bin_nnz=[0, 20_000, 1_000_000, A.nnz - 1_020_000, 0, 0])
+    b200sp.b200sp_set_option("spmm_flat", 1)
+    try:
+        assert not any(b200sp.b200sp_spmm_by_bundles(stats, k, beta, dtype) for beta in (0.0, 1.25))
+        B, Y0 = rng.standard_normal(n * k).astype(np.float32), rng.standard_normal(A.m * k).astype(np.float32)
+        Y, Y_ref, S = run_spmm(A, B, k, None, 1.0, 0.0, dtype)
+        assert_within(Y, Y_ref, S, dtype)
+        Y, Y_ref, S = run_spmm(A, B, k, Y0, -0.5, 1.25, dtype)
+        y0f = Y0 if dtype == "f32" else gen.bf16_to_f32(gen.to_bf16(Y0))
+        assert_within(Y, Y_ref, S, dtype, 1.0, np.abs(1.25 * y0f.astype(np.float64)).reshape(A.m, k))
+    finally:
+        b200sp.b200sp_set_option("spmm_flat", 2)
