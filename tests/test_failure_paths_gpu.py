@@ -150,6 +150,34 @@ def test_spmm_by_shares_without_its_scratch_goes_by_rows(dtype):
 
 
 @needs_plain_build
+@pytest.mark.parametrize("dtype,k,rows,length,beta,allocations", [
+    ("bf16", 50, 60_000, None, 0.0, 2), ("f32", 33, 60_000, None, 0.5, 2),                # the padded copy of B, what tiles leave unfinished
+    ("bf16", 64, 60_000, None, 0.0, 1), ("bf16", 40, 150_000, 7, 0.5, 1),                 # the latter; rows of one length go by rows then
+    ("bf16", 8, 700_000, None, 0.0, 2), ("bf16", 40, 1_200_000, 7, 0.0, 2)])              # above 2^23 items the shares first
+def test_spmm_side_by_side_without_one_of_its_allocations(dtype, k, rows, length, beta, allocations):
+    rng = np.random.default_rng(4)
+    n = 30_000
+    if length:
+        A = gen.uniform_rows(rows, n, length, 2)
+    else:
+        lens = rng.integers(1, 24, rows)
+        lens[:2] = 700, 1500
+        A = gen.random_csr(rows, n, lens, seed=k, sort_cols=True)
+    B, vals, Y0 = (store(a, dtype) for a in (rng.standard_normal(n * k).astype(np.float32), A.vals, rng.standard_normal(A.m * k).astype(np.float32)))
+    d = [to_dev(a) for a in (A.row_ptr, A.col_idx, vals, B)]
+    some = np.sort(rng.choice(A.m, 5000, replace=False))
+    ref, S = oracle.spmm_csr(A.m, n, k, A.row_ptr, A.col_idx, vals, B, Y0 if beta else None, 1.0, beta, dtype, rows=some, nthreads=oracle.max_threads())
+    y0f = (Y0 if dtype == "f32" else gen.bf16_to_f32(Y0)).astype(np.float64).reshape(A.m, k)[some]
+    for nth in range(1, allocations + 1):
+        plan = b200sp.b200sp_plan_create(A.m, n, A.nnz, d[0])
+        assert b200sp.b200sp_spmm_by_bundles(b200sp.b200sp_plan_info(plan), k, beta, dtype)
+        Y = to_dev(Y0).clone()
+        failing(nth, lambda: b200sp.b200sp_spmm(plan, k, d[1], d[2], d[3], Y, 1.0, beta, dtype))
+        assert_within(to_host(Y, dtype).reshape(A.m, k)[some], ref, S, dtype, 1.0, np.abs(beta * y0f), what="allocation %d" % nth)
+        b200sp.b200sp_plan_destroy(plan)
+
+
+@needs_plain_build
 def test_csc_without_memory_for_one_of_its_parts():
     """12 bytes per nonzero were enough for both operations: SpMV does without its places, SpMM takes their memory back."""
     rng = np.random.default_rng(7)
