@@ -190,3 +190,22 @@ def test_every_form_that_the_rules_take(dtype, full, holes):
             Y, Y_ref, S = run_spmm(A, B, k, Y0 if beta else None, -0.5 if beta else 1.0, beta, dtype)
             y0f = Y0 if dtype == "f32" else gen.bf16_to_f32(gen.to_bf16(Y0))
             assert_within(Y, Y_ref, S, dtype, 1.0, np.abs(beta * y0f.astype(np.float64)).reshape(A.m, k), what="k=%d beta=%g" % (k, beta))
+
+
+@pytest.mark.parametrize("k,beta,lens", [
+    (32, 0.5, np.concatenate([np.repeat([0, 3], 5000), [30_000], np.full(200, 32), np.full(200, 33), np.zeros(3000, np.int64)])),     # regions of 24 items, the shortest
+    (16, 0.0, np.concatenate([np.repeat([2, 5], 9000), [150_000], np.full(200, 33), np.full(400, 32), np.full(30, 87)])),             # just above the least number of items
+    (64, 0.5, np.concatenate([np.repeat([0, 9], 60_000), [400_000], np.full(100, 1000)]))],
+    ids=["regions_of_24", "least_items", "long_regions"])
+def test_positive_data_stays_below_the_literal_fp32_bound(k, beta, lens):
+    """All-positive data, where rounding errors do not cancel: a row over hundreds of tiles, pieces at the limit of the cooperative ones, full regions.  A row over T tiles adds at
+    most 128 products in a chain, five levels of a tree, eight partial sums and a chain of T / 16 trees of 16: 600 tiles are 183 additions, 0.36 of the literal bound if all erred
+    the same way."""
+    n = 20_000
+    A = gen.random_csr(len(lens), n, lens, seed=8, allow_dup=True)
+    rng = np.random.default_rng(2)
+    A.vals[:] = rng.random(A.nnz).astype(np.float32) + 0.01
+    B = rng.random(n * k).astype(np.float32) + 0.01
+    assert by_bundles(A, k, beta, "f32")
+    Y, Y_ref, S = run_spmm(A, B, k, np.zeros(A.m * k, np.float32), 1.0, beta, "f32")
+    assert assert_within(Y, Y_ref, S, "f32") < 0.5
