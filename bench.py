@@ -915,7 +915,7 @@ def main():
                     b200sp.b200sp_set_option("x_l2_window", 0)
                     b200sp.b200sp_cache_clear()
                     torch.cuda.empty_cache()
-        # SpMM on the power-law matrix (not one of the five configurations): the nnz-balanced kernel that the plan picks for uneven rows
+        # SpMM on the power-law matrix (not one of the five configurations): the nnz-balanced kernels that the plan picks for uneven rows
         try:
             cache = {}
             wpl = gen.workload("c3k64")
@@ -927,7 +927,7 @@ def main():
                     "algorithmic_bytes": r["algorithmic_bytes"], "nnz": r["nnz"], "copies": r["copies"],
                     "cusparse_ms": round(r["cusparse_ms"], 5) if isinstance(r["cusparse_ms"], float) else r["cusparse_ms"],
                     "line_read_bound_ms": round(wpl.A.nnz * 64 * (4 if dt == "f32" else 2) / lr * 1e3, 5),
-                    "note": "R-MAT scale 22 pattern (61 % empty rows, rows up to 57 k) times a dense 2^22 x 64 B: spmm_merge_kernel"}
+                    "note": "R-MAT scale 22 pattern (61 % empty rows, rows up to 57 k) times a dense 2^22 x 64 B: " + ("spmm_merge_kernel" if dt == "f32" else "spmm_bundle_kernel")}
                 del r
                 b200sp.b200sp_cache_clear()
                 torch.cuda.empty_cache()

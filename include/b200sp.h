@@ -42,7 +42,10 @@
  *  - Device memory the library needs (plan scratch, the staging buffers of the "host" entry
  *    points, and per-call scratch for SpMM, taken and returned in the order of `stream`: where SpMM goes by
  *    equal shares (uneven rows, or k > 16 that is no multiple of 16 bytes) 8 bytes per dense column and
- *    256 .. 4096 rows + nonzeros, the fewer the smaller the matrix (without that memory it goes by rows); on matrices with so few
+ *    256 .. 4096 rows + nonzeros, the fewer the smaller the matrix (without that memory it goes by rows); where it has warps walk several rows side
+ *    by side (narrow rows of B, and larger matrices with rows all of one odd length) the same for 192 .. 2560 rows + nonzeros, and with k no multiple
+ *    of 16 bytes a copy of B in rows of whole 128-byte lines, n * 128 * ceil(k * bytes per value / 128) bytes (without that memory it goes by equal shares, or
+ *    by rows); on matrices with so few
  *    columns that a slice of B is kept in shared memory a re-laid copy of A, about (2 + bytes per
  *    value) * (nnz + 3 m) bytes, plus 8 m bytes kept with the plan) comes from a
  *    stream-ordered memory pool of its own, one per device, created at first use.  The pool keeps up to 1 GiB of freed memory for the next call (option "pool_keep_mb",
@@ -116,7 +119,7 @@ int spmm_csr(int64_t m, int64_t n, int64_t nnz, int64_t k, const int32_t* row_pt
  * (a merge-path search over rows + nonzeros), all on the device and in one launch.  From the same statistics it decides
  * whether SpMM gives every row to a group of eight lanes (even rows) or cuts rows + nonzeros into equal shares per warp
  * (uneven rows: many empty rows, a share of the nonzeros in rows of more than 128, or a longest row far above the mean; with few
- * columns only where the rows differ enough for it to pay).  What only some SpMM kernels need is
+ * columns only where the rows differ enough for it to pay), or has a warp walk several rows at a time (narrow rows of B).  What only some SpMM kernels need is
  * built on the first SpMM call that uses them, in stream order: the lists of rows of 129-1024 and of more than 1024 nonzeros,
  * the shares of large matrices, and the order of the rows by length that SpMM uses when A has so few columns that a slice
  * of B is kept in shared memory.

@@ -26,7 +26,9 @@ extern "C" {
  *   "spmm_flat"      SpMM by equal shares of rows + nonzeros per warp instead of by rows (nnz-balanced, with carries between warps and
  *                    CTAs): 1 = always, 0 = never, 2 = when the rows are uneven (5 % or more of the nonzeros in rows longer than
  *                    128, a quarter or more of the rows empty, or a longest row far above the mean; with few columns only where the
- *                    rows differ enough, b200sp_spmm_by_shares) or k > 16 is no multiple of 16 bytes (default)
+ *                    rows differ enough, b200sp_spmm_by_shares) or k > 16 is no multiple of 16 bytes (default).  1 and 2: with
+ *                    narrow rows of B and enough rows + nonzeros a warp walks several rows side by side
+ *                    (b200sp_spmm_by_bundles), else one nonzero after the other; 2 only: rows all of one odd length as well
  *   "spmm_stage_a"   the k-sliced SpMM kernel's warps first copy their rows' (col, val) pairs into shared memory: 1 = yes, 0 = no,
  *                    2 = for BF16 storage only (default: measured 5-6 % faster there and 2-3 % slower for FP32), and there a kernel
  *                    with four lanes a row and 32 bytes of B per load instead, without staging, where it is faster: k a multiple
@@ -102,7 +104,7 @@ int b200sp_get_option(const char* name, int* value);
 int b200sp_spmm_by_shares(const b200sp_plan_info_t* info, int64_t k, float beta, int dtype);
 
 /* 1 if SpMM has its warps walk several rows of about equal length side by side, 16 bytes of B per lane: of the calls that go by shares those with
- * narrow rows of B (k a multiple of 16 bytes, or odd widths through a padded copy of B, which takes up to 128 n more bytes than B for the call), and rows all of
+ * narrow rows of B (k a multiple of 16 bytes, or odd widths through a copy of B in rows of whole 128-byte lines where B is read often enough to pay for it), and rows all of
  * one short length that is no multiple of four (these only while "spmm_sliced", "spmm_flat", "spmm_stage_a" and "spmm_ranges" have their default values).  Larger
  * matrices only; B kept in shared memory comes before it.  0 if not, under the present switches.  A rule of the host: no device needed. */
 int b200sp_spmm_by_bundles(const b200sp_plan_info_t* info, int64_t k, float beta, int dtype);

@@ -15,7 +15,8 @@ namespace b200sp {
 
 constexpr int kBundleLong = 32;      // longer pieces of rows are split over the lane groups
 // Resident CTAs per SM: 4 loads of 16 bytes per lane in flight, and more warps rather than more loads (R-MAT 2^22, k = 64 FP32: 968 us with 4 CTAs, 824 with 5, 797 with 6;
-// 8 loads and 3 CTAs 990 us).  BF16 has eight sums a lane and spills at six.
+// 8 loads and 3 CTAs 990 us).  Some forms spill a little for it (FP32 at six with beta == 0 and 8 or 16 lanes 20 bytes stored and up to 64 loaded a thread, BF16 at five
+// with narrow ragged rows up to 32 / 48); BF16, with eight sums a lane, spills much more at six.
 template <typename T> constexpr int kBundleCtas = sizeof(T) == 4 ? 6 : 5;
 // Most merge items per warp: no lane adds more than 128 products of a long piece in one chain, and the shared memory of the resident warps leaves L1 room
 // for what is in flight (320 items: 27 KB a CTA).
